@@ -908,36 +908,434 @@ static constexpr long long RQ_MAX = 1 << 16;
 // tuning knob (gqf_region_groups, 8 by default).
 
 
-// read-only: per region, the slots its groups add, and whether the data they
-// push stays before the region after next (two slots of margin) and before
-// the table's end
+// ---------------------------------------------------------------------------
+// One warp per region (batches that cannot fill the chip with threads). A
+// run's group grows or shrinks one slot at a time; opening a slot at p moves
+// the slots from p to the first empty slot E right by one, closing one moves
+// the slots up to the next gap left. Either way the remainders of the span,
+// its run-end words and its offsets are each moved by all lanes at once:
+//   remainders [p, E) -> [p + 1, E]; run-end bits likewise; the offset of
+//   every block j with x <= 64 j < E changes by one (x: the group's quotient;
+//   every run that such a block's offset names ends inside the span).
+// The span's end is found by one load per lane: block j's record alone (its
+// offset covers all runs of quotients <= 64 j) says where its gaps are.
+// Bound by the latency of the dependent loads of an update: about 8 of them
+// instead of some 4 per run of the cluster. 1000 inserts and 1000 removes at
+// 85 % of 2^20 slots: 938 + 608 us with a thread per region.
+// ---------------------------------------------------------------------------
+// slots that c more copies of fingerprint fp take, or -1 on an inconsistent table
 template <int R>
-__global__ void gqf_insert_precheck(GView g, const uint64_t *__restrict__ ufp, const uint32_t *__restrict__ ustart,
-                                    const uint32_t *__restrict__ rlo, uint64_t nreg, uint64_t rq,
-                                    unsigned long long *bad)
+__device__ __forceinline__ int gv_slots_added(const GView &g, uint64_t fp, uint64_t c, long long r0)
 {
+    long long s, e, p;
+    uint64_t c_old;
+    uint32_t ol;
+    if (!gv_locate<R>(g, (long long)(fp >> R), (uint32_t)(fp & ((1ull << R) - 1ull)), r0, s, e, p, c_old, ol)) return -1;
+    return (int)enc_len(c_old + c, R) - (int)ol;
+}
+
+// first b in [lo, 64] (lo >= 1) such that every run of a quotient below
+// 64 j + b ends below it, from block j's record; 65 when there is none
+__device__ __forceinline__ int gv_block_gap(const Meta &m, int lo)
+{
+    const unsigned off = m.off;
+    if (off >= 64) return 65;
+    const unsigned long long occ = m.occ & ~1ull;  // the offset covers bit 0
+    const unsigned long long rend = off == 63 ? 0ull : m.rend & (~0ull << (off + 1));
+    int b = lo > (int)off + 1 ? lo : (int)off + 1;
+    while (b <= 64) {
+        const unsigned long long below = b == 64 ? ~0ull : (1ull << b) - 1ull;
+        int open = __popcll(occ & below) - __popcll(rend & below);  // runs begun and not ended below b
+        if (open <= 0) return b;
+        unsigned long long t = rend & ~below;
+        while (--open && t) t &= t - 1;
+        if (!t) break;
+        b = __ffsll((long long)t);  // one past the run end that closes them
+    }
+    return 65;
+}
+
+// first empty slot of block j at or after 64 j + lo (lo >= 0), or 64
+__device__ __forceinline__ int gv_block_empty(const Meta &m, int lo)
+{
+    if (lo <= 0) {
+        if (m.off == 0 && !(m.rend & 1ull)) return 0;
+        lo = 1;
+    }
+    while (lo < 64) {
+        const int b = gv_block_gap(m, lo);
+        if (b >= 64) break;
+        if (!((m.occ >> b) & 1ull)) return b;
+        lo = b + 1;  // a run starts there, at its home slot
+    }
+    return 64;
+}
+
+// first empty slot >= lo (EMPTY) or first gap >= lo, in the blocks [jb, jend)
+// (jb at most lo's block); -1 when there is none. All lanes call it and get
+// the result; `m` keeps the record of block jb + lane of the last round.
+template <bool EMPTY>
+__device__ __forceinline__ long long gvw_find(const GView &g, long long lo, long long &jb, long long jend, Meta &m)
+{
+    const int lane = threadIdx.x & 31;
+    for (; jb < jend; jb += 32) {
+        const long long j = jb + lane;
+        int b = 99;
+        m.occ = m.rend = 0;
+        m.off = 0;
+        if (j < jend) {
+            m.occ = g.meta[j].occ;
+            m.rend = g.meta[j].rend;
+            m.off = g.meta[j].off;
+            const long long l = lo - 64 * j;
+            if (l <= 64) b = EMPTY ? gv_block_empty(m, l > 0 ? (int)l : 0) : gv_block_gap(m, l > 1 ? (int)l : 1);
+        }
+        const unsigned hit = __ballot_sync(0xffffffffu, b <= (EMPTY ? 63 : 64));
+        if (hit) {
+            const int src = __ffs(hit) - 1;
+            return 64 * (jb + src) + __shfl_sync(0xffffffffu, b, src);
+        }
+    }
+    return -1;
+}
+
+static constexpr int GVW_U = 8;  // slots a lane moves per round
+
+// The run-end words and offsets of a span move one slot: right (OPEN: [p, E)
+// to [p + 1, E]) or left ((p, E] to [p, E - 1]); bit p (OPEN) or E is then 0,
+// and the offset of every block j with x <= 64 j < E changes by one. m: the
+// record of block jb + lane, as gvw_find read it.
+template <bool OPEN>
+__device__ __forceinline__ void gvw_shift_meta(const GView &g, long long x, long long p, long long E, long long jb,
+                                               const Meta &m)
+{
+    const int lane = threadIdx.x & 31;
+    const long long w0 = p >> 6, w1 = E >> 6;
+    // the bits of word w after the move, from its own and its neighbour's
+    auto moved_word = [&](long long w, unsigned long long bits, unsigned long long next) {
+        unsigned long long mask = ~0ull, moved = OPEN ? (bits << 1) | (next >> 63) : (bits >> 1) | (next << 63);
+        if (w == w1) {
+            mask &= ~0ull >> (63 - (int)(E & 63));
+            if (!OPEN) moved &= ~(1ull << (E & 63));
+        }
+        if (w == w0) {
+            mask &= ~0ull << (p & 63);
+            if (OPEN) moved &= ~(1ull << (p & 63));
+        }
+        return (bits & ~mask) | (moved & mask);
+    };
+    if (jb == w0 && w1 - w0 < 32) {  // the find's first round holds the whole span
+        const unsigned long long next = OPEN ? __shfl_up_sync(0xffffffffu, m.rend, 1)
+                                             : __shfl_down_sync(0xffffffffu, m.rend, 1);
+        const long long w = w0 + lane;
+        if (w <= w1) {
+            g.meta[w].rend = moved_word(w, m.rend, next);
+            if (64 * w >= x && 64 * w < E) g.meta[w].off = OPEN ? m.off + 1 : m.off - 1;
+        }
+        for (long long j = ((x + 63) >> 6) + lane; j < w0; j += 32) g.meta[j].off += OPEN ? 1 : -1;
+        __syncwarp();
+        return;
+    }
+    for (long long k = 0; k <= w1 - w0; k += 32) {  // away from the side that the bits come from
+        const long long w = OPEN ? w1 - k - lane : w0 + k + lane;
+        const bool in = w >= w0 && w <= w1;
+        unsigned long long bits = 0, next = 0;
+        if (in) {
+            bits = g.meta[w].rend;
+            if (OPEN ? w > w0 : w < w1) next = g.meta[OPEN ? w - 1 : w + 1].rend;
+        }
+        __syncwarp();
+        if (in) g.meta[w].rend = moved_word(w, bits, next);
+        __syncwarp();
+    }
+    for (long long j = ((x + 63) >> 6) + lane; 64 * j < E; j += 32) g.meta[j].off += OPEN ? 1 : -1;
+    __syncwarp();
+}
+
+// Opens slot p in the run of x (had: x has a run; append: p is one past its
+// end). False when no empty slot is left below block jend.
+template <int R>
+__device__ __forceinline__ bool gvw_open(const GView &g, long long x, long long p, bool had, bool append,
+                                         long long jend)
+{
+    const int lane = threadIdx.x & 31;
+    Meta m;
+    long long jb = p >> 6;
+    const long long E = gvw_find<true>(g, p, jb, jend, m);
+    if (E < 0) return false;
+    for (long long hi = E; hi > p; hi -= 32 * GVW_U) {  // from the top: each chunk is read before it is overwritten
+        uint32_t v[GVW_U];
+#pragma unroll
+        for (int u = 0; u < GVW_U; u++) {
+            const long long q = hi - 1 - lane - 32 * u;
+            if (q >= p) v[u] = rd_slot<R>(g.rem, (uint64_t)q);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < GVW_U; u++) {
+            const long long q = hi - 1 - lane - 32 * u;
+            if (q >= p) wr_slot<R>(g.rem, (uint64_t)q + 1, v[u]);
+        }
+        __syncwarp();
+    }
+    gvw_shift_meta<true>(g, x, p, E, jb, m);
+    if (lane == 0) {
+        if (!had) {
+            g.meta[x >> 6].occ |= 1ull << (x & 63);
+            gv_rend_put(g, p, true);
+        } else if (append) {
+            gv_rend_put(g, p - 1, false);
+            gv_rend_put(g, p, true);
+        }
+    }
+    __syncwarp();
+    return true;
+}
+
+// Closes slot p of the run [s, e] of x. False when no gap is found below
+// block jend.
+template <int R>
+__device__ __forceinline__ bool gvw_close(const GView &g, long long x, long long p, long long s, long long e,
+                                          long long jend)
+{
+    const int lane = threadIdx.x & 31;
+    Meta m;
+    long long jb = p >> 6;
+    const long long L = gvw_find<false>(g, e + 1, jb, jend, m) - 1;  // the last slot that moves
+    if (L < e) return false;
+    for (long long lo = p; lo < L; lo += 32 * GVW_U) {  // from the bottom
+        uint32_t v[GVW_U];
+#pragma unroll
+        for (int u = 0; u < GVW_U; u++) {
+            const long long q = lo + lane + 32 * u;
+            if (q < L) v[u] = rd_slot<R>(g.rem, (uint64_t)q + 1);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < GVW_U; u++) {
+            const long long q = lo + lane + 32 * u;
+            if (q < L) wr_slot<R>(g.rem, (uint64_t)q, v[u]);
+        }
+        __syncwarp();
+    }
+    gvw_shift_meta<false>(g, x, p, L, jb, m);
+    if (lane == 0) {
+        wr_slot<R>(g.rem, (uint64_t)L, 0u);
+        if (s == e) g.meta[x >> 6].occ &= ~(1ull << (x & 63));
+        else if (p == e) gv_rend_put(g, e - 1, true);  // its bit went with the slot
+    }
+    __syncwarp();
+    return true;
+}
+
+// add c copies of fingerprint fp (the whole warp calls it)
+template <int R>
+__device__ __forceinline__ bool gvw_insert(const GView &g, uint64_t fp, uint64_t c, long long r0, long long jend)
+{
+    const long long x = (long long)(fp >> R);
+    const uint32_t v = (uint32_t)(fp & ((1ull << R) - 1ull));
+    bool had = gv_occ(g, x);
+    long long s, e, p;
+    uint64_t c_old;
+    uint32_t ol;
+    if (!gv_locate<R>(g, x, v, r0, s, e, p, c_old, ol)) return false;
+    const uint64_t cn = c_old + c;
+    const uint32_t nl = enc_len(cn, R);
+    __syncwarp();
+    for (uint32_t k = ol; k < nl; k++, e++) {
+        if (!gvw_open<R>(g, x, p + k, had, p + k == e + 1, jend)) return false;
+        had = true;
+    }
+    if ((threadIdx.x & 31) == 0) gv_put_group<R>(g, p, v, cn);
+    __syncwarp();
+    return true;
+}
+
+// remove min(c, d) copies of fingerprint fp (the whole warp calls it);
+// returns the number removed
+template <int R>
+__device__ __forceinline__ uint64_t gvw_delete(const GView &g, uint64_t fp, uint64_t d, long long jend,
+                                               unsigned long long *status)
+{
+    const long long x = (long long)(fp >> R);
+    const uint32_t v = (uint32_t)(fp & ((1ull << R) - 1ull));
+    if (x >= g.N || !gv_occ(g, x)) return 0;
+    long long s, e, p;
+    uint64_t c;
+    uint32_t ol;
+    if (!gv_locate<R>(g, x, v, x, s, e, p, c, ol)) {
+        if ((threadIdx.x & 31) == 0) atomicOr(status, GQF_ST_INTERNAL);
+        return 0;
+    }
+    if (c == 0) return 0;
+    const uint64_t rm = c < d ? c : d;
+    const uint32_t nl = c > rm ? enc_len(c - rm, R) : 0u;
+    __syncwarp();
+    for (uint32_t k = ol; k > nl; k--, e--)
+        if (!gvw_close<R>(g, x, p + nl, s, e, jend)) {
+            if ((threadIdx.x & 31) == 0) atomicOr(status, GQF_ST_INTERNAL);
+            return rm;
+        }
+    if (nl && (threadIdx.x & 31) == 0) gv_put_group<R>(g, p, v, c - rm);
+    __syncwarp();
+    return rm;
+}
+
+// blocks that a warp of region reg may touch: those of it and of the next one
+__device__ __forceinline__ long long gvw_jend(const GView &g, uint64_t reg, uint64_t rq)
+{
+    const long long j = (long long)((reg + 2) * rq >> 6);
+    return (long long)((reg + 2) * rq) >= g.N || j > g.nblk ? g.nblk : j;
+}
+
+// read-only: does every region's pushed data stop before the region after
+// next (two slots of margin) and before the table's end? A lane locates a
+// group each, the warp finds where the data stops. Odd regions run second and
+// find fewer empty slots than the pre-check does: those that the even regions
+// beside them take are counted in with their own. seen: regions with groups,
+// and those of them whose last group has no empty slot left in its block.
+template <int R>
+__global__ void __launch_bounds__(128) gqf_insert_precheck_warp(GView g, const uint64_t *__restrict__ ufp,
+                                                                const uint32_t *__restrict__ ustart,
+                                                                const uint32_t *__restrict__ rlo, uint64_t nreg,
+                                                                uint64_t rq, unsigned long long *bad, unsigned *seen)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned regions = 0, crowded = 0;
+    for (uint64_t reg = blockIdx.x * (uint64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); reg < nreg;
+         reg += (uint64_t)gridDim.x * (blockDim.x >> 5)) {
+        const uint32_t k0 = rlo[reg], k1 = rlo[reg + 1];
+        if (k0 == k1) continue;
+        const bool odd = reg & 1;
+        const uint32_t a0 = odd ? rlo[reg - 1] : k0, a1 = odd && reg + 1 < nreg ? rlo[reg + 2] : k1;
+        const long long jend = gvw_jend(g, reg, rq);
+        const long long limit = jend == g.nblk ? g.nslots - 1 : 64 * jend - 2;
+        unsigned need = 0;
+        bool ok = true;
+        for (uint32_t k = a0 + lane; k < a1; k += 32) {
+            const long long r0 = (long long)((k < k0 ? reg - 1 : (k < k1 ? reg : reg + 1)) * rq);
+            const int d = gv_slots_added<R>(g, ufp[k], ustart[k + 1] - ustart[k], r0);
+            ok &= d >= 0;
+            need += (unsigned)d;
+        }
+        need = __reduce_add_sync(0xffffffffu, need);
+        ok = __all_sync(0xffffffffu, ok);
+        // that many empty slots from the last group's quotient to the limit: a
+        // lane counts a block's
+        const long long x = (long long)(ufp[k1 - 1] >> R);
+        unsigned empty = 0;
+        for (long long jb = x >> 6; jb < jend && ok && empty < need; jb += 32) {
+            const long long j = jb + lane;
+            unsigned c = 0;
+            if (j < jend) {
+                const Meta m = g.meta[j];
+                for (int b = x > 64 * j ? (int)(x - 64 * j) : 0; c < need; b++, c++) {
+                    b = gv_block_empty(m, b);
+                    if (b >= 64 || 64 * j + b > limit) break;
+                }
+            }
+            if (jb == (x >> 6) && c == 0) crowded++;  // lane 0: none left in x's block
+            empty += __reduce_add_sync(0xffffffffu, c);
+        }
+        ok &= empty >= need;
+        regions++;
+        if (!ok && lane == 0) atomicExch(bad, 1ull);
+    }
+    if (lane == 0 && regions) {
+        atomicAdd(&seen[0], regions);
+        if (crowded) atomicAdd(&seen[1], crowded);
+    }
+}
+
+template <int R>
+__global__ void __launch_bounds__(128) gqf_insert_phase_warp(GView g, const uint64_t *__restrict__ ufp,
+                                                             const uint32_t *__restrict__ ustart,
+                                                             const uint32_t *__restrict__ rlo, uint64_t nreg,
+                                                             uint64_t rq, int phase, unsigned long long *status)
+{
+    for (uint64_t i = blockIdx.x * (uint64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);;
+         i += (uint64_t)gridDim.x * (blockDim.x >> 5)) {
+        const uint64_t reg = 2 * i + (uint64_t)phase;
+        if (reg >= nreg) return;
+        const long long jend = gvw_jend(g, reg, rq);
+        for (uint32_t k = rlo[reg]; k < rlo[reg + 1]; k++)
+            if (!gvw_insert<R>(g, ufp[k], ustart[k + 1] - ustart[k], (long long)(reg * rq), jend) &&
+                (threadIdx.x & 31) == 0)
+                atomicOr(status, ST_INTERNAL);
+    }
+}
+
+template <int R>
+__global__ void __launch_bounds__(128) gqf_delete_phase_warp(GView g, const uint64_t *__restrict__ ufp,
+                                                             const uint32_t *__restrict__ ustart,
+                                                             const uint32_t *__restrict__ rlo, uint64_t nreg,
+                                                             uint64_t rq, int phase, uint32_t *removed,
+                                                             unsigned long long *status)
+{
+    for (uint64_t i = blockIdx.x * (uint64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);;
+         i += (uint64_t)gridDim.x * (blockDim.x >> 5)) {
+        const uint64_t reg = 2 * i + (uint64_t)phase;
+        if (reg >= nreg) return;
+        const long long jend = gvw_jend(g, reg, rq);
+        for (uint32_t k = rlo[reg + 1]; k > rlo[reg]; k--) {
+            const uint32_t gi = k - 1;
+            const uint64_t rmv = gvw_delete<R>(g, ufp[gi], ustart[gi + 1] - ustart[gi], jend, status);
+            if (removed && (threadIdx.x & 31) == 0) removed[gi] = (uint32_t)rmv;
+        }
+    }
+}
+
+// read-only: the slots that each region's groups add (`need`, all ones when
+// the table is inconsistent)
+template <int R>
+__global__ void gqf_insert_need(GView g, const uint64_t *__restrict__ ufp, const uint32_t *__restrict__ ustart,
+                                const uint32_t *__restrict__ rlo, uint64_t nreg, uint64_t rq, uint32_t *need)
+{
+    for (uint64_t reg = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; reg < nreg;
+         reg += (uint64_t)gridDim.x * blockDim.x) {
+        uint32_t sum = 0;
+        for (uint32_t k = rlo[reg]; k < rlo[reg + 1]; k++) {
+            const int d = gv_slots_added<R>(g, ufp[k], ustart[k + 1] - ustart[k], (long long)(reg * rq));
+            if (d < 0) {
+                sum = ~0u;
+                break;
+            }
+            sum += (uint32_t)d;
+        }
+        need[reg] = sum;
+    }
+}
+
+// read-only: whether the data that each region pushes stops before the region
+// after next (two slots of margin) and before the table's end. Odd regions run
+// second, so the slots that the even regions beside them take count as theirs.
+template <int R>
+__global__ void gqf_insert_precheck(GView g, const uint64_t *__restrict__ ufp, const uint32_t *__restrict__ rlo,
+                                    const uint32_t *__restrict__ needs, uint64_t nreg, uint64_t rq,
+                                    unsigned long long *bad, unsigned *seen)
+{
+    unsigned regions = 0, crowded = 0;
     for (uint64_t reg = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; reg < nreg;
          reg += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t k0 = rlo[reg], k1 = rlo[reg + 1];
         if (k0 == k1) continue;
-        const long long r0 = (long long)(reg * rq);
         long long limit = (long long)((reg + 2) * rq) - 2;
         if (limit > g.nslots - 1) limit = g.nslots - 1;
-        long long need = 0;
-        for (uint32_t k = k0; k < k1; k++) {
-            const uint64_t fp = ufp[k];
-            long long s, e, p;
-            uint64_t c_old;
-            uint32_t ol;
-            if (!gv_locate<R>(g, (long long)(fp >> R), (uint32_t)(fp & ((1ull << R) - 1ull)), r0, s, e, p, c_old, ol)) {
-                atomicExch(bad, 1ull);
-                return;
-            }
-            need += (long long)enc_len(c_old + (uint64_t)(ustart[k + 1] - ustart[k]), R) - (long long)ol;
-        }
+        long long need = needs[reg];
+        if (reg & 1) need += (long long)needs[reg - 1] + (reg + 1 < nreg ? needs[reg + 1] : 0u);
         // the data all of them push stops, at the latest, where the data pushed
         // from the last one stops
-        if (gv_push_end(g, (long long)(ufp[k1 - 1] >> R), need, r0, limit) < 0) atomicExch(bad, 1ull);
+        const long long x = (long long)(ufp[k1 - 1] >> R);
+        const long long end = need >= 0xffffffffll ? -1 : gv_push_end(g, x, need, (long long)(reg * rq), limit);
+        if (end < 0) atomicExch(bad, 1ull);
+        regions++;
+        if (end < 0 || gv_block_empty(g.meta[x >> 6], (int)(x & 63)) > 63) crowded++;
+    }
+    regions = __reduce_add_sync(0xffffffffu, regions);
+    crowded = __reduce_add_sync(0xffffffffu, crowded);
+    if ((threadIdx.x & 31) == 0 && regions) {
+        atomicAdd(&seen[0], regions);
+        if (crowded) atomicAdd(&seen[1], crowded);
     }
 }
 
@@ -975,27 +1373,41 @@ __global__ void gqf_region_ranges(const uint64_t *__restrict__ ufp, const uint32
 }
 
 // read-only: the largest reach (cluster tail end - home slot + 1) over the
-// groups to delete, capped just above RQ_MAX
+// groups to delete, capped just above RQ_MAX. The cluster of x ends before
+// the first gap at or after x + 1; a block's gaps are read off its own record
+// (gv_block_gap), so a thread makes one load per 64 slots of cluster instead
+// of two dependent ones per run (1000 groups at 85 % load: 90 -> 18 us). seen:
+// stored groups, and those of them whose cluster runs past their block.
 template <int R>
 __global__ void gqf_delete_precheck(GView g, const uint64_t *__restrict__ ufp, const uint32_t *pm,
-                                    unsigned long long *reach)
+                                    unsigned long long *reach, unsigned *seen)
 {
     const uint64_t m = *pm;
     unsigned long long mine = 0;
+    unsigned found = 0, crowded = 0;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
         const long long x = (long long)(ufp[i] >> R);
         if (x >= g.N || !gv_occ(g, x)) continue;
-        long long prev = gv_runend_of(g, x), y = x;
-        while (prev >= 0 && prev - x < RQ_MAX) {
-            const long long yn = gv_next_occ(g, y, prev + 1);
-            if (yn < 0) break;
-            prev = gv_next_runend(g, prev + 1);
-            y = yn;
+        unsigned long long r = (unsigned long long)RQ_MAX + 1;
+        int lo = (int)(x & 63) + 1;
+        for (long long j = x >> 6; j < g.nblk && 64 * j - x <= RQ_MAX; j++, lo = 1) {
+            const int b = gv_block_gap(g.meta[j], lo);
+            if (b <= 64) {
+                r = (unsigned long long)(64 * j + b - x);
+                break;
+            }
+            if (j == (x >> 6)) crowded++;
         }
-        const unsigned long long r = prev < 0 ? (unsigned long long)RQ_MAX + 1 : (unsigned long long)(prev - x + 1);
+        found++;
         mine = r > mine ? r : mine;
     }
     if (mine) atomicMax(reach, mine);
+    found = __reduce_add_sync(0xffffffffu, found);
+    crowded = __reduce_add_sync(0xffffffffu, crowded);
+    if ((threadIdx.x & 31) == 0 && found) {
+        atomicAdd(&seen[0], found);
+        if (crowded) atomicAdd(&seen[1], crowded);
+    }
 }
 
 template <int R>
@@ -1381,10 +1793,49 @@ static int read_dev(const T *d, T *h, cudaStream_t st)
     return FILTER_OK;
 }
 
+// Regions by warp or by thread. A warp's update costs the latency of some ten
+// dependent loads whatever the cluster; a thread's costs that per run that it
+// moves, but 32 of them share a warp. Insert and remove of m keys, threads /
+// warps in us: 2^24 slots at 40, 70, 85, 93 % load, m = 2^14: 329 / 349,
+// 639 / 471, 2732 / 620, 22541 / 1037; m = 2^17: 554 / 692, 1333 / 959, then
+// the merge; 2^27 slots, m = 2^18: 717 / 1205, 1381 / 1693, 5532 / 4356, 53200
+// / 5608. So warps up to 2^14 groups, and up to 2^18 when a quarter of the
+// clusters run past their 64-slot block (the pre-checks count those; about
+// 80 % load). At such loads the merge takes over at one group per 256 slots
+// instead of the tuned bound (2^27 slots at 85 %, 2^20 groups: 13.8 ms in
+// place by threads, 8.3 ms merged).
+static constexpr uint64_t GVW_FEW = 1u << 14, GVW_MOST = 1u << 18;
+
+// the smallest region tried: about one group each when warps take them anyway
+static uint64_t first_region(uint64_t m, uint64_t N)
+{
+    uint64_t rq = RQ_MIN;
+    while (m <= GVW_FEW && rq < (uint64_t)RQ_MAX / 4 && m * rq * 4 <= N) rq <<= 2;
+    return rq;
+}
+
+// what a pre-check found: its verdict (a region that cannot, or the reach),
+// and its counts of places and of crowded ones
+struct Precheck {
+    unsigned long long verdict;
+    unsigned seen[2];
+    bool crowded() const { return (uint64_t)seen[1] * 4 >= seen[0] && seen[0]; }
+    bool warps(uint64_t m) const { return m <= GVW_FEW || (m <= GVW_MOST && crowded()); }
+    bool merge(uint64_t m, uint64_t N) const { return crowded() && m * RQ_MIN > N; }
+};
+static_assert(offsetof(DevCounters, pend) == offsetof(DevCounters, overflow) + 8, "a pre-check's words are read together");
+
+static int clear_precheck(DevCounters *ctr, cudaStream_t st)
+{
+    GF_CUDA(cudaMemsetAsync(&ctr->overflow, 0, sizeof(Precheck), st));
+    return FILTER_OK;
+}
+
 // Small batches go in place over even-odd regions; `done` is false when the
 // pre-check found, at every region size tried, a region whose inserts could
-// reach the region after next (or the table's end).
-static int gqf_insert_in_place(filter *F, const uint32_t *cstart, uint64_t n, uint32_t m, cudaStream_t st,
+// reach the region after next (or the table's end). m: at least the number
+// of groups.
+static int gqf_insert_in_place(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m, cudaStream_t st,
                                bool &done)
 {
     GqfState &Q = F->gqf;
@@ -1393,35 +1844,50 @@ static int gqf_insert_in_place(filter *F, const uint32_t *cstart, uint64_t n, ui
             (long long)Q.nblk};
     int rc = FILTER_OK;
     // a few region sizes, growing fourfold; dense batches go to the merge
-    for (uint64_t rq = RQ_MIN; rq <= (uint64_t)RQ_MAX / 4 && (uint64_t)m * rq <= gqf_region_groups(F->tune) * Q.N; rq <<= 2) {
+    Precheck pc{};
+    for (uint64_t rq = first_region(m, Q.N);
+         rq <= (uint64_t)RQ_MAX / 4 && m * rq <= gqf_region_groups(F->tune) * Q.N; rq <<= 2) {
         const uint64_t nreg = (Q.N + rq - 1) / rq;
         {
             gf::TraceScope ts_("gqf_region_ranges", nreg + 1, st);
             gqf_region_ranges<<<grid_for(nreg + 1, 256, 4), 256, 0, st>>>(Q.ufp, Q.flags + n, Q.N, Q.r, rq, nreg,
                                                                          Q.tile_lo);
         }
-        GF_CUDA(cudaMemsetAsync(&F->ctr->overflow, 0, 8, st));
-        {
+        if ((rc = clear_precheck(F->ctr, st))) return rc;
+        unsigned long long *d_bad = &F->ctr->overflow;
+        if (pc.warps(m)) {  // as the last try saw the clusters
+            gf::TraceScope ts_("gqf_insert_precheck_warp", nreg, st);
+            const int gr = grid_for(nreg * 32, 128, 16);
+            if (Q.r == 8) gqf_insert_precheck_warp<8><<<gr, 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq, d_bad,
+                                                                          F->ctr->pend);
+            else gqf_insert_precheck_warp<16><<<gr, 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq, d_bad,
+                                                                  F->ctr->pend);
+        } else {
+            // the look-back state is free outside a merge, and has a word per 256 quotients
+            uint32_t *need = reinterpret_cast<uint32_t *>(Q.tile_state);
+            const int gr = grid_for(nreg, 128, 8);
+            {
+                gf::TraceScope ts_("gqf_insert_need", nreg, st);
+                if (Q.r == 8) gqf_insert_need<8><<<gr, 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq, need);
+                else gqf_insert_need<16><<<gr, 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq, need);
+            }
             gf::TraceScope ts_("gqf_insert_precheck", nreg, st);
-            if (Q.r == 8)
-                gqf_insert_precheck<8><<<grid_for(nreg, 128, 8), 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq,
-                                                                               &F->ctr->overflow);
-            else
-                gqf_insert_precheck<16><<<grid_for(nreg, 128, 8), 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq,
-                                                                                &F->ctr->overflow);
+            if (Q.r == 8) gqf_insert_precheck<8><<<gr, 128, 0, st>>>(g, Q.ufp, Q.tile_lo, need, nreg, rq, d_bad, F->ctr->pend);
+            else gqf_insert_precheck<16><<<gr, 128, 0, st>>>(g, Q.ufp, Q.tile_lo, need, nreg, rq, d_bad, F->ctr->pend);
         }
-        unsigned long long bad = 0;
-        if ((rc = read_dev(&F->ctr->overflow, &bad, st))) return rc;
-        if (bad) continue;
+        if ((rc = read_dev(reinterpret_cast<const Precheck *>(&F->ctr->overflow), &pc, st))) return rc;
+        if (pc.merge(m, Q.N)) break;
+        if (pc.verdict) continue;
+        const bool warps = pc.warps(m);
         const uint64_t half = (nreg + 1) / 2;
         for (int ph = 0; ph < 2; ph++) {
             gf::TraceScope ts_("gqf_insert_phase", half, st);
-            if (Q.r == 8)
-                gqf_insert_phase<8><<<grid_for(half, 128, 8), 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq, ph,
-                                                                            &F->ctr->status);
-            else
-                gqf_insert_phase<16><<<grid_for(half, 128, 8), 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq,
-                                                                             ph, &F->ctr->status);
+            unsigned long long *status = &F->ctr->status;
+            const int gw = grid_for(half * 32, 128, 16), gt = grid_for(half, 128, 8);
+            if (Q.r == 8 && warps) gqf_insert_phase_warp<8><<<gw, 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq, ph, status);
+            else if (warps) gqf_insert_phase_warp<16><<<gw, 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq, ph, status);
+            else if (Q.r == 8) gqf_insert_phase<8><<<gt, 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq, ph, status);
+            else gqf_insert_phase<16><<<gt, 128, 0, st>>>(g, Q.ufp, cstart, Q.tile_lo, nreg, rq, ph, status);
         }
         GF_CUDA(cudaGetLastError());
         done = true;
@@ -1465,11 +1931,16 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
         GF_CUDA(cudaGetLastError());
         cstart = cs;
     }
-    // small batches: in place, region by region; larger ones: the merge
+    // small batches: in place, region by region; larger ones: the merge. The
+    // keys bound the groups, whose number is read back only when that decides.
     {
-        uint32_t m = 0;
-        if ((rc = read_dev(Q.flags + n, &m, st))) return rc;
-        if ((uint64_t)m * RQ_MIN <= gqf_region_groups(F->tune) * Q.N && !Q.merge_only) {
+        uint64_t m = n;
+        if (m * RQ_MIN > gqf_region_groups(F->tune) * Q.N && !Q.merge_only) {
+            uint32_t groups = 0;
+            if ((rc = read_dev(Q.flags + n, &groups, st))) return rc;
+            m = groups;
+        }
+        if (m * RQ_MIN <= gqf_region_groups(F->tune) * Q.N && !Q.merge_only) {
             bool done = false;
             if ((rc = gqf_insert_in_place(F, cstart, n, m, st, done))) return rc;
             if (done) {
@@ -1529,23 +2000,30 @@ int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cud
     gqf_prepare(F, keys, n, status != nullptr, st, &sidx);
     int rc = FILTER_OK;
     // small batches: in place, cluster by cluster; large ones: full merge
-    uint32_t m = 0;
-    if ((rc = read_dev(Q.flags + n, &m, st))) return rc;
+    uint64_t m = n;  // at least the number of groups
+    if (m * RQ_MIN > gqf_region_groups(F->tune) * Q.N) {
+        uint32_t groups = 0;
+        if ((rc = read_dev(Q.flags + n, &groups, st))) return rc;
+        m = groups;
+    }
     bool done = false;
-    if ((uint64_t)m * RQ_MIN <= gqf_region_groups(F->tune) * Q.N) {
+    if (m * RQ_MIN <= gqf_region_groups(F->tune) * Q.N) {
         GView g{reinterpret_cast<Meta *>(Q.meta[Q.cur]), Q.rem[Q.cur], (long long)Q.N, (long long)Q.nslots,
                 (long long)Q.nblk};
-        GF_CUDA(cudaMemsetAsync(&F->ctr->overflow, 0, 8, st));
+        if ((rc = clear_precheck(F->ctr, st))) return rc;
         {
             gf::TraceScope ts_("gqf_delete_precheck", m, st);
-            if (Q.r == 8) gqf_delete_precheck<8><<<grid_for(m, 256, 8), 256, 0, st>>>(g, Q.ufp, Q.flags + n, &F->ctr->overflow);
-            else gqf_delete_precheck<16><<<grid_for(m, 256, 8), 256, 0, st>>>(g, Q.ufp, Q.flags + n, &F->ctr->overflow);
+            const int gr = grid_for(m, 256, 8);
+            unsigned long long *reach = &F->ctr->overflow;
+            if (Q.r == 8) gqf_delete_precheck<8><<<gr, 256, 0, st>>>(g, Q.ufp, Q.flags + n, reach, F->ctr->pend);
+            else gqf_delete_precheck<16><<<gr, 256, 0, st>>>(g, Q.ufp, Q.flags + n, reach, F->ctr->pend);
         }
-        unsigned long long reach = 0;
-        if ((rc = read_dev(&F->ctr->overflow, &reach, st))) return rc;
-        uint64_t rq = RQ_MIN;
-        while ((unsigned long long)rq < reach) rq <<= 1;
-        if (rq <= (uint64_t)RQ_MAX && (uint64_t)m * rq <= gqf_region_groups(F->tune) * Q.N) {
+        Precheck pc{};
+        if ((rc = read_dev(reinterpret_cast<const Precheck *>(&F->ctr->overflow), &pc, st))) return rc;
+        const bool warps = pc.warps(m);
+        uint64_t rq = first_region(m, Q.N);
+        while ((unsigned long long)rq < pc.verdict) rq <<= 1;
+        if (!pc.merge(m, Q.N) && rq <= (uint64_t)RQ_MAX && m * rq <= gqf_region_groups(F->tune) * Q.N) {
             const uint64_t nreg = (Q.N + rq - 1) / rq;
             {
                 gf::TraceScope ts_("gqf_region_ranges", nreg + 1, st);
@@ -1553,14 +2031,19 @@ int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cud
                                                                              Q.tile_lo);
             }
             const uint64_t half = (nreg + 1) / 2;
+            uint32_t *removed = status ? Q.removed : nullptr;
             for (int ph = 0; ph < 2; ph++) {
                 gf::TraceScope ts_("gqf_delete_phase", half, st);
-                if (Q.r == 8)
-                    gqf_delete_phase<8><<<grid_for(half, 128, 8), 128, 0, st>>>(g, Q.ufp, Q.ustart, Q.tile_lo, nreg, ph,
-                                                                                status ? Q.removed : nullptr, &F->ctr->status);
+                unsigned long long *sw = &F->ctr->status;
+                const int gw = grid_for(half * 32, 128, 16), gt = grid_for(half, 128, 8);
+                if (Q.r == 8 && warps)
+                    gqf_delete_phase_warp<8><<<gw, 128, 0, st>>>(g, Q.ufp, Q.ustart, Q.tile_lo, nreg, rq, ph, removed, sw);
+                else if (warps)
+                    gqf_delete_phase_warp<16><<<gw, 128, 0, st>>>(g, Q.ufp, Q.ustart, Q.tile_lo, nreg, rq, ph, removed, sw);
+                else if (Q.r == 8)
+                    gqf_delete_phase<8><<<gt, 128, 0, st>>>(g, Q.ufp, Q.ustart, Q.tile_lo, nreg, ph, removed, sw);
                 else
-                    gqf_delete_phase<16><<<grid_for(half, 128, 8), 128, 0, st>>>(g, Q.ufp, Q.ustart, Q.tile_lo, nreg, ph,
-                                                                                 status ? Q.removed : nullptr, &F->ctr->status);
+                    gqf_delete_phase<16><<<gt, 128, 0, st>>>(g, Q.ufp, Q.ustart, Q.tile_lo, nreg, ph, removed, sw);
             }
             GF_CUDA(cudaGetLastError());
             done = true;
