@@ -2187,8 +2187,16 @@ static int dst_grid(const PhaseDst &P, uint64_t n, uint64_t ndst)
 // straddle word boundaries). A block is B slots of F bits packed
 // little-endian into whole 32-byte sectors (gf_packed.cuh); the phases and
 // their grouping are the ones above, only the per-block steps and the query
-// read and write packed slots. One thread per block, as in the 32-byte path;
-// the per-block candidate and tag lists live in local memory.
+// read and write packed slots.
+//
+// A block's step is shared by 4, 8 or 16 lanes: its words and candidates go
+// through shared memory, each candidate ranks itself among the others and finds
+// its slot by binary search, and a bit map of the new (or removed) slots tells
+// each lane what its slots of the new block hold. Bound by instructions; a
+// thread per block kept the candidate and tag lists (up to 4 KB) in local
+// memory. 128 slots of 16 bits, 2^22 slots: the block steps of removing half in
+// four batches 1822 us with threads, 153 with the lanes; of eight inserts to
+// 90 % 398 and 212 us.
 // ---------------------------------------------------------------------------
 template <int F, int B>
 struct GBlk : Packed<F, B> {
@@ -2196,6 +2204,8 @@ struct GBlk : Packed<F, B> {
     static constexpr int WORDS = Packed<F, B>::WORDS;
     static constexpr int BYTES = WORDS * 4;
     static_assert(BYTES % 32 == 0, "whole sectors");
+    static constexpr int LANES = B <= 32 ? 4 : (B <= 64 ? 8 : 16);  // that share a block's step
+    static constexpr uint32_t CAND = 8 * LANES;                      // candidates the step stages
 
     __device__ __forceinline__ void load(const uint8_t *blocks, uint64_t b, bool ro)
     {
@@ -2232,6 +2242,248 @@ struct GBlk : Packed<F, B> {
     }
 };
 
+// entries of the ascending v[0 .. n) below t
+template <class Get>
+__device__ __forceinline__ uint32_t count_below(uint32_t n, uint32_t t, Get v)
+{
+    uint32_t lo = 0, hi = n;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (v(mid) < t) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// The steps of a block with more candidates than its lanes stage (a hot key),
+// by one thread: insert returns the largest accepted record; remove passes the
+// unmatched on itself
+template <int F, int B>
+__device__ __noinline__ uint64_t gblock_insert_many(uint8_t *blocks, uint64_t b, uint32_t f0, uint32_t k,
+                                                    const uint64_t *rec, uint32_t cnt)
+{
+    uint64_t a[B];
+    int have = 0;
+    for (uint32_t q = 0; q < cnt; q++) have = topk_push(a, have, (int)k, rec[q]);
+    uint32_t nv[B];
+    for (uint32_t q = 0; q < k; q++) nv[q] = (uint32_t)(a[q] >> 32);
+    GBlk<F, B> blk;
+    blk.load(blocks, b, false);
+    blk.merge_sorted((int)f0, nv, (int)k);
+    blk.store(blocks, b);
+    return a[k - 1];
+}
+
+template <int F, int B>
+__device__ __noinline__ uint32_t gblock_remove_many(uint8_t *blocks, uint64_t b, uint32_t f0, const uint64_t *rec,
+                                                    uint32_t cnt, uint32_t *pend32, unsigned *npend)
+{
+    uint32_t dt[B], dc[B], used[B], removed = 0;
+    uint64_t thr[B];
+    int ndt = 0;
+    GBlk<F, B> blk;
+    blk.load(blocks, b, false);
+    for (int p = 0; p < (int)f0; p++) {  // copies of a tag are adjacent
+        const uint32_t t = blk.get(p);
+        if (ndt > 0 && dt[ndt - 1] == t) {
+            dc[ndt - 1]++;
+        } else {
+            dt[ndt] = t;
+            dc[ndt] = 1;
+            ndt++;
+        }
+    }
+    for (int d = 0; d < ndt; d++) {
+        uint64_t a[B];
+        int have = 0;
+        const uint64_t lo = (uint64_t)dt[d] << 32, hi = lo | 0xffffffffull;
+        for (uint32_t q = 0; q < cnt; q++)
+            if (rec[q] >= lo && rec[q] <= hi) have = topk_push(a, have, (int)dc[d], rec[q]);
+        used[d] = (uint32_t)have;
+        thr[d] = have ? a[have - 1] : 0;
+        removed += (uint32_t)have;
+    }
+    if (removed) {
+        GBlk<F, B> out;
+        out.clear();
+        int o = 0;
+        for (int d = 0; d < ndt; d++)
+            for (uint32_t c = used[d]; c < dc[d]; c++) out.set(o++, dt[d]);
+        out.store(blocks, b);
+    }
+    if (removed < cnt) {
+        uint32_t slot = atomicAdd(npend, cnt - removed);
+        for (uint32_t q = 0; q < cnt; q++) {
+            const uint32_t t = (uint32_t)(rec[q] >> 32);
+            bool matched = false;
+            for (int d = 0; d < ndt; d++)
+                if (dt[d] == t && used[d] > 0 && rec[q] <= thr[d]) matched = true;
+            if (!matched) pend32[slot++] = (uint32_t)rec[q];
+        }
+    }
+    return f0 - removed;
+}
+
+// One phase over its blocks. Insert (DEL = false): the k smallest (tag, index)
+// candidates that fit under `cap` join the block; rejects go on as in
+// tcf_block_insert. Remove: per tag, the smallest candidates take one copy
+// each; the unmatched go on.
+template <int F, int B, bool DEL>
+__global__ void __launch_bounds__(TPB) tcf_gblock_step(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
+                                                       const uint64_t *__restrict__ rec, int phase, uint32_t cap,
+                                                       uint32_t *pend32, uint64_t *pend64, unsigned *npend,
+                                                       unsigned long long *units)
+{
+    using Blk = GBlk<F, B>;
+    constexpr int L = Blk::LANES, NG = TPB / L, RM = (B + 31) / 32;
+    constexpr uint32_t CAND = Blk::CAND;
+    constexpr int S = (B + L - 1) / L;  // slots per lane: gl, gl + L, ..
+    __shared__ uint64_t s_rec[NG][CAND];
+    __shared__ __align__(16) Blk s_blk[NG];
+    constexpr bool BYTEWISE = F == 8 || F == 16;  // the new block's slots are its words
+    using Slot = typename std::conditional<F == 8, uint8_t, uint16_t>::type;
+    __shared__ uint16_t s_new[NG][B];
+    __shared__ __align__(16) Slot s_out[NG][BYTEWISE ? Blk::BYTES / sizeof(Slot) : B];
+    __shared__ uint32_t s_map[NG][RM];  // insert: the new slots; remove: the removed ones
+    const int gl = threadIdx.x % L, g = threadIdx.x / L;
+    const uint64_t nd = phase_count(P, G.nb);
+    if (P.dlist) note_units(units, nd);  // units: blocks with candidates
+    const uint64_t stride = (uint64_t)gridDim.x * NG;
+    auto old = [&](uint32_t i) -> uint32_t {
+        if constexpr (F == 16) return reinterpret_cast<const uint16_t *>(s_blk[g].w)[i];
+        else if constexpr (F == 8) return reinterpret_cast<const uint8_t *>(s_blk[g].w)[i];
+        else return s_blk[g].get((int)i);
+    };
+    auto fresh = [&](uint32_t i) { return (uint32_t)s_new[g][i]; };
+    if (BYTEWISE)
+        for (int i = B + gl; i < Blk::BYTES / (int)sizeof(Slot); i += L) s_out[g][i] = 0;  // past the last slot
+    // whole warps step together: a warp's lanes all reach its barriers
+    for (uint64_t j0 = blockIdx.x * (uint64_t)NG + (threadIdx.x & ~31u) / L; j0 < nd; j0 += stride) {
+        const uint64_t j = j0 + (threadIdx.x & 31) / L;
+        uint32_t s = 0, e = 0, f0 = 0, k = 0;
+        uint64_t b = 0;
+        if (j < nd) b = phase_dst(P, j, s, e);
+        const uint32_t cnt = e - s;
+        const bool staged = cnt > 0 && cnt <= CAND;
+        uint64_t r[8];
+        uint32_t left = 0;  // bit u: candidate gl + u L goes on
+        if (cnt) f0 = fill[b];
+        if (staged) {
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                if (u * L >= (int)cnt) break;
+                const uint32_t q = gl + u * L;
+                r[u] = q < cnt ? rec[s + q] : ~0ull;
+                if (q < cnt) s_rec[g][q] = r[u];
+            }
+            for (int w = gl; w < Blk::WORDS / 4; w += L)
+                reinterpret_cast<uint4 *>(s_blk[g].w)[w] = reinterpret_cast<const uint4 *>(blocks + b * Blk::BYTES)[w];
+            for (int w = gl; w < RM; w += L) s_map[g][w] = 0;
+        }
+        if (!DEL) k = cap > f0 ? min(cnt, cap - f0) : 0u;
+        __syncwarp();
+        if (staged) {
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                if (u * L >= (int)cnt) break;
+                uint32_t rank = 0;  // smaller candidates (DEL: of the same tag)
+                for (uint32_t i = 0; i < cnt; i++) {
+                    const uint64_t x = s_rec[g][i];
+                    rank += x < r[u] && (!DEL || (x >> 32) == (r[u] >> 32));
+                }
+                if (gl + u * L >= (int)cnt) continue;
+                const uint32_t tag = (uint32_t)(r[u] >> 32);
+                if (!DEL) {
+                    if (rank < k) s_new[g][rank] = (uint16_t)tag;
+                    else left |= 1u << u;
+                } else {
+                    const uint32_t at = count_below(f0, tag, old) + rank;
+                    if (at < f0 && old(at) == tag) atomicOr(&s_map[g][at >> 5], 1u << (at & 31));
+                    else left |= 1u << u;
+                }
+            }
+        }
+        __syncwarp();
+        if (!DEL && staged) {
+            // an accepted tag lands behind the old ones up to it and the accepted before it
+            for (uint32_t i = gl; i < k; i += L) {
+                const uint32_t at = i + count_below(f0, fresh(i) + 1, old);
+                atomicOr(&s_map[g][at >> 5], 1u << (at & 31));
+            }
+        }
+        __syncwarp();
+        uint32_t f1 = f0;  // the new fill
+        if (staged) {
+            uint32_t map[RM], pre[RM + 1];
+            pre[0] = 0;
+#pragma unroll
+            for (int w = 0; w < RM; w++) {
+                map[w] = s_map[g][w];
+                pre[w + 1] = pre[w] + __popc(map[w]);
+            }
+            f1 = DEL ? f0 - pre[RM] : f0 + k;
+#pragma unroll
+            for (int u = 0; u < S; u++) {
+                const int w = u * L / 32;  // the slots of one u share a map word
+                const uint32_t i = gl + u * L, m = map[w] >> ((u * L) % 32);
+                if (i >= (uint32_t)B) break;
+                const uint32_t before = pre[w] + __popc(map[w] & ((1u << (i & 31)) - 1u));
+                if (!DEL) {
+                    s_out[g][i] = (Slot)(i >= f1 ? 0u : ((m >> gl) & 1u) ? fresh(before) : old(i - before));
+                } else {
+                    if (i < f0 && !((m >> gl) & 1u)) s_out[g][i - before] = (Slot)old(i);
+                    if (i >= f1) s_out[g][i] = 0;
+                }
+            }
+        }
+        __syncwarp();
+        if (staged && f1 != f0) {
+            for (int w = gl; w < Blk::WORDS; w += L) {
+                uint32_t x = 0;
+                if constexpr (BYTEWISE) {
+                    x = reinterpret_cast<const uint32_t *>(s_out[g])[w];
+                } else {
+                    for (int i = 32 * w / F; i < B && F * i < 32 * (w + 1); i++) {
+                        const int o = F * i - 32 * w;
+                        x |= o >= 0 ? (uint32_t)s_out[g][i] << o : (uint32_t)s_out[g][i] >> -o;
+                    }
+                }
+                reinterpret_cast<uint32_t *>(blocks + b * Blk::BYTES)[w] = x;
+            }
+            if (gl == 0) fill[b] = (uint8_t)f1;
+        }
+        uint64_t thr = 0;
+        const bool many = cnt > CAND && gl == 0;
+        uint32_t nleft = __popc(left);
+        if (many) {
+            if (DEL) {
+                f1 = gblock_remove_many<F, B>(blocks, b, f0, rec + s, cnt, pend32, npend);
+            } else if (k) {
+                thr = gblock_insert_many<F, B>(blocks, b, f0, k, rec + s, cnt);
+                f1 = f0 + k;
+            }
+            if (f1 != f0) fill[b] = (uint8_t)f1;
+            if (!DEL) nleft = cnt - k;
+        }
+        uint32_t slot = warp_reserve(npend, nleft);
+        auto pass_on = [&](uint64_t x) {
+            if (!DEL && phase == 1) pend64[slot++] = ((b ^ tcf_g((uint32_t)(x >> 32), G.nb)) << 32) | (uint32_t)x;  // the other block
+            else pend32[slot++] = (uint32_t)x;
+        };
+#pragma unroll
+        for (int u = 0; u < 8; u++)
+            if ((left >> u) & 1u) pass_on(r[u]);
+        if (many && !DEL)
+            for (uint32_t q = s; q < e; q++)
+                if (k == 0 || rec[q] > thr) pass_on(rec[q]);
+        __syncwarp();  // the group's shared memory is free again
+    }
+}
+
+// The insert of blocks of up to 21 slots, a thread each: a block gets a
+// candidate or two, too few for lanes to share (2^24 slots filled to 90 %:
+// blocks of 8 slots 2.43 ms by threads, 3.45 by lanes; 21 slots of 12 bits
+// 2.44 and 3.18; 32 slots of 16 bits 1.99 and 1.96)
 template <int F, int B>
 __global__ void __launch_bounds__(TPB) tcf_gblock_insert(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
                                                          const uint64_t *__restrict__ rec, int phase, uint32_t cap,
@@ -2279,90 +2531,66 @@ __global__ void __launch_bounds__(TPB) tcf_gblock_insert(TcfGeom G, uint8_t *blo
     }
 }
 
-// per distinct stored tag, the smallest candidates with that tag remove one copy each
-template <int F, int B>
-__global__ void __launch_bounds__(TPB) tcf_gblock_remove(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
-                                                         const uint64_t *__restrict__ rec, uint32_t *pend32,
-                                                         unsigned *npend, unsigned long long *units)
-{
-    const uint64_t nd = phase_count(P, G.nb);
-    if (P.dlist) note_units(units, nd);
-    const uint64_t stride = (uint64_t)gridDim.x * TPB;
-    for (uint64_t j0 = blockIdx.x * (uint64_t)TPB + (threadIdx.x & ~31u); j0 < nd; j0 += stride) {
-        const uint64_t j = j0 + (threadIdx.x & 31);
-        uint32_t s = 0, e = 0, removed = 0;
-        uint32_t dt[B], dc[B], used[B];
-        uint64_t thr[B];
-        int ndt = 0;
-        if (j < nd) {
-            const uint64_t b = phase_dst(P, j, s, e);
-            if (s != e) {
-                const uint32_t f0 = fill[b];
-                GBlk<F, B> blk;
-                blk.load(blocks, b, false);
-                for (int p = 0; p < (int)f0; p++) {  // copies of a tag are adjacent
-                    const uint32_t t = blk.get(p);
-                    if (ndt > 0 && dt[ndt - 1] == t) {
-                        dc[ndt - 1]++;
-                    } else {
-                        dt[ndt] = t;
-                        dc[ndt] = 1;
-                        ndt++;
-                    }
-                }
-                for (int d = 0; d < ndt; d++) {
-                    uint64_t a[B];
-                    int have = 0;
-                    const uint64_t lo = (uint64_t)dt[d] << 32, hi = lo | 0xffffffffull;
-                    for (uint32_t q = s; q < e; q++) {
-                        const uint64_t r = rec[q];
-                        if (r >= lo && r <= hi) have = topk_push(a, have, (int)dc[d], r);
-                    }
-                    used[d] = (uint32_t)have;
-                    thr[d] = have ? a[have - 1] : 0;
-                    removed += (uint32_t)have;
-                }
-                if (removed) {
-                    GBlk<F, B> out;
-                    out.clear();
-                    int o = 0;
-                    for (int d = 0; d < ndt; d++)
-                        for (uint32_t c = used[d]; c < dc[d]; c++) out.set(o++, dt[d]);
-                    out.store(blocks, b);
-                    fill[b] = (uint8_t)(f0 - removed);
-                }
-            }
-        }
-        const uint32_t nunm = (e - s) - removed;  // unmatched candidates go on
-        uint32_t slot = warp_reserve(npend, nunm);
-        if (nunm == 0) continue;
-        for (uint32_t q = s; q < e; q++) {
-            const uint64_t r = rec[q];
-            const uint32_t t = (uint32_t)(r >> 32);
-            bool matched = false;
-            for (int d = 0; d < ndt; d++)
-                if (dt[d] == t && used[d] > 0 && r <= thr[d]) matched = true;
-            if (!matched) pend32[slot++] = (uint32_t)r;
-        }
-    }
-}
-
+// A thread per key reads a 32-byte block; a wider one is read by one lane per
+// 16 bytes, so that a load instruction covers whole lines (128 slots of 16
+// bits: 32 lines a load with a thread per key, 2 to 4 this way; 2^21 queries
+// of 2^22 slots 218 and GQUERY us). The second block only for keys not in the
+// first.
 template <int F, int B>
 __global__ void __launch_bounds__(TPB) tcf_gquery_kernel(const uint64_t *__restrict__ keys, uint64_t n, TcfGeom G,
                                                          const uint8_t *__restrict__ blocks,
                                                          const uint64_t *__restrict__ bk, const DevCounters *ctr,
                                                          uint8_t *__restrict__ out)
 {
+    constexpr int L = GBlk<F, B>::BYTES / 16, KW = 32 / L;  // lanes per block, keys of one load
     const bool backing = ctr->backing != 0;
-    for (uint64_t i = blockIdx.x * (uint64_t)TPB + threadIdx.x; i < n; i += (uint64_t)gridDim.x * TPB) {
-        const KeyInfo k = tcf_keyinfo(__ldcs(keys + i), G);
-        GBlk<F, B> x;
-        x.load(blocks, k.b1, true);
-        bool hit = x.has(k.t);
-        if (!hit) {
-            x.load(blocks, k.b2, true);
-            hit = x.has(k.t);
+    const int lane = threadIdx.x & 31;
+    for (uint64_t i0 = blockIdx.x * (uint64_t)TPB + (threadIdx.x & ~31u); i0 < n; i0 += (uint64_t)gridDim.x * TPB) {
+        const uint64_t i = i0 + lane;
+        KeyInfo k{0, 0, 0};
+        if (i < n) k = tcf_keyinfo(__ldcs(keys + i), G);
+        bool hit = false;
+        if constexpr (L == 2) {
+            GBlk<F, B> x;
+            if (i < n) {
+                x.load(blocks, k.b1, true);
+                hit = x.has(k.t);
+                if (!hit) {
+                    x.load(blocks, k.b2, true);
+                    hit = x.has(k.t);
+                }
+            }
+        } else {
+            static_assert(F == 16 || F == 8, "wide blocks of whole bytes");
+            const uint4 *base = reinterpret_cast<const uint4 *>(blocks) + lane % L;
+            for (int side = 0; side < 2; side++) {
+                if (!__any_sync(0xffffffffu, !hit && i < n)) break;
+                constexpr int U = L < 8 ? L : 8;  // loads in flight
+                for (int r0 = 0; r0 < L; r0 += U) {
+                    uint4 v[U];
+                    uint32_t t[U];
+#pragma unroll
+                    for (int u = 0; u < U; u++) {
+                        const int src = (r0 + u) * KW + lane / L;
+                        const uint32_t b = __shfl_sync(0xffffffffu, (uint32_t)(side ? k.b2 : k.b1), src);  // nb <= 2^32
+                        t[u] = __shfl_sync(0xffffffffu, hit ? 0u : k.t, src);
+                        const bool want = t[u] != 0;
+                        t[u] = F == 16 ? (t[u] | (t[u] << 16)) : t[u] * 0x01010101u;
+                        v[u] = want ? __ldg(base + (uint64_t)b * L) : make_uint4(0, 0, 0, 0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; u++) {
+                        const uint32_t m = F == 16 ? __vcmpeq2(v[u].x, t[u]) | __vcmpeq2(v[u].y, t[u]) |
+                                                         __vcmpeq2(v[u].z, t[u]) | __vcmpeq2(v[u].w, t[u])
+                                                   : __vcmpeq4(v[u].x, t[u]) | __vcmpeq4(v[u].y, t[u]) |
+                                                         __vcmpeq4(v[u].z, t[u]) | __vcmpeq4(v[u].w, t[u]);
+                        const unsigned any = __ballot_sync(0xffffffffu, m != 0);
+                        if (lane / KW == r0 + u && !hit && k.t) hit = ((any >> (lane % KW * L)) & ((1u << L) - 1u)) != 0;
+                    }
+                }
+            }
         }
+        if (i >= n) continue;
         if (!hit && backing) {
             const uint64_t e = tcf_entry(k, G.f);
             const ulonglong2 *p = reinterpret_cast<const ulonglong2 *>(bk + tcf_bucket_of(e, G) * BK_W);
@@ -2374,6 +2602,20 @@ __global__ void __launch_bounds__(TPB) tcf_gquery_kernel(const uint64_t *__restr
         }
         __stcs(out + i, (uint8_t)(hit ? 1 : 0));
     }
+}
+
+// one phase's per-block steps of a packed geometry
+template <int F, int B, bool DEL>
+static void gblock_phase(const TcfBulk &T, const PhaseDst &P, uint64_t n, int phase, uint32_t cap, uint32_t *pend32,
+                         uint64_t *pend64, unsigned *npend, unsigned long long *units, cudaStream_t st)
+{
+    const uint64_t nd = P.dlist && n < T.G.nb ? n : T.G.nb;
+    if constexpr (!DEL && B <= 21)
+        tcf_gblock_insert<F, B><<<grid_for(nd, TPB, 8), TPB, 0, st>>>(T.G, T.blocks, T.fill, P, T.rec, phase, cap, pend32,
+                                                                       pend64, npend, units);
+    else
+        tcf_gblock_step<F, B, DEL><<<grid_for(nd * GBlk<F, B>::LANES, TPB, 8), TPB, 0, st>>>(
+            T.G, T.blocks, T.fill, P, T.rec, phase, cap, pend32, pend64, npend, units);
 }
 
 // The per-block counting-sort path: each phase groups its candidates by
@@ -2396,8 +2638,7 @@ static void tcf_bulk_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
             tcf_block_insert<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, 0, G.tsc, T.pend0,
                                                                        nullptr, &np[0], T.prep, ts_.units());
         else
-            tcf_gblock_insert<F, GB><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, 0, G.tsc,
-                                                                           T.pend0, nullptr, &np[0], ts_.units());
+            gblock_phase<F, GB, false>(T, P, n, 0, G.tsc, T.pend0, nullptr, &np[0], ts_.units(), st);
     }
     // B: the less full of b1, b2 under the post-A fills
     P = group_phase<SRC_PEND_U32, DST_TARGET>(T, keys, n, T.pend0, &np[0], 1, nullptr, st);
@@ -2407,8 +2648,7 @@ static void tcf_bulk_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
             tcf_block_insert<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, 1, G.B, nullptr,
                                                                        T.pend1, &np[1], T.prep, ts_.units());
         else
-            tcf_gblock_insert<F, GB><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, 1, G.B,
-                                                                           nullptr, T.pend1, &np[1], ts_.units());
+            gblock_phase<F, GB, false>(T, P, n, 1, G.B, nullptr, T.pend1, &np[1], ts_.units(), st);
     }
     // C: the other block
     P = group_phase<SRC_PEND_U64, DST_ALT>(T, keys, n, T.pend1, &np[1], 2, nullptr, st);
@@ -2418,8 +2658,7 @@ static void tcf_bulk_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
             tcf_block_insert<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, 2, G.B, T.pend2,
                                                                        nullptr, &np[2], T.prep, ts_.units());
         else
-            tcf_gblock_insert<F, GB><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, 2, G.B,
-                                                                           T.pend2, nullptr, &np[2], ts_.units());
+            gblock_phase<F, GB, false>(T, P, n, 2, G.B, T.pend2, nullptr, &np[2], ts_.units(), st);
     }
     // D: backing buckets
     P = group_phase<SRC_PEND_U32, DST_BUCKET>(T, keys, n, T.pend2, &np[2], 3, T.pend0, st);
@@ -2445,8 +2684,7 @@ static void tcf_bulk_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
             tcf_block_remove<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, T.pend0, &np[0],
                                                                        ts_.units());
         else
-            tcf_gblock_remove<F, GB><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, T.pend0,
-                                                                           &np[0], ts_.units());
+            gblock_phase<F, GB, true>(T, P, n, 0, 0, T.pend0, nullptr, &np[0], ts_.units(), st);
     }
     // 2: secondary block
     P = group_phase<SRC_PEND_U32, DST_B2>(T, keys, n, T.pend0, &np[0], 1, nullptr, st);
@@ -2456,8 +2694,7 @@ static void tcf_bulk_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
             tcf_block_remove<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, T.pend2, &np[2],
                                                                        ts_.units());
         else
-            tcf_gblock_remove<F, GB><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, T.pend2,
-                                                                           &np[2], ts_.units());
+            gblock_phase<F, GB, true>(T, P, n, 0, 0, T.pend2, nullptr, &np[2], ts_.units(), st);
     }
     // 3: backing bucket; what is left is not found
     P = group_phase<SRC_PEND_U32, DST_BUCKET>(T, keys, n, T.pend2, &np[2], 2, T.pend0, st);
