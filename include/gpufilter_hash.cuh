@@ -48,6 +48,7 @@ GF_HASH_FN PHash phash_of(uint32_t p, uint64_t seed)
 GF_HASH_FN uint64_t fold_p(uint64_t x, const PHash &H)
 {
     if (H.p >= 64) return x;
+    if (H.p >= 32) return (x & H.mask) ^ (x >> H.p);  // two chunks; the usual widths, without a loop
     uint64_t r = 0;
     while (x) {
         r ^= x & H.mask;

@@ -40,6 +40,8 @@ namespace gf {
 static constexpr int MT = 256;          // merge threads per CTA
 static constexpr int QPT = 8;           // quotients per thread
 static constexpr int TQ = MT * QPT;     // quotients per tile
+static constexpr uint32_t TQ_LOG = 11;
+static_assert(TQ == 1 << TQ_LOG, "a tile is a span of top bits");
 static constexpr int TBLK = TQ / 64;    // blocks per tile
 static constexpr int OLDBUF = 3072;     // staged old slots
 static constexpr int GSMALL = 640;      // staged new groups of a tile that has old runs
@@ -61,7 +63,8 @@ struct MergeArgs {
     const uint64_t *ufp;
     const uint32_t *ustart;
     const uint32_t *pm;      // number of groups (device)
-    const uint32_t *tlo;     // first group of each tile (ntiles + 1 entries)
+    const uint32_t *tlo;     // first group of each tile,
+    const uint32_t *thi;     // and the end of its groups
     uint64_t m_limit;        // use groups [0, min(m, m_limit))
     uint32_t *removed;       // delete: copies removed per group
     unsigned long long *ts;  // look-back state: [0] tile counter, then one status word per tile
@@ -318,7 +321,7 @@ __device__ __forceinline__ void merge_tile(const MergeArgs &a, MergeSmem<R> &S, 
     if (tid < TBLK) S.occ[tid] = (j0 + tid < a.nblk) ? a.meta_old[j0 + tid].occ : 0ull;
     if (tid == TBLK) {
         S.glo = a.tlo[tile];
-        S.ghi = a.tlo[tile + 1];
+        S.ghi = a.thi[tile];
     }
     __syncthreads();
     const uint32_t mybyte = (uint32_t)(S.occ[tid >> 3] >> ((tid & 7) * 8)) & 0xffu;
@@ -886,6 +889,34 @@ __global__ void gqf_tile_ranges(const uint64_t *__restrict__ ufp, const uint32_t
             else hi = mid;
         }
         tlo[t] = (uint32_t)lo;
+    }
+}
+
+// the same for groups left in their units, each unit 2^span whole tiles: the
+// search stays in the tile's unit
+__global__ void gqf_unit_tile_ranges(const uint64_t *__restrict__ ufp, MsdUnits units, uint64_t N, uint32_t r,
+                                     uint32_t span, uint64_t ntiles, uint32_t *tlo, uint32_t *thi)
+{
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < ntiles; t += (uint64_t)gridDim.x * blockDim.x) {
+        uint32_t lo = 0, hi = 0;
+        if (t * TQ < N) {
+            const uint64_t u = t >> span;
+            lo = units.st[u];
+            hi = lo + units.distinct[u];
+            for (int side = 0; side < 2 && span; side++) {  // the tile's first group, then the next tile's
+                const uint64_t key = ((t + side) * TQ) << r;
+                uint32_t a = lo, b = hi;
+                while (a < b) {
+                    const uint32_t mid = (a + b) >> 1;
+                    if (ufp[mid] < key) a = mid + 1;
+                    else b = mid;
+                }
+                if (side) hi = a;
+                else lo = a;
+            }
+        }
+        tlo[t] = lo;
+        thi[t] = hi;
     }
 }
 
@@ -1646,11 +1677,11 @@ static uint64_t tail_slots(uint32_t q)
     return s;
 }
 
-// entries of the range array: one per merge tile or per smallest region, plus one
+// entries of the range array: two per merge tile or one per smallest region, plus one
 uint64_t gqf_tile_lo_words(const GqfState &Q)
 {
     const uint64_t nreg = (Q.N + RQ_MIN - 1) / RQ_MIN;
-    return (Q.ntiles > nreg ? Q.ntiles : nreg) + 1;
+    return (2 * Q.ntiles > nreg ? 2 * Q.ntiles : nreg) + 1;
 }
 
 int gqf_setup(filter *F, uint64_t &table_bytes, uint64_t &scratch_bytes, bool plan_only)
@@ -1781,9 +1812,12 @@ __global__ void __launch_bounds__(SM_T) gqf_small_prepare(const uint64_t *__rest
 
 // sort + reduce: leaves groups in ufp / ustart, group count in flags[n]. The
 // sort carries the batch indices (need_idx: statuses) or a caller's per-key
-// values (vals, without statuses); either ends in idx_b in sorted order.
+// values (vals, without statuses); either ends in idx_b in sorted order. With
+// `units`, groups bound for the merge may be left in their units: *in_units
+// says whether they were.
 static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_idx, cudaStream_t st,
-                        uint32_t **sorted_idx, const uint32_t *vals = nullptr)
+                        uint32_t **sorted_idx, const uint32_t *vals = nullptr, MsdUnits *units = nullptr,
+                        bool *in_units = nullptr)
 {
     GqfState &Q = F->gqf;
     *sorted_idx = Q.idx_b;
@@ -1794,6 +1828,20 @@ static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_i
                                                            Q.ustart, need_idx ? Q.flags : nullptr, Q.flags + n);
         return;
     }
+    if (!need_idx && !vals) {
+        auto groups = [&](MsdUnits *in) {
+            return msd_groups(keys, n, &Q.H, Q.p, Q.q > TQ_LOG ? Q.q - TQ_LOG : 0u, Q.fp_a, Q.fp_b, Q.ufp, Q.ustart,
+                              Q.flags + n, Q.radix_tmp, radix_tmp_words(F->cfg.max_batch), F->ctr, st, in);
+        };
+        // in place of the table, a batch needs its groups in one list; one
+        // twice past that bound may still turn out to have few distinct keys
+        const bool dense = n * RQ_MIN > 4 * gqf_region_groups(F->tune) * Q.N || Q.merge_only;
+        if (units && dense && groups(units)) {
+            *in_units = true;
+            return;
+        }
+        if (groups(nullptr)) return;
+    }
     fingerprint_for_sort(keys, n, Q.H, Q.fp_a, need_idx ? Q.idx_a : nullptr, Q.p, Q.radix_tmp, st);
     radix_sort_u64(Q.fp_a, Q.fp_b, Q.fp_c, need_idx ? Q.idx_a : vals, Q.idx_b, Q.idx_c, n, Q.p, Q.radix_tmp,
                    F->scan_tmp, F->ctr, st, true);
@@ -1802,8 +1850,9 @@ static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_i
 }
 
 // cstart: group g adds (or removes) cstart[g + 1] - cstart[g] copies
+// units: the groups' units where they were left in place (msd_groups)
 static int gqf_merge(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m_limit, int del, int dry,
-                     cudaStream_t st)
+                     cudaStream_t st, const MsdUnits *units = nullptr)
 {
     GqfState &Q = F->gqf;
     const int nb = Q.cur ^ 1;
@@ -1816,6 +1865,7 @@ static int gqf_merge(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m_l
     a.ustart = cstart;
     a.pm = Q.flags + n;
     a.tlo = Q.tile_lo;
+    a.thi = units ? Q.tile_lo + Q.ntiles : Q.tile_lo + 1;
     a.m_limit = m_limit;
     a.removed = del ? Q.removed : nullptr;
     a.ts = Q.tile_state;
@@ -1833,7 +1883,11 @@ static int gqf_merge(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m_l
     GF_CUDA(cudaMemsetAsync(&F->ctr->overflow, 0, 8, st));
     GF_CUDA(cudaMemsetAsync(&F->ctr->gqf_end, 0xff, 8, st));  // -1
     if (!dry) GF_CUDA(cudaMemsetAsync(Q.meta[nb], 0, Q.nblk * 32, st));
-    {
+    if (units) {
+        gf::TraceScope ts_("gqf_tile_ranges", Q.ntiles + 1, st);
+        gqf_unit_tile_ranges<<<grid_for(Q.ntiles, 256, 4), 256, 0, st>>>(Q.ufp, *units, Q.N, Q.r, Q.q - TQ_LOG - units->k,
+                                                                         Q.ntiles, Q.tile_lo, Q.tile_lo + Q.ntiles);
+    } else {
         gf::TraceScope ts_("gqf_tile_ranges", Q.ntiles + 1, st);
         gqf_tile_ranges<<<grid_for(Q.ntiles + 1, 256, 4), 256, 0, st>>>(Q.ufp, Q.flags + n, m_limit, Q.N, Q.r,
                                                                        Q.ntiles, Q.tile_lo);
@@ -1966,7 +2020,9 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
     uint32_t *sidx = nullptr;
     // counts without statuses ride through the sort in place of the indices
     const bool carry = counts != nullptr && status == nullptr;
-    gqf_prepare(F, keys, n, status != nullptr, st, &sidx, carry ? counts : nullptr);
+    MsdUnits units{};
+    bool in_units = false;
+    gqf_prepare(F, keys, n, status != nullptr, st, &sidx, carry ? counts : nullptr, counts ? nullptr : &units, &in_units);
     int rc;
     // the copies each group adds: its keys, or the sum of their counts
     const uint32_t *cstart = Q.ustart;
@@ -1995,7 +2051,7 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
     }
     // small batches: in place, region by region; larger ones: the merge. The
     // keys bound the groups, whose number is read back only when that decides.
-    {
+    if (!in_units) {
         uint64_t m = n;
         if (m * RQ_MIN > gqf_region_groups(F->tune) * Q.N && !Q.merge_only) {
             uint32_t groups = 0;
@@ -2016,12 +2072,13 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
             }
         }
     }
-    rc = gqf_merge(F, cstart, n, ~0ull, 0, 0, st);
+    rc = gqf_merge(F, cstart, n, ~0ull, 0, 0, st, in_units ? &units : nullptr);
     if (rc) return rc;
     unsigned long long ovf = 0;
     if ((rc = read_dev(&F->ctr->overflow, &ovf, st))) return rc;
     uint64_t m_keep = ~0ull;
     if (ovf) {
+        if (in_units) gqf_prepare(F, keys, n, false, st, &sidx);  // one list, whose prefixes are tried
         // keep the longest prefix of the sorted groups that fits (dry runs)
         uint32_t m = 0;
         if ((rc = read_dev(Q.flags + n, &m, st))) return rc;
@@ -2059,17 +2116,19 @@ int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cud
     if (n == 0) return FILTER_OK;
     GqfState &Q = F->gqf;
     uint32_t *sidx = nullptr;
-    gqf_prepare(F, keys, n, status != nullptr, st, &sidx);
+    MsdUnits units{};
+    bool in_units = false;
+    gqf_prepare(F, keys, n, status != nullptr, st, &sidx, nullptr, &units, &in_units);
     int rc = FILTER_OK;
     // small batches: in place, cluster by cluster; large ones: full merge
     uint64_t m = n;  // at least the number of groups
-    if (m * RQ_MIN > gqf_region_groups(F->tune) * Q.N) {
+    if (!in_units && m * RQ_MIN > gqf_region_groups(F->tune) * Q.N) {
         uint32_t groups = 0;
         if ((rc = read_dev(Q.flags + n, &groups, st))) return rc;
         m = groups;
     }
     bool done = false;
-    if (m * RQ_MIN <= gqf_region_groups(F->tune) * Q.N) {
+    if (!in_units && m * RQ_MIN <= gqf_region_groups(F->tune) * Q.N) {
         GView g{reinterpret_cast<Meta *>(Q.meta[Q.cur]), Q.rem[Q.cur], (long long)Q.N, (long long)Q.nslots,
                 (long long)Q.nblk};
         if ((rc = clear_precheck(F->ctr, st))) return rc;
@@ -2112,7 +2171,7 @@ int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cud
         }
     }
     if (!done) {
-        if ((rc = gqf_merge(F, Q.ustart, n, ~0ull, 1, 0, st))) return rc;
+        if ((rc = gqf_merge(F, Q.ustart, n, ~0ull, 1, 0, st, in_units ? &units : nullptr))) return rc;
         Q.cur ^= 1;
     }
     if (status) {
@@ -2552,6 +2611,7 @@ int gqf_group_setup(filter_group *GR, const filter_config *cfgs, uint64_t &bytes
                 a.ustart = Q.ustart;
                 a.pm = nullptr;
                 a.tlo = Q.tile_lo + tile0[m];
+                a.thi = a.tlo + 1;
                 a.m_limit = ~0ull;
                 a.removed = del ? Q.removed : nullptr;
                 a.ts = Q.tile_state + tile0[m];

@@ -232,6 +232,55 @@ struct Arena {
 };
 
 // ---------------------------------------------------------------------------
+// Decoupled look-back: tiles publish (flag << 32) | value words, flag 1 = tile
+// aggregate, 2 = inclusive prefix, and are taken in ticket order.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned long long ld_volatile(const unsigned long long *p)
+{
+    return *(const volatile unsigned long long *)p;
+}
+
+// Warp 0 of tile `tile`: publish the tile's total, look back over 32
+// predecessors at a time for the exclusive prefix, publish the inclusive one.
+// All 32 lanes call it and get the prefix. A wait that reaches SPIN_LIMIT
+// records ST_TIMEOUT and gives up (prefix then incomplete).
+__device__ __forceinline__ uint32_t lookback_prefix(unsigned long long *st, uint64_t tile, uint32_t total,
+                                    unsigned long long *status, uint32_t limit = SPIN_LIMIT)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t prefix = 0;
+    if (tile == 0) {
+        if (lane == 0) atomicExch(&st[0], (2ull << 32) | total);
+        return 0;
+    }
+    if (lane == 0) atomicExch(&st[tile], (1ull << 32) | total);
+    int64_t jtop = (int64_t)tile - 1;
+    uint32_t spins = 0;
+    while (true) {
+        const int64_t j = jtop - lane;
+        unsigned long long w2 = 2ull << 32;  // before tile 0: inclusive prefix 0
+        if (j >= 0) {
+            w2 = ld_volatile(&st[j]);
+            while ((w2 >> 32) == 0 && ++spins <= limit) w2 = ld_volatile(&st[j]);
+        }
+        const uint32_t flag = (uint32_t)(w2 >> 32);
+        if (__ballot_sync(0xffffffffu, flag == 0)) {
+            if (lane == 0) atomicOr(status, ST_TIMEOUT);
+            break;
+        }
+        const unsigned incl_mask = __ballot_sync(0xffffffffu, flag == 2);
+        const int L = incl_mask ? __ffs(incl_mask) - 1 : 31;
+        uint32_t part = (lane <= L) ? (uint32_t)w2 : 0u;
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        prefix += part;
+        if (incl_mask) break;
+        jtop -= 32;
+    }
+    if (lane == 0) atomicExch(&st[tile], (2ull << 32) | (uint32_t)(prefix + total));
+    return prefix;
+}
+
+// ---------------------------------------------------------------------------
 // Generic device primitives (gf_prims.cu)
 // ---------------------------------------------------------------------------
 // In-place-safe exclusive scan of n uint32 (out may equal in). Needs
@@ -260,6 +309,23 @@ void radix_sort_u64(const uint64_t *keys_in, uint64_t *keys_out, uint64_t *keys_
 // takes for its first pass
 void fingerprint_for_sort(const uint64_t *keys, uint64_t n, const PHash &H, uint64_t *fp, uint32_t *idx,
                           uint32_t bits, uint32_t *tmp, cudaStream_t st);
+
+// Distinct sorted values of n keys and the copies before each (gf_msd.cu): for
+// each group g, uniq[g] ascending and start[g] = the keys below it, start[m] =
+// n and *m_out = m. The values are the keys' fingerprints (H set), or the keys
+// themselves, of `bits` bits. buf_a and buf_b: n words each, spent; keys may be
+// buf_b. tmp: 32-bit words of scratch. With units_out, the groups stay in units
+// of their top k <= max_k bits: those of unit u are uniq / start [st[u], st[u] +
+// distinct[u]), with start[st[u] + distinct[u]] = st[u + 1] behind them, in tmp
+// until its next use. False (and nothing enqueued) for the sizes that it does
+// not take.
+struct MsdUnits {
+    const uint32_t *st, *distinct;
+    uint32_t k;
+};
+bool msd_groups(const uint64_t *keys, uint64_t n, const PHash *H, uint32_t bits, uint32_t max_k, uint64_t *buf_a,
+                uint64_t *buf_b, uint64_t *uniq, uint32_t *start, uint32_t *m_out, uint32_t *tmp, uint64_t tmp_words,
+                DevCounters *ctr, cudaStream_t st, MsdUnits *units_out);
 
 // Kernel tracing: a TraceScope around a launch records CUDA events before and
 // after it when tracing is on. Launches whose work is only known on the device

@@ -98,51 +98,6 @@ static_assert(SCAN_TILE <= 65536, "positions inside a tile fit 16 bits");
 
 size_t scan_tmp_words(uint64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE + 2; }
 
-__device__ __forceinline__ unsigned long long ld_volatile(const unsigned long long *p)
-{
-    return *(const volatile unsigned long long *)p;
-}
-
-// Warp 0 of tile `tile`: publish the tile's total, look back over 32
-// predecessors at a time for the exclusive prefix, publish the inclusive one.
-// All 32 lanes call it and get the prefix. A wait that reaches SPIN_LIMIT
-// records ST_TIMEOUT and gives up (prefix then incomplete).
-__device__ uint32_t lookback_prefix(unsigned long long *st, uint64_t tile, uint32_t total,
-                                    unsigned long long *status, uint32_t limit = SPIN_LIMIT)
-{
-    const int lane = threadIdx.x & 31;
-    uint32_t prefix = 0;
-    if (tile == 0) {
-        if (lane == 0) atomicExch(&st[0], (2ull << 32) | total);
-        return 0;
-    }
-    if (lane == 0) atomicExch(&st[tile], (1ull << 32) | total);
-    int64_t jtop = (int64_t)tile - 1;
-    uint32_t spins = 0;
-    while (true) {
-        const int64_t j = jtop - lane;
-        unsigned long long w2 = 2ull << 32;  // before tile 0: inclusive prefix 0
-        if (j >= 0) {
-            w2 = ld_volatile(&st[j]);
-            while ((w2 >> 32) == 0 && ++spins <= limit) w2 = ld_volatile(&st[j]);
-        }
-        const uint32_t flag = (uint32_t)(w2 >> 32);
-        if (__ballot_sync(0xffffffffu, flag == 0)) {
-            if (lane == 0) atomicOr(status, ST_TIMEOUT);
-            break;
-        }
-        const unsigned incl_mask = __ballot_sync(0xffffffffu, flag == 2);
-        const int L = incl_mask ? __ffs(incl_mask) - 1 : 31;
-        uint32_t part = (lane <= L) ? (uint32_t)w2 : 0u;
-        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        prefix += part;
-        if (incl_mask) break;
-        jtop -= 32;
-    }
-    if (lane == 0) atomicExch(&st[tile], (2ull << 32) | (uint32_t)(prefix + total));
-    return prefix;
-}
-
 __global__ void __launch_bounds__(SCAN_T) scan_kernel(const uint32_t *in, uint32_t *out, uint64_t n,
                                                       unsigned long long *tmp,
                                                       unsigned long long *status)
@@ -377,7 +332,7 @@ static_assert(RS_TILE < (1 << 16), "tile positions fit the 16-bit counters");
 size_t radix_tmp_words(uint64_t n)
 {
     uint64_t tiles = (n + RS_TILE - 1) / RS_TILE;
-    return tiles * RS_MAXB + 1;
+    return tiles * RS_MAXB + 1 + 6 * RS_MAXB;  // with room for the small arrays of msd_groups
 }
 
 // Per-tile digit counts. Each warp counts into its own shared histogram
