@@ -70,11 +70,20 @@ BYTES_PER_UNIT = {
     "tcf_bucket_remove": 136.0,
     "tcf_tile_hist": 8.0,        # key read (tile histogram through shared memory)
     "tcf_tile_hist_pend": 12.0,  # pending record read
-    "tcf_tile_part": 20.0,       # key read + 12-byte record write
-    "tcf_tile_part_pend": 24.0,  # record read + record write
-    "tcf_tile_part2": 24.0,      # record read + record write (second partition pass)
-    "tcf_tile_insert": 1.0,      # unit = algorithmic byte, counted on the device: 12 per candidate read and
-    "tcf_tile_remove": 1.0,      # per candidate left, 32 per block read, 32 per block written, 2 per fill
+    "tcf_tile_part": 16.0,       # key read + 8-byte record write
+    "tcf_tile_part_pend": 20.0,  # pending record read + record write
+    "tcf_tile_hist2": 8.0,       # record read (second partition pass)
+    "tcf_tile_part2": 16.0,      # record read + record write
+    "tcf_tile_insert": 1.0,      # unit = algorithmic byte, counted on the device: 8 per candidate read, 12 per
+    "tcf_tile_remove": 1.0,      # candidate left, 32 per block read, 32 per block written, 2 per fill
+    "msd_hist1": 8.0,            # key read
+    "msd_part": 16.0,            # key read + fingerprint write
+    "msd_hist2": 8.0,            # fingerprint read
+    "msd_part2": 16.0,           # fingerprint read + write
+    "msd_units": 8.0,            # fingerprint read (group writes not counted)
+    "gqf_small_prepare": 8.0,    # key read
+    "tcf_small_insert": 104.0,   # key + two 32 B blocks read + one written
+    "tcf_small_remove": 104.0,
     "batch_gather": 16.0,        # key read + key write
     "batch_scatter": 9.0,        # result read + write (1 byte; counts: 16)
     "gqf_group_commit": 192.0,   # per 64-slot block: 32 B metadata + 64 B remainders, read and written (r = 8)

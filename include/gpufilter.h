@@ -126,11 +126,12 @@ int filter_destroy(filter_t *f);
  *     per block, an 8-byte record per key, scattered); fastest while that
  *     scratch stays in the L2. FILTER_TCF_PATH_TILED: a partition by tile of
  *     consecutive blocks in coalesced passes, then a shared-memory sort per
- *     tile; fastest for large tables and batches. FILTER_TCF_PATH_AUTO takes
- *     TILED when the table has at least tcf_tiled_min_blocks blocks and the
- *     batch at least as many keys (0: 2^23).
+ *     tile. FILTER_TCF_PATH_AUTO takes TILED when the table has at least
+ *     tcf_tiled_min_blocks blocks and the batch at least as many keys; with
+ *     tcf_tiled_min_blocks = 0, for tables of 2^22 blocks or more, and for
+ *     removes of four keys a block or more on tables of 2^12 blocks or more.
  *   tcf_tile_target: tiled path, the expected candidates per tile, 128 ..
- *     1024 (0: 1024).
+ *     1024 (0: 2048).
  *   gqf_region_groups: GQF batches with at most this many distinct
  *     fingerprints per 256 quotients on average are inserted or removed in
  *     place (even-odd regions); denser ones take the merge (0: 8).

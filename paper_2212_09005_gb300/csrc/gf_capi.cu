@@ -36,15 +36,24 @@ bool tuning_valid(const filter_tuning &t)
     return true;
 }
 
-bool tcf_tiled(const filter_tuning &t, uint64_t nb, uint64_t n)
+bool tcf_tiled(const filter_tuning &t, uint64_t nb, uint64_t n, bool del)
 {
     if (t.tcf_path == FILTER_TCF_PATH_BLOCK) return false;
     if (t.tcf_path == FILTER_TCF_PATH_TILED) return true;
-    const uint64_t m = t.tcf_tiled_min_blocks ? t.tcf_tiled_min_blocks : (1ull << 23);
-    return nb >= m && n >= m;
+    if (t.tcf_tiled_min_blocks) return nb >= t.tcf_tiled_min_blocks && n >= t.tcf_tiled_min_blocks;
+    // From 2^22 blocks the counters and records of the counting sort leave the
+    // L2: a 2^28-slot table takes 2^24 keys to 90 % load in 13.9 ms by unit, in
+    // 32.7 by block, and 65533 of them a call 0.11 and 0.18 ms an insert and
+    // remove; at 2^22 blocks 3.80 against 4.30 and 0.072 against 0.077. Below,
+    // inserts are as fast by block or faster (2^20 blocks, 2^21 keys: 1.33 ms
+    // against 1.48). Removes of four keys a block or more are faster by unit on
+    // any table, the unit step needing no scratch per block (2^20 blocks, 2^22
+    // keys: 0.67 ms against 0.87; 2^12 blocks, 2^14 keys 126 us against 139;
+    // 8-bit tags 0.77 ms against 1.72).
+    return nb >= (1ull << 22) || (del && nb >= (1ull << 12) && n >= 4 * nb);
 }
 
-uint32_t tcf_tile_target(const filter_tuning &t) { return t.tcf_tile_target ? t.tcf_tile_target : 1024u; }
+uint32_t tcf_tile_target(const filter_tuning &t) { return t.tcf_tile_target ? t.tcf_tile_target : 2048u; }
 uint64_t gqf_region_groups(const filter_tuning &t) { return t.gqf_region_groups ? t.gqf_region_groups : 8u; }
 
 }  // namespace gf

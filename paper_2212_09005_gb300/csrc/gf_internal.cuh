@@ -41,14 +41,15 @@ struct DevCounters {
     unsigned long long backing;
     unsigned long long overflow;  // GQF merge: 1 if a run would pass the tail
     unsigned int pend[8];         // TCF: pending-list lengths per phase
-    unsigned int tile_ctr[4];     // dynamic tile counters
-    long long gqf_end;            // GQF merge: end of the last run (dry runs)
-    unsigned int touched[4];      // TCF sparse phases: touched destinations (cursor must follow)
+    unsigned int touched[4];      // TCF sparse phases: touched destinations
     unsigned int cursor[4];       // TCF sparse phases: records placed so far
+    unsigned int bar, pad;        // arrivals at the barriers of a cooperative launch
+    long long gqf_end;            // GQF merge: end of the last run (dry runs)
     unsigned long long wflag;     // GQF counted insert: 1 if some count was 0
 };
-static_assert(offsetof(DevCounters, cursor) == offsetof(DevCounters, touched) + sizeof(DevCounters::touched),
-              "touched and cursor are cleared together");
+// a TCF bulk call clears its words, pend to bar, at once
+static constexpr size_t CALL_WORDS_BYTES = 18 * sizeof(unsigned int);
+static_assert(offsetof(DevCounters, gqf_end) == offsetof(DevCounters, pend) + CALL_WORDS_BYTES, "pend to bar are adjacent");
 
 // ---------------------------------------------------------------------------
 // Hashing (paper Sec. 5.1 fingerprint h; Sec. 4 block/tag hash). Bijective:
@@ -98,67 +99,6 @@ __host__ __device__ __forceinline__ uint64_t tcf_bucket_of(uint64_t e, const Tcf
 {
     return tcf_bucket(e & ~(uint64_t)G.vmask, G.nbk);
 }
-
-// ---------------------------------------------------------------------------
-// One-dimensional bulk copies between global and shared memory (the TMA's
-// cp.async.bulk, sm_90 and later), completed through an mbarrier. Addresses
-// 16-byte aligned, sizes a multiple of 16 bytes.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-// one arrival that also announces `bytes` of copies completing on the barrier
-__device__ __forceinline__ void mbar_arrive_expect(uint64_t *bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// the phase with this parity completed, or false after `limit` tries
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, uint32_t limit)
-{
-    for (uint32_t i = 0; i < limit; i++)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
-
-__device__ __forceinline__ void bulk_load(void *dst_smem, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst_smem)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
-__device__ __forceinline__ void bulk_store(void *dst, const void *src_smem, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src_smem)),
-                 "r"(bytes)
-                 : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-
-// the shared-memory sources of this thread's bulk stores have been read
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// this thread's bulk stores are complete
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// this thread's shared-memory writes become visible to the bulk copies
-__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
 // Filter groups: member m of a group call owns keys [off[m], off[m + 1]).
@@ -310,6 +250,146 @@ void radix_sort_u64(const uint64_t *keys_in, uint64_t *keys_out, uint64_t *keys_
 void fingerprint_for_sort(const uint64_t *keys, uint64_t n, const PHash &H, uint64_t *fp, uint32_t *idx,
                           uint32_t bits, uint32_t *tmp, cudaStream_t st);
 
+// ---------------------------------------------------------------------------
+// Partition of 64-bit values into units by their top bits (gf_msd.cu), in one
+// or two passes of at most MP_BINS bins; the order inside a bin is free.
+// ---------------------------------------------------------------------------
+static constexpr int MP_T = 512;             // threads of a partition tile
+static constexpr int MP_I = 8;               // values per thread
+static constexpr int MP_TILE = MP_T * MP_I;
+static constexpr int MP_BINS = 512;          // most bins of a pass
+
+// scratch of one partition: words of one array, the first `zero_words` of them
+// cleared before each
+struct MsdScratch {
+    uint32_t *cnt1;     // first pass: values per bin
+    uint32_t *misc;     // [0] unit ticket, [1] squeezed chunks, [2] oversized units, [3] CTAs done
+    uint64_t *look;     // look-back words of the units
+    uint32_t *cnt2;     // second pass: values per unit
+    uint32_t *st1, *cur1, *tile1, *htile1;  // first-pass bins: starts, cursors, first tiles of either kind
+    uint32_t *st2, *cur2;                   // units: starts, cursors
+    uint32_t *chunk0;   // a squeezed unit's first chunk
+    uint32_t *distinct; // the units' distinct values
+    uint32_t *big;      // units of more than big_cap values (null: not listed)
+    uint32_t big_cap, chunk;                // values of a listed unit above which it goes by chunks
+    uint32_t *chunk_unit, *chunk_cnt;       // chunks: their unit, the pairs left
+    uint64_t zero_words, words;
+};
+MsdScratch msd_scratch(uint32_t *base, uint64_t n, uint32_t k, bool two, bool lookback, bool big);
+
+// the second pass: the values of `in`, in first-pass bins, into the units of
+// their digit (value >> shift) & (2^bits2 - 1); n: at least their number
+void msd_second_pass(const MsdScratch &s, const uint64_t *in, uint64_t *out, uint64_t n, uint32_t nb1, uint32_t shift,
+                     uint32_t bits2, const char *hist_name, const char *part_name, cudaStream_t st);
+
+// exclusive scan of one value per thread of a CTA of T threads
+template <int T>
+__device__ __forceinline__ uint32_t cta_scan(uint32_t v, uint32_t *s_warp)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    __syncthreads();
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    uint32_t pre = 0;
+#pragma unroll
+    for (int w = 0; w < T / 32; w++) pre += w < warp ? s_warp[w] : 0u;
+    return pre + incl - v;
+}
+
+// oversized units are listed, those of more than a chunk chunk by chunk too
+__device__ __forceinline__ void list_big(const MsdScratch &s, uint32_t unit, uint32_t c)
+{
+    if (!s.big || c <= s.big_cap) return;
+    s.big[atomicAdd(&s.misc[2], 1u)] = unit;
+    if (c <= s.chunk) return;
+    const uint32_t m = (c + s.chunk - 1) / s.chunk, at = atomicAdd(&s.misc[1], m);
+    s.chunk0[unit] = at;
+    for (uint32_t i = 0; i < m; i++) s.chunk_unit[at + i] = unit;
+}
+
+// The end of a first histogram (MP_T threads a CTA, the shared counts added to
+// s.cnt1): the last CTA turns the counts into starts, cursors and tiles of the
+// nb bins, and leaves the counts at zero.
+static constexpr int MH_TILE = 4 * MP_TILE;  // values a CTA counts in the second histogram
+__device__ __forceinline__ void hist_end(const MsdScratch &s, uint32_t nb, bool two)
+{
+    static_assert(MP_BINS == MP_T, "a thread per bin");
+    __shared__ uint32_t s_warp[MP_T / 32];
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&s.misc[3], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const uint32_t b = threadIdx.x, c = b < nb ? __ldcg(&s.cnt1[b]) : 0u;
+    const uint32_t st = cta_scan<MP_T>(c, s_warp);
+    const uint32_t tiles = (c + MP_TILE - 1) / MP_TILE, t0 = cta_scan<MP_T>(tiles, s_warp);
+    const uint32_t htiles = (c + MH_TILE - 1) / MH_TILE, h0 = cta_scan<MP_T>(htiles, s_warp);
+    if (b == 0) s.misc[3] = 0;
+    if (b >= nb) return;
+    s.cnt1[b] = 0;
+    s.st1[b] = s.cur1[b] = st;
+    s.tile1[b] = t0;
+    s.htile1[b] = h0;
+    if (b == nb - 1) {
+        s.st1[nb] = st + c;
+        s.tile1[nb] = t0 + tiles;
+        s.htile1[nb] = h0 + htiles;
+    }
+    if (!two) list_big(s, b, c);
+}
+
+// One partition tile: the cnt values v (value r * MP_T + t of the tile in
+// thread t) are ranked by bin, staged in bin order and written as runs. The
+// room in each bin is one returning global atomic per tile and bin, issued
+// before the staging that hides it. HOT: a warp's values may all share a bin.
+struct PartSmem {
+    uint64_t key[MP_TILE];
+    uint32_t cnt[MP_BINS];    // values per bin, then the bins' tile starts
+    uint32_t delta[MP_BINS];  // global start - tile start
+    uint32_t warp[MP_T / 32];
+};
+template <bool HOT, class Digit>
+__device__ __forceinline__ void part_tile(PartSmem &S, const uint64_t (&v)[MP_I], uint32_t cnt, uint32_t nb,
+                                          Digit digit, uint32_t *cur, uint64_t *__restrict__ out)
+{
+    const int lane = threadIdx.x & 31;
+    for (uint32_t b = threadIdx.x; b < nb; b += MP_T) S.cnt[b] = 0;
+    __syncthreads();
+    uint32_t rank[MP_I];
+#pragma unroll
+    for (int r = 0; r < MP_I; r++) {
+        const uint32_t d = r * MP_T + threadIdx.x < cnt ? digit(v[r], r) : nb;
+        const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
+        if (HOT && __all_sync(0xffffffffu, d == d0)) {  // one update for the warp's values
+            uint32_t b = 0;
+            if (lane == 0 && d0 < nb) b = atomicAdd(&S.cnt[d0], 32u);
+            rank[r] = __shfl_sync(0xffffffffu, b, 0) + lane;
+        } else if (d < nb) {
+            rank[r] = atomicAdd(&S.cnt[d], 1u);
+        }
+    }
+    __syncthreads();
+    const uint32_t c = threadIdx.x < nb ? S.cnt[threadIdx.x] : 0u;
+    uint32_t room = 0;
+    if (c) room = atomicAdd(&cur[threadIdx.x], c);
+    const uint32_t st = cta_scan<MP_T>(c, S.warp);
+    if (threadIdx.x < nb) S.cnt[threadIdx.x] = st;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < MP_I; r++)
+        if (r * MP_T + threadIdx.x < cnt) S.key[S.cnt[digit(v[r], r)] + rank[r]] = v[r];
+    if (c) S.delta[threadIdx.x] = room - st;
+    __syncthreads();
+}
+
 // Distinct sorted values of n keys and the copies before each (gf_msd.cu): for
 // each group g, uniq[g] ascending and start[g] = the keys below it, start[m] =
 // n and *m_out = m. The values are the keys' fingerprints (H set), or the keys
@@ -390,8 +470,8 @@ struct TcfState {
     uint32_t *tcount;  // one per CTA of a phase launch
     uint32_t *dlist;   // max_batch
     uint64_t *seg;     // max_batch: start << 32 | count
-    // tiled phases: per-tile counts and cursors, and a second pending list
-    uint32_t *tcur;    // 2 * ceil(nb / 32) + 264
+    // unit phases: the partition's scratch, and a second pending list
+    uint32_t *tcur;    // tcf_unit_words(max_batch)
     uint64_t *pb;      // max_batch
     uint32_t *pbi;     // max_batch
 };
@@ -464,8 +544,8 @@ struct filter_group {
 namespace gf {
 // tuning values with the defaults filled in; false if one is out of range
 bool tuning_valid(const filter_tuning &t);
-// TCF bulk calls: the tiled path for this table and batch?
-bool tcf_tiled(const filter_tuning &t, uint64_t nb, uint64_t n);
+// TCF bulk calls: the tiled path for this table, batch and direction?
+bool tcf_tiled(const filter_tuning &t, uint64_t nb, uint64_t n, bool del);
 bool tcf_geom_supported(uint32_t f, uint32_t B);
 uint32_t tcf_tile_target(const filter_tuning &t);
 uint64_t gqf_region_groups(const filter_tuning &t);

@@ -22,11 +22,6 @@
 
 namespace gf {
 
-static constexpr int MP_T = 512;                // threads of a partition tile
-static constexpr int MP_I = 8;                  // keys per thread
-static constexpr int MP_TILE = MP_T * MP_I;
-static constexpr int MP_BINS = 512;             // most bins of a pass
-static constexpr int MH_TILE = 4 * MP_TILE;     // keys a CTA counts in the second histogram
 static constexpr int MU_T = 256;                // threads of a unit, a chunk or an oversized unit
 static constexpr uint32_t MU_CAP = 2560;        // keys that a unit sorts in shared memory
 static constexpr uint32_t MU_BBITS = 12, MU_BUCKETS = 1u << MU_BBITS;  // buckets of that sort
@@ -40,24 +35,7 @@ static constexpr uint32_t EMPTY = 0xffffffffu;  // (values below have at most 31
 
 static_assert(MP_BINS <= MP_T, "a thread per bin");
 
-// ---------------------------------------------------------------------------
-// Scratch: one array of words, the first `zero_words` of them cleared per call
-// ---------------------------------------------------------------------------
-struct MsdScratch {
-    uint32_t *cnt1;     // first pass: keys per bin
-    uint32_t *misc;     // [0] unit ticket, [1] squeezed chunks, [2] oversized units
-    uint64_t *look;     // look-back words of the units
-    uint32_t *cnt2;     // second pass: keys per unit
-    uint32_t *st1, *cur1, *tile1, *htile1;  // first-pass bins: starts, cursors, first tiles of either kind
-    uint32_t *st2, *cur2;                   // units: starts, cursors
-    uint32_t *chunk0;   // a squeezed unit's first chunk
-    uint32_t *distinct; // the units' distinct values
-    uint32_t *big;      // oversized units
-    uint32_t *chunk_unit, *chunk_cnt;       // chunks: their unit, the pairs left
-    uint64_t zero_words, words;
-};
-
-static MsdScratch msd_scratch(uint32_t *base, uint64_t n, uint32_t k, bool two, bool lookback)
+MsdScratch msd_scratch(uint32_t *base, uint64_t n, uint32_t k, bool two, bool lookback, bool big)
 {
     MsdScratch s;
     uint64_t at = 0;
@@ -78,11 +56,16 @@ static MsdScratch msd_scratch(uint32_t *base, uint64_t n, uint32_t k, bool two, 
     s.htile1 = take(MP_BINS + 1);
     s.st2 = take(two ? units + 1 : 0);
     s.cur2 = take(two ? units : 0);
-    s.chunk0 = take(units);
-    s.distinct = take(units);
-    s.big = take(n / MU_CAP + 1);
-    s.chunk_unit = take(chunks);
-    s.chunk_cnt = take(chunks);
+    s.chunk0 = s.distinct = s.big = s.chunk_unit = s.chunk_cnt = nullptr;
+    if (big) {
+        s.chunk0 = take(units);
+        s.distinct = take(units);
+        s.big = take(n / MU_CAP + 1);
+        s.chunk_unit = take(chunks);
+        s.chunk_cnt = take(chunks);
+    }
+    s.big_cap = MU_CAP;
+    s.chunk = MS_CHUNK;
     s.words = at;
     return s;
 }
@@ -99,9 +82,10 @@ __device__ __forceinline__ uint64_t msd_value(uint64_t key, const PHash &H)
 // keys per first-pass bin (value >> shift), one shared histogram per CTA
 template <bool HASH>
 __global__ void __launch_bounds__(MP_T) msd_hist1(const uint64_t *__restrict__ keys, uint64_t n, PHash H,
-                                                  uint32_t shift, uint32_t nb, uint32_t *cnt)
+                                                  uint32_t shift, uint32_t nb, MsdScratch s, bool two, uint32_t *m_out)
 {
     __shared__ uint32_t h[MP_BINS];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *m_out = 0;  // (the units count into it)
     for (uint32_t b = threadIdx.x; b < nb; b += MP_T) h[b] = 0;
     __syncthreads();
     const uint64_t step = (uint64_t)gridDim.x * MP_TILE;
@@ -120,59 +104,8 @@ __global__ void __launch_bounds__(MP_T) msd_hist1(const uint64_t *__restrict__ k
     }
     __syncthreads();
     for (uint32_t b = threadIdx.x; b < nb; b += MP_T)
-        if (h[b]) atomicAdd(&cnt[b], h[b]);
-}
-
-// exclusive scan of one value per thread of a CTA of T threads
-template <int T>
-__device__ __forceinline__ uint32_t cta_scan(uint32_t v, uint32_t *s_warp)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    __syncthreads();
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    uint32_t pre = 0;
-#pragma unroll
-    for (int w = 0; w < T / 32; w++) pre += w < warp ? s_warp[w] : 0u;
-    return pre + incl - v;
-}
-
-// oversized units are listed, those of more than MS_CHUNK keys chunk by chunk too
-__device__ __forceinline__ void list_big(const MsdScratch &s, uint32_t unit, uint32_t c)
-{
-    if (c <= MU_CAP) return;
-    s.big[atomicAdd(&s.misc[2], 1u)] = unit;
-    if (c <= MS_CHUNK) return;
-    const uint32_t m = (c + MS_CHUNK - 1) / MS_CHUNK, at = atomicAdd(&s.misc[1], m);
-    s.chunk0[unit] = at;
-    for (uint32_t i = 0; i < m; i++) s.chunk_unit[at + i] = unit;
-}
-
-// starts, cursors and tiles of the first-pass bins (one CTA)
-__global__ void __launch_bounds__(MP_BINS) msd_scan1(MsdScratch s, uint32_t nb, bool two, uint32_t *m_out)
-{
-    if (threadIdx.x == 0) *m_out = 0;  // (the units count into it)
-    __shared__ uint32_t s_warp[MP_BINS / 32];
-    const uint32_t b = threadIdx.x, c = b < nb ? s.cnt1[b] : 0u;
-    const uint32_t st = cta_scan<MP_BINS>(c, s_warp);
-    const uint32_t tiles = (c + MP_TILE - 1) / MP_TILE, t0 = cta_scan<MP_BINS>(tiles, s_warp);
-    const uint32_t htiles = (c + MH_TILE - 1) / MH_TILE, h0 = cta_scan<MP_BINS>(htiles, s_warp);
-    if (b >= nb) return;
-    s.st1[b] = s.cur1[b] = st;
-    s.tile1[b] = t0;
-    s.htile1[b] = h0;
-    if (b == nb - 1) {
-        s.st1[nb] = st + c;
-        s.tile1[nb] = t0 + tiles;
-        s.htile1[nb] = h0 + htiles;
-    }
-    if (!two) list_big(s, b, c);
+        if (h[b]) atomicAdd(&s.cnt1[b], h[b]);
+    hist_end(s, nb, two);
 }
 
 // the bin whose tiles hold tile t, or nb past the last tile
@@ -222,7 +155,8 @@ __global__ void __launch_bounds__(MP_T) msd_hist2(const uint64_t *__restrict__ v
         if (h[b]) atomicAdd(&s.cnt2[(j << bits2) + b], h[b]);
 }
 
-// starts and cursors of the units of first-pass bin blockIdx.x
+// starts and cursors of the units of first-pass bin blockIdx.x; the counts are
+// left at zero
 __global__ void __launch_bounds__(MP_BINS) msd_scan2(MsdScratch s, uint32_t nb1, uint32_t bits2)
 {
     __shared__ uint32_t s_warp[MP_BINS / 32];
@@ -230,28 +164,24 @@ __global__ void __launch_bounds__(MP_BINS) msd_scan2(MsdScratch s, uint32_t nb1,
     const uint32_t c = b < (1u << bits2) ? s.cnt2[u] : 0u;
     const uint32_t st = s.st1[j] + cta_scan<MP_BINS>(c, s_warp);
     if (b >= (1u << bits2)) return;
+    s.cnt2[u] = 0;
     s.st2[u] = s.cur2[u] = st;
     if (u == (nb1 << bits2) - 1) s.st2[u + 1] = st + c;
     list_big(s, u, c);
 }
 
 // ---------------------------------------------------------------------------
-// A partition pass: a tile's keys are ranked by bin, staged in bin order and
-// written as runs. FIRST: tiles of the batch, keys hashed when HASH; else
-// tiles of a first-pass bin, whose keys go to its units. The room in each bin
-// is one returning global atomic per tile and bin, issued before the staging
-// that hides it. Bound by the shared-memory pipe (80 % busy with the rank
-// atomics and the staging; 16 bytes a key at 4.4 TB/s); 48 warps per SM.
+// A partition pass. FIRST: tiles of the batch, keys hashed when HASH; else
+// tiles of a first-pass bin, whose keys go to its units. Bound by the
+// shared-memory pipe (80 % busy with the rank atomics and the staging; 16 bytes
+// a key at 4.4 TB/s); 48 warps per SM.
 // ---------------------------------------------------------------------------
 template <bool FIRST, bool HASH>
 __global__ void __launch_bounds__(MP_T, 3) msd_part(const uint64_t *__restrict__ in, uint32_t n, PHash H, MsdScratch s,
                                                     uint32_t nb1, uint32_t shift, uint32_t bits,
                                                     uint64_t *__restrict__ out)
 {
-    __shared__ uint64_t s_key[MP_TILE];
-    __shared__ uint32_t s_cnt[MP_BINS];    // keys per bin, then the bins' tile starts
-    __shared__ uint32_t s_delta[MP_BINS];  // global start - tile start
-    __shared__ uint32_t s_warp[MP_T / 32];
+    __shared__ PartSmem S;
     const uint32_t nb = 1u << bits;
     uint32_t base, end;
     uint32_t *cur;
@@ -267,49 +197,40 @@ __global__ void __launch_bounds__(MP_T, 3) msd_part(const uint64_t *__restrict__
         cur = s.cur2 + ((uint64_t)j << bits);
     }
     const uint32_t cnt = end - base < MP_TILE ? end - base : MP_TILE;
-    const int lane = threadIdx.x & 31;
     uint64_t v[MP_I];
 #pragma unroll
     for (int r = 0; r < MP_I; r++) {
         const uint32_t i = r * MP_T + threadIdx.x;
         v[r] = i < cnt ? __ldcs(in + base + i) : 0ull;
     }
-    for (uint32_t b = threadIdx.x; b < nb; b += MP_T) s_cnt[b] = 0;
-    __syncthreads();
-    uint32_t rank[MP_I];
+    if (FIRST)
 #pragma unroll
-    for (int r = 0; r < MP_I; r++) {
-        if (FIRST) v[r] = msd_value<HASH>(v[r], H);
-        const uint32_t d = r * MP_T + threadIdx.x < cnt ? (uint32_t)(v[r] >> shift) & (nb - 1) : nb;
-        const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
-        if (!FIRST && __all_sync(0xffffffffu, d == d0)) {  // a hot unit: one update for the warp's keys
-            uint32_t b = 0;
-            if (lane == 0 && d0 < nb) b = atomicAdd(&s_cnt[d0], 32u);
-            rank[r] = __shfl_sync(0xffffffffu, b, 0) + lane;
-        } else if (d < nb) {
-            rank[r] = atomicAdd(&s_cnt[d], 1u);
-        }
-    }
-    __syncthreads();
-    const uint32_t c = threadIdx.x < nb ? s_cnt[threadIdx.x] : 0u;
-    uint32_t room = 0;
-    if (c) room = atomicAdd(&cur[threadIdx.x], c);
-    const uint32_t st = cta_scan<MP_T>(c, s_warp);
-    if (threadIdx.x < nb) s_cnt[threadIdx.x] = st;
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < MP_I; r++)
-        if (r * MP_T + threadIdx.x < cnt) s_key[s_cnt[(uint32_t)(v[r] >> shift) & (nb - 1)] + rank[r]] = v[r];
-    if (c) s_delta[threadIdx.x] = room - st;
-    __syncthreads();
+        for (int r = 0; r < MP_I; r++) v[r] = msd_value<HASH>(v[r], H);
+    part_tile<!FIRST>(S, v, cnt, nb, [=](uint64_t x, int) { return (uint32_t)(x >> shift) & (nb - 1); }, cur, out);
 #pragma unroll
     for (int r = 0; r < MP_I; r++) {
         const uint32_t i = r * MP_T + threadIdx.x;
         if (i < cnt) {
-            const uint64_t x = s_key[i];
-            __stcs(out + (s_delta[(uint32_t)(x >> shift) & (nb - 1)] + i), x);
+            const uint64_t x = S.key[i];
+            __stcs(out + (S.delta[(uint32_t)(x >> shift) & (nb - 1)] + i), x);
         }
     }
+}
+
+void msd_second_pass(const MsdScratch &s, const uint64_t *in, uint64_t *out, uint64_t n, uint32_t nb1, uint32_t shift,
+                     uint32_t bits2, const char *hist_name, const char *part_name, cudaStream_t st)
+{
+    {
+        TraceScope ts_(hist_name, n, st);
+        msd_hist2<<<(unsigned)((n + MH_TILE - 1) / MH_TILE) + nb1, MP_T, 0, st>>>(in, s, nb1, shift, bits2);
+    }
+    {
+        TraceScope ts_("msd_scan2", (uint64_t)nb1 << bits2, st);
+        msd_scan2<<<nb1, MP_BINS, 0, st>>>(s, nb1, bits2);
+    }
+    TraceScope ts_(part_name, n, st);
+    msd_part<false, false><<<(unsigned)((n + MP_TILE - 1) / MP_TILE) + nb1, MP_T, 0, st>>>(in, (uint32_t)n, PHash{}, s, nb1,
+                                                                                         shift, bits2, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -729,7 +650,7 @@ bool msd_groups(const uint64_t *keys, uint64_t n, const PHash *H, uint32_t bits,
     const bool two = k > 9;
     const uint32_t b1 = two ? (k + 1) / 2 : k, b2 = k - b1, rbits = bits - k;
     if (k == 0 || k > 18 || rbits > 31) return false;
-    const MsdScratch s = msd_scratch(tmp, n, k, two, ordered);
+    const MsdScratch s = msd_scratch(tmp, n, k, two, ordered, true);
     if (s.words > tmp_words) return false;
     const PHash h = H ? *H : PHash{};
     const uint32_t units = 1u << k;
@@ -739,31 +660,15 @@ bool msd_groups(const uint64_t *keys, uint64_t n, const PHash *H, uint32_t bits,
     {
         TraceScope ts_("msd_hist1", n, st);
         const int g = grid_for(tiles * (uint64_t)MP_T, MP_T, 4);
-        if (H) msd_hist1<true><<<g, MP_T, 0, st>>>(keys, n, h, bits - b1, 1u << b1, s.cnt1);
-        else msd_hist1<false><<<g, MP_T, 0, st>>>(keys, n, h, bits - b1, 1u << b1, s.cnt1);
-    }
-    {
-        TraceScope ts_("msd_scan1", 1u << b1, st);
-        msd_scan1<<<1, MP_BINS, 0, st>>>(s, 1u << b1, two, m_out);
+        if (H) msd_hist1<true><<<g, MP_T, 0, st>>>(keys, n, h, bits - b1, 1u << b1, s, two, m_out);
+        else msd_hist1<false><<<g, MP_T, 0, st>>>(keys, n, h, bits - b1, 1u << b1, s, two, m_out);
     }
     {
         TraceScope ts_("msd_part", n, st);
         if (H) msd_part<true, true><<<tiles, MP_T, 0, st>>>(keys, (uint32_t)n, h, s, 0, bits - b1, b1, buf_a);
         else msd_part<true, false><<<tiles, MP_T, 0, st>>>(keys, (uint32_t)n, h, s, 0, bits - b1, b1, buf_a);
     }
-    if (two) {
-        const unsigned nb1 = 1u << b1;
-        {
-            TraceScope ts_("msd_hist2", n, st);
-            msd_hist2<<<(unsigned)((n + MH_TILE - 1) / MH_TILE) + nb1, MP_T, 0, st>>>(buf_a, s, nb1, rbits, b2);
-        }
-        {
-            TraceScope ts_("msd_scan2", units, st);
-            msd_scan2<<<nb1, MP_BINS, 0, st>>>(s, nb1, b2);
-        }
-        TraceScope ts_("msd_part2", n, st);
-        msd_part<false, false><<<tiles + nb1, MP_T, 0, st>>>(buf_a, (uint32_t)n, h, s, nb1, rbits, b2, buf_b);
-    }
+    if (two) msd_second_pass(s, buf_a, buf_b, n, 1u << b1, rbits, b2, "msd_hist2", "msd_part2", st);
     const uint32_t *ust = two ? s.st2 : s.st1;
     if (n > MS_CHUNK) {
         TraceScope ts_("msd_squeeze", 0, st);

@@ -408,10 +408,10 @@ __device__ __forceinline__ void cta_chunk(uint64_t n, uint64_t &c0, uint64_t &c1
 // candidates, as in the later phases) also list each destination the first
 // time it is hit, per CTA chunk, in tlist[c0 ..] with the count in tcount.
 template <int SRC, int DST, bool SPARSE>
-__global__ void __launch_bounds__(TPB) tcf_group_hist(const uint64_t *__restrict__ keys, const TcfPrep prep,
-                                                      uint64_t n_keys, const void *pend, const unsigned *npend,
-                                                      TcfGeom G, const uint8_t *fill, uint32_t *cnt,
-                                                      uint32_t *tlist, uint32_t *tcount, unsigned long long *units)
+__device__ __forceinline__ void tcf_group_hist_body(const uint64_t *__restrict__ keys, const TcfPrep prep,
+                                                    uint64_t n_keys, const void *pend, const unsigned *npend,
+                                                    TcfGeom G, const uint8_t *fill, uint32_t *cnt, uint32_t *tlist,
+                                                    uint32_t *tcount, unsigned long long *units)
 {
     const uint64_t n = (SRC == SRC_KEYS) ? n_keys : (uint64_t)*npend;
     note_units(units, n);
@@ -445,14 +445,23 @@ __global__ void __launch_bounds__(TPB) tcf_group_hist(const uint64_t *__restrict
     }
 }
 
+template <int SRC, int DST, bool SPARSE>
+__global__ void __launch_bounds__(TPB) tcf_group_hist(const uint64_t *__restrict__ keys, const TcfPrep prep,
+                                                      uint64_t n_keys, const void *pend, const unsigned *npend,
+                                                      TcfGeom G, const uint8_t *fill, uint32_t *cnt,
+                                                      uint32_t *tlist, uint32_t *tcount, unsigned long long *units)
+{
+    tcf_group_hist_body<SRC, DST, SPARSE>(keys, prep, n_keys, pend, npend, G, fill, cnt, tlist, tcount, units);
+}
+
 // Sparse phases: every touched destination gets a contiguous segment of the
 // record array (CTA-wide scan of the counts, one atomic per 256 destinations)
 // and an entry in the dense touched list. Same grid as the histogram.
-__global__ void __launch_bounds__(TPB) tcf_alloc(const unsigned *npend, uint64_t n_keys,
-                                                 const uint32_t *__restrict__ tlist,
-                                                 const uint32_t *__restrict__ tcount, const uint32_t *cnt,
-                                                 uint32_t *off, uint32_t *dlist, uint64_t *seg, unsigned *cursor,
-                                                 unsigned *nlist, unsigned long long *units)
+__device__ __forceinline__ void tcf_alloc_body(const unsigned *npend, uint64_t n_keys,
+                                               const uint32_t *__restrict__ tlist,
+                                               const uint32_t *__restrict__ tcount, const uint32_t *cnt,
+                                               uint32_t *off, uint32_t *dlist, uint64_t *seg, unsigned *cursor,
+                                               unsigned *nlist, unsigned long long *units)
 {
     __shared__ uint32_t s_w[TPB / 32];
     __shared__ uint32_t s_base, s_lbase;
@@ -495,14 +504,22 @@ __global__ void __launch_bounds__(TPB) tcf_alloc(const unsigned *npend, uint64_t
     }
 }
 
+__global__ void __launch_bounds__(TPB) tcf_alloc(const unsigned *npend, uint64_t n_keys,
+                                                 const uint32_t *__restrict__ tlist,
+                                                 const uint32_t *__restrict__ tcount, const uint32_t *cnt,
+                                                 uint32_t *off, uint32_t *dlist, uint64_t *seg, unsigned *cursor,
+                                                 unsigned *nlist, unsigned long long *units)
+{
+    tcf_alloc_body(npend, n_keys, tlist, tcount, cnt, off, dlist, seg, cursor, nlist, units);
+}
+
 // rec = (tag << 32) | batch index, or the backing entry with the index in recI
 template <int SRC, int DST>
-__global__ void __launch_bounds__(TPB) tcf_group_scatter(const uint64_t *__restrict__ keys, const TcfPrep prep,
-                                                         uint64_t n_keys, const void *pend, const unsigned *npend,
-                                                         TcfGeom G,
-                                                         const uint8_t *fill, uint32_t *cnt,
-                                                         const uint32_t *__restrict__ off, uint64_t *rec,
-                                                         uint32_t *recI, unsigned long long *units)
+__device__ __forceinline__ void tcf_group_scatter_body(const uint64_t *__restrict__ keys, const TcfPrep prep,
+                                                       uint64_t n_keys, const void *pend, const unsigned *npend,
+                                                       TcfGeom G, const uint8_t *fill, uint32_t *cnt,
+                                                       const uint32_t *__restrict__ off, uint64_t *rec,
+                                                       uint32_t *recI, unsigned long long *units)
 {
     const uint64_t n = (SRC == SRC_KEYS) ? n_keys : (uint64_t)*npend;
     note_units(units, n);
@@ -523,6 +540,17 @@ __global__ void __launch_bounds__(TPB) tcf_group_scatter(const uint64_t *__restr
             rec[pos] = ((uint64_t)k.t << 32) | i;
         }
     }
+}
+
+template <int SRC, int DST>
+__global__ void __launch_bounds__(TPB) tcf_group_scatter(const uint64_t *__restrict__ keys, const TcfPrep prep,
+                                                         uint64_t n_keys, const void *pend, const unsigned *npend,
+                                                         TcfGeom G,
+                                                         const uint8_t *fill, uint32_t *cnt,
+                                                         const uint32_t *__restrict__ off, uint64_t *rec,
+                                                         uint32_t *recI, unsigned long long *units)
+{
+    tcf_group_scatter_body<SRC, DST>(keys, prep, n_keys, pend, npend, G, fill, cnt, off, rec, recI, units);
 }
 
 // ---------------------------------------------------------------------------
@@ -644,11 +672,10 @@ struct RejSink {
 // every lane reaches the sink's reserve in every iteration and its flush
 // after the last one.
 template <int F>
-__global__ void __launch_bounds__(TPB) tcf_block_insert(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
-                                                        const uint64_t *__restrict__ rec, int phase,
-                                                        uint32_t cap, uint32_t *pend32, uint64_t *pend64,
-                                                        unsigned *npend, const TcfPrep prep,
-                                                        unsigned long long *units)
+__device__ __forceinline__ void tcf_block_insert_body(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
+                                                      const uint64_t *__restrict__ rec, int phase, uint32_t cap,
+                                                      uint32_t *pend32, uint64_t *pend64, unsigned *npend,
+                                                      const TcfPrep prep, unsigned long long *units)
 {
     constexpr int B = Blk<F>::B;
     __shared__ uint64_t s_sink[TPB / 32][SINK_CAP];
@@ -735,6 +762,16 @@ __global__ void __launch_bounds__(TPB) tcf_block_insert(TcfGeom G, uint8_t *bloc
         }
     }
     sink.flush();
+}
+
+template <int F>
+__global__ void __launch_bounds__(TPB) tcf_block_insert(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
+                                                        const uint64_t *__restrict__ rec, int phase,
+                                                        uint32_t cap, uint32_t *pend32, uint64_t *pend64,
+                                                        unsigned *npend, const TcfPrep prep,
+                                                        unsigned long long *units)
+{
+    tcf_block_insert_body<F>(G, blocks, fill, P, rec, phase, cap, pend32, pend64, npend, prep, units);
 }
 
 // One backing bucket q: cnt candidates (entry(j), index(j)) taken in (entry,
@@ -857,10 +894,10 @@ __device__ __forceinline__ void bucket_remove_step(const TcfGeom &G, uint64_t *b
 }
 
 // backing buckets of a phase: candidates (entry in rec, index in recI)
-__global__ void __launch_bounds__(TPB) tcf_bucket_insert(TcfGeom G, uint64_t *bk, PhaseDst P,
-                                                         const uint64_t *__restrict__ rec,
-                                                         const uint32_t *__restrict__ recI, uint8_t *status,
-                                                         DevCounters *ctr, unsigned long long *units)
+__device__ __forceinline__ void tcf_bucket_insert_body(TcfGeom G, uint64_t *bk, PhaseDst P,
+                                                       const uint64_t *__restrict__ rec,
+                                                       const uint32_t *__restrict__ recI, uint8_t *status,
+                                                       DevCounters *ctr, unsigned long long *units)
 {
     const uint64_t nd = phase_count(P, G.nbk);
     note_units(units, nd);  // units: buckets with candidates
@@ -873,14 +910,22 @@ __global__ void __launch_bounds__(TPB) tcf_bucket_insert(TcfGeom G, uint64_t *bk
     }
 }
 
+__global__ void __launch_bounds__(TPB) tcf_bucket_insert(TcfGeom G, uint64_t *bk, PhaseDst P,
+                                                         const uint64_t *__restrict__ rec,
+                                                         const uint32_t *__restrict__ recI, uint8_t *status,
+                                                         DevCounters *ctr, unsigned long long *units)
+{
+    tcf_bucket_insert_body(G, bk, P, rec, recI, status, ctr, units);
+}
+
 // ---------------------------------------------------------------------------
 // Bulk delete: per-block matching. For each tag present c times in the block,
 // the c smallest (tag, index) candidates with that tag remove one copy each.
 // ---------------------------------------------------------------------------
 template <int F>
-__global__ void __launch_bounds__(TPB) tcf_block_remove(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
-                                                        const uint64_t *__restrict__ rec, uint32_t *pend32,
-                                                        unsigned *npend, unsigned long long *units)
+__device__ __forceinline__ void tcf_block_remove_body(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
+                                                      const uint64_t *__restrict__ rec, uint32_t *pend32,
+                                                      unsigned *npend, unsigned long long *units)
 {
     constexpr int B = Blk<F>::B;
     __shared__ uint64_t s_sink[TPB / 32][SINK_CAP];
@@ -1006,11 +1051,19 @@ __global__ void __launch_bounds__(TPB) tcf_block_remove(TcfGeom G, uint8_t *bloc
     sink.flush();
 }
 
+template <int F>
+__global__ void __launch_bounds__(TPB) tcf_block_remove(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
+                                                        const uint64_t *__restrict__ rec, uint32_t *pend32,
+                                                        unsigned *npend, unsigned long long *units)
+{
+    tcf_block_remove_body<F>(G, blocks, fill, P, rec, pend32, npend, units);
+}
+
 // backing buckets of a remove
-__global__ void __launch_bounds__(TPB) tcf_bucket_remove(TcfGeom G, uint64_t *bk, PhaseDst P,
-                                                         const uint64_t *__restrict__ rec,
-                                                         const uint32_t *__restrict__ recI, uint8_t *status,
-                                                         DevCounters *ctr, unsigned long long *units)
+__device__ __forceinline__ void tcf_bucket_remove_body(TcfGeom G, uint64_t *bk, PhaseDst P,
+                                                       const uint64_t *__restrict__ rec,
+                                                       const uint32_t *__restrict__ recI, uint8_t *status,
+                                                       DevCounters *ctr, unsigned long long *units)
 {
     const uint64_t nd = phase_count(P, G.nbk);
     note_units(units, nd);  // units: buckets with candidates
@@ -1021,6 +1074,113 @@ __global__ void __launch_bounds__(TPB) tcf_bucket_remove(TcfGeom G, uint64_t *bk
         bucket_remove_step(G, bk, q, e - s, [&](uint32_t i) { return rec[s + i]; },
                            [&](uint32_t i) { return recI[s + i]; }, status, ctr);
     }
+}
+
+__global__ void __launch_bounds__(TPB) tcf_bucket_remove(TcfGeom G, uint64_t *bk, PhaseDst P,
+                                                         const uint64_t *__restrict__ rec,
+                                                         const uint32_t *__restrict__ recI, uint8_t *status,
+                                                         DevCounters *ctr, unsigned long long *units)
+{
+    tcf_bucket_remove_body(G, bk, P, rec, recI, status, ctr, units);
+}
+
+// ---------------------------------------------------------------------------
+// The later phases of a call in one cooperative launch: what the launches of
+// the sparse path do one after another (histogram, segments, scatter and steps
+// of the less full block, the other block and the backing buckets), with a
+// barrier of the grid in each launch's place, and an end as soon as a phase has
+// no candidates. Eleven launches cost about 45 us whatever they have to do.
+// ---------------------------------------------------------------------------
+// Every CTA of the grid arrives at *bar; thread 0 waits for the n-th round of
+// them. False when the wait gave up (the status word then shows a timeout).
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned round, unsigned long long *status)
+{
+    __shared__ bool s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned want = round * gridDim.x;
+        __threadfence();
+        atomicAdd(bar, 1u);
+        bool ok = false;
+        for (uint32_t i = 0; i < SPIN_LIMIT && !ok; i++) {
+            unsigned got;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(bar) : "memory");
+            ok = got >= want;
+        }
+        if (!ok) atomicOr(status, ST_TIMEOUT);
+        __threadfence();
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok;
+}
+
+// what the phases work on
+struct SparseArgs {
+    const uint64_t *keys;
+    uint64_t n;
+    TcfGeom G;
+    TcfPrep prep;
+    uint8_t *blocks, *fill;
+    uint64_t *bk;
+    uint32_t *cnt, *off, *tlist, *tcount, *dlist, *pend0, *pend2;
+    uint64_t *rec, *pend1, *seg;
+    uint8_t *status;
+    DevCounters *ctr;
+    uint32_t unit_min;  // more candidates than this of the first phase here went by unit
+};
+
+// groups the candidates of one phase by the destinations that they touch
+template <int SRC, int DST>
+__device__ __forceinline__ bool sparse_group(const SparseArgs &A, const void *pend, const unsigned *npend, int slot,
+                                             uint32_t *recI, unsigned &round, PhaseDst &P)
+{
+    DevCounters *c = A.ctr;
+    tcf_group_hist_body<SRC, DST, true>(A.keys, A.prep, A.n, pend, npend, A.G, A.fill, A.cnt, A.tlist, A.tcount, nullptr);
+    if (!grid_barrier(&c->bar, ++round, &c->status)) return false;
+    tcf_alloc_body(npend, A.n, A.tlist, A.tcount, A.cnt, A.off, A.dlist, A.seg, &c->cursor[slot], &c->touched[slot], nullptr);
+    if (!grid_barrier(&c->bar, ++round, &c->status)) return false;
+    tcf_group_scatter_body<SRC, DST>(A.keys, A.prep, A.n, pend, npend, A.G, A.fill, A.cnt, A.off, A.rec, recI, nullptr);
+    if (!grid_barrier(&c->bar, ++round, &c->status)) return false;
+    P = PhaseDst{nullptr, A.dlist, A.seg, &c->touched[slot]};
+    return true;
+}
+
+__device__ __forceinline__ unsigned ld_now(const unsigned *p) { return *(const volatile unsigned *)p; }
+
+template <int F>
+__global__ void __launch_bounds__(TPB, 4) tcf_sparse_insert_coop(const SparseArgs A)
+{
+    unsigned *np = A.ctr->pend, round = 0;
+    PhaseDst P;
+    if (ld_now(&np[0]) == 0) return;  // (the same in every CTA)
+    if (ld_now(&np[0]) <= A.unit_min) {
+        if (!sparse_group<SRC_PEND_U32, DST_TARGET>(A, A.pend0, &np[0], 1, nullptr, round, P)) return;
+        tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 1, A.G.B, nullptr, A.pend1, &np[1], A.prep, nullptr);
+        if (!grid_barrier(&A.ctr->bar, ++round, &A.ctr->status) || ld_now(&np[1]) == 0) return;
+        if (!sparse_group<SRC_PEND_U64, DST_ALT>(A, A.pend1, &np[1], 2, nullptr, round, P)) return;
+        tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 2, A.G.B, A.pend2, nullptr, &np[2], A.prep, nullptr);
+        if (!grid_barrier(&A.ctr->bar, ++round, &A.ctr->status)) return;
+    }
+    if (ld_now(&np[2]) == 0) return;
+    if (!sparse_group<SRC_PEND_U32, DST_BUCKET>(A, A.pend2, &np[2], 3, A.pend0, round, P)) return;
+    tcf_bucket_insert_body(A.G, A.bk, P, A.rec, A.pend0, A.status, A.ctr, nullptr);
+}
+
+template <int F>
+__global__ void __launch_bounds__(TPB, 4) tcf_sparse_remove_coop(const SparseArgs A)
+{
+    unsigned *np = A.ctr->pend, round = 0;
+    PhaseDst P;
+    if (ld_now(&np[0]) == 0) return;
+    if (ld_now(&np[0]) <= A.unit_min) {
+        if (!sparse_group<SRC_PEND_U32, DST_B2>(A, A.pend0, &np[0], 1, nullptr, round, P)) return;
+        tcf_block_remove_body<F>(A.G, A.blocks, A.fill, P, A.rec, A.pend2, &np[2], nullptr);
+        if (!grid_barrier(&A.ctr->bar, ++round, &A.ctr->status)) return;
+    }
+    if (ld_now(&np[2]) == 0) return;
+    if (!sparse_group<SRC_PEND_U32, DST_BUCKET>(A, A.pend2, &np[2], 2, A.pend0, round, P)) return;
+    tcf_bucket_remove_body(A.G, A.bk, P, A.rec, A.pend0, A.status, A.ctr, nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -1148,714 +1308,685 @@ __global__ void __launch_bounds__(SM_T) tcf_small(const uint64_t *__restrict__ k
 }
 
 // ---------------------------------------------------------------------------
-// Tiled bulk phases. A phase groups its candidates by destination block in
-// two steps that keep every global write coalesced: a partition by tile (TB
-// consecutive blocks) in one or two counting passes, each staging a chunk of
-// candidates in shared memory in bin order before writing it out, then one
-// CTA per tile that sorts the tile's candidates by block in shared memory and
-// runs the per-block step (accept into the sorted block, or remove) with the
-// block loaded and stored by consecutive threads. A candidate record is
-// (dest << 16 | slot, batch index); inside a tile it becomes the per-block
-// record (slot << 32 | index) that the per-block steps take in (slot, index)
-// order. The partition passes write to L2-sized runs instead of scattering 8
-// bytes per key over a batch-sized array, which is what keeps large batches
-// (2^24 keys into 2^24 blocks) off the DRAM read-modify-write path.
+// Bulk phases by unit. A phase's candidates are partitioned by the top bits of
+// their destination block (one or two passes whose writes are runs, gf_msd.cu)
+// into units of two thousand candidates and their stretch of blocks; one CTA
+// per unit groups its candidates by block in shared memory, and a thread per
+// block that has some takes its step. A candidate is one word: the low bits of its
+// block, its slot and its batch index; the partition implies the bits above.
+// Against a counting sort by block (a counter, an offset and a scattered
+// record per block and key) every global write is a run, nothing is sized by
+// the table, and a phase's time goes with its candidates.
 // ---------------------------------------------------------------------------
-static constexpr int TT_TPB = 256;      // threads of the partition and tile kernels
-static constexpr int TT_CH = 2048;      // items per partition chunk (8 per thread)
-static constexpr int TT_BINS = 512;     // shared-memory bins of a partition chunk
-static constexpr uint32_t TT_CAP = 2048;  // candidates a tile stages in shared memory (8 per thread)
-static constexpr uint32_t TT_TB_MAX = 2048;
-static constexpr uint64_t TT_LEFT = 1ull << 63;  // stage entry: the candidate is left for the next phase
+static constexpr int TU_T = 512;             // threads of a unit
+static constexpr uint32_t TU_CAP = 3072;     // candidates that a unit holds in shared memory
+static constexpr int TU_PER = TU_CAP / TU_T;
+static constexpr uint32_t TU_BBITS = 12, TU_BUCKETS = 1u << TU_BBITS;  // buckets they are grouped by: a block or a few
+static constexpr uint32_t TU_HOT = 64;       // candidates of one bucket above which the CTA takes them
+static uint64_t tcf_unit_words(uint64_t max_n);  // scratch words of calls of up to max_n keys
+static MsdScratch tu_scratch(uint32_t *base, uint64_t max_n);
 
-// words of the tile counters a filter needs: counts (nt + 1), high-bin
-// cursors (nh) and tile cursors (nt), at the smallest tile size
-static uint64_t tt_counter_words(uint64_t nb) { return 2 * ((nb + 31) / 32) + 256 + 8; }
-
-// tile geometry of one call: tiles of 2^tb_log blocks; lo > 0: two passes,
-// the first by tile >> lo (nh bins), the second by tile
-struct TtGeom {
-    uint64_t nb, nt, nh;
-    uint32_t tb_log, lo;
+// geometry of one phase: 2^k units of 2^lbits blocks each
+struct TuGeom {
+    uint32_t k, b1, b2;      // unit bits, in one (b2 = 0) or two passes
+    uint32_t lbits;          // bits of a block inside its unit
+    uint32_t sbits, ibits;   // slot and index bits of a record
 };
 
 // where a phase's candidates come from: the call's keys (hashed here, or the
 // prepared keys of a group call), or a pending list (rec, idx) of n_dev items
-struct TtSrc {
+struct TuSrc {
     const uint64_t *keys;
-    const uint64_t *rec;
+    const uint64_t *rec;     // dest << 16 | slot
     const uint32_t *idx;
-    const unsigned *n_dev;  // pending lists: their length on the device
-    uint64_t n;             // keys: their number; pending lists: an upper bound
+    const unsigned *n_dev;   // pending lists: their length on the device,
+    uint32_t n_min;          // taken for zero up to this many (the cooperative launch takes them)
+    uint64_t n;              // keys: their number; pending lists: an upper bound
 };
 
-enum TtSrcKind : int { TT_KEYS = 0, TT_PEND = 1 };
-enum TtRule : int { TT_SAME = 0, TT_TARGET = 1 };              // dest: the record's block, or the less full
-enum TtNext : int { TT_NX_SAME = 0, TT_NX_OTHER = 1, TT_NX_IDX = 2 };  // what a reject becomes
+enum TuSrcKind : int { TU_KEYS = 0, TU_TARGET = 1, TU_SAME = 2 };      // dest: b1; the less full block; the record's
+enum TuNext : int { TU_NX_SAME = 0, TU_NX_OTHER = 1, TU_NX_IDX = 2 };  // what a candidate left becomes
 
-__device__ __forceinline__ uint64_t tt_count(const TtSrc &s) { return s.n_dev ? (uint64_t)*s.n_dev : s.n; }
+__device__ __forceinline__ uint64_t tu_count(const TuSrc &s)
+{
+    if (!s.n_dev) return s.n;
+    const unsigned m = *s.n_dev;
+    return m > s.n_min ? m : 0;
+}
 
 // the other block of the pair of candidate (b, slot, idx): b1 ^ b2 = g(tag)
 // for a single filter; group calls read the prepared pair
-__device__ __forceinline__ uint64_t tt_other(uint64_t b, uint32_t slot, uint32_t i, const TcfGeom &G,
-                                            const TcfPrep &P)
+__device__ __forceinline__ uint64_t tu_other(uint64_t b, uint32_t slot, uint32_t i, const TcfGeom &G, const TcfPrep &P)
 {
     if (P.bt) return (P.bt[i] >> 32) + P.b2[i] - b;
     return b ^ tcf_g(slot >> G.vbits, G.nb);
 }
 
-// candidate j of a phase as (dest << 16 | slot, index)
-template <int SRC, int RULE>
-__device__ __forceinline__ void tt_item(const TtSrc &s, uint64_t j, const TcfGeom &G, const TcfPrep &P,
-                                        const uint8_t *fill, uint64_t &rec, uint32_t &idx)
+// candidate j: its destination block; rec = its record
+template <int SRC>
+__device__ __forceinline__ uint64_t tu_item(const TuSrc &s, uint64_t j, const TcfGeom &G, const TcfPrep &P,
+                                            const uint8_t *fill, const TuGeom &U, uint64_t &rec)
 {
-    if (SRC == TT_KEYS) {
-        idx = (uint32_t)j;
+    uint64_t b;
+    uint32_t slot, idx = (uint32_t)j;
+    if (SRC == TU_KEYS) {
         if (P.bt) {
             const uint64_t v = P.bt[j];
-            rec = ((v >> 32) << 16) | (uint32_t)(v & 0xffffu);
+            b = v >> 32;
+            slot = (uint32_t)v;
         } else {
-            KeyInfo k = tcf_keyinfo(s.keys[j], G);
+            KeyInfo k = tcf_keyinfo(__ldcs(s.keys + j), G);
             if (P.vals) k.t |= P.vals[j] & G.vmask;
-            rec = (k.b1 << 16) | k.t;
+            b = k.b1;
+            slot = k.t;
         }
-        return;
+    } else {
+        const uint64_t r = s.rec[j];
+        idx = s.idx[j];
+        b = r >> 16;
+        slot = (uint32_t)(r & 0xffffu);
+        if (SRC == TU_TARGET) {
+            const uint64_t b2 = tu_other(b, slot, idx, G, P);
+            if (fill[b] > fill[b2]) b = b2;
+        }
     }
-    rec = s.rec[j];
-    idx = s.idx[j];
-    if (RULE == TT_TARGET) {
-        const uint64_t b1 = rec >> 16;
-        const uint32_t slot = (uint32_t)(rec & 0xffffu);
-        const uint64_t b2 = tt_other(b1, slot, idx, G, P);
-        const uint64_t d = fill[b1] <= fill[b2] ? b1 : b2;
-        rec = (d << 16) | slot;
+    rec = (b << (U.sbits + U.ibits)) | ((uint64_t)slot << U.ibits) | idx;  // (bits above 64 are the first pass's)
+    return b;
+}
+
+template <int SRC>
+__global__ void __launch_bounds__(MP_T) tu_hist(const TuSrc s, TcfGeom G, TcfPrep P, const uint8_t *fill, TuGeom U,
+                                                MsdScratch M, unsigned long long *units)
+{
+    __shared__ uint32_t h[MP_BINS];
+    const uint64_t n = tu_count(s);
+    note_units(units, n);
+    const uint32_t nb = 1u << U.b1, shift = U.lbits + U.b2;
+    for (uint32_t b = threadIdx.x; b < nb; b += MP_T) h[b] = 0;
+    __syncthreads();
+    for (uint64_t base = (uint64_t)blockIdx.x * MP_TILE; base < n; base += (uint64_t)gridDim.x * MP_TILE) {
+        uint64_t b[MP_I];
+#pragma unroll
+        for (int r = 0; r < MP_I; r++) {
+            const uint64_t j = base + r * MP_T + threadIdx.x;
+            uint64_t rec;
+            b[r] = j < n ? tu_item<SRC>(s, j, G, P, fill, U, rec) : 0;
+        }
+#pragma unroll
+        for (int r = 0; r < MP_I; r++)
+            if (base + r * MP_T + threadIdx.x < n) atomicAdd(&h[(uint32_t)(b[r] >> shift)], 1u);
+    }
+    __syncthreads();
+    for (uint32_t b = threadIdx.x; b < nb; b += MP_T)
+        if (h[b]) atomicAdd(&M.cnt1[b], h[b]);
+    hist_end(M, nb, U.b2 > 0);
+}
+
+// the first pass: a tile's records to the bins of their blocks' top bits
+template <int SRC>
+__global__ void __launch_bounds__(MP_T, 3) tu_part(const TuSrc s, TcfGeom G, TcfPrep P, const uint8_t *fill, TuGeom U,
+                                                   MsdScratch M, uint64_t *__restrict__ out, unsigned long long *units)
+{
+    __shared__ PartSmem S;
+    const uint64_t n = tu_count(s), base = (uint64_t)blockIdx.x * MP_TILE;
+    note_units(units, n);
+    if (base >= n) return;
+    const uint32_t cnt = n - base < MP_TILE ? (uint32_t)(n - base) : MP_TILE, shift = U.lbits + U.b2;
+    const uint32_t nb = 1u << U.b1, rshift = shift + U.sbits + U.ibits;
+    const bool whole = rshift + U.b1 <= 64;
+    uint64_t v[MP_I];
+    uint16_t bin[MP_I];
+#pragma unroll
+    for (int r = 0; r < MP_I; r++) {
+        const uint32_t i = r * MP_T + threadIdx.x;
+        if (i < cnt) bin[r] = (uint16_t)(tu_item<SRC>(s, base + i, G, P, fill, U, v[r]) >> shift);
+    }
+    part_tile<false>(S, v, cnt, nb, [&](uint64_t, int r) { return (uint32_t)bin[r]; }, M.cur1, out);
+#pragma unroll
+    for (int r = 0; r < MP_I; r++) {
+        const uint32_t i = r * MP_T + threadIdx.x;
+        if (i >= cnt) continue;
+        const uint64_t x = S.key[i];
+        uint32_t b;
+        if (whole) {
+            b = (uint32_t)(x >> rshift);
+        } else {  // the record does not hold its bin's bits: the last bin that starts at or before it
+            uint32_t hi = nb;
+            b = 0;
+            while (hi - b > 1) {
+                const uint32_t mid = (b + hi) >> 1;
+                if (S.cnt[mid] <= i) b = mid;
+                else hi = mid;
+            }
+        }
+        out[S.delta[b] + i] = x;
     }
 }
 
-// Counter words of a phase: cnt[nt + 1] | hcur[nh] | tcur[nt] | done.
-struct TtCtr {
-    uint32_t *cnt, *hcur, *tcur, *done;
+struct TuSmem {
+    uint32_t cnt[TU_BUCKETS / 2 + 4];  // per bucket, two to a word: records, then the first position
+    uint64_t a[TU_CAP];                // records by bucket
+    uint16_t head[TU_CAP], left[TU_CAP];  // buckets with records; positions of the records left
+    uint16_t hot[TU_CAP / TU_HOT];
+    uint32_t warp[TU_T / 32];
+    unsigned long long red[TU_T / 32];
+    uint32_t nhead, nleft, nhot, base;
+    unsigned long long bytes;
 };
 
-__device__ __forceinline__ TtCtr tt_ctr(uint32_t *base, const TtGeom &tg)
+// Groups a unit's n records (record r * TU_T + t in thread t) by bucket into
+// S.a and lists the buckets that have some in S.head. All threads pass its
+// barriers.
+__device__ __forceinline__ void tu_group(TuSmem &S, const uint64_t (&key)[TU_PER], uint32_t n, uint32_t shift)
 {
-    TtCtr c;
-    c.cnt = base;
-    c.hcur = base + tg.nt + 1;
-    c.tcur = c.hcur + tg.nh;
-    c.done = c.tcur + tg.nt;
-    return c;
+    const uint16_t *first = reinterpret_cast<const uint16_t *>(S.cnt);
+    for (uint32_t k = threadIdx.x; k < TU_BUCKETS / 8; k += TU_T) reinterpret_cast<uint4 *>(S.cnt)[k] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    uint32_t at[TU_PER];  // bucket << 16 | rank
+#pragma unroll
+    for (int r = 0; r < TU_PER; r++) {
+        if (r * TU_T >= n) break;
+        if (r * TU_T + threadIdx.x < n) {
+            const uint32_t bk = (uint32_t)(key[r] >> shift), sh = (bk & 1u) * 16u;
+            at[r] = (bk << 16) | ((atomicAdd(&S.cnt[bk >> 1], 1u << sh) >> sh) & 0xffffu);  // (no half carries)
+        }
+    }
+    __syncthreads();
+    {
+        // one scan for the buckets' starts and the places in the list: counts
+        // below 2^16 each, so that records and buckets share a word
+        uint4 *w = reinterpret_cast<uint4 *>(S.cnt) + threadIdx.x;
+        static_assert(TU_BUCKETS / 8 == TU_T, "four words per thread");
+        const uint4 y = *w;
+        uint32_t x[4] = {y.x, y.y, y.z, y.w}, sum = 0, some = 0;  // some: bit q set where bucket q has records
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint32_t lo = x[q] & 0xffffu, hi = x[q] >> 16;
+            some |= (lo ? 1u << (2 * q) : 0u) | (hi ? 2u << (2 * q) : 0u);
+            x[q] = sum | ((sum + lo) << 16);
+            sum += lo + hi;
+        }
+        const uint32_t pre = cta_scan<TU_T>(sum | (__popc(some) << 16), S.warp), p2 = (pre & 0xffffu) * 0x00010001u;
+        *w = make_uint4(x[0] + p2, x[1] + p2, x[2] + p2, x[3] + p2);
+        uint32_t h = pre >> 16;
+        if (threadIdx.x == TU_T - 1) {
+            S.cnt[TU_BUCKETS / 2] = n;
+            S.nhead = h + __popc(some);
+        }
+        for (; some; some &= some - 1) S.head[h++] = (uint16_t)(threadIdx.x * 8 + __ffs(some) - 1);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < TU_PER; r++) {
+        if (r * TU_T >= n) break;
+        if (r * TU_T + threadIdx.x < n) S.a[first[at[r] >> 16] + (at[r] & 0xffffu)] = key[r];
+    }
+    __syncthreads();
 }
 
-// Per-tile candidate counts, from a shared histogram when the tiles fit in
-// it. The last CTA to finish turns them into the tiles' offsets toff[0 ..
-// nt] (toff[nt] = all candidates) and clears the counts and `done`; `reset`
-// (first phase of a call) also clears the call's pending-list lengths and
-// bucket-phase cursors. Every counter word is zero between phases (the tile
-// kernel clears the partition cursors), whatever tile geometry a call uses.
-template <int SRC, int RULE>
-__global__ void __launch_bounds__(TT_TPB) tt_hist(const TtSrc s, TcfGeom G, TcfPrep P, const uint8_t *fill,
-                                                  TtGeom tg, uint32_t *ctr_words, uint32_t *toff,
-                                                  DevCounters *reset, unsigned long long *units)
+// smallest over the CTA; S.red is free again after the next barrier
+__device__ __forceinline__ uint64_t tu_min(TuSmem &S, uint64_t m)
 {
-    extern __shared__ uint32_t s_h[];
-    __shared__ uint32_t s_wsum[TT_TPB / 32];
-    __shared__ bool s_last;
-    const TtCtr C = tt_ctr(ctr_words, tg);
-    const uint64_t n = tt_count(s);
-    note_units(units, n);
-    if (n == 0) return;  // an empty phase: the later kernels of the phase see n = 0 and do nothing
-    // a shared histogram pays off when each CTA has enough items for its bins
-    const bool shared = tg.nt <= 8192 && n * 8 >= (uint64_t)gridDim.x * tg.nt;
-    if (shared) {
-        for (uint32_t t = threadIdx.x; t < tg.nt; t += TT_TPB) s_h[t] = 0;
-        __syncthreads();
-    }
-    for (uint64_t j = blockIdx.x * (uint64_t)TT_TPB + threadIdx.x; j < n; j += (uint64_t)gridDim.x * TT_TPB) {
-        uint64_t rec;
-        uint32_t idx;
-        tt_item<SRC, RULE>(s, j, G, P, fill, rec, idx);
-        const uint32_t t = (uint32_t)((rec >> 16) >> tg.tb_log);
-        if (shared) atomicAdd(&s_h[t], 1u);
-        else atomicAdd(&C.cnt[t], 1u);
-    }
-    if (shared) {
-        __syncthreads();
-        for (uint32_t t = threadIdx.x; t < tg.nt; t += TT_TPB)
-            if (s_h[t]) atomicAdd(&C.cnt[t], s_h[t]);
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(C.done, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    // the last CTA: exclusive scan of cnt[0 .. nt] into toff, in chunks of
-    // 16 counts per thread with a running carry
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr uint32_t PER = 16;
-    uint32_t carry = 0;
-    for (uint64_t c0 = 0; c0 <= tg.nt; c0 += (uint64_t)TT_TPB * PER) {
-        const uint64_t b0 = c0 + (uint64_t)threadIdx.x * PER;
-        uint32_t v[PER], sum = 0;
 #pragma unroll
-        for (uint32_t k = 0; k < PER; k++) {
-            v[k] = (b0 + k <= tg.nt) ? __ldcg(C.cnt + b0 + k) : 0u;
-            sum += v[k];
-        }
-        uint32_t incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) s_wsum[warp] = incl;
-        __syncthreads();
-        uint32_t run = carry + incl - sum, tot = 0;
-        for (int w = 0; w < TT_TPB / 32; w++) {
-            if (w < warp) run += s_wsum[w];
-            tot += s_wsum[w];
-        }
-#pragma unroll
-        for (uint32_t k = 0; k < PER; k++) {
-            if (b0 + k <= tg.nt) toff[b0 + k] = run;
-            run += v[k];
-        }
-        carry += tot;
-        __syncthreads();
-    }
-    // clear the counts for the next phase (the partition cursors are
-    // cleared by the tile kernel, after the passes that use them)
-    for (uint64_t k = threadIdx.x; k <= tg.nt; k += TT_TPB) ctr_words[k] = 0;
-    if (reset && threadIdx.x == 0) {
-        for (int k = 0; k < 8; k++) reset->pend[k] = 0;
-        for (int k = 0; k < 4; k++) reset->touched[k] = reset->cursor[k] = 0;
+    for (int o = 16; o > 0; o >>= 1) {
+        const uint64_t y = __shfl_xor_sync(0xffffffffu, m, o);
+        m = y < m ? y : m;
     }
     __syncthreads();
-    if (threadIdx.x == 0) *C.done = 0;
+    if ((threadIdx.x & 31) == 0) S.red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    m = S.red[0];
+#pragma unroll
+    for (int w = 1; w < TU_T / 32; w++) m = S.red[w] < m ? S.red[w] : m;
+    return m;
 }
 
-// One partition pass. PASS 0: the only pass, bins are tiles; PASS 1: bins are
-// tile >> lo, each bin's region the span of its tiles; PASS 2: the pass-1
-// output, bins are tiles relative to the chunk's first high bin (a chunk that
-// reaches past TT_BINS of them places the rest by global atomics). toff: the
-// tiles' scanned offsets; hcur / tcur: the running cursors of the high bins
-// and of the tiles (zero at the start of the phase).
-template <int SRC, int RULE, int PASS>
-__global__ void __launch_bounds__(TT_TPB, 4) tt_part(const TtSrc s, TcfGeom G, TcfPrep P, const uint8_t *fill,
-                                                  TtGeom tg, const uint32_t *__restrict__ toff, uint32_t *ctr_words,
-                                                  uint64_t *__restrict__ orec, uint32_t *__restrict__ oidx,
-                                                  unsigned long long *units)
+// where a unit's candidates left go
+struct TuOut {
+    uint64_t *rec;
+    uint32_t *idx;
+    unsigned *n;
+    uint64_t cap;
+    unsigned long long *status;
+};
+
+template <int NEXT>
+__device__ __forceinline__ void tu_leave(const TuOut &O, uint64_t pos, uint64_t b, uint32_t slot, uint32_t i,
+                                         const TcfGeom &G, const TcfPrep &P)
 {
-    const TtCtr C = tt_ctr(ctr_words, tg);
-    uint32_t *hcur = C.hcur, *tcur = C.tcur;
-    __shared__ uint32_t s_cnt[TT_BINS], s_start[TT_BINS], s_base[TT_BINS];
-    __shared__ uint64_t s_rec[TT_CH];
-    __shared__ uint32_t s_idx[TT_CH];
-    __shared__ uint16_t s_bin[TT_CH];
-    __shared__ uint32_t s_wsum[TT_TPB / 32];
-    __shared__ uint64_t s_tbase;
-    constexpr int IPT = TT_CH / TT_TPB;
-    const uint64_t n = tt_count(s);
-    note_units(units, n);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (uint64_t c0 = (uint64_t)blockIdx.x * TT_CH; c0 < n; c0 += (uint64_t)gridDim.x * TT_CH) {
-        for (int b = threadIdx.x; b < TT_BINS; b += TT_TPB) s_cnt[b] = 0;
-        if (PASS == 2 && threadIdx.x == 0) s_tbase = ((s.rec[c0] >> 16) >> (tg.tb_log + tg.lo)) << tg.lo;
-        __syncthreads();
-        uint64_t rec[IPT];
-        uint32_t idx[IPT], rank[IPT];
-        uint32_t bin[IPT];
-#pragma unroll
-        for (int q = 0; q < IPT; q++) {
-            const uint64_t j = c0 + threadIdx.x + (uint64_t)q * TT_TPB;
-            bin[q] = 0xffffffffu;
-            if (j < n) {
-                tt_item<SRC, RULE>(s, j, G, P, fill, rec[q], idx[q]);
-                const uint64_t t = (rec[q] >> 16) >> tg.tb_log;
-                const uint64_t b = PASS == 1 ? (t >> tg.lo) : (PASS == 2 ? t - s_tbase : t);
-                if (b < TT_BINS && t < tg.nt) {
-                    bin[q] = (uint32_t)b;
-                    rank[q] = atomicAdd(&s_cnt[b], 1u);
-                } else if (PASS == 2 && t < tg.nt) {  // a tile far past the chunk's first high bin
-                    const uint32_t pos = toff[t] + atomicAdd(&tcur[t], 1u);
-                    if (pos < toff[tg.nt]) {
-                        orec[pos] = rec[q];
-                        oidx[pos] = idx[q];
-                    }
-                }
-            }
+    if (pos >= O.cap) {  // more left than the pending list holds
+        atomicOr(O.status, ST_INTERNAL);
+        return;
+    }
+    O.idx[pos] = i;
+    if (NEXT != TU_NX_IDX) O.rec[pos] = ((NEXT == TU_NX_OTHER ? tu_other(b, slot, i, G, P) : b) << 16) | slot;
+}
+
+// A block with many candidates (a hot key): the CTA reads them once per stored
+// slot, for the next smallest each time. v: c records, some of them the
+// block's; lb: the block inside the unit.
+template <int F, bool DEL, int NEXT>
+__device__ __noinline__ void tu_hot_block(TuSmem &S, const uint64_t *v, uint32_t c, uint64_t b, uint32_t lb,
+                                          const TcfGeom &G, const TcfPrep &P, const TuGeom &U, uint8_t *blocks,
+                                          uint8_t *fill, uint32_t cap, const TuOut &O)
+{
+    constexpr int B = Blk<F>::B;
+    __shared__ uint32_t s_tag[B];
+    __shared__ uint64_t s_thr[B];
+    const uint32_t tsh = U.ibits, bsh = U.ibits + U.sbits, smask = (1u << U.sbits) - 1u, lmask = (1u << U.lbits) - 1u;
+    const uint64_t rmask = bsh + U.lbits >= 64 ? ~0ull : (1ull << (bsh + U.lbits)) - 1ull;
+    const uint32_t f0 = fill[b];
+    Blk<F> blk;
+    blk.load(blocks, b);
+    auto mine = [&](uint64_t x) { return ((uint32_t)(x >> bsh) & lmask) == lb; };
+    // the smallest record of the block that `want` accepts and is above `prev`
+    auto next = [&](uint64_t prev, bool any, auto want) {
+        uint64_t m = ~0ull;
+        for (uint32_t i = threadIdx.x; i < c; i += TU_T) {
+            const uint64_t x = v[i] & rmask;
+            if (mine(x) && (any || x > prev) && want(x) && x < m) m = x;
         }
-        __syncthreads();
-        // bin starts inside the chunk (exclusive scan, 2 bins per thread) and
-        // each bin's global base, one atomic per non-empty bin
-        {
-            const uint32_t a = s_cnt[2 * threadIdx.x], b = s_cnt[2 * threadIdx.x + 1];
-            uint32_t incl = a + b;
+        return tu_min(S, m);
+    };
+    uint32_t used = 0;  // entries of s_tag / s_thr (DEL), accepted records
+    uint64_t thr = 0;
+    if (!DEL) {
+        const uint32_t k = cap > f0 ? cap - f0 : 0u;
+        for (uint32_t j = 0; j < k; j++) {
+            const uint64_t m = next(thr, j == 0, [](uint64_t) { return true; });
+            if (m == ~0ull) break;  // (the same in every thread)
+            thr = m;
+            used++;
+            uint64_t r8[8] = {((thr >> tsh) & smask) << 32, 0, 0, 0, 0, 0, 0, 0};
+            blk.merge_new(f0 + j, 1, r8);
+        }
+        if (used && threadIdx.x == 0) {
+            blk.store(blocks, b);
+            fill[b] = (uint8_t)(f0 + used);
+        }
+    } else {
+        const uint32_t lm = G.vmask;
+        Blk<F> old = blk;
+        uint32_t removed = 0;
+        bool left = true;  // candidates of the current tag
+        uint64_t prev = 0;
+        for (uint32_t p = 0; p < f0; p++) {  // a stored copy each; copies of a tag are adjacent
+            uint32_t t = 0;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            if (lane == 31) s_wsum[warp] = incl;
+            for (int q = 0; q < B; q++)
+                if (q == (int)p) t = old.tag(q);
+            t &= ~lm;
+            const bool again = used > 0 && s_tag[used - 1] == t;
             __syncthreads();
-            uint32_t pre = 0;
-            for (int w = 0; w < warp; w++) pre += s_wsum[w];
-            const uint32_t ex = pre + incl - a - b;
-            s_start[2 * threadIdx.x] = ex;
-            s_start[2 * threadIdx.x + 1] = ex + a;
-#pragma unroll
-            for (int k = 0; k < 2; k++) {
-                const uint32_t bb = 2 * threadIdx.x + k, c = k ? b : a;
-                if (!c) continue;
-                if (PASS == 1) {
-                    s_base[bb] = toff[(uint64_t)bb << tg.lo] + atomicAdd(&hcur[bb], c);
-                } else {
-                    const uint64_t t = PASS == 2 ? s_tbase + bb : bb;
-                    s_base[bb] = toff[t] + atomicAdd(&tcur[t], c);
+            if (!again) {
+                left = true;
+                if (threadIdx.x == 0) {
+                    s_tag[used] = t;
+                    s_thr[used] = 0;  // none matched (a record is never 0: tags are at least 2)
+                }
+                used++;
+            }
+            if (left) {
+                const uint64_t m = next(prev, !again, [&](uint64_t x) { return ((uint32_t)(x >> tsh) & smask) == t; });
+                left = m != ~0ull;
+                if (left) {
+                    prev = m;
+                    if (threadIdx.x == 0) s_thr[used - 1] = m;
+                    const uint32_t sm = blk.eq_slots(t, Blk<F>::lane_mask(G.vmask));
+                    if (sm) blk.delete_at(__ffs(sm) - 1);
+                    removed++;
                 }
             }
+            __syncthreads();
         }
-        __syncthreads();
+        if (removed && threadIdx.x == 0) {
+            blk.store(blocks, b);
+            fill[b] = (uint8_t)(f0 - removed);
+        }
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < c; i += TU_T) {
+        const uint64_t x = v[i] & rmask;
+        if (!mine(x)) continue;
+        const uint32_t slot = (uint32_t)(x >> tsh) & smask;
+        bool took = !DEL && used && x <= thr;
+        if (DEL)
+            for (uint32_t d = 0; d < used; d++) took |= s_tag[d] == slot && x <= s_thr[d];
+        if (!took) tu_leave<NEXT>(O, atomicAdd(O.n, 1u), b, slot, (uint32_t)x & (uint32_t)((1ull << U.ibits) - 1ull), G, P);
+    }
+    __syncthreads();
+}
+
+// Inserts a tag into the sorted tags of a 16-bit block, all lanes less one, so
+// that empty ones are the largest: lane i becomes max(lane i - 1, min(lane i,
+// tag)). tt: the tag less one in both lanes.
+__device__ __forceinline__ void insert_tag16(uint32_t (&w)[8], uint32_t tt)
+{
 #pragma unroll
-        for (int q = 0; q < IPT; q++) {
-            if (bin[q] != 0xffffffffu) {
-                const uint32_t p = s_start[bin[q]] + rank[q];
-                s_rec[p] = rec[q];
-                s_idx[p] = idx[q];
-                s_bin[p] = (uint16_t)bin[q];
-            }
-        }
-        __syncthreads();
-        const uint32_t total = s_start[TT_BINS - 1] + s_cnt[TT_BINS - 1];
-        const uint32_t lim = toff[tg.nt];
-        for (uint32_t p = threadIdx.x; p < total; p += TT_TPB) {
-            const uint32_t b = s_bin[p];
-            const uint32_t pos = s_base[b] + (p - s_start[b]);
-            if (pos < lim) {  // positions past the counted total would mean counts that disagree
-                orec[pos] = s_rec[p];
-                oidx[pos] = s_idx[p];
-            }
-        }
-        __syncthreads();
+    for (int q = 7; q >= 0; q--) {
+        const uint32_t below = q ? __funnelshift_l(w[q - 1], w[q], 16) : w[0] << 16;
+        uint32_t m;
+        asm("min.u16x2 %0, %1, %2;" : "=r"(m) : "r"(w[q]), "r"(tt));
+        asm("max.u16x2 %0, %1, %2;" : "=r"(w[q]) : "r"(m), "r"(below));
     }
 }
 
-// block-wide exclusive scan of v[0 .. m) in place, v[m] = the total; m <= TT_TB_MAX
-__device__ __forceinline__ void tt_block_scan(uint32_t *v, uint32_t m, uint32_t *s_wsum)
+__device__ __forceinline__ void add_lanes16(uint32_t (&w)[8], uint32_t x)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // chunks of TT_TPB entries in order, one entry per thread, with a carry
-    uint32_t carry = 0;
-    for (uint32_t k0 = 0; k0 <= m; k0 += TT_TPB) {
-        const uint32_t i = k0 + threadIdx.x;
-        const uint32_t x = i < m ? v[i] : 0u;
-        uint32_t incl = x;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) s_wsum[warp] = incl;
-        __syncthreads();
-        uint32_t pre = carry, tot = 0;
-        for (int w = 0; w < TT_TPB / 32; w++) {
-            if (w < warp) pre += s_wsum[w];
-            tot += s_wsum[w];
-        }
-        if (i <= m) v[i] = pre + incl - x;
-        carry += tot;
-        __syncthreads();
-    }
+    for (int q = 0; q < 8; q++) asm("add.u16x2 %0, %0, %1;" : "+r"(w[q]) : "r"(x));
 }
 
-// Per-block steps with more than 8 candidates (rare: hot blocks), kept out
-// of line so that the common path stays light on registers. Insert: the k
-// smallest candidates join the sorted block (f0 tags); remove: for each
-// stored tag present d times, the d smallest candidates with that tag take
-// one copy each. Left candidates get `mark` in place. Return the new fill.
-template <int F>
-__device__ __noinline__ uint32_t tt_insert_many(uint8_t *blocks, uint64_t b, uint32_t f0, uint32_t k, uint64_t *cand,
-                                                uint32_t c, uint64_t mark)
+// Removes the first lane whose tag part (lm) is tt's from the sorted lanes of a
+// 16-bit block (EMPTY ones last): lanes of at least that tag take the next one.
+__device__ __forceinline__ bool remove_tag16(uint32_t (&w)[8], uint32_t tt, uint32_t lm)
 {
-    constexpr int B = Blk<F>::B;
-    Blk<F> blk;
-    blk.load(blocks, b);
-    uint64_t a[MAXSEL];
-    int have = 0;
-    for (uint32_t q = 0; q < c; q++) have = topk_push(a, have, (int)k, cand[q]);
-    const uint64_t thr = a[k - 1];
-    uint32_t t_out[B];
-    int ia = 0, ib = 0;
-#pragma unroll
-    for (int p = 0; p < B; p++) {
-        const uint32_t ta = (ia < (int)f0) ? blk.tag(ia) : 0xffffffffu;
-        const uint32_t tb = (ib < (int)k) ? (uint32_t)(a[ib] >> 32) : 0xffffffffu;
-        if (ta == 0xffffffffu && tb == 0xffffffffu) {
-            t_out[p] = 0;
-        } else if (ta <= tb) {
-            t_out[p] = ta;
-            ia++;
-        } else {
-            t_out[p] = tb;
-            ib++;
-        }
-    }
-    blk.pack(t_out);
-    blk.store(blocks, b);
-    for (uint32_t q = 0; q < c; q++)
-        if (cand[q] > thr) cand[q] |= mark;
-    return f0 + k;
-}
-
-template <int F>
-__device__ __noinline__ uint32_t tt_remove_many(uint8_t *blocks, uint64_t b, uint32_t f0, uint64_t *cand, uint32_t c,
-                                                uint32_t vmask, uint64_t mark)
-{
-    constexpr int B = Blk<F>::B;
-    Blk<F> blk;
-    blk.load(blocks, b);
-    uint32_t tags[B], dt[B], dp[B], dc[B], used[B];
-    uint64_t dthr[B];
-    int ndt = 0, removed = 0;
-#pragma unroll
-    for (int p = 0; p < B; p++) tags[p] = blk.tag(p);
-    for (int p = 0; p < (int)f0; p++) {
-        const uint32_t mt = tags[p] & ~vmask;
-        if (ndt > 0 && dt[ndt - 1] == mt) {
-            dc[ndt - 1]++;
-        } else {
-            dt[ndt] = mt;
-            dp[ndt] = (uint32_t)p;
-            dc[ndt] = 1;
-            ndt++;
-        }
-    }
-    for (int d = 0; d < ndt; d++) {
-        uint64_t a[MAXSEL];
-        int have = 0;
-        const uint64_t lo = (uint64_t)dt[d] << 32, hi = lo | 0xffffffffull;
-        for (uint32_t q = 0; q < c; q++) {
-            const uint64_t r = cand[q];
-            if (r >= lo && r <= hi) have = topk_push(a, have, (int)dc[d], r);
-        }
-        used[d] = (uint32_t)have;
-        dthr[d] = have ? a[have - 1] : 0;
-    }
-    uint32_t t_out[B];
-    int o = 0;
-    for (int d = 0; d < ndt; d++) {
-        for (uint32_t q = used[d]; q < dc[d]; q++) t_out[o++] = tags[dp[d] + q];
-        removed += (int)used[d];
-    }
-    for (int p = o; p < B; p++) t_out[p] = 0;
-    for (uint32_t q = 0; q < c; q++) {
-        const uint64_t r = cand[q];
-        const uint32_t t = (uint32_t)(r >> 32);
-        bool matched = false;
-        for (int d = 0; d < ndt; d++)
-            if (dt[d] == t && used[d] > 0 && r <= dthr[d]) matched = true;
-        if (!matched) cand[q] = r | mark;
-    }
-    if (removed) {
-        blk.pack(t_out);
-        blk.store(blocks, b);
-    }
-    return f0 - (uint32_t)removed;
-}
-
-// The per-block step of one block: candidates cand[0 .. c) (slot << 32 |
-// index, any order), the block's fill f0. Insert: the k smallest that fit
-// under `cap` join the sorted block. Remove: each candidate removes one copy
-// of its tag, smallest first. Candidates that are left get TT_LEFT | lb << 48
-// in place. Returns the new fill.
-template <int F, int OP>
-__device__ __forceinline__ uint32_t tt_block_step(uint8_t *blocks, uint64_t b, uint32_t lb, uint32_t f0, uint32_t cap,
-                                                  uint64_t *cand, uint32_t c, uint32_t lm, uint32_t vmask,
-                                                  uint64_t &bytes)
-{
-    const uint64_t mark = TT_LEFT | ((uint64_t)lb << 48);
-    if (OP == 0) {
-        const uint32_t k = cap > f0 ? min(c, cap - f0) : 0u;
-        if (k == 0) {
-            for (uint32_t q = 0; q < c; q++) cand[q] |= mark;
-            return f0;
-        }
-        bytes += 66;
-        if (c > 8) return tt_insert_many<F>(blocks, b, f0, k, cand, c, mark);
-        Blk<F> blk;
-        blk.load(blocks, b);
-        uint64_t r8[8];
-#pragma unroll
-        for (int q = 0; q < 8; q++) r8[q] = q < (int)c ? cand[q] : ~0ull;
-        sort_small(r8, c);
-        blk.merge_new(f0, k, r8);
-        blk.store(blocks, b);
-#pragma unroll
-        for (int q = 0; q < 8; q++)
-            if (q < (int)c) cand[q] = q < (int)k ? r8[q] : (r8[q] | mark);
-        return f0 + k;
-    }
-    bytes += 32;
-    if (c > 8) {
-        const uint32_t f1 = tt_remove_many<F>(blocks, b, f0, cand, c, vmask, mark);
-        if (f1 != f0) bytes += 34;
-        return f1;
-    }
-    Blk<F> blk;
-    blk.load(blocks, b);
-    int removed = 0;
-    uint64_t r8[8];
-#pragma unroll
-    for (int q = 0; q < 8; q++) r8[q] = (uint32_t)q < c ? cand[q] : ~0ull;
-    sort_small(r8, c);
+    uint32_t none = 0x00010001u;  // a half is 0 once a lane of it matched
 #pragma unroll
     for (int q = 0; q < 8; q++) {
-        if ((uint32_t)q < c) {
-            const uint32_t sm = blk.eq_slots((uint32_t)(r8[q] >> 32), lm);
-            if (sm) {
-                blk.delete_at(__ffs(sm) - 1);
-                removed++;
-                cand[q] = r8[q];
-            } else {
-                cand[q] = r8[q] | mark;
-            }
-        }
+        uint32_t m;
+        asm("min.u16x2 %0, %1, %2;" : "=r"(m) : "r"((w[q] & lm) ^ tt), "r"(0x00010001u));
+        none &= m;
     }
-    if (removed) {
-        blk.store(blocks, b);
-        bytes += 34;
+    if (none == 0x00010001u) return false;
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+        const uint32_t x = w[q] & lm, next = q < 7 ? __funnelshift_r(w[q], w[q + 1], 16) : w[7] >> 16;
+        uint32_t m;
+        asm("max.u16x2 %0, %1, %2;" : "=r"(m) : "r"(x), "r"(tt));
+        asm("min.u16x2 %0, %1, %2;" : "=r"(m) : "r"(m - x), "r"(0x00010001u));  // 1: below the tag
+        m *= 0xffffu;
+        w[q] = (w[q] & m) | (next & ~m);
     }
-    return f0 - (uint32_t)removed;
+    return true;
 }
 
-// One CTA per tile (looping over tiles): the tile's candidates are counted
-// per block with their rank (shared atomics, the records held in registers),
-// placed in block order in shared memory (a tile with more than TT_CAP of
-// them is staged in the spare record buffer `gstage` at the same offsets and
-// read twice), each block with candidates takes its step, and the candidates
-// left are written out with one reservation per tile. A dense tile (at least
-// one candidate per TT_DENSE blocks) moves its blocks into shared memory with
-// one bulk copy, issued before the staging so that the two overlap, and back
-// with one bulk store; a sparse one reads and writes only the blocks it
-// touches. What a candidate left becomes (NEXT): the same block's record
-// (phase A rejects: phase B finds their target), the other block's record
-// (phase B rejects, remove misses in b1), or its batch index (for the
-// backing-bucket phase). n_dev: the phase's candidate count when it comes from
-// a pending list (the kernel returns at once for an empty phase). units:
-// algorithmic bytes (12 per candidate read and per candidate left, 32 per
-// block read, 32 per block written, 2 per fill read and written).
-static constexpr uint32_t TT_DENSE = 4;
-
-template <int F, int OP, int NEXT>
-__global__ void __launch_bounds__(TT_TPB, 4) tt_tile(TcfGeom G, TcfPrep P, uint8_t *blocks, uint8_t *fill, TtGeom tg,
-                                                  const uint32_t *__restrict__ toff, const uint64_t *__restrict__ rec,
-                                                  const uint32_t *__restrict__ ridx, uint64_t *gstage, uint32_t cap,
-                                                  uint64_t *orec, uint32_t *oidx, unsigned *nout, uint64_t out_cap,
-                                                  const unsigned *n_dev, uint32_t *ctr_words,
-                                                  unsigned long long *status, unsigned long long *units)
+// The steps of bucket [s, e) of S.a by one thread, block by block in ascending
+// order (ONE: a bucket is a block). Insert: the candidates that fit under
+// `cap`, smallest first, join the sorted block; their order matters only where
+// some do not fit. Remove: each candidate, smallest first, takes the first copy
+// of its tag. Those left are listed in S.left. Returns the algorithmic bytes
+// (64 per block changed, 32 per block only read, 2 per fill).
+template <int F, bool DEL, bool ONE>
+__device__ __forceinline__ uint32_t tu_bucket(TuSmem &S, uint32_t s, uint32_t e, uint32_t lb, uint64_t b0,
+                                              const TcfGeom &G, uint32_t tsh, uint32_t bsh, uint32_t smask,
+                                              uint8_t *blocks, uint8_t *fill, uint32_t cap)
 {
-    constexpr uint32_t RPT = TT_CAP / TT_TPB;
-    if (n_dev && *n_dev == 0) return;  // an empty phase: nothing was counted or placed
-    extern __shared__ __align__(128) uint64_t s_mem[];
-    const uint32_t TB = 1u << tg.tb_log;
-    uint8_t *s_blocks = reinterpret_cast<uint8_t *>(s_mem);                     // TB x 32 bytes
-    uint64_t *s_stage = s_mem + TB * 4;                                         // TT_CAP entries
-    uint32_t *s_start = reinterpret_cast<uint32_t *>(s_stage + TT_CAP);         // TB + 1
-    uint8_t *s_fill = reinterpret_cast<uint8_t *>(s_start + TB + 1);            // TB
-    __shared__ uint32_t s_wsum[TT_TPB / 32];
-    __shared__ uint32_t s_base;
-    __shared__ unsigned long long s_bytes;
-    __shared__ __align__(8) uint64_t s_bar;
-    {
-        // the partition passes of this phase are done with their cursors
-        const TtCtr C = tt_ctr(ctr_words, tg);
-        const uint64_t w = tg.nh + tg.nt;
-        for (uint64_t k = blockIdx.x * (uint64_t)TT_TPB + threadIdx.x; k < w; k += (uint64_t)gridDim.x * TT_TPB)
-            C.hcur[k] = 0;
-    }
-    if (threadIdx.x == 0) mbar_init(&s_bar, 1);
-    __syncthreads();
-    uint32_t parity = 0;
-    bool stores_pending = false;  // thread 0: a bulk store may still read s_blocks
-    const uint32_t lm = Blk<F>::lane_mask(G.vmask);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (uint64_t T = blockIdx.x; T < tg.nt; T += gridDim.x) {
-        const uint32_t s = toff[T], e = toff[T + 1];
-        if (s == e) continue;
-        const uint64_t b0 = T << tg.tb_log;
-        const uint32_t nblk = (uint32_t)min((uint64_t)TB, tg.nb - b0);
-        const uint32_t cnt = e - s;
-        const bool in_smem = cnt <= TT_CAP;
-        const bool dense = (uint64_t)cnt * TT_DENSE >= nblk;
-        uint64_t *stage = in_smem ? s_stage : gstage + s;
-        if (dense && threadIdx.x == 0) {
-            if (stores_pending) bulk_wait_read();  // the previous tile's store has read s_blocks
-            stores_pending = false;
-            mbar_arrive_expect(&s_bar, nblk * 32);
-            bulk_load(s_blocks, blocks + b0 * 32, nblk * 32, &s_bar);
+    uint32_t done = 0, bytes = 0;
+    do {
+        uint32_t m = e - s;  // the block's candidates
+        if (!ONE) {
+            uint32_t mn = 0xffffffffu;
+            for (uint32_t j = s; j < e; j++) {
+                const uint32_t x = (uint32_t)(S.a[j] >> bsh);
+                if (done == 0 || x > lb) mn = min(mn, x);
+            }
+            lb = mn;
+            m = 0;
+            for (uint32_t j = s; j < e; j++) m += (uint32_t)(S.a[j] >> bsh) == lb;
         }
-        for (uint32_t k = threadIdx.x; k <= nblk; k += TT_TPB) s_start[k] = 0;
-        if (dense)
-            for (uint32_t k = threadIdx.x; k < nblk; k += TT_TPB) s_fill[k] = fill[b0 + k];
-        if (threadIdx.x == 0) s_bytes = 0;
-        __syncthreads();
-        uint64_t rv[RPT];
-        uint32_t rank[RPT];
-        if (in_smem) {
-#pragma unroll
-            for (uint32_t q = 0; q < RPT; q++) {
-                const uint32_t r = s + threadIdx.x + q * TT_TPB;
-                rank[q] = 0xffffffffu;
-                if (r < e) {
-                    const uint64_t v = rec[r];
-                    const uint64_t lb = (v >> 16) - b0;
-                    if (lb >= nblk) {  // a record outside its tile: report, never index with it
-                        atomicOr(status, ST_INTERNAL);
-                        continue;
-                    }
-                    rank[q] = atomicAdd(&s_start[lb], 1u);
-                    rv[q] = (lb << 48) | ((v & 0xffffu) << 32) | ridx[r];
-                }
+        done += m;
+        const uint64_t b = b0 + lb;
+        const uint32_t f0 = min((uint32_t)fill[b], (uint32_t)Blk<F>::B);
+        Blk<F> blk;
+        blk.load(blocks, b);
+        bytes += 34;
+        auto mine = [&](uint64_t x) { return ONE || (uint32_t)(x >> bsh) == lb; };
+        // the smallest of the block's candidates above prev (or of all)
+        auto next = [&](uint64_t prev, bool any) {
+            uint64_t q = ~0ull;
+            for (uint32_t j = s; j < e; j++) {
+                const uint64_t x = S.a[j];
+                if (mine(x) && (any || x > prev) && x < q) q = x;
             }
-        } else {
-            for (uint32_t r = s + threadIdx.x; r < e; r += TT_TPB) {
-                const uint64_t lb = (rec[r] >> 16) - b0;
-                if (lb < nblk) atomicAdd(&s_start[lb], 1u);
-                else atomicOr(status, ST_INTERNAL);
-            }
-        }
-        __syncthreads();
-        tt_block_scan(s_start, nblk, s_wsum);
-        if (in_smem) {
-#pragma unroll
-            for (uint32_t q = 0; q < RPT; q++) {
-                const uint32_t r = s + threadIdx.x + q * TT_TPB;
-                if (r < e && rank[q] != 0xffffffffu) {
-                    const uint32_t lb = (uint32_t)(rv[q] >> 48);
-                    const uint32_t p = s_start[lb] + rank[q];
-                    if (p < cnt) stage[p] = rv[q] & 0x0000ffffffffffffull;
-                    else atomicOr(status, ST_INTERNAL);
-                }
-            }
-        } else {
-            // ranks come from a second pass: the counts above turned into
-            // starts, then advanced per placed candidate and restored
-            for (uint32_t r = s + threadIdx.x; r < e; r += TT_TPB) {
-                const uint64_t v = rec[r];
-                const uint64_t lb = (v >> 16) - b0;
-                if (lb >= nblk) continue;
-                const uint32_t p = atomicAdd(&s_start[lb], 1u);
-                if (p < cnt) stage[p] = ((v & 0xffffu) << 32) | ridx[r];
-                else atomicOr(status, ST_INTERNAL);
-            }
-            __syncthreads();
-            // s_start[lb] now holds the end of block lb, the start of lb + 1
-            constexpr uint32_t PB = TT_TB_MAX / TT_TPB;
-            uint32_t prev[PB];
-#pragma unroll
-            for (uint32_t j = 0; j < PB; j++) {
-                const uint32_t k = threadIdx.x + j * TT_TPB;
-                prev[j] = (k < nblk && k > 0) ? s_start[k - 1] : 0u;
-            }
-            __syncthreads();
-#pragma unroll
-            for (uint32_t j = 0; j < PB; j++) {
-                const uint32_t k = threadIdx.x + j * TT_TPB;
-                if (k < nblk) s_start[k] = prev[j];
-            }
-        }
-        if (dense) {
-            // the tile's blocks have arrived (a bounded wait: give up on the
-            // whole kernel, reporting a timeout, rather than spin for ever)
-            const bool ok = mbar_wait_bounded(&s_bar, parity, SPIN_LIMIT);
-            parity ^= 1u;
-            if (__syncthreads_or(!ok)) {
-                if (threadIdx.x == 0) atomicOr(status, ST_TIMEOUT);
-                break;
-            }
-        } else {
-            __syncthreads();
-        }
-        // each block with candidates takes its step
-        uint8_t *blk_base = dense ? s_blocks : blocks;
-        uint64_t bytes = 0;
-        for (uint32_t k = threadIdx.x; k < nblk; k += TT_TPB) {
-            const uint32_t c = s_start[k + 1] - s_start[k];
-            if (!c) continue;
-            const uint64_t b = b0 + k;
-            const uint32_t f0 = dense ? s_fill[k] : fill[b];
-            if (s_start[k + 1] > cnt || s_start[k + 1] < s_start[k] || f0 > (uint32_t)Blk<F>::B) {
-                atomicOr(status, ST_INTERNAL);
-                continue;
-            }
-            bytes += 12ull * c + 2;
-            const uint32_t f1 = tt_block_step<F, OP>(blk_base, dense ? k : b, k, f0, cap, stage + s_start[k], c, lm,
-                                                     G.vmask, bytes);
-            if (f1 != f0) fill[b] = (uint8_t)f1;
-        }
-        if (dense) {
-            fence_async_shared();  // the block writes above, before the bulk store reads them
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                bulk_store(blocks + b0 * 32, s_blocks, nblk * 32);
-                stores_pending = true;
-            }
-        } else {
-            __syncthreads();
-        }
-        // the candidates left, written out in stage order with one reservation
-        for (uint32_t c0 = 0; c0 < cnt; c0 += TT_CAP) {
-            const uint32_t i0 = c0 + threadIdx.x * RPT;
-            uint32_t mine = 0;
-#pragma unroll
-            for (uint32_t q = 0; q < RPT; q++)
-                if (i0 + q < cnt && (stage[i0 + q] & TT_LEFT)) mine++;
-            uint32_t incl = mine;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            if (lane == 31) s_wsum[warp] = incl;
-            __syncthreads();
-            uint32_t pre = 0, tot = 0;
-            for (int w = 0; w < TT_TPB / 32; w++) {
-                if (w < warp) pre += s_wsum[w];
-                tot += s_wsum[w];
-            }
-            if (threadIdx.x == 0 && tot) s_base = atomicAdd(nout, tot);
-            __syncthreads();
-            uint32_t pos = s_base + pre + incl - mine;
-            if (mine) {
-#pragma unroll
-                for (uint32_t q = 0; q < RPT; q++) {
-                    if (i0 + q >= cnt) break;
-                    const uint64_t v = stage[i0 + q];
-                    if (!(v & TT_LEFT)) continue;
-                    const uint32_t sl = (uint32_t)(v >> 32) & 0xffffu, i = (uint32_t)v;
-                    if (pos >= out_cap) {  // more left than the pending list holds
-                        atomicOr(status, ST_INTERNAL);
-                        break;
-                    }
-                    if (NEXT == TT_NX_IDX) {
-                        oidx[pos++] = i;
+            return q;
+        };
+        if (!DEL) {
+            const uint32_t k = cap > f0 ? min(m, cap - f0) : 0u;
+            uint64_t thr = 0;
+            if (k) {
+                if constexpr (F == 16) {
+                    add_lanes16(blk.w, 0xffffffffu);
+                    if (k == m) {
+                        for (uint32_t j = s; j < e; j++) {
+                            const uint64_t x = S.a[j];
+                            if (mine(x)) insert_tag16(blk.w, (((uint32_t)(x >> tsh) & smask) - 1) * 0x00010001u);
+                        }
                     } else {
-                        const uint64_t b = b0 + ((v >> 48) & 0x7fffu);
-                        const uint64_t d = NEXT == TT_NX_OTHER ? tt_other(b, sl, i, G, P) : b;
-                        orec[pos] = (d << 16) | sl;
-                        oidx[pos++] = i;
+                        for (uint32_t at = 0; at < k; at++) {
+                            thr = next(thr, at == 0);
+                            insert_tag16(blk.w, (((uint32_t)(thr >> tsh) & smask) - 1) * 0x00010001u);
+                        }
+                    }
+                    add_lanes16(blk.w, 0x00010001u);
+                } else {
+                    for (uint32_t at = 0; at < k; at += 8) {
+                        uint64_t r8[8];
+#pragma unroll
+                        for (uint32_t q = 0; q < 8; q++) {
+                            r8[q] = 0;
+                            if (at + q < k) {
+                                thr = next(thr, at + q == 0);
+                                r8[q] = ((thr >> tsh) & smask) << 32;
+                            }
+                        }
+                        blk.merge_new(f0 + at, min(8u, k - at), r8);
                     }
                 }
+                blk.store(blocks, b);
+                fill[b] = (uint8_t)(f0 + k);
+                bytes += 32;
             }
-            bytes += 12ull * mine;
-            __syncthreads();
+            if (k < m) {
+                uint32_t pos = atomicAdd(&S.nleft, m - k);
+                for (uint32_t j = s; j < e; j++) {
+                    const uint64_t x = S.a[j];
+                    if (mine(x) && (k == 0 || x > thr)) S.left[pos++] = (uint16_t)j;
+                }
+            }
+        } else {
+            uint32_t removed = 0;
+            uint64_t prev = 0;
+            for (uint32_t q = 0; q < m; q++) {
+                prev = e - s == 1 ? S.a[s] : next(prev, q == 0);
+                const uint32_t tag = (uint32_t)(prev >> tsh) & smask, lm = Blk<F>::lane_mask(G.vmask);
+                bool hit;
+                if constexpr (F == 16) {
+                    hit = remove_tag16(blk.w, tag * 0x00010001u, lm);
+                } else {
+                    const uint32_t sm = blk.eq_slots(tag, lm);
+                    hit = sm != 0;
+                    if (hit) blk.delete_at(__ffs(sm) - 1);
+                }
+                if (hit) {
+                    removed++;
+                } else {
+                    uint32_t j = s;
+                    while (S.a[j] != prev) j++;
+                    S.left[atomicAdd(&S.nleft, 1u)] = (uint16_t)j;
+                }
+            }
+            if (removed) {
+                blk.store(blocks, b);
+                fill[b] = (uint8_t)(f0 - removed);
+                bytes += 32;
+            }
         }
-        if (units && bytes) atomicAdd(&s_bytes, bytes);
-        __syncthreads();
-        if (units && threadIdx.x == 0 && s_bytes) atomicAdd(units, s_bytes);
+    } while (!ONE && done < e - s);
+    return bytes;
+}
+
+// the candidates that a unit's steps left in S.left, with one reservation
+template <int NEXT>
+__device__ __forceinline__ void tu_emit(TuSmem &S, const TuOut &O, uint64_t b0, const TcfGeom &G, const TcfPrep &P,
+                                        const TuGeom &U)
+{
+    const uint32_t nleft = S.nleft;
+    if (threadIdx.x == 0 && nleft) S.base = atomicAdd(O.n, nleft);
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < nleft; i += TU_T) {
+        const uint64_t x = S.a[S.left[i]];
+        tu_leave<NEXT>(O, (uint64_t)S.base + i, b0 + (x >> (U.ibits + U.sbits)),
+                       (uint32_t)(x >> U.ibits) & ((1u << U.sbits) - 1u), (uint32_t)(x & ((1ull << U.ibits) - 1ull)), G, P);
     }
-    if (threadIdx.x == 0 && stores_pending) bulk_wait_all();
+}
+
+// the arguments of a phase's steps (a kernel parameter that functions out of
+// line read in place)
+struct TuStep {
+    TcfGeom G;
+    TcfPrep P;
+    TuGeom U;
+    uint8_t *blocks, *fill;
+    const uint32_t *ust;   // the units' first records
+    uint32_t nunits, cap;
+    const uint64_t *v;     // records by unit
+    TuOut O;
+    TuSrc src;
+    unsigned long long *units;
+};
+
+// the hot buckets in S.hot, by the whole CTA, block by block
+template <int F, bool DEL, int NEXT>
+__device__ __noinline__ void tu_hot_buckets(TuSmem &S, const TuStep &A, uint64_t b0)
+{
+    const uint32_t bsh = A.U.ibits + A.U.sbits;
+    const uint16_t *first = reinterpret_cast<const uint16_t *>(S.cnt);
+    for (uint32_t h = 0; h < S.nhot; h++) {
+        const uint32_t bk = S.hot[h], s = first[bk], e = first[bk + 1];
+        uint64_t last = 0;
+        for (bool any = true;; any = false) {
+            uint64_t m = ~0ull;
+            for (uint32_t j = s + threadIdx.x; j < e; j += TU_T) {
+                const uint64_t x = S.a[j] >> bsh;
+                if ((any || x > last) && x < m) m = x;
+            }
+            last = tu_min(S, m);
+            if (last == ~0ull) break;
+            tu_hot_block<F, DEL, NEXT>(S, S.a + s, e - s, b0 + last, (uint32_t)last, A.G, A.P, A.U, A.blocks, A.fill, A.cap,
+                                       A.O);
+        }
+    }
+    __syncthreads();
+}
+
+// A unit with more candidates than fit: ranges of blocks that do, found by
+// counting, take the same steps; a block that alone has more goes by the CTA.
+template <int F, bool DEL, int NEXT>
+__device__ __noinline__ void tu_big_unit(TuSmem &S, const TuStep &A, uint32_t unit)
+{
+    const TuGeom &U = A.U;
+    const uint32_t tsh = U.ibits, bsh = U.ibits + U.sbits, smask = (1u << U.sbits) - 1u, lmask = (1u << U.lbits) - 1u;
+    const uint64_t rmask = bsh + U.lbits >= 64 ? ~0ull : (1ull << (bsh + U.lbits)) - 1ull;
+    const uint32_t bkshift = bsh + (U.lbits > TU_BBITS ? U.lbits - TU_BBITS : 0u);
+    const uint16_t *first = reinterpret_cast<const uint16_t *>(S.cnt);
+    const uint64_t b0 = (uint64_t)unit << U.lbits;
+    const uint64_t *w = A.v + A.ust[unit];
+    const uint32_t all = A.ust[unit + 1] - A.ust[unit], end = 1u << U.lbits;
+    uint32_t lo = 0, range = end;
+    while (lo < end) {
+        uint32_t n = 0;
+        while (true) {
+            uint32_t m = 0;
+            for (uint32_t i = threadIdx.x; i < all; i += TU_T) m += ((uint32_t)(w[i] >> bsh) & lmask) - lo < range;
+            const uint32_t before = cta_scan<TU_T>(m, S.warp);
+            if (threadIdx.x == TU_T - 1) S.base = before + m;
+            __syncthreads();
+            n = S.base;
+            __syncthreads();
+            if (n <= TU_CAP || range == 1) break;
+            range >>= 1;
+        }
+        if (n > TU_CAP) {
+            tu_hot_block<F, DEL, NEXT>(S, w, all, b0 + lo, lo, A.G, A.P, U, A.blocks, A.fill, A.cap, A.O);
+        } else if (n) {
+            if (threadIdx.x == 0) S.base = S.nleft = S.nhot = 0;
+            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < all; i += TU_T)
+                if (((uint32_t)(w[i] >> bsh) & lmask) - lo < range) S.a[atomicAdd(&S.base, 1u)] = w[i] & rmask;
+            __syncthreads();
+            uint64_t key[TU_PER];
+#pragma unroll
+            for (int r = 0; r < TU_PER; r++)
+                if (r * TU_T + threadIdx.x < n) key[r] = S.a[r * TU_T + threadIdx.x];
+            tu_group(S, key, n, bkshift);
+            for (uint32_t h = threadIdx.x; h < S.nhead; h += TU_T) {
+                const uint32_t bk = S.head[h], s = first[bk], e = first[bk + 1];
+                if (e - s > TU_HOT) S.hot[atomicAdd(&S.nhot, 1u)] = (uint16_t)bk;
+                else tu_bucket<F, DEL, false>(S, s, e, bk, b0, A.G, tsh, bsh, smask, A.blocks, A.fill, A.cap);
+            }
+            __syncthreads();
+            tu_emit<NEXT>(S, A.O, b0, A.G, A.P, U);
+            tu_hot_buckets<F, DEL, NEXT>(S, A, b0);
+        }
+        lo += range;
+        while (range < end && lo % (2 * range) == 0) range <<= 1;  // wider again where it may be
+    }
+}
+
+// One CTA per unit (staying for more, the next one's records on their way):
+// group the candidates by block, then a thread per block with candidates takes
+// its step. units: algorithmic bytes (tu_bucket's, 8 per candidate read, 12 per
+// candidate left). Bound by instructions and the latency of the blocks' loads:
+// 2^22 candidates on 2^22 blocks 81 us, 2^24 on 2^24 291 us (3.7 TB/s of
+// algorithmic bytes).
+template <int F, bool DEL, int NEXT, bool ONE>
+__global__ void __launch_bounds__(TU_T, 3) tcf_unit_step(const __grid_constant__ TuStep A)
+{
+    if (tu_count(A.src) == 0) return;
+    __shared__ __align__(16) TuSmem S;
+    const uint32_t tsh = A.U.ibits, bsh = A.U.ibits + A.U.sbits, smask = (1u << A.U.sbits) - 1u;
+    const uint64_t rmask = bsh + A.U.lbits >= 64 ? ~0ull : (1ull << (bsh + A.U.lbits)) - 1ull;
+    const uint32_t bkshift = ONE ? bsh : bsh + A.U.lbits - TU_BBITS;
+    const uint16_t *first = reinterpret_cast<const uint16_t *>(S.cnt);
+    uint64_t key[TU_PER];
+    uint32_t u = blockIdx.x, c = 0;
+    unsigned long long total = 0;
+    auto fetch = [&] {
+        const uint32_t s0 = A.ust[u];
+        c = A.ust[u + 1] - s0;
+        if (c > TU_CAP) return;
+#pragma unroll
+        for (int r = 0; r < TU_PER; r++) {
+            if (r * TU_T >= c) break;
+            if (r * TU_T + threadIdx.x < c) key[r] = __ldcs(A.v + s0 + r * TU_T + threadIdx.x) & rmask;
+        }
+    };
+    if (u < A.nunits) fetch();
+    while (u < A.nunits) {
+        const uint32_t unit = u, n = c;
+        const uint64_t b0 = (uint64_t)unit << A.U.lbits;
+        u += gridDim.x;
+        if (n == 0) {
+            if (u < A.nunits) fetch();
+            continue;
+        }
+        __syncthreads();  // everything of the last unit is done
+        if (n > TU_CAP) {
+            tu_big_unit<F, DEL, NEXT>(S, A, unit);
+            if (u < A.nunits) fetch();
+            continue;
+        }
+        if (threadIdx.x == 0) S.nleft = S.nhot = 0;
+        tu_group(S, key, n, bkshift);
+        if (u < A.nunits) fetch();  // the next unit's records
+        const uint32_t heads = S.nhead;
+        uint32_t bytes = 0;
+        for (uint32_t h = threadIdx.x; h < heads; h += TU_T) {
+            const uint32_t bk = S.head[h], s = first[bk], e = first[bk + 1];
+            if (e - s > TU_HOT) S.hot[atomicAdd(&S.nhot, 1u)] = (uint16_t)bk;
+            else bytes += tu_bucket<F, DEL, ONE>(S, s, e, bk, b0, A.G, tsh, bsh, smask, A.blocks, A.fill, A.cap);
+        }
+        __syncthreads();
+        if (A.units) total += bytes + (threadIdx.x == 0 ? 8ull * n + 12ull * S.nleft : 0ull);
+        tu_emit<NEXT>(S, A.O, b0, A.G, A.P, A.U);
+        if (S.nhot) tu_hot_buckets<F, DEL, NEXT>(S, A, b0);
+    }
+    if (A.units) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) total += __shfl_down_sync(0xffffffffu, total, o);
+        if ((threadIdx.x & 31) == 0 && total) atomicAdd(A.units, total);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2056,7 +2187,7 @@ int tcf_setup(filter *F, uint64_t &table_bytes, uint64_t &scratch_bytes, bool pl
     piece(T.tcount, (uint64_t)sm_count() * 8);
     piece(T.dlist, M);
     piece(T.seg, M);
-    piece(T.tcur, tt_counter_words(T.G.nb));
+    piece(T.tcur, tcf_unit_words(M));
     piece(T.pb, M);
     piece(T.pbi, M);
     piece(F->scan_tmp, scan_tmp_words(groups));
@@ -2072,7 +2203,7 @@ int tcf_clear(filter *F, cudaStream_t st)
     GF_CUDA(cudaMemsetAsync(T.bk, 0, T.G.nbk * BK_W * 8, st));
     GF_CUDA(cudaMemsetAsync(T.fill, 0, T.G.nb, st));
     GF_CUDA(cudaMemsetAsync(T.cnt, 0, groups * 4, st));
-    GF_CUDA(cudaMemsetAsync(T.tcur, 0, tt_counter_words(T.G.nb) * 4, st));
+    GF_CUDA(cudaMemsetAsync(T.tcur, 0, tu_scratch(nullptr, F->cfg.max_batch).zero_words * 4, st));
     GF_CUDA(cudaMemsetAsync(F->ctr, 0, sizeof(DevCounters), st));
     return FILTER_OK;
 }
@@ -2093,9 +2224,9 @@ struct TcfBulk {
     uint32_t *tlist, *tcount, *dlist;
     uint64_t *seg;
     uint64_t max_n;  // entries of every per-key scratch list (max_batch)
-    uint32_t tile_target;  // tiled path: expected candidates per tile
-    uint32_t *tcur;  // tiled phases: tile counts and cursors
-    uint64_t *pb;    // tiled phases: the second pending list
+    uint32_t tile_target;  // unit path: most candidates per unit on average
+    uint32_t *tcur;  // unit phases: the partition's scratch
+    uint64_t *pb;    // unit phases: the second pending list
     uint32_t *pbi;
     uint64_t *scan_tmp;
     DevCounters *ctr;
@@ -2618,6 +2749,31 @@ static void gblock_phase(const TcfBulk &T, const PhaseDst &P, uint64_t n, int ph
             T.G, T.blocks, T.fill, P, T.rec, phase, cap, pend32, pend64, npend, units);
 }
 
+template <int F, int GB = 0>
+static void tcf_sparse_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, cudaStream_t st);
+template <int F, int GB = 0>
+static void tcf_sparse_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, cudaStream_t st);
+
+// the later phases in one launch; at most four CTAs per SM, which its launch
+// bounds keep resident together
+template <int F, bool DEL>
+static void tcf_sparse_coop(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, uint32_t unit_min,
+                            cudaStream_t st)
+{
+    SparseArgs A{keys, n, T.G, T.prep, T.blocks, T.fill, T.bk, T.cnt, T.off, T.tlist, T.tcount, T.dlist, T.pend0, T.pend2,
+                 T.rec, T.pend1, T.seg, status, T.ctr, unit_min};
+    void *args[] = {&A};
+    gf::TraceScope ts_(DEL ? "tcf_sparse_remove" : "tcf_sparse_insert", n, st);
+    const void *kernel = DEL ? (const void *)tcf_sparse_remove_coop<F> : (const void *)tcf_sparse_insert_coop<F>;
+    cudaLaunchCooperativeKernel(kernel, dim3(grid_for(n, TPB * 2, 4)), dim3(TPB), args, 0, st);
+}
+
+// Tables whose later phases go by one launch: ten launches less a call (2^12
+// blocks, 2^14 keys a call: an insert and a remove 51 and 40 us, 62 and 46
+// with kernels of their own; 2^16 blocks, 2^16 keys: 49 and 46 us, 80 and 63).
+// Smaller ones keep the kernels, which a trace shows by phase.
+static constexpr uint64_t COOP_MIN_BLOCKS = 1ull << 12;
+
 // The per-block counting-sort path: each phase groups its candidates by
 // destination block (counts, scan, scatter) and one thread per block takes
 // its step. Its scratch (a counter and an offset per block, a record per
@@ -2628,8 +2784,7 @@ static void tcf_bulk_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
     const TcfGeom G = T.G;
     DevCounters *ctr = T.ctr;
     unsigned *np = ctr->pend;
-    cudaMemsetAsync(np, 0, sizeof(ctr->pend), st);
-    cudaMemsetAsync(ctr->touched, 0, sizeof(ctr->touched) + sizeof(ctr->cursor), st);  // adjacent fields
+    cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
     // A: shortcut into b1
     PhaseDst P = group_phase<SRC_KEYS, DST_B1>(T, keys, n, nullptr, nullptr, 0, nullptr, st);
     {
@@ -2640,8 +2795,21 @@ static void tcf_bulk_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
         else
             gblock_phase<F, GB, false>(T, P, n, 0, G.tsc, T.pend0, nullptr, &np[0], ts_.units(), st);
     }
+    if constexpr (GB == 0)
+        if (G.nb >= COOP_MIN_BLOCKS) return tcf_sparse_coop<F, false>(T, keys, n, status, 0xffffffffu, st);
+    tcf_sparse_insert<F, GB>(T, keys, n, status, st);
+}
+
+// phases B to D of an insert, whose candidates T.pend0 lists by index: a
+// counting sort over the blocks that they touch
+template <int F, int GB>
+static void tcf_sparse_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, cudaStream_t st)
+{
+    const TcfGeom G = T.G;
+    DevCounters *ctr = T.ctr;
+    unsigned *np = ctr->pend;
     // B: the less full of b1, b2 under the post-A fills
-    P = group_phase<SRC_PEND_U32, DST_TARGET>(T, keys, n, T.pend0, &np[0], 1, nullptr, st);
+    PhaseDst P = group_phase<SRC_PEND_U32, DST_TARGET>(T, keys, n, T.pend0, &np[0], 1, nullptr, st);
     {
         gf::TraceScope ts_("tcf_block_insert_sparse", 0, st, true);
         if constexpr (GB == 0)
@@ -2674,8 +2842,7 @@ static void tcf_bulk_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
     const TcfGeom G = T.G;
     DevCounters *ctr = T.ctr;
     unsigned *np = ctr->pend;
-    cudaMemsetAsync(np, 0, sizeof(ctr->pend), st);
-    cudaMemsetAsync(ctr->touched, 0, sizeof(ctr->touched) + sizeof(ctr->cursor), st);  // adjacent fields
+    cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
     // 1: primary block
     PhaseDst P = group_phase<SRC_KEYS, DST_B1>(T, keys, n, nullptr, nullptr, 0, nullptr, st);
     {
@@ -2686,8 +2853,20 @@ static void tcf_bulk_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
         else
             gblock_phase<F, GB, true>(T, P, n, 0, 0, T.pend0, nullptr, &np[0], ts_.units(), st);
     }
+    if constexpr (GB == 0)
+        if (G.nb >= COOP_MIN_BLOCKS) return tcf_sparse_coop<F, true>(T, keys, n, status, 0xffffffffu, st);
+    tcf_sparse_remove<F, GB>(T, keys, n, status, st);
+}
+
+// phases 2 and 3 of a remove, likewise
+template <int F, int GB>
+static void tcf_sparse_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, cudaStream_t st)
+{
+    const TcfGeom G = T.G;
+    DevCounters *ctr = T.ctr;
+    unsigned *np = ctr->pend;
     // 2: secondary block
-    P = group_phase<SRC_PEND_U32, DST_B2>(T, keys, n, T.pend0, &np[0], 1, nullptr, st);
+    PhaseDst P = group_phase<SRC_PEND_U32, DST_B2>(T, keys, n, T.pend0, &np[0], 1, nullptr, st);
     {
         gf::TraceScope ts_("tcf_block_remove_sparse", 0, st, true);
         if constexpr (GB == 0)
@@ -2731,136 +2910,119 @@ static void tcf_custom_bulk(const TcfBulk &W, const uint64_t *keys, uint64_t n, 
 }
 
 // ---------------------------------------------------------------------------
-// Tiled phases: host side
+// Unit phases: host side
 // ---------------------------------------------------------------------------
-// Tiles of TB blocks, TB the largest power of two in [32, TT_TB_MAX] that
-// keeps a tile's expected candidates (n keys spread over nb blocks) at or
-// below `target` (at most half of TT_CAP, so that a tile's records fit its
-// shared-memory stage with room for the spread); partitioned in one pass up
-// to 256 tiles and in two above (at most 256 high bins).
-static TtGeom tt_geom(uint64_t nb, uint64_t n, uint32_t target)
+// units of at most `target` candidates on average (2048: a uniform phase's
+// largest unit is far below what a CTA holds), one pass up to 2^9 of them
+static TuGeom tu_geom(const TcfGeom &G, uint64_t n, uint32_t target)
 {
-    TtGeom g;
-    g.nb = nb;
-    uint32_t tl = 5;
-    while ((1u << (tl + 1)) <= TT_TB_MAX && (n << (tl + 1)) <= (uint64_t)target * nb) tl++;
-    g.tb_log = tl;
-    g.nt = (nb + (1ull << tl) - 1) >> tl;
-    uint32_t lg = 0;
-    while ((1ull << lg) < g.nt) lg++;
-    g.lo = g.nt <= 256 ? 0 : ((lg + 1) / 2 > lg - 8 ? (lg + 1) / 2 : lg - 8);
-    g.nh = g.lo ? (g.nt + (1ull << g.lo) - 1) >> g.lo : g.nt;
-    return g;
+    TuGeom U;
+    uint32_t lgnb = 0;
+    while ((1ull << lgnb) < G.nb) lgnb++;
+    U.k = 0;
+    while (U.k < lgnb && U.k < 18 && (n >> U.k) > target) U.k++;
+    U.b1 = U.k > 9 ? (U.k + 1) / 2 : U.k;
+    U.b2 = U.k - U.b1;
+    U.lbits = lgnb - U.k;
+    U.sbits = G.f;
+    U.ibits = 1;
+    while ((1ull << U.ibits) < n) U.ibits++;
+    return U;
 }
 
-template <int F, int OP, int NEXT>
-static void tt_tile_launch(const TcfBulk &T, const TtGeom &tg, const unsigned *n_dev, const uint64_t *rec,
-                           const uint32_t *ridx, uint64_t *gstage, uint32_t cap, uint64_t *orec, uint32_t *oidx,
-                           unsigned *nout, const char *name, cudaStream_t st)
+// the record holds what the first pass does not imply
+static bool tu_takes(const TcfGeom &G, uint64_t n, uint32_t target)
 {
-    const size_t TB = (size_t)1 << tg.tb_log;
-    const size_t smem = TB * 32 + TT_CAP * 8 + (TB + 1) * 4 + TB;
-    cudaFuncSetAttribute(tt_tile<F, OP, NEXT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(TT_TB_MAX * 32 + TT_CAP * 8 + (TT_TB_MAX + 1) * 4 + TT_TB_MAX));
-    const uint64_t grid = tg.nt < (uint64_t)sm_count() * 8 ? tg.nt : (uint64_t)sm_count() * 8;
-    gf::TraceScope ts_(name, 0, st, true);
-    tt_tile<F, OP, NEXT><<<(unsigned)grid, TT_TPB, smem, st>>>(T.G, T.prep, T.blocks, T.fill, tg, T.off, rec, ridx,
-                                                               gstage, cap, orec, oidx, nout, T.max_n, n_dev, T.tcur,
-                                                               &T.ctr->status, ts_.units());
+    const TuGeom U = tu_geom(G, n, target);
+    return n <= (1ull << 28) && U.lbits <= 31 && U.lbits + U.b2 + U.sbits + U.ibits <= 64;
 }
 
-// group one phase's candidates by tile: counts (their last CTA scans them
-// into T.off and clears the counters), then one or two partition passes;
-// returns the buffers holding the grouped records (and the spare pair,
-// which the tile kernel may use for a hot tile)
-template <int SRC, int RULE>
-static void tt_group(const TcfBulk &T, const TtGeom &tg, const TtSrc &src, DevCounters *reset, const uint64_t **grec,
-                     const uint32_t **gidx, uint64_t **spare, cudaStream_t st)
+// The partition's scratch for calls of up to max_n keys: one layout for all of
+// them, so that the counts, zero between phases, stay where they are.
+static MsdScratch tu_scratch(uint32_t *base, uint64_t max_n)
 {
-    const bool keys = SRC == TT_KEYS;
-    const int ghist = grid_for(src.n, TT_TPB * 16, 4);
+    uint32_t k = 0;
+    while (k < 18 && (max_n >> k) > 128) k++;  // the smallest target
+    return msd_scratch(base, max_n, k, true, false, false);
+}
+static uint64_t tcf_unit_words(uint64_t max_n) { return tu_scratch(nullptr, max_n).words; }
+
+// one phase: partition the candidates (n: at most as many), step every unit
+template <int F, bool DEL, int SRC, int NEXT>
+static void tu_phase(const TcfBulk &T, const TuSrc &src, uint64_t n, uint32_t cap, uint64_t *orec, uint32_t *oidx,
+                     unsigned *nout, cudaStream_t st)
+{
+    const TuGeom U = tu_geom(T.G, n, T.tile_target);
+    const MsdScratch M = tu_scratch(T.tcur, T.max_n);
+    const bool keys = SRC == TU_KEYS;
+    const uint32_t nb1 = 1u << U.b1;
+    const uint64_t tiles = (n + MP_TILE - 1) / MP_TILE;
     {
-        gf::TraceScope ts_(keys ? "tcf_tile_hist" : "tcf_tile_hist_pend", keys ? src.n : 0, st, !keys);
-        tt_hist<SRC, RULE><<<ghist, TT_TPB, tg.nt <= 8192 ? tg.nt * 4 : 0, st>>>(src, T.G, T.prep, T.fill, tg, T.tcur,
-                                                                                T.off, reset, ts_.units());
-    }
-    const int gpart = grid_for((src.n + TT_CH - 1) / TT_CH * TT_TPB, TT_TPB, 6);
-    if (tg.lo == 0) {
-        gf::TraceScope ts_(keys ? "tcf_tile_part" : "tcf_tile_part_pend", keys ? src.n : 0, st, !keys);
-        tt_part<SRC, RULE, 0><<<gpart, TT_TPB, 0, st>>>(src, T.G, T.prep, T.fill, tg, T.off, T.tcur, T.rec, T.tlist,
-                                                        ts_.units());
-        *grec = T.rec;
-        *gidx = T.tlist;
-        *spare = T.seg;
-        return;
+        gf::TraceScope ts_(keys ? "tcf_tile_hist" : "tcf_tile_hist_pend", keys ? n : 0, st, !keys);
+        tu_hist<SRC><<<grid_for(tiles * MP_T, MP_T, 4), MP_T, 0, st>>>(src, T.G, T.prep, T.fill, U, M, ts_.units());
     }
     {
-        gf::TraceScope ts_(keys ? "tcf_tile_part" : "tcf_tile_part_pend", keys ? src.n : 0, st, !keys);
-        tt_part<SRC, RULE, 1><<<gpart, TT_TPB, 0, st>>>(src, T.G, T.prep, T.fill, tg, T.off, T.tcur, T.rec, T.tlist,
-                                                        ts_.units());
+        gf::TraceScope ts_(keys ? "tcf_tile_part" : "tcf_tile_part_pend", keys ? n : 0, st, !keys);
+        tu_part<SRC><<<(unsigned)tiles, MP_T, 0, st>>>(src, T.G, T.prep, T.fill, U, M, T.rec, ts_.units());
     }
-    TtSrc s2{nullptr, T.rec, T.tlist, src.n_dev, src.n};
-    {
-        gf::TraceScope ts_("tcf_tile_part2", 0, st, true);
-        tt_part<TT_PEND, TT_SAME, 2><<<gpart, TT_TPB, 0, st>>>(s2, T.G, T.prep, T.fill, tg, T.off, T.tcur, T.seg,
-                                                               T.dlist, ts_.units());
-    }
-    *grec = T.seg;
-    *gidx = T.dlist;
-    *spare = T.rec;
+    if (U.b2)
+        msd_second_pass(M, T.rec, T.seg, n, nb1, U.lbits + U.sbits + U.ibits, U.b2, "tcf_tile_hist2", "tcf_tile_part2", st);
+    gf::TraceScope ts_(DEL ? "tcf_tile_remove" : "tcf_tile_insert", 0, st, true);
+    const TuStep A{T.G, T.prep, U, T.blocks, T.fill, U.b2 ? M.st2 : M.st1, 1u << U.k, cap, U.b2 ? T.seg : T.rec,
+                   TuOut{orec, oidx, nout, T.max_n, &T.ctr->status}, src, ts_.units()};
+    const int g = grid_for((uint64_t)TU_T << U.k, TU_T, 3);
+    if (U.lbits <= TU_BBITS) tcf_unit_step<F, DEL, NEXT, true><<<g, TU_T, 0, st>>>(A);
+    else tcf_unit_step<F, DEL, NEXT, false><<<g, TU_T, 0, st>>>(A);
+}
+
+// Candidates of the first phase of all keys up to which the later phases go by
+// touched destinations, in one cooperative launch: their counters and records
+// stay in the L2 up to 2^22 blocks, whatever their number; on larger tables
+// more than one key in sixteen goes by unit (2^28 slots, 2^24 keys at 90 %
+// load: 1.41 ms by destination, 0.64 by unit; on the first batches 0.02 and
+// 0.13).
+static uint32_t tu_unit_min(const TcfBulk &T, uint64_t n)
+{
+    return T.G.nb > (1ull << 22) ? (uint32_t)(n / 16) : 0xffffffffu;
 }
 
 template <int F>
-static void tcf_tiled_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, cudaStream_t st)
+static void tcf_unit_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, cudaStream_t st)
 {
     const TcfGeom G = T.G;
-    DevCounters *ctr = T.ctr;
-    unsigned *np = ctr->pend;
-    const TtGeom tg = tt_geom(G.nb, n, T.tile_target);
-    const uint64_t *gr;
-    const uint32_t *gi;
-    uint64_t *sp;
-    // A: shortcut into b1 while fill < 3B/4; rejects keep b1 (the counts'
-    // last CTA also clears the call's pending-list lengths)
-    tt_group<TT_KEYS, TT_SAME>(T, tg, TtSrc{keys, nullptr, nullptr, nullptr, n}, ctr, &gr, &gi, &sp, st);
-    tt_tile_launch<F, 0, TT_NX_SAME>(T, tg, nullptr, gr, gi, sp, G.tsc, T.pend1, T.pend0, &np[0], "tcf_tile_insert", st);
-    // B: the less full of b1, b2 under the post-A fills; rejects go to the other block
-    tt_group<TT_PEND, TT_TARGET>(T, tg, TtSrc{nullptr, T.pend1, T.pend0, &np[0], n}, nullptr, &gr, &gi, &sp, st);
-    tt_tile_launch<F, 0, TT_NX_OTHER>(T, tg, &np[0], gr, gi, sp, G.B, T.pb, T.pbi, &np[1], "tcf_tile_insert", st);
-    // C: the other block; rejects go to the backing buckets by index
-    tt_group<TT_PEND, TT_SAME>(T, tg, TtSrc{nullptr, T.pb, T.pbi, &np[1], n}, nullptr, &gr, &gi, &sp, st);
-    tt_tile_launch<F, 0, TT_NX_IDX>(T, tg, &np[1], gr, gi, sp, G.B, nullptr, T.pend2, &np[2], "tcf_tile_insert", st);
-    // D: backing buckets
-    PhaseDst P = group_phase<SRC_PEND_U32, DST_BUCKET>(T, keys, n, T.pend2, &np[2], 3, T.pend0, st);
-    {
-        gf::TraceScope ts_("tcf_bucket_insert", 0, st, true);
-        tcf_bucket_insert<<<dst_grid(P, n, G.nbk), TPB, 0, st>>>(G, T.bk, P, T.rec, T.pend0, status, ctr, ts_.units());
+    unsigned *np = T.ctr->pend;
+    const uint32_t unit_min = tu_unit_min(T, n);
+    cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
+    // A: shortcut into b1 while fill < 3B/4; rejects keep b1
+    tu_phase<F, false, TU_KEYS, TU_NX_SAME>(T, TuSrc{keys, nullptr, nullptr, nullptr, 0, n}, n, G.tsc, T.pend1, T.pend0,
+                                            &np[0], st);
+    if (unit_min != 0xffffffffu) {
+        // B: the less full of b1, b2 under the post-A fills; rejects go to the other block
+        tu_phase<F, false, TU_TARGET, TU_NX_OTHER>(T, TuSrc{nullptr, T.pend1, T.pend0, &np[0], unit_min, n}, n, G.B, T.pb,
+                                                   T.pbi, &np[1], st);
+        // C: the other block; rejects go to the backing buckets by index
+        tu_phase<F, false, TU_SAME, TU_NX_IDX>(T, TuSrc{nullptr, T.pb, T.pbi, &np[1], 0, n}, n, G.B, nullptr, T.pend2,
+                                               &np[2], st);
     }
+    // B and C of fewer candidates, and D: backing buckets
+    tcf_sparse_coop<F, false>(T, keys, n, status, unit_min, st);
 }
 
 template <int F>
-static void tcf_tiled_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, cudaStream_t st)
+static void tcf_unit_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, cudaStream_t st)
 {
-    const TcfGeom G = T.G;
-    DevCounters *ctr = T.ctr;
-    unsigned *np = ctr->pend;
-    const TtGeom tg = tt_geom(G.nb, n, T.tile_target);
-    const uint64_t *gr;
-    const uint32_t *gi;
-    uint64_t *sp;
+    unsigned *np = T.ctr->pend;
+    const uint32_t unit_min = tu_unit_min(T, n);
+    cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
     // 1: primary block; misses go on to the secondary block
-    tt_group<TT_KEYS, TT_SAME>(T, tg, TtSrc{keys, nullptr, nullptr, nullptr, n}, ctr, &gr, &gi, &sp, st);
-    tt_tile_launch<F, 1, TT_NX_OTHER>(T, tg, nullptr, gr, gi, sp, 0, T.pend1, T.pend0, &np[0], "tcf_tile_remove", st);
+    tu_phase<F, true, TU_KEYS, TU_NX_OTHER>(T, TuSrc{keys, nullptr, nullptr, nullptr, 0, n}, n, 0, T.pend1, T.pend0, &np[0],
+                                            st);
     // 2: secondary block; misses go to the backing buckets by index
-    tt_group<TT_PEND, TT_SAME>(T, tg, TtSrc{nullptr, T.pend1, T.pend0, &np[0], n}, nullptr, &gr, &gi, &sp, st);
-    tt_tile_launch<F, 1, TT_NX_IDX>(T, tg, &np[0], gr, gi, sp, 0, nullptr, T.pend2, &np[2], "tcf_tile_remove", st);
-    // 3: backing bucket; what is left is not found
-    PhaseDst P = group_phase<SRC_PEND_U32, DST_BUCKET>(T, keys, n, T.pend2, &np[2], 2, T.pend0, st);
-    {
-        gf::TraceScope ts_("tcf_bucket_remove", 0, st, true);
-        tcf_bucket_remove<<<dst_grid(P, n, G.nbk), TPB, 0, st>>>(G, T.bk, P, T.rec, T.pend0, status, ctr,
-                                                                 ts_.units());
-    }
+    if (unit_min != 0xffffffffu)
+        tu_phase<F, true, TU_SAME, TU_NX_IDX>(T, TuSrc{nullptr, T.pend1, T.pend0, &np[0], unit_min, n}, n, 0, nullptr,
+                                              T.pend2, &np[2], st);
+    // 2 of fewer candidates, and 3: backing bucket; what is left is not found
+    tcf_sparse_coop<F, true>(T, keys, n, status, unit_min, st);
 }
 
 // Batches that one CTA takes whole (32-byte blocks); false for the others.
@@ -2896,10 +3058,10 @@ int tcf_insert(filter *F, const uint64_t *keys, const uint8_t *vals, uint64_t n,
             else tcf_point_insert<8><<<g, TPB, 0, st>>>(keys, vals, n, T.G, T.blocks, T.bk, status, F->ctr);
         }
     } else {
-        const bool tiled = !tcf_custom(T.G) && tcf_tiled(F->tune, T.G.nb, n);
+        const bool tiled = !tcf_custom(T.G) && tcf_tiled(F->tune, T.G.nb, n, false) && tu_takes(T.G, n, tcf_tile_target(F->tune));
         if (tcf_custom(T.G)) tcf_custom_bulk(W, keys, n, status, false, st);
-        else if (T.G.f == 16) tiled ? tcf_tiled_insert<16>(W, keys, n, status, st) : tcf_bulk_insert<16>(W, keys, n, status, st);
-        else tiled ? tcf_tiled_insert<8>(W, keys, n, status, st) : tcf_bulk_insert<8>(W, keys, n, status, st);
+        else if (T.G.f == 16) tiled ? tcf_unit_insert<16>(W, keys, n, status, st) : tcf_bulk_insert<16>(W, keys, n, status, st);
+        else tiled ? tcf_unit_insert<8>(W, keys, n, status, st) : tcf_bulk_insert<8>(W, keys, n, status, st);
     }
     GF_CUDA(cudaGetLastError());
     return FILTER_OK;
@@ -2923,10 +3085,10 @@ int tcf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cud
             else tcf_point_remove<8><<<g, TPB, 0, st>>>(keys, n, T.G, T.blocks, T.bk, status, F->ctr);
         }
     } else {
-        const bool tiled = !tcf_custom(T.G) && tcf_tiled(F->tune, T.G.nb, n);
+        const bool tiled = !tcf_custom(T.G) && tcf_tiled(F->tune, T.G.nb, n, true) && tu_takes(T.G, n, tcf_tile_target(F->tune));
         if (tcf_custom(T.G)) tcf_custom_bulk(W, keys, n, status, true, st);
-        else if (T.G.f == 16) tiled ? tcf_tiled_remove<16>(W, keys, n, status, st) : tcf_bulk_remove<16>(W, keys, n, status, st);
-        else tiled ? tcf_tiled_remove<8>(W, keys, n, status, st) : tcf_bulk_remove<8>(W, keys, n, status, st);
+        else if (T.G.f == 16) tiled ? tcf_unit_remove<16>(W, keys, n, status, st) : tcf_bulk_remove<16>(W, keys, n, status, st);
+        else tiled ? tcf_unit_remove<8>(W, keys, n, status, st) : tcf_bulk_remove<8>(W, keys, n, status, st);
     }
     GF_CUDA(cudaGetLastError());
     return FILTER_OK;
@@ -3125,7 +3287,7 @@ int tcf_group_setup(filter_group *GR, const filter_config *cfgs, uint64_t &bytes
     piece(T.tcount, (uint64_t)sm_count() * 8);
     piece(T.dlist, M);
     piece(T.seg, M);
-    piece(T.tcur, tt_counter_words(nb_tot));
+    piece(T.tcur, tcf_unit_words(M));
     piece(T.pb, M);
     piece(T.pbi, M);
     piece(GR->prep.bt, M);
@@ -3181,7 +3343,7 @@ int tcf_group_clear(filter_group *GR, cudaStream_t st)
     GF_CUDA(cudaMemsetAsync(T.bk, 0, T.G.nbk * BK_W * 8, st));
     GF_CUDA(cudaMemsetAsync(T.fill, 0, T.G.nb, st));
     GF_CUDA(cudaMemsetAsync(T.cnt, 0, groups * 4, st));
-    GF_CUDA(cudaMemsetAsync(T.tcur, 0, tt_counter_words(T.G.nb) * 4, st));
+    GF_CUDA(cudaMemsetAsync(T.tcur, 0, tu_scratch(nullptr, GR->max_total).zero_words * 4, st));
     GF_CUDA(cudaMemsetAsync(GR->ctr, 0, sizeof(DevCounters), st));
     return FILTER_OK;
 }
@@ -3211,13 +3373,13 @@ int tcf_group_op(filter_group *GR, int op, const uint64_t *off, const uint64_t *
         return FILTER_OK;
     }
     if (out) GF_CUDA(cudaMemsetAsync(out, 0, n, st));
-    const bool tiled = tcf_tiled(GR->tune, T.G.nb, n);
+    const bool tiled = tcf_tiled(GR->tune, T.G.nb, n, op != GROUP_INSERT) && tu_takes(T.G, n, tcf_tile_target(GR->tune));
     if (op == GROUP_INSERT) {
-        if (T.G.f == 16) tiled ? tcf_tiled_insert<16>(W, nullptr, n, out, st) : tcf_bulk_insert<16>(W, nullptr, n, out, st);
-        else tiled ? tcf_tiled_insert<8>(W, nullptr, n, out, st) : tcf_bulk_insert<8>(W, nullptr, n, out, st);
+        if (T.G.f == 16) tiled ? tcf_unit_insert<16>(W, nullptr, n, out, st) : tcf_bulk_insert<16>(W, nullptr, n, out, st);
+        else tiled ? tcf_unit_insert<8>(W, nullptr, n, out, st) : tcf_bulk_insert<8>(W, nullptr, n, out, st);
     } else {
-        if (T.G.f == 16) tiled ? tcf_tiled_remove<16>(W, nullptr, n, out, st) : tcf_bulk_remove<16>(W, nullptr, n, out, st);
-        else tiled ? tcf_tiled_remove<8>(W, nullptr, n, out, st) : tcf_bulk_remove<8>(W, nullptr, n, out, st);
+        if (T.G.f == 16) tiled ? tcf_unit_remove<16>(W, nullptr, n, out, st) : tcf_bulk_remove<16>(W, nullptr, n, out, st);
+        else tiled ? tcf_unit_remove<8>(W, nullptr, n, out, st) : tcf_bulk_remove<8>(W, nullptr, n, out, st);
     }
     GF_CUDA(cudaGetLastError());
     return FILTER_OK;

@@ -7,9 +7,11 @@ multiset (Section 5). They only trade launch count against memory traffic,
 and where the trade-off turns over is a property of the device, so it is
 measured rather than assumed:
 
-  tcf_path            per-block counting sort (one CTA per 2^k blocks, keys
-                      sorted in shared memory) or tiled (one partition of the
-                      whole batch by tile, one CTA per tile of blocks);
+  tcf_path            per-block counting sort (a counter and a record segment
+                      per block) or tiled (one partition of the whole batch by
+                      tile, one CTA per tile of blocks); left to the library's
+                      rule on table, batch and direction unless one of the two
+                      alone is faster;
   tcf_tile_target     candidates per tile the tiled path aims for;
   gqf_region_groups   how many 64-slot groups a batch may touch per key
                       before the GQF leaves the in-place path for a merge.
@@ -80,7 +82,8 @@ def struct(knobs: dict):
 # ---------------------------------------------------------------------------
 # Measurement
 # ---------------------------------------------------------------------------
-TCF_CANDIDATES = ((1, 0), (2, 256), (2, 512), (2, 1024))  # (tcf_path, tile target)
+TCF_CANDIDATES = ((0, 0), (1, 0), (2, 512), (2, 1024))    # (tcf_path, tile target)
+AUTO_MARGIN = 0.97  # what a forced path's time must be below, of the rule's
 GQF_CANDIDATES = (4, 8, 16, 32, 64, 128)                  # region groups
 
 
@@ -94,6 +97,15 @@ def _timed(torch, fn, reps=2):
         ms = sum(a.elapsed_time(b) for a, b in pairs)
         best = ms if best is None else min(best, ms)
     return best
+
+
+def _path_name(path: int, target: int) -> str:
+    return ("auto", "block", f"tiled_{target}")[path]
+
+
+def _best_path(res: dict) -> str:
+    best = min(res, key=res.get)
+    return best if res[best] < AUTO_MARGIN * res["auto"] else "auto"
 
 
 def tune_tcf(lg: int, keys, torch) -> dict:
@@ -126,12 +138,11 @@ def tune_tcf(lg: int, keys, torch) -> dict:
             return [(a, m), (m, z)]
 
         run()  # warm-up
-        res[f"{'block' if path == 1 else 'tiled'}{'' if path == 1 else '_' + str(target)}"] = round(
-            _timed(torch, run), 3)
+        res[_path_name(path, target)] = round(_timed(torch, run), 3)
     F.close()
-    best = min(res, key=res.get)
-    if best == "block":
-        knobs = {"tcf_path": 1}
+    best = _best_path(res)
+    if best in ("auto", "block"):
+        knobs = {"tcf_path": 0 if best == "auto" else 1}
     else:  # tiled when a batch has at least one key per block, else per-block
         knobs = {"tcf_path": 0, "tcf_tiled_min_blocks": nb, "tcf_tile_target": int(best.split("_")[1])}
     return {**knobs, "ms": res, "batch": b}
@@ -164,7 +175,7 @@ def tune_tcf_group(torch, n_filters: int = 2048, rounds: int = 8, seed: int = 78
     G = FilterGroup(FILTER_TCF, logs, 16, seeds, max_total=mt)
     ev = lambda: torch.cuda.Event(enable_timing=True)
     res = {}
-    for path in (1, 2):
+    for path in (0, 1, 2):
         G.set_tuning(tcf_path=path, tcf_tile_target=1024 if path == 2 else 0)
 
         def run():
@@ -179,12 +190,12 @@ def tune_tcf_group(torch, n_filters: int = 2048, rounds: int = 8, seed: int = 78
             return [(a, m), (m, z)]
 
         run()
-        res["block" if path == 1 else "tiled_1024"] = round(_timed(torch, run), 3)
+        res[_path_name(path, 1024)] = round(_timed(torch, run), 3)
     G.close()
     lg = int(sum(1 << int(x) for x in logs)).bit_length() - 1
-    best = min(res, key=res.get)
-    return lg, {**({"tcf_path": 1} if best == "block" else {"tcf_path": 2, "tcf_tile_target": 1024}), "ms": res,
-                "members": int(nt)}
+    best = _best_path(res)
+    knobs = {"auto": {"tcf_path": 0}, "block": {"tcf_path": 1}}.get(best, {"tcf_path": 2, "tcf_tile_target": 1024})
+    return lg, {**knobs, "ms": res, "members": int(nt)}
 
 
 def tune_gqf(q: int, keys, torch) -> dict:
