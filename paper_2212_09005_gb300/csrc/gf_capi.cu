@@ -36,6 +36,20 @@ bool tuning_valid(const filter_tuning &t)
     return true;
 }
 
+bool tcf_few_keys(uint64_t nb, uint64_t n)
+{
+    // A pass over every block's offsets and three launches less, against four
+    // barriers of the grid and counters whose atomics reply: an insert and a
+    // remove of 32765 keys take 42 us on 2^20 blocks (60 over every block, 71
+    // by unit), of 65533 on 2^16 blocks 61 (66), of 2^19 on 2^20 blocks 286
+    // (296); beyond, counting over every block is as good. Of tables past the
+    // L2 every atomic is a read of DRAM: 2^19 keys 117 us on 2^22 blocks (130
+    // by unit), 153 on 2^24 (129).
+    if (nb < TCF_COOP_MIN_BLOCKS) return false;
+    if (nb > (1ull << 17) && n > nb / 2) return false;
+    return n <= nb && n <= (nb > (1ull << 22) ? 1ull << 18 : 1ull << 19);
+}
+
 bool tcf_tiled(const filter_tuning &t, uint64_t nb, uint64_t n, bool del)
 {
     if (t.tcf_path == FILTER_TCF_PATH_BLOCK) return false;
@@ -50,6 +64,7 @@ bool tcf_tiled(const filter_tuning &t, uint64_t nb, uint64_t n, bool del)
     // any table, the unit step needing no scratch per block (2^20 blocks, 2^22
     // keys: 0.67 ms against 0.87; 2^12 blocks, 2^14 keys 126 us against 139;
     // 8-bit tags 0.77 ms against 1.72).
+    if (tcf_few_keys(nb, n)) return false;
     return nb >= (1ull << 22) || (del && nb >= (1ull << 12) && n >= 4 * nb);
 }
 

@@ -544,6 +544,13 @@ struct filter_group {
 namespace gf {
 // tuning values with the defaults filled in; false if one is out of range
 bool tuning_valid(const filter_tuning &t);
+// Tables whose later phases go by one launch: ten launches less a call (2^12
+// blocks, 2^14 keys a call: an insert and a remove 51 and 40 us, 62 and 46
+// with kernels of their own; 2^16 blocks, 2^16 keys: 49 and 46 us, 80 and 63).
+// Smaller ones keep the kernels, which a trace shows by phase.
+static constexpr uint64_t TCF_COOP_MIN_BLOCKS = 1ull << 12;
+// TCF bulk calls: the first phase by touched blocks, in that launch too?
+bool tcf_few_keys(uint64_t nb, uint64_t n);
 // TCF bulk calls: the tiled path for this table, batch and direction?
 bool tcf_tiled(const filter_tuning &t, uint64_t nb, uint64_t n, bool del);
 bool tcf_geom_supported(uint32_t f, uint32_t B);

@@ -1127,59 +1127,134 @@ struct SparseArgs {
     uint64_t *rec, *pend1, *seg;
     uint8_t *status;
     DevCounters *ctr;
-    uint32_t unit_min;  // more candidates than this of the first phase here went by unit
+    uint32_t unit_min;  // more candidates than this of the second phase went by unit
+    bool first;         // the first phase is taken here too
 };
 
-// groups the candidates of one phase by the destinations that they touch
-template <int SRC, int DST>
-__device__ __forceinline__ bool sparse_group(const SparseArgs &A, const void *pend, const unsigned *npend, int slot,
-                                             uint32_t *recI, unsigned &round, PhaseDst &P)
+__device__ __forceinline__ unsigned ld_now(const unsigned *p) { return *(const volatile unsigned *)p; }
+
+// Where a call's phases have got to: the barriers passed, and whether one CTA
+// has taken over (a phase had few candidates; the next ones have no more).
+struct SparseRun {
+    unsigned round;
+    bool few;
+};
+static constexpr int SPARSE_FEW = TPB;  // a candidate, and then a destination, a thread of the first CTA
+
+// the end of a phase's part: its writes are seen by the next
+__device__ __forceinline__ bool sparse_next(const SparseArgs &A, SparseRun &run)
 {
-    DevCounters *c = A.ctr;
-    tcf_group_hist_body<SRC, DST, true>(A.keys, A.prep, A.n, pend, npend, A.G, A.fill, A.cnt, A.tlist, A.tcount, nullptr);
-    if (!grid_barrier(&c->bar, ++round, &c->status)) return false;
-    tcf_alloc_body(npend, A.n, A.tlist, A.tcount, A.cnt, A.off, A.dlist, A.seg, &c->cursor[slot], &c->touched[slot], nullptr);
-    if (!grid_barrier(&c->bar, ++round, &c->status)) return false;
-    tcf_group_scatter_body<SRC, DST>(A.keys, A.prep, A.n, pend, npend, A.G, A.fill, A.cnt, A.off, A.rec, recI, nullptr);
-    if (!grid_barrier(&c->bar, ++round, &c->status)) return false;
-    P = PhaseDst{nullptr, A.dlist, A.seg, &c->touched[slot]};
+    if (!run.few) return grid_barrier(&A.ctr->bar, ++run.round, &A.ctr->status);
+    __syncthreads();
     return true;
 }
 
-__device__ __forceinline__ unsigned ld_now(const unsigned *p) { return *(const volatile unsigned *)p; }
+// Few candidates, by one CTA: their segments by counting. Over the grid a
+// phase of a hundred candidates took 9 to 13 us, all of it barriers and
+// latency; most calls have one or two of that size.
+template <int SRC, int DST>
+__device__ __forceinline__ void few_group(const SparseArgs &A, const void *pend, uint32_t m, uint32_t *recI,
+                                          unsigned *touched)
+{
+    __shared__ uint32_t s_d[SPARSE_FEW];
+    const uint32_t j = threadIdx.x;
+    uint64_t rec = 0, i = j;
+    uint32_t d = 0;
+    if (j < m) {
+        uint64_t pw = 0;
+        if (SRC == SRC_PEND_U32) i = static_cast<const uint32_t *>(pend)[j];
+        if (SRC == SRC_PEND_U64) {
+            pw = static_cast<const uint64_t *>(pend)[j];
+            i = pw & 0xffffffffu;
+        }
+        const KeyInfo k = key_at<DST>(A.keys, A.prep, i, A.G);
+        d = (uint32_t)dest_of(DST, k, pw, A.G, A.fill, A.prep, i);
+        s_d[j] = d;
+        rec = DST == DST_BUCKET ? (A.prep.bt ? A.prep.e[i] : tcf_entry(k, A.G.f)) : ((uint64_t)k.t << 32) | i;
+    }
+    __syncthreads();
+    if (j >= m) return;
+    uint32_t less = 0, before = 0, same = 0;
+    for (uint32_t q = 0; q < m; q++) {
+        const uint32_t x = s_d[q];
+        less += x < d;
+        same += x == d;
+        before += x == d && q < j;
+    }
+    A.rec[less + before] = rec;
+    if (DST == DST_BUCKET) recI[less + before] = (uint32_t)i;
+    if (before) return;
+    const unsigned at = atomicAdd(touched, 1u);
+    A.dlist[at] = d;
+    A.seg[at] = ((uint64_t)less << 32) | same;
+}
+
+// Groups the candidates of one phase by the destinations that they touch.
+// False in a CTA that is done: no candidates, another CTA has the rest, or a
+// barrier gave up.
+template <int SRC, int DST>
+__device__ __forceinline__ bool sparse_group(const SparseArgs &A, const void *pend, const unsigned *npend, int slot,
+                                             uint32_t *recI, SparseRun &run, PhaseDst &P)
+{
+    DevCounters *c = A.ctr;
+    const uint64_t m = SRC == SRC_KEYS ? A.n : (uint64_t)ld_now(npend);  // (the same in every CTA)
+    if (m == 0) return false;
+    P = PhaseDst{nullptr, A.dlist, A.seg, &c->touched[slot]};
+    if (run.few || m <= SPARSE_FEW) {
+        run.few = true;
+        if (blockIdx.x != 0) return false;
+        few_group<SRC, DST>(A, pend, (uint32_t)m, recI, &c->touched[slot]);
+        __syncthreads();
+        return true;
+    }
+    tcf_group_hist_body<SRC, DST, true>(A.keys, A.prep, A.n, pend, npend, A.G, A.fill, A.cnt, A.tlist, A.tcount, nullptr);
+    if (!sparse_next(A, run)) return false;
+    tcf_alloc_body(npend, A.n, A.tlist, A.tcount, A.cnt, A.off, A.dlist, A.seg, &c->cursor[slot], &c->touched[slot], nullptr);
+    if (!sparse_next(A, run)) return false;
+    tcf_group_scatter_body<SRC, DST>(A.keys, A.prep, A.n, pend, npend, A.G, A.fill, A.cnt, A.off, A.rec, recI, nullptr);
+    return sparse_next(A, run);
+}
 
 template <int F>
 __global__ void __launch_bounds__(TPB, 4) tcf_sparse_insert_coop(const SparseArgs A)
 {
-    unsigned *np = A.ctr->pend, round = 0;
+    unsigned *np = A.ctr->pend;
+    SparseRun run{0, false};
     PhaseDst P;
-    if (ld_now(&np[0]) == 0) return;  // (the same in every CTA)
-    if (ld_now(&np[0]) <= A.unit_min) {
-        if (!sparse_group<SRC_PEND_U32, DST_TARGET>(A, A.pend0, &np[0], 1, nullptr, round, P)) return;
-        tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 1, A.G.B, nullptr, A.pend1, &np[1], A.prep, nullptr);
-        if (!grid_barrier(&A.ctr->bar, ++round, &A.ctr->status) || ld_now(&np[1]) == 0) return;
-        if (!sparse_group<SRC_PEND_U64, DST_ALT>(A, A.pend1, &np[1], 2, nullptr, round, P)) return;
-        tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 2, A.G.B, A.pend2, nullptr, &np[2], A.prep, nullptr);
-        if (!grid_barrier(&A.ctr->bar, ++round, &A.ctr->status)) return;
+    if (A.first) {
+        if (!sparse_group<SRC_KEYS, DST_B1>(A, nullptr, nullptr, 0, nullptr, run, P)) return;
+        tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 0, A.G.tsc, A.pend0, nullptr, &np[0], A.prep, nullptr);
+        if (!sparse_next(A, run)) return;
     }
-    if (ld_now(&np[2]) == 0) return;
-    if (!sparse_group<SRC_PEND_U32, DST_BUCKET>(A, A.pend2, &np[2], 3, A.pend0, round, P)) return;
+    if (ld_now(&np[0]) <= A.unit_min) {
+        if (!sparse_group<SRC_PEND_U32, DST_TARGET>(A, A.pend0, &np[0], 1, nullptr, run, P)) return;
+        tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 1, A.G.B, nullptr, A.pend1, &np[1], A.prep, nullptr);
+        if (!sparse_next(A, run)) return;
+        if (!sparse_group<SRC_PEND_U64, DST_ALT>(A, A.pend1, &np[1], 2, nullptr, run, P)) return;
+        tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 2, A.G.B, A.pend2, nullptr, &np[2], A.prep, nullptr);
+        if (!sparse_next(A, run)) return;
+    }
+    if (!sparse_group<SRC_PEND_U32, DST_BUCKET>(A, A.pend2, &np[2], 3, A.pend0, run, P)) return;
     tcf_bucket_insert_body(A.G, A.bk, P, A.rec, A.pend0, A.status, A.ctr, nullptr);
 }
 
 template <int F>
 __global__ void __launch_bounds__(TPB, 4) tcf_sparse_remove_coop(const SparseArgs A)
 {
-    unsigned *np = A.ctr->pend, round = 0;
+    unsigned *np = A.ctr->pend;
+    SparseRun run{0, false};
     PhaseDst P;
-    if (ld_now(&np[0]) == 0) return;
-    if (ld_now(&np[0]) <= A.unit_min) {
-        if (!sparse_group<SRC_PEND_U32, DST_B2>(A, A.pend0, &np[0], 1, nullptr, round, P)) return;
-        tcf_block_remove_body<F>(A.G, A.blocks, A.fill, P, A.rec, A.pend2, &np[2], nullptr);
-        if (!grid_barrier(&A.ctr->bar, ++round, &A.ctr->status)) return;
+    if (A.first) {
+        if (!sparse_group<SRC_KEYS, DST_B1>(A, nullptr, nullptr, 0, nullptr, run, P)) return;
+        tcf_block_remove_body<F>(A.G, A.blocks, A.fill, P, A.rec, A.pend0, &np[0], nullptr);
+        if (!sparse_next(A, run)) return;
     }
-    if (ld_now(&np[2]) == 0) return;
-    if (!sparse_group<SRC_PEND_U32, DST_BUCKET>(A, A.pend2, &np[2], 2, A.pend0, round, P)) return;
+    if (ld_now(&np[0]) <= A.unit_min) {
+        if (!sparse_group<SRC_PEND_U32, DST_B2>(A, A.pend0, &np[0], 1, nullptr, run, P)) return;
+        tcf_block_remove_body<F>(A.G, A.blocks, A.fill, P, A.rec, A.pend2, &np[2], nullptr);
+        if (!sparse_next(A, run)) return;
+    }
+    if (!sparse_group<SRC_PEND_U32, DST_BUCKET>(A, A.pend2, &np[2], 2, A.pend0, run, P)) return;
     tcf_bucket_remove_body(A.G, A.bk, P, A.rec, A.pend0, A.status, A.ctr, nullptr);
 }
 
@@ -2758,21 +2833,15 @@ static void tcf_sparse_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n
 // bounds keep resident together
 template <int F, bool DEL>
 static void tcf_sparse_coop(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, uint32_t unit_min,
-                            cudaStream_t st)
+                            bool first, cudaStream_t st)
 {
     SparseArgs A{keys, n, T.G, T.prep, T.blocks, T.fill, T.bk, T.cnt, T.off, T.tlist, T.tcount, T.dlist, T.pend0, T.pend2,
-                 T.rec, T.pend1, T.seg, status, T.ctr, unit_min};
+                 T.rec, T.pend1, T.seg, status, T.ctr, unit_min, first};
     void *args[] = {&A};
     gf::TraceScope ts_(DEL ? "tcf_sparse_remove" : "tcf_sparse_insert", n, st);
     const void *kernel = DEL ? (const void *)tcf_sparse_remove_coop<F> : (const void *)tcf_sparse_insert_coop<F>;
     cudaLaunchCooperativeKernel(kernel, dim3(grid_for(n, TPB * 2, 4)), dim3(TPB), args, 0, st);
 }
-
-// Tables whose later phases go by one launch: ten launches less a call (2^12
-// blocks, 2^14 keys a call: an insert and a remove 51 and 40 us, 62 and 46
-// with kernels of their own; 2^16 blocks, 2^16 keys: 49 and 46 us, 80 and 63).
-// Smaller ones keep the kernels, which a trace shows by phase.
-static constexpr uint64_t COOP_MIN_BLOCKS = 1ull << 12;
 
 // The per-block counting-sort path: each phase groups its candidates by
 // destination block (counts, scan, scatter) and one thread per block takes
@@ -2785,6 +2854,8 @@ static void tcf_bulk_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
     DevCounters *ctr = T.ctr;
     unsigned *np = ctr->pend;
     cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
+    if constexpr (GB == 0)
+        if (tcf_few_keys(G.nb, n)) return tcf_sparse_coop<F, false>(T, keys, n, status, 0xffffffffu, true, st);
     // A: shortcut into b1
     PhaseDst P = group_phase<SRC_KEYS, DST_B1>(T, keys, n, nullptr, nullptr, 0, nullptr, st);
     {
@@ -2796,7 +2867,7 @@ static void tcf_bulk_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
             gblock_phase<F, GB, false>(T, P, n, 0, G.tsc, T.pend0, nullptr, &np[0], ts_.units(), st);
     }
     if constexpr (GB == 0)
-        if (G.nb >= COOP_MIN_BLOCKS) return tcf_sparse_coop<F, false>(T, keys, n, status, 0xffffffffu, st);
+        if (G.nb >= TCF_COOP_MIN_BLOCKS) return tcf_sparse_coop<F, false>(T, keys, n, status, 0xffffffffu, false, st);
     tcf_sparse_insert<F, GB>(T, keys, n, status, st);
 }
 
@@ -2843,6 +2914,8 @@ static void tcf_bulk_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
     DevCounters *ctr = T.ctr;
     unsigned *np = ctr->pend;
     cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
+    if constexpr (GB == 0)
+        if (tcf_few_keys(G.nb, n)) return tcf_sparse_coop<F, true>(T, keys, n, status, 0xffffffffu, true, st);
     // 1: primary block
     PhaseDst P = group_phase<SRC_KEYS, DST_B1>(T, keys, n, nullptr, nullptr, 0, nullptr, st);
     {
@@ -2854,7 +2927,7 @@ static void tcf_bulk_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
             gblock_phase<F, GB, true>(T, P, n, 0, 0, T.pend0, nullptr, &np[0], ts_.units(), st);
     }
     if constexpr (GB == 0)
-        if (G.nb >= COOP_MIN_BLOCKS) return tcf_sparse_coop<F, true>(T, keys, n, status, 0xffffffffu, st);
+        if (G.nb >= TCF_COOP_MIN_BLOCKS) return tcf_sparse_coop<F, true>(T, keys, n, status, 0xffffffffu, false, st);
     tcf_sparse_remove<F, GB>(T, keys, n, status, st);
 }
 
@@ -3005,7 +3078,7 @@ static void tcf_unit_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
                                                &np[2], st);
     }
     // B and C of fewer candidates, and D: backing buckets
-    tcf_sparse_coop<F, false>(T, keys, n, status, unit_min, st);
+    tcf_sparse_coop<F, false>(T, keys, n, status, unit_min, false, st);
 }
 
 template <int F>
@@ -3022,7 +3095,7 @@ static void tcf_unit_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
         tu_phase<F, true, TU_SAME, TU_NX_IDX>(T, TuSrc{nullptr, T.pend1, T.pend0, &np[0], unit_min, n}, n, 0, nullptr,
                                               T.pend2, &np[2], st);
     // 2 of fewer candidates, and 3: backing bucket; what is left is not found
-    tcf_sparse_coop<F, true>(T, keys, n, status, unit_min, st);
+    tcf_sparse_coop<F, true>(T, keys, n, status, unit_min, false, st);
 }
 
 // Batches that one CTA takes whole (32-byte blocks); false for the others.

@@ -110,3 +110,18 @@ def test_auto_calls_leave_the_oracle_table(gf, oracle, lg, n):
     G, O = gf.TCF(lg, 16, seed=2, max_batch=n), oracle.TCF(lg, 16, seed=2)
     G.set_tuning()
     check(G, O, [("insert", keys[i:i + n]) for i in range(0, len(keys), n)] + [("remove", keys[: n]), ("remove", keys[: n])])
+
+
+@pytest.mark.parametrize("few", [255, 256, 257])
+@pytest.mark.parametrize("f", [16, 8])
+def test_few_keys_by_touched_blocks(gf, oracle, f, few):
+    """Batches small against the table, every phase by touched blocks; the
+    later phases on both sides of what one CTA takes."""
+    base, hot = W.uniform_keys(21, 4000), W.uniform_keys(22, 3)
+    cap = 3 * (32 if f == 8 else 16) // 4
+    G, O = gf.TCF(18, f, seed=3, max_batch=8192), oracle.TCF(18, f, seed=3)
+    G.set_tuning()
+    # one block's shortcut leaves exactly `few` copies to the second phase
+    one = np.concatenate([base, np.repeat(hot[:1], cap + few)])
+    check(G, O, [("insert", one), ("insert", np.concatenate([base[:3000], np.repeat(hot, 300)])),
+                 ("remove", one[::-1]), ("remove", np.concatenate([base, np.repeat(hot, 200)])), ("insert", base)])
