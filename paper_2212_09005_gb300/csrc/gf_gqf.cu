@@ -109,7 +109,7 @@ struct MergeSmem {
     long long wA[MT / 32], wB[MT / 32];
     long long prev_end_old, os0, ein, w0, w1, tileP;
     unsigned long long glo, ghi;
-    unsigned int tile, kold, oldlen, err, gcap, nmix;
+    unsigned int kold, oldlen, err, gcap, nmix;
 };
 
 // staged groups: GSMALL of them, or (no old runs) as many as fill oend, old and gsm
@@ -307,10 +307,107 @@ __device__ __forceinline__ unsigned long long ld_vol(const unsigned long long *p
     return *(const volatile unsigned long long *)p;
 }
 
-// One tile of one filter. `tile` is the filter's own tile index; S.err is 0.
-template <int R>
-__device__ __forceinline__ void merge_tile(const MergeArgs &a, MergeSmem<R> &S, const uint64_t tile)
+// Decoupled look-back over tiles, CTA-wide: MT predecessors per round. (TA, TB):
+// the tile's aggregate; returns the end of the last run before the tile.
+// One status word per tile: bits 62-63 flag (1 aggregate, 2 inclusive end);
+// aggregate payload (A - Q0 + 1) << 31 | B, with 0 in the A field for a tile
+// without runs; inclusive payload P + 1. A tile whose aggregate does not fit
+// publishes only its inclusive end.
+__device__ __forceinline__ long long tile_lookback(unsigned long long *st, DevCounters *ctr, const uint64_t tile,
+                                                   const long long Q0, const long long TA, const long long TB)
 {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned full = 0xffffffffu;
+    __shared__ long long lbA[MT / 32], lbB[MT / 32], lbP;
+    __shared__ int lb_incl;
+    __shared__ unsigned lb_timeout;
+    const long long arel = (TA == NEG_INF) ? 0 : TA - Q0 + 1;
+    const bool packable = TB < (1ll << 31) && arel >= 0 && arel < (1ll << 31);
+    if (tid == 0) {
+        lb_timeout = 0;
+        if (tile > 0 && packable)
+            atomicExch(&st[tile], (1ull << 62) | ((unsigned long long)arel << 31) | (unsigned long long)TB);
+    }
+    long long ein = -1;
+    if (tile > 0) {
+        long long gA = NEG_INF, gB = 0;  // composition of the newer tiles of earlier rounds
+        long long jtop = (long long)tile - 1;
+        while (true) {
+            const long long j = jtop - tid;
+            unsigned long long wd = 2ull << 62;  // before tile 0: inclusive end -1
+            if (j >= 0) {
+                wd = ld_vol(&st[j]);
+                uint32_t spins = 0, ns = 32;
+                while ((wd >> 62) == 0) {
+                    if (++spins > (SPIN_LIMIT >> 2)) {
+                        lb_timeout = 1;
+                        break;
+                    }
+                    __nanosleep(ns);
+                    if (ns < 512) ns <<= 1;
+                    wd = ld_vol(&st[j]);
+                }
+            }
+            const unsigned flag = (unsigned)(wd >> 62);
+            if (tid == 0) lb_incl = MT;
+            __syncthreads();
+            if (flag == 2) atomicMin(&lb_incl, tid);
+            __syncthreads();
+            const int Lc = lb_incl;
+            long long A = NEG_INF, Bv = 0;
+            if (tid < Lc && flag == 1) {
+                const unsigned long long ar = (wd >> 31) & 0x7fffffffull;
+                Bv = (long long)(wd & 0x7fffffffull);
+                A = ar ? (long long)ar - 1 + j * TQ : NEG_INF;
+            }
+            // ordered composition, thread tid + 1 being the older tile
+            for (int o = 1; o < 32; o <<= 1) {
+                long long oA = __shfl_down_sync(full, A, o), oB = __shfl_down_sync(full, Bv, o);
+                if (lane + o < 32) {
+                    agg_combine(oA, oB, A, Bv);
+                    A = oA;
+                    Bv = oB;
+                }
+            }
+            if (lane == 0) {
+                lbA[warp] = A;
+                lbB[warp] = Bv;
+            }
+            if (tid == Lc) lbP = (long long)(wd & ((1ull << 62) - 1ull)) - 1;
+            __syncthreads();
+            long long WA = NEG_INF, WB = 0;
+            for (int w = MT / 32 - 1; w >= 0; w--) agg_combine(WA, WB, lbA[w], lbB[w]);
+            agg_combine(WA, WB, gA, gB);
+            if (lb_timeout) {
+                if (tid == 0) atomicOr(&ctr->status, ST_TIMEOUT);
+                break;
+            }
+            if (Lc < MT) {
+                long long v = lbP + WB;
+                ein = v > WA ? v : WA;
+                break;
+            }
+            gA = WA;
+            gB = WB;
+            jtop -= MT;
+        }
+    }
+    if (tid == 0) {
+        const long long v = ein + TB;
+        const long long P = v > TA ? v : TA;
+        atomicExch(&st[tile], (2ull << 62) | (unsigned long long)(P + 1));
+        atomicMax(&ctr->gqf_end, P);
+    }
+    return ein;
+}
+
+// One tile of one filter of any size: whatever does not fit merge_tile's
+// stages. `tile` is the filter's own tile index.
+template <int R>
+__device__ __noinline__ void merge_tile_any(const MergeArgs &a, MergeSmem<R> &S, const uint64_t tile)
+{
+    if (threadIdx.x == 0) S.err = 0;
+    __syncthreads();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long Q0 = (long long)tile * TQ;
     const uint64_t j0 = tile * TBLK;
@@ -573,98 +670,17 @@ __device__ __forceinline__ void merge_tile(const MergeArgs &a, MergeSmem<R> &S, 
         xA = pA;
         xB = pB;
     }
-    // 8. decoupled look-back over tiles, CTA-wide: MT predecessors per round.
-    // One status word per tile: bits 62-63 flag (1 aggregate, 2 inclusive end);
-    // aggregate payload (A - Q0 + 1) << 31 | B, with 0 in the A field for a tile
-    // without runs; inclusive payload P + 1. A tile whose aggregate does not fit
-    // publishes only its inclusive end.
+    // 8. decoupled look-back
     {
-        const unsigned full = 0xffffffffu;
-        __shared__ long long lbA[MT / 32], lbB[MT / 32], lbP;
-        __shared__ int lb_incl;
-        __shared__ unsigned lb_timeout;
         long long TA = NEG_INF, TB = 0;
         for (int w = 0; w < MT / 32; w++) agg_combine(TA, TB, S.wA[w], S.wB[w]);
-        unsigned long long *st = a.ts + 1;
-        const long long arel = (TA == NEG_INF) ? 0 : TA - Q0 + 1;
-        const bool packable = TB < (1ll << 31) && arel >= 0 && arel < (1ll << 31);
-        if (tid == 0) {
-            lb_timeout = 0;
-            if (tile > 0 && packable)
-                atomicExch(&st[tile], (1ull << 62) | ((unsigned long long)arel << 31) | (unsigned long long)TB);
-        }
-        long long ein = -1;
-        if (tile > 0) {
-            long long gA = NEG_INF, gB = 0;  // composition of the newer tiles of earlier rounds
-            long long jtop = (long long)tile - 1;
-            while (true) {
-                const long long j = jtop - tid;
-                unsigned long long wd = 2ull << 62;  // before tile 0: inclusive end -1
-                if (j >= 0) {
-                    wd = ld_vol(&st[j]);
-                    uint32_t spins = 0, ns = 32;
-                    while ((wd >> 62) == 0) {
-                        if (++spins > (SPIN_LIMIT >> 2)) {
-                            lb_timeout = 1;
-                            break;
-                        }
-                        __nanosleep(ns);
-                        if (ns < 512) ns <<= 1;
-                        wd = ld_vol(&st[j]);
-                    }
-                }
-                const unsigned flag = (unsigned)(wd >> 62);
-                if (tid == 0) lb_incl = MT;
-                __syncthreads();
-                if (flag == 2) atomicMin(&lb_incl, tid);
-                __syncthreads();
-                const int Lc = lb_incl;
-                long long A = NEG_INF, Bv = 0;
-                if (tid < Lc && flag == 1) {
-                    const unsigned long long ar = (wd >> 31) & 0x7fffffffull;
-                    Bv = (long long)(wd & 0x7fffffffull);
-                    A = ar ? (long long)ar - 1 + j * TQ : NEG_INF;
-                }
-                // ordered composition, thread tid + 1 being the older tile
-                for (int o = 1; o < 32; o <<= 1) {
-                    long long oA = __shfl_down_sync(full, A, o), oB = __shfl_down_sync(full, Bv, o);
-                    if (lane + o < 32) {
-                        agg_combine(oA, oB, A, Bv);
-                        A = oA;
-                        Bv = oB;
-                    }
-                }
-                if (lane == 0) {
-                    lbA[warp] = A;
-                    lbB[warp] = Bv;
-                }
-                if (tid == Lc) lbP = (long long)(wd & ((1ull << 62) - 1ull)) - 1;
-                __syncthreads();
-                long long WA = NEG_INF, WB = 0;
-                for (int w = MT / 32 - 1; w >= 0; w--) agg_combine(WA, WB, lbA[w], lbB[w]);
-                agg_combine(WA, WB, gA, gB);
-                if (lb_timeout) {
-                    if (tid == 0) atomicOr(&a.ctr->status, ST_TIMEOUT);
-                    break;
-                }
-                if (Lc < MT) {
-                    long long v = lbP + WB;
-                    ein = v > WA ? v : WA;
-                    break;
-                }
-                gA = WA;
-                gB = WB;
-                jtop -= MT;
-            }
-        }
+        const long long ein = tile_lookback(a.ts + 1, a.ctr, tile, Q0, TA, TB);
         if (tid == 0) {
             long long v = ein + TB;
             long long P = v > TA ? v : TA;
-            atomicExch(&st[tile], (2ull << 62) | (unsigned long long)(P + 1));
+            if (P >= (long long)a.nslots) atomicExch(&a.ctr->overflow, 1ull);
             S.ein = ein;
             S.tileP = P;
-            atomicMax(&a.ctr->gqf_end, P);
-            if (P >= (long long)a.nslots) atomicExch(&a.ctr->overflow, 1ull);
             long long w0 = Q0 > ein + 1 ? Q0 : ein + 1;
             long long w1 = slot_end > P + 1 ? slot_end : P + 1;
             if (w1 > (long long)a.nslots) w1 = (long long)a.nslots;
@@ -817,6 +833,447 @@ __device__ __forceinline__ void merge_tile(const MergeArgs &a, MergeSmem<R> &S, 
     }
 }
 
+// ---------------------------------------------------------------------------
+// The usual tile: at most FCAP old slots and new groups. Its entries (quotient,
+// remainder, count) are laid out in order with room for every old slot and new
+// group, and each thread then places a stretch of them in one go; all positions
+// are 32-bit, from Q0. A thread per new group walks the old run of its quotient
+// to its place; a thread per old run writes that run's groups, moved up by the
+// new ones before them.
+// Bound by instructions: 2^24 slots of 8 bits, from empty to 45 % load 109 us,
+// on to 90 % 291, a third of the first keys removed 262; by quotients, the runs
+// with old and new groups merged once for their length and again for their
+// place, these took 174, 528 and 475 (2^28 slots: 1.76, 4.27 and 3.96 ms, and
+// 2.55, 8.51 and 7.50).
+// ---------------------------------------------------------------------------
+static constexpr uint32_t FCAP = 3072;
+static constexpr uint32_t FOUT = FCAP + 64;  // staged new slots, from a multiple of 64
+static constexpr uint32_t F_QBITS = 53, F_RBITS = 37;  // an entry: quotient, remainder (16 bits), count
+static constexpr unsigned long long F_CMASK = (1ull << F_RBITS) - 1ull;
+static constexpr int F_NONE = -(1 << 30);
+
+template <int R>
+struct FastSmem {
+    using T = typename SlotIO<R>::T;
+    unsigned long long m[FCAP];                 // entries in order; 0: none here
+    union {
+        uint32_t ins[FCAP / 2 + 4];             // new groups that go before an old slot, then those up to it (16 bits each)
+        T out[FOUT];
+    };
+    T old[FCAP + 16];                           // old slots, from a multiple of 16 bytes
+    uint16_t oend[TQ];                          // old run ends from os0
+    uint32_t dead[FCAP / 32 + 1];               // old groups that a new one's entry stands for
+    uint32_t occ[TQ / 32], wpre[TQ / 32 + 1], nocc[TQ / 32], off[TBLK], rend[FOUT / 32];
+    uint32_t sel[MT / 32];
+    int wA[MT / 32], wB[MT / 32], wQ[MT / 32];
+    long long prev_end, os0;
+    uint32_t glo, ghi, yfirst, oldlen, err;
+};
+
+// the group of an old run [.., e] at slot p: its value, count and slots
+template <class T>
+__device__ __forceinline__ uint32_t old_group(const T *old, uint32_t p, uint32_t e, uint32_t r, uint32_t &v, uint64_t &c)
+{
+    v = old[p];
+    c = 1;
+    if (p + 2 > e || old[p + 1] != v) return 1;
+    uint32_t nd = old[p + 2];
+    if (p + 2 + nd > e) nd = e - p - 2;  // malformed: stay in the run
+    uint64_t acc = 0;
+    for (uint32_t d = 0; d < nd; d++) acc = (acc << r) | old[p + 3 + d];
+    c = acc + 2;
+    return 3 + nd;
+}
+
+template <int R>
+__device__ __forceinline__ void fast_put(FastSmem<R> &S, const MergeArgs &a, long long Q0, int wa, int pos, uint32_t v)
+{
+    const uint32_t d = (uint32_t)(pos - wa);
+    if (d < FOUT) S.out[d] = (typename SlotIO<R>::T)v;
+    else if (Q0 + pos < (long long)a.nslots) wr_slot<R>(a.rem_new, (uint64_t)(Q0 + pos), v);
+}
+
+template <int R>
+__device__ __forceinline__ void fast_rend(FastSmem<R> &S, const MergeArgs &a, long long Q0, int wa, int pos)
+{
+    const uint32_t d = (uint32_t)(pos - wa);
+    if (d < FOUT) atomicOr(&S.rend[d >> 5], 1u << (d & 31));
+    else if (Q0 + pos < (long long)a.nslots) atomicOr(&a.meta_new[(Q0 + pos) >> 6].rend, 1ull << ((Q0 + pos) & 63));
+}
+
+// offsets of the blocks whose first quotient is in [from, to): runs up to there end at pe
+template <int R>
+__device__ __forceinline__ void fast_offsets(FastSmem<R> &S, int from, int to, int pe)
+{
+    for (int j = (from + 63) >> 6; 64 * j < to; j++) S.off[j] = pe > 64 * j ? (uint32_t)(pe - 64 * j) : 0u;
+}
+
+// false (nothing written): the tile does not fit
+template <int R>
+__device__ __forceinline__ bool merge_tile(const MergeArgs &a, FastSmem<R> &S, const uint64_t tile)
+{
+    using T = typename SlotIO<R>::T;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long Q0 = (long long)tile * TQ;
+    const uint64_t j0 = tile * TBLK;
+    // occupieds, and the runs before each word of them
+    if (tid < TBLK) {
+        const unsigned long long w = j0 + tid < a.nblk ? a.meta_old[j0 + tid].occ : 0ull;
+        S.occ[2 * tid] = (uint32_t)w;
+        S.occ[2 * tid + 1] = (uint32_t)(w >> 32);
+        const uint32_t c = __popcll(w);
+        uint32_t incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        S.wpre[2 * tid] = incl - c;
+        S.wpre[2 * tid + 1] = incl - c + __popc((uint32_t)w);
+        if (tid == TBLK - 1) S.wpre[TQ / 32] = incl;
+        const uint32_t any = __ballot_sync(0xffffffffu, w != 0);
+        if (any && lane == __ffs(any) - 1) S.yfirst = 64 * lane + __ffsll((long long)w) - 1;
+    } else if (tid == TBLK) {
+        S.glo = a.tlo[tile];
+        S.ghi = a.thi[tile];
+        S.err = 0;
+        S.oldlen = 0;
+    }
+    for (int p = tid; p < (int)(FCAP / 32 + 1); p += MT) S.dead[p] = 0;
+    for (int p = tid; p < (int)(FOUT / 32); p += MT) S.rend[p] = 0;
+    if (tid < TQ / 32) S.nocc[tid] = 0;
+    __syncthreads();
+    const uint32_t kold = S.wpre[TQ / 32], glo = S.glo, ghi = S.ghi, nn = ghi - glo;
+    if (!a.del && nn > FCAP) return false;
+    if (kold > 0) {
+        // the run before the tile's first, and where its old slots start
+        const long long base = Q0 + (long long)a.meta_old[j0].off;
+        const bool q0occ = S.occ[0] & 1u;
+        const long long sp = q0occ ? base : base + 1;
+        if (tid == 0) {
+            long long pe = base;
+            if (q0occ) {
+                // last runend in [Q0, base - 1]; Q0 is a multiple of 64
+                pe = Q0 - 1;
+                for (long long p = base - 1; p >= Q0;) {
+                    const long long w = p >> 6;
+                    const unsigned pb = (unsigned)(p & 63);
+                    const unsigned long long bits = a.meta_old[w].rend & (pb == 63 ? ~0ull : ((1ull << (pb + 1)) - 1ull));
+                    if (bits) {
+                        pe = 64 * w + 63 - __clzll((long long)bits);
+                        break;
+                    }
+                    p = 64 * w - 1;
+                }
+            }
+            const long long y = Q0 + S.yfirst;
+            S.os0 = y > pe + 1 ? y : pe + 1;
+        }
+        __syncthreads();
+        const long long os0 = S.os0;
+        // old run ends: select over runends after the offset of block j0, each
+        // thread taking 16 bits of one of 64 words a round
+        const unsigned quarter = tid & 3;
+        uint32_t found = 0;
+        for (long long w0 = sp >> 6; found < kold; w0 += MT / 4) {
+            const long long ww = w0 + (tid >> 2);
+            unsigned long long bits = (ww < (long long)a.nblk) ? a.meta_old[ww].rend : 0ull;
+            if (ww == (sp >> 6)) bits &= (~0ull) << (sp & 63);
+            uint32_t b16 = (uint32_t)(bits >> (16 * quarter)) & 0xffffu;
+            const uint32_t c = __popc(b16);
+            uint32_t incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (lane == 31) S.sel[warp] = incl;
+            __syncthreads();
+            uint32_t pre = 0, tot = 0;
+#pragma unroll
+            for (int v = 0; v < MT / 32; v++) {
+                const uint32_t x = S.sel[v];
+                pre += v < warp ? x : 0u;
+                tot += x;
+            }
+            uint32_t idx = found + pre + incl - c;
+            const long long at = ww * 64 + 16 * quarter - os0;
+            while (b16 && idx < kold) {
+                const long long e = at + __ffs(b16) - 1;
+                S.oend[idx] = (uint16_t)(e < 0 || e > 0xffff ? 0xffff : e);
+                if (idx == kold - 1) S.oldlen = e < 0 || e >= (long long)FCAP ? ~0u : (uint32_t)e + 1u;
+                b16 &= b16 - 1;
+                idx++;
+            }
+            found += tot;
+            __syncthreads();  // sel is rewritten by the next round
+            if (found < kold && w0 + MT / 4 >= (long long)a.nblk) return false;  // (the same decision in every thread)
+        }
+        const uint32_t oldlen = S.oldlen;
+        if (oldlen > FCAP || oldlen + (a.del ? 0u : nn) > FCAP) return false;
+        // the old slots; entries and counters are cleared
+        constexpr uint32_t SPC = 16 / sizeof(T);
+        const long long a0 = os0 & ~(long long)(SPC - 1);
+        const uint32_t chunks = (uint32_t)(os0 - a0 + oldlen + SPC - 1) / SPC;
+        if (reinterpret_cast<uintptr_t>(a.rem_old) % 16)  // (a caller's image)
+            for (uint32_t i = tid; i < chunks * SPC; i += MT) S.old[i] = (T)rd_slot<R>(a.rem_old, (uint64_t)a0 + i);
+        else
+            for (uint32_t i = tid; i < chunks; i += MT)
+                reinterpret_cast<uint4 *>(S.old)[i] = reinterpret_cast<const uint4 *>(a.rem_old + a0 * (long long)sizeof(T))[i];
+        const uint32_t len = oldlen + (a.del ? 0u : nn);
+        for (uint32_t i = tid; i < len; i += MT) S.m[i] = 0;
+        if (!a.del)
+            for (uint32_t i = tid; i < oldlen / 2 + 2; i += MT) S.ins[i] = 0;
+        __syncthreads();
+    }
+    const uint32_t oldlen = kold ? S.oldlen : 0u;
+    const int y0 = (int)(Q0 - S.os0);  // quotient y is y0 + y from os0 (with old runs)
+    const T *old = S.old + ((uint32_t)S.os0 & (16 / sizeof(T) - 1));
+    bool big = false;  // a count that an entry does not hold
+    // new groups
+    for (uint32_t i0 = tid; i0 < nn; i0 += GB * MT) {
+        uint64_t fv[GB];
+        uint32_t s0[GB], s1[GB];
+#pragma unroll
+        for (int u = 0; u < GB; u++) {
+            const uint32_t g = glo + i0 + u * MT;
+            if (g < ghi) {
+                fv[u] = a.ufp[g];
+                s0[u] = a.ustart[g];
+                s1[u] = a.ustart[g + 1];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < GB; u++) {
+            const uint32_t i = i0 + u * MT, g = glo + i;
+            if (g >= ghi) break;
+            uint32_t y, rem;
+            uint64_t cnt;
+            decode_group<R>(a, Q0, fv[u], s0[u], s1[u], y, rem, cnt);
+            const unsigned long long key = ((unsigned long long)y << F_QBITS) | ((unsigned long long)rem << F_RBITS);
+            if (kold == 0) {
+                if (!a.del) S.m[i] = key | cnt;
+                else if (a.removed) a.removed[g] = 0;
+                continue;
+            }
+            const uint32_t w = S.occ[y >> 5], k = S.wpre[y >> 5] + __popc(w & ((1u << (y & 31)) - 1u));
+            uint32_t p = k ? S.oend[k - 1] + 1u : 0u;
+            bool match = false;
+            uint64_t oc = 0;
+            if ((w >> (y & 31)) & 1u) {
+                const uint32_t e = S.oend[k];
+                if (k) p = max((int)p, y0 + (int)y);
+                uint32_t v = 0;
+                while (p <= e) {
+                    const uint32_t l = old_group(old, p, e, R, v, oc);
+                    if (v >= rem) break;
+                    p += l;
+                }
+                match = p <= e && v == rem;
+            }
+            p = min(p, oldlen);  // (further on only in a malformed table)
+            if (match) atomicOr(&S.dead[p >> 5], 1u << (p & 31));
+            if (a.del) {
+                const uint64_t rm = !match ? 0 : oc < cnt ? oc : cnt;
+                if (a.removed) a.removed[g] = (uint32_t)rm;
+                if (match && oc > rm) S.m[p] = key | (oc - rm);
+                big |= match && oc - rm > F_CMASK;
+            } else {
+                cnt += match ? oc : 0;
+                big |= cnt > F_CMASK;
+                S.m[p + i] = key | (cnt & F_CMASK);
+                atomicAdd(&S.ins[p >> 1], 1u << (16 * (p & 1)));
+            }
+        }
+    }
+    if (kold > 0) {
+        if (!a.del && nn) {
+            // new groups before each old slot's place
+            __syncthreads();
+            constexpr uint32_t PW = (FCAP / 2 + MT - 1) / MT;
+            uint32_t v[PW], sum = 0;
+#pragma unroll
+            for (uint32_t j = 0; j < PW; j++) {
+                const uint32_t i = tid * PW + j;
+                v[j] = 2 * i < oldlen ? S.ins[i] : 0u;
+                sum += (v[j] & 0xffffu) + (v[j] >> 16);
+            }
+            uint32_t incl = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (lane == 31) S.sel[warp] = incl;
+            __syncthreads();
+            uint32_t run = incl - sum;
+#pragma unroll
+            for (int x = 0; x < MT / 32; x++) run += x < warp ? S.sel[x] : 0u;
+#pragma unroll
+            for (uint32_t j = 0; j < PW; j++) {
+                const uint32_t i = tid * PW + j;
+                if (2 * i >= oldlen) break;
+                const uint32_t lo = run + (v[j] & 0xffffu), hi = lo + (v[j] >> 16);
+                S.ins[i] = lo | (hi << 16);
+                run = hi;
+            }
+        }
+        __syncthreads();
+        // old groups, a thread per run
+        const uint16_t *pre = reinterpret_cast<const uint16_t *>(S.ins);
+        const bool moved = !a.del && nn;
+        for (int y = tid; y < TQ; y += MT) {
+            const uint32_t w = S.occ[y >> 5];
+            if (!((w >> (y & 31)) & 1u)) continue;
+            const uint32_t k = S.wpre[y >> 5] + __popc(w & ((1u << (y & 31)) - 1u)), e = S.oend[k];
+            uint32_t p = k ? (uint32_t)max((int)S.oend[k - 1] + 1, y0 + y) : 0u;
+            while (p <= e) {
+                uint32_t v;
+                uint64_t c;
+                const uint32_t l = old_group(old, p, e, R, v, c);
+                if (!((S.dead[p >> 5] >> (p & 31)) & 1u)) {
+                    big |= c > F_CMASK;
+                    S.m[moved ? p + pre[p] : p] =
+                        ((unsigned long long)y << F_QBITS) | ((unsigned long long)v << F_RBITS) | (c & F_CMASK);
+                }
+                p += l;
+            }
+        }
+    }
+    if (__syncthreads_or(big)) return false;
+    // a thread's stretch: the end of its runs by the operator of the placement
+    const uint32_t len = oldlen + (a.del ? 0u : nn), per = ((len + MT - 1) / MT) | 1u;
+    const uint32_t i0 = min(tid * per, len), i1 = min(i0 + per, len);
+    int A = F_NONE, B = 0, lq = -1;
+    for (uint32_t i = i0; i < i1; i++) {
+        const unsigned long long x = S.m[i];
+        const uint64_t c = x & F_CMASK;
+        if (c == 0) continue;
+        lq = (int)(x >> F_QBITS);
+        const int L = (int)enc_len(c, R);
+        A = max(lq + L - 1, A + L);
+        B += L;
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int pA = __shfl_up_sync(0xffffffffu, A, o), pB = __shfl_up_sync(0xffffffffu, B, o);
+        const int pq = __shfl_up_sync(0xffffffffu, lq, o);
+        if (lane >= o) {
+            A = max(A, pA + B);
+            B += pB;
+            lq = max(lq, pq);
+        }
+    }
+    if (lane == 31) {
+        S.wA[warp] = A;
+        S.wB[warp] = B;
+        S.wQ[warp] = lq;
+    }
+    int xA = __shfl_up_sync(0xffffffffu, A, 1), xB = __shfl_up_sync(0xffffffffu, B, 1);
+    int xq = __shfl_up_sync(0xffffffffu, lq, 1);
+    if (lane == 0) {
+        xA = F_NONE;
+        xB = 0;
+        xq = -1;
+    }
+    __syncthreads();
+    int tA = F_NONE, tB = 0, tq = -1, wA = F_NONE, wB = 0, wq = -1;
+#pragma unroll
+    for (int w = 0; w < MT / 32; w++) {
+        if (w == warp) {
+            wA = tA;
+            wB = tB;
+            wq = tq;
+        }
+        tA = max(S.wA[w], tA + S.wB[w]);
+        tB += S.wB[w];
+        tq = max(tq, S.wQ[w]);
+    }
+    xA = max(xA, wA + xB);
+    xB += wB;
+    xq = max(xq, wq);
+    const long long ein = tile_lookback(a.ts + 1, a.ctr, tile, Q0, tA < 0 ? NEG_INF : Q0 + tA, (long long)tB);
+    if (ein - Q0 > (1ll << 29)) return false;  // (publishing the tile's words twice does no harm)
+    const int er = (int)max(ein - Q0, -1ll);
+    const int P = max(er + tB, tA);
+    if (tid == 0 && max(ein + tB, tA < 0 ? NEG_INF : Q0 + tA) >= (long long)a.nslots) atomicExch(&a.ctr->overflow, 1ull);
+    if (a.dry) return true;
+    // the tile writes the new slots [w0, w1)
+    const int last = (int)min((long long)a.nslots - Q0, 1ll << 30);
+    const int w0 = min(er + 1, last), w1 = max(w0, min(max(P + 1, TQ), last));
+    const int wa = w0 & ~63;
+    for (uint32_t i = tid; i < FOUT * sizeof(T) / 16; i += MT) reinterpret_cast<uint4 *>(S.out)[i] = make_uint4(0, 0, 0, 0);
+    for (int p = wa + (int)FOUT + tid; p < w1; p += MT) wr_slot<R>(a.rem_new, (uint64_t)(Q0 + p), 0u);
+    __syncthreads();
+    {
+        int f = max(er + xB, xA) + 1, pq = xq;
+        for (uint32_t i = i0; i < i1; i++) {
+            const unsigned long long x = S.m[i];
+            const uint64_t c = x & F_CMASK;
+            if (c == 0) continue;
+            const int y = (int)(x >> F_QBITS);
+            const uint32_t v = (uint32_t)(x >> F_RBITS) & 0xffffu;
+            if (y != pq) {
+                if (pq >= 0) fast_rend(S, a, Q0, wa, f - 1);
+                fast_offsets(S, pq < 0 ? 0 : pq, y, f - 1);
+                atomicOr(&S.nocc[y >> 5], 1u << (y & 31));
+                pq = y;
+                f = max(f, y);
+            }
+            fast_put(S, a, Q0, wa, f++, v);
+            if (c == 1) continue;
+            const uint64_t z = c - 2;
+            const uint32_t nd = ndig(z, R);
+            fast_put(S, a, Q0, wa, f++, v);
+            fast_put(S, a, Q0, wa, f++, nd);
+            for (uint32_t d = 0; d < nd; d++) fast_put(S, a, Q0, wa, f++, (uint32_t)(z >> (R * (nd - 1 - d))) & ((1u << R) - 1u));
+        }
+        if (tid == 0) {
+            if (tq >= 0) fast_rend(S, a, Q0, wa, P);
+            fast_offsets(S, max(tq, 0), TQ, P);
+        }
+    }
+    __syncthreads();
+    // out with it: whole 16 bytes, the edges slot by slot
+    constexpr int SPC = 16 / (int)sizeof(T);
+    const bool aligned = reinterpret_cast<uintptr_t>(a.rem_new) % 16 == 0;
+    for (int c = tid; c < (int)FOUT / SPC; c += MT) {
+        const int s = wa + c * SPC;
+        if (s >= w1) break;
+        if (aligned && s >= w0 && s + SPC <= w1) {
+            reinterpret_cast<uint4 *>(a.rem_new + (Q0 + s) * (long long)sizeof(T))[0] = reinterpret_cast<const uint4 *>(S.out)[c];
+        } else {
+            for (int p = max(s, w0); p < min(s + SPC, w1); p++) wr_slot<R>(a.rem_new, (uint64_t)(Q0 + p), S.out[p - wa]);
+        }
+    }
+    const long long wblk = (Q0 + wa) >> 6;
+    for (int p = tid; p < (int)FOUT / 64; p += MT) {
+        const unsigned long long bits = S.rend[2 * p] | ((unsigned long long)S.rend[2 * p + 1] << 32);
+        if (bits && wblk + p < (long long)a.nblk) atomicOr(&a.meta_new[wblk + p].rend, bits);
+    }
+    if (tid < TBLK && j0 + tid < a.nblk) {
+        a.meta_new[j0 + tid].occ = S.nocc[2 * tid] | ((unsigned long long)S.nocc[2 * tid + 1] << 32);
+        a.meta_new[j0 + tid].off = S.off[tid];
+    }
+    return true;
+}
+
+// both forms of a tile share their memory
+template <int R>
+union MergeShared {
+    FastSmem<R> fast;
+    MergeSmem<R> any;
+    __device__ MergeShared() {}
+};
+
+template <int R>
+__device__ __forceinline__ void merge_one(const MergeArgs &a, MergeShared<R> &S, const uint64_t tile)
+{
+    if (merge_tile<R>(a, S.fast, tile)) return;
+    __syncthreads();
+    merge_tile_any<R>(a, S.any, tile);
+}
+
 // Tiles are taken from a counter in launch order, so every tile a look-back
 // waits on has already been scheduled.
 // Traced launches record their algorithmic bytes on the device: the old
@@ -829,19 +1286,20 @@ __device__ __forceinline__ void merge_units(unsigned long long *units, uint64_t 
 }
 
 template <int R>
-__global__ void __launch_bounds__(MT, MERGE_CTAS) gqf_merge_kernel(MergeArgs a, unsigned long long *units)
+__global__ void __launch_bounds__(MT, MERGE_CTAS) gqf_merge_kernel(const __grid_constant__ MergeArgs a,
+                                                                   unsigned long long *units)
 {
-    __shared__ MergeSmem<R> S;
+    __shared__ __align__(16) MergeShared<R> S;
+    __shared__ unsigned s_tile;
     if (threadIdx.x == 0) {
-        S.tile = (unsigned)atomicAdd(&a.ts[0], 1ull);
-        S.err = 0;
-        if (units && S.tile == 0) {
+        s_tile = (unsigned)atomicAdd(&a.ts[0], 1ull);
+        if (units && s_tile == 0) {
             const uint64_t m = *a.pm;
             merge_units<R>(units, a.nslots, m < a.m_limit ? m : a.m_limit);
         }
     }
     __syncthreads();
-    merge_tile<R>(a, S, S.tile);
+    merge_one<R>(a, S, s_tile);
 }
 
 // Group merge: the tiles of all member filters, concatenated. tab[m] holds
@@ -853,22 +1311,22 @@ __global__ void __launch_bounds__(MT, MERGE_CTAS) gqf_merge_group_kernel(const M
                                                              unsigned long long *tctr, uint64_t slots,
                                                              const uint32_t *pm, unsigned long long *units)
 {
-    __shared__ MergeSmem<R> S;
+    __shared__ __align__(16) MergeShared<R> S;
     __shared__ MergeArgs A;
+    __shared__ unsigned s_tile;
     if (threadIdx.x == 0) {
-        S.tile = (unsigned)atomicAdd(tctr, 1ull);
-        S.err = 0;
-        if (units && S.tile == 0) merge_units<R>(units, slots, *pm);
+        s_tile = (unsigned)atomicAdd(tctr, 1ull);
+        if (units && s_tile == 0) merge_units<R>(units, slots, *pm);
     }
     __syncthreads();
     static_assert(sizeof(MergeArgs) % 8 == 0, "MergeArgs copies as 64-bit words");
     {
-        const unsigned long long *src = reinterpret_cast<const unsigned long long *>(tab + tile_member[S.tile]);
+        const unsigned long long *src = reinterpret_cast<const unsigned long long *>(tab + tile_member[s_tile]);
         unsigned long long *dst = reinterpret_cast<unsigned long long *>(&A);
         for (int w = threadIdx.x; w < (int)(sizeof(MergeArgs) / 8); w += MT) dst[w] = src[w];
     }
     __syncthreads();
-    merge_tile<R>(A, S, S.tile - A.tile0);
+    merge_one<R>(A, S, s_tile - A.tile0);
 }
 
 // first group of every tile: successor search of the tile's first fingerprint
