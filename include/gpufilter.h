@@ -135,7 +135,9 @@ int filter_destroy(filter_t *f);
  *     1024 (0: 2048).
  *   gqf_region_groups: GQF batches with at most this many distinct
  *     fingerprints per 256 quotients on average are inserted or removed in
- *     place (even-odd regions); denser ones take the merge (0: 8).
+ *     place (even-odd regions); denser ones take the merge (0: by the table's
+ *     size, from one per 512 quotients at 2^22 slots to one per 32 from 2^27,
+ *     and fewer when its clusters are long).
  * filter_set_tuning / filter_group_set_tuning: FILTER_ERR_ARG for values out
  * of range. filter_get_tuning: the current settings (0 fields = defaults).
  */

@@ -71,6 +71,23 @@ bool tcf_tiled(const filter_tuning &t, uint64_t nb, uint64_t n, bool del)
 uint32_t tcf_tile_target(const filter_tuning &t) { return t.tcf_tile_target ? t.tcf_tile_target : 2048u; }
 uint64_t gqf_region_groups(const filter_tuning &t) { return t.gqf_region_groups ? t.gqf_region_groups : 8u; }
 
+uint64_t gqf_in_place_most(const filter_tuning &t, uint64_t N)
+{
+    if (t.gqf_region_groups) return t.gqf_region_groups * (N / 256);
+    // A merge costs its launches and 13 ps a slot; in place, a group costs the
+    // more the longer the clusters. A remove and an insert in us, merged / in
+    // place at 60 % / in place at 85 % load: 2^20 slots, 1024 groups 148 / 172
+    // / 294; 2^22, 8192 251 / 212 / 541; 2^24, 65536 586 / 527 / 1334; 2^26,
+    // 2^20 2000 / 1717 / (refused); 2^28, 2^23 7756 / 8404 / (refused). The
+    // bounds are for tables that are not crowded; crowded ones, told by the
+    // pre-check or before it, merge from fewer.
+    uint64_t most = N / 32;  // 8 per 256 quotients
+    if (N < (1ull << 27)) most = N / 256 * (N >> 24);
+    if (N < (1ull << 24)) most = N / 512;
+    if (N < (1ull << 22)) most = N / 64;
+    return most;
+}
+
 }  // namespace gf
 
 extern "C" {

@@ -2214,6 +2214,25 @@ int gqf_clear(filter *F, cudaStream_t st)
     return FILTER_OK;
 }
 
+// How long the clusters are, by a sample of the blocks' offsets: one CTA of
+// SM_T threads, a block each, into out[0].
+__device__ __forceinline__ void crowd_sample(const Meta *__restrict__ meta, uint64_t nblk, unsigned *out)
+{
+    const uint32_t off = min(meta[(uint64_t)threadIdx.x * nblk / SM_T].off, 64u);
+    if (threadIdx.x == 0) out[0] = 0;
+    __syncthreads();
+    const uint32_t sum = __reduce_add_sync(0xffffffffu, off);
+    if ((threadIdx.x & 31) == 0 && sum) atomicAdd(out, sum);
+}
+
+// the same by itself, with the batch's number of groups beside it
+__global__ void __launch_bounds__(SM_T) gqf_crowd_sample(const Meta *__restrict__ meta, uint64_t nblk, const uint32_t *pm,
+                                                         unsigned *out)
+{
+    crowd_sample(meta, nblk, out);
+    if (threadIdx.x == 0) out[1] = *pm;
+}
+
 // sort + reduce of at most GQF_SMALL keys by one CTA: what gqf_prepare leaves,
 // in one launch instead of 16 (1000 keys, p = 28: 101 -> 11 us). A sorted value
 // is fingerprint << 12 | batch index, 64 bits at the most (q <= 36, r <= 16).
@@ -2224,8 +2243,10 @@ static_assert(GQF_SMALL == 1 << 12, "the batch index takes 12 bits");
 __global__ void __launch_bounds__(SM_T) gqf_small_prepare(const uint64_t *__restrict__ keys, uint32_t n, PHash H,
                                                           const uint32_t *__restrict__ vals, uint32_t *sorted,
                                                           bool want_idx, uint64_t *ufp, uint32_t *ustart,
-                                                          uint32_t *run_of, uint32_t *m_out)
+                                                          uint32_t *run_of, uint32_t *m_out, const Meta *__restrict__ meta,
+                                                          uint64_t nblk, unsigned *crowd)
 {
+    if (crowd) crowd_sample(meta, nblk, crowd);
     extern __shared__ __align__(16) uint64_t s_small[];
     __shared__ uint32_t s_warp[32];
     uint64_t *a = s_small;
@@ -2265,6 +2286,7 @@ __global__ void __launch_bounds__(SM_T) gqf_small_prepare(const uint64_t *__rest
     if (threadIdx.x == 0) {
         ustart[m] = n;
         *m_out = m;
+        if (crowd) crowd[1] = m;
     }
 }
 
@@ -2283,7 +2305,9 @@ static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_i
         cudaFuncSetAttribute(gqf_small_prepare, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GQF_SMALL_SMEM);
         gf::TraceScope ts_("gqf_small_prepare", n, st);
         gqf_small_prepare<<<1, SM_T, GQF_SMALL_SMEM, st>>>(keys, (uint32_t)n, Q.H, vals, Q.idx_b, need_idx, Q.ufp,
-                                                           Q.ustart, need_idx ? Q.flags : nullptr, Q.flags + n);
+                                                           Q.ustart, need_idx ? Q.flags : nullptr, Q.flags + n,
+                                                           reinterpret_cast<const Meta *>(Q.meta[Q.cur]), Q.nblk,
+                                                           Q.merge_only ? nullptr : &F->ctr->pend[2]);
         return;
     }
     if (!need_idx && !vals) {
@@ -2293,7 +2317,7 @@ static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_i
         };
         // in place of the table, a batch needs its groups in one list; one
         // twice past that bound may still turn out to have few distinct keys
-        const bool dense = n * RQ_MIN > 4 * gqf_region_groups(F->tune) * Q.N || Q.merge_only;
+        const bool dense = n > 4 * gqf_in_place_most(F->tune, Q.N) || Q.merge_only;
         if (units && dense && groups(units)) {
             *in_units = true;
             return;
@@ -2398,6 +2422,53 @@ struct Precheck {
     bool merge(uint64_t m, uint64_t N) const { return crowded() && m * RQ_MIN > N; }
 };
 static_assert(offsetof(DevCounters, pend) == offsetof(DevCounters, overflow) + 8, "a pre-check's words are read together");
+
+template <class T>
+static int read_dev(const T *d, T *h, cudaStream_t st);
+
+// Crowded tables merge from fewer groups, and without a pre-check. late: slots
+// that a block's offset is late, per mille: 820 at 70 % load, 1600 at 80 %, 2400
+// at 85 %. A remove and an insert in us, in place / merged: 2^20 slots, 1024
+// groups at 85 % 294 / 155; 2^22, 4096 at 85 % 383 / 259; 2^24, 2^15 at 85 % 917
+// / 650; 2^28 at 80 %, 2^19 4064 / 7750 and 2^21 11314 / 7844, at 90 %, 2^19
+// 24345 / 7800.
+static uint64_t gqf_crowded_most(uint64_t N, uint64_t late)
+{
+    if (late < 1300) return ~0ull;
+    if (N < (1ull << 24)) return N <= (1ull << 20) ? N / 4096 : N / 2048;
+    return late >= 2200 ? N / 1024 : N <= (1ull << 25) ? N / 512 : N / 256;
+}
+
+// Whether a batch of at most m groups goes in place as far as the table's load
+// says; m becomes its number of groups when that was read.
+static int gqf_goes_in_place(filter *F, uint64_t n, bool small, uint64_t &m, bool &in_place, cudaStream_t st)
+{
+    GqfState &Q = F->gqf;
+    const uint64_t most = gqf_in_place_most(F->tune, Q.N);
+    in_place = !Q.merge_only;
+    if (!in_place) return FILTER_OK;
+    if (F->tune.gqf_region_groups || m <= gqf_crowded_most(Q.N, ~0ull)) {  // the load does not matter
+        if (m > most) {
+            uint32_t groups = 0;
+            const int rc = read_dev(Q.flags + n, &groups, st);
+            if (rc) return rc;
+            m = groups;
+        }
+        in_place = m <= most;
+        return FILTER_OK;
+    }
+    if (!small) {
+        gf::TraceScope ts_("gqf_crowd_sample", SM_T, st);
+        gqf_crowd_sample<<<1, SM_T, 0, st>>>(reinterpret_cast<const Meta *>(Q.meta[Q.cur]), Q.nblk, Q.flags + n, &F->ctr->pend[2]);
+    }
+    alignas(8) unsigned seen[2] = {0, 0};  // slots late, groups
+    const int rc = read_dev(reinterpret_cast<const unsigned long long *>(&F->ctr->pend[2]),
+                            reinterpret_cast<unsigned long long *>(seen), st);
+    if (rc) return rc;
+    m = seen[1];
+    in_place = m <= most && m <= gqf_crowded_most(Q.N, (uint64_t)seen[0] * 1000 / SM_T);
+    return FILTER_OK;
+}
 
 static int clear_precheck(DevCounters *ctr, cudaStream_t st)
 {
@@ -2511,12 +2582,9 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
     // keys bound the groups, whose number is read back only when that decides.
     if (!in_units) {
         uint64_t m = n;
-        if (m * RQ_MIN > gqf_region_groups(F->tune) * Q.N && !Q.merge_only) {
-            uint32_t groups = 0;
-            if ((rc = read_dev(Q.flags + n, &groups, st))) return rc;
-            m = groups;
-        }
-        if (m * RQ_MIN <= gqf_region_groups(F->tune) * Q.N && !Q.merge_only) {
+        bool in_place = false;
+        if ((rc = gqf_goes_in_place(F, n, n <= GQF_SMALL, m, in_place, st))) return rc;
+        if (in_place) {
             bool done = false;
             if ((rc = gqf_insert_in_place(F, cstart, n, m, st, done))) return rc;
             if (done) {
@@ -2580,13 +2648,10 @@ int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cud
     int rc = FILTER_OK;
     // small batches: in place, cluster by cluster; large ones: full merge
     uint64_t m = n;  // at least the number of groups
-    if (!in_units && m * RQ_MIN > gqf_region_groups(F->tune) * Q.N) {
-        uint32_t groups = 0;
-        if ((rc = read_dev(Q.flags + n, &groups, st))) return rc;
-        m = groups;
-    }
+    bool in_place = false;
+    if (!in_units && (rc = gqf_goes_in_place(F, n, n <= GQF_SMALL, m, in_place, st))) return rc;
     bool done = false;
-    if (!in_units && m * RQ_MIN <= gqf_region_groups(F->tune) * Q.N) {
+    if (in_place) {
         GView g{reinterpret_cast<Meta *>(Q.meta[Q.cur]), Q.rem[Q.cur], (long long)Q.N, (long long)Q.nslots,
                 (long long)Q.nblk};
         if ((rc = clear_precheck(F->ctr, st))) return rc;

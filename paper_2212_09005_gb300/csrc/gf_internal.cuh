@@ -556,6 +556,8 @@ bool tcf_tiled(const filter_tuning &t, uint64_t nb, uint64_t n, bool del);
 bool tcf_geom_supported(uint32_t f, uint32_t B);
 uint32_t tcf_tile_target(const filter_tuning &t);
 uint64_t gqf_region_groups(const filter_tuning &t);
+// the most groups that a batch updates in place of the table
+uint64_t gqf_in_place_most(const filter_tuning &t, uint64_t N);
 int tcf_group_setup(filter_group *G, const filter_config *cfgs, uint64_t &bytes, bool plan_only);
 int tcf_group_clear(filter_group *G, cudaStream_t st);
 int tcf_group_op(filter_group *G, int op, const uint64_t *off, const uint64_t *keys, uint64_t n, uint8_t *out,

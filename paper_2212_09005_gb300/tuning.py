@@ -13,8 +13,10 @@ measured rather than assumed:
                       rule on table, batch and direction unless one of the two
                       alone is faster;
   tcf_tile_target     candidates per tile the tiled path aims for;
-  gqf_region_groups   how many 64-slot groups a batch may touch per key
-                      before the GQF leaves the in-place path for a merge.
+  gqf_region_groups   how many distinct fingerprints a batch may have per 256
+                      quotients before the GQF leaves the in-place path for a
+                      merge; left to the library's rule on the table's size
+                      unless one bound is faster.
 
 `autotune()` times each choice on synthetic filters of every size class and
 writes `tuning.json` next to this file; `Filter` and `FilterGroup` apply the
@@ -83,8 +85,8 @@ def struct(knobs: dict):
 # Measurement
 # ---------------------------------------------------------------------------
 TCF_CANDIDATES = ((0, 0), (1, 0), (2, 512), (2, 1024))    # (tcf_path, tile target)
-AUTO_MARGIN = 0.97  # what a forced path's time must be below, of the rule's
-GQF_CANDIDATES = (4, 8, 16, 32, 64, 128)                  # region groups
+AUTO_MARGIN = 0.97  # what another choice's time must be below, of the library's own
+GQF_CANDIDATES = (0, 1, 4, 8, 16)                          # region groups
 
 
 def _timed(torch, fn, reps=2):
@@ -200,12 +202,12 @@ def tune_tcf_group(torch, n_filters: int = 2048, rounds: int = 8, seed: int = 78
 
 def tune_gqf(q: int, keys, torch) -> dict:
     """A GQF with 2^q home slots filled to 90 % in one batch; then a batch
-    of min(2^24, n/16) distinct stored keys is removed and inserted again:
+    of min(2^24, n/100) distinct stored keys is removed and inserted again:
     the region bound with the least total time for the two."""
     from . import GQF
 
     n = int(0.9 * (1 << q))
-    b = min(1 << 24, n // 16)
+    b = min(1 << 24, n // 100)
     F = GQF(q, 8, seed=q, max_batch=n)
     sub = keys[:b]
     ev = lambda: torch.cuda.Event(enable_timing=True)
@@ -228,6 +230,8 @@ def tune_gqf(q: int, keys, torch) -> dict:
         res[str(g)] = round(_timed(torch, run), 3)
     F.close()
     best = min(res, key=res.get)
+    if res[best] > AUTO_MARGIN * res["0"]:
+        best = "0"
     return {"gqf_region_groups": int(best), "ms": res, "batch": b}
 
 

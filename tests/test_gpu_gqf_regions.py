@@ -33,6 +33,7 @@ def test_updates_equal_oracle(gf, oracle, q, r, load, m):
     fresh = W.uniform_keys(200 + q, m)
     again = np.concatenate([base[: m // 2 + 1], fresh[: m // 2]])  # counters grow by 1, then by 2
     O, G = oracle.GQF(q, r, seed=q), gf.GQF(q, r, seed=q, max_batch=max(len(base), 4 * m + 4))
+    G.set_tuning(gqf_region_groups=8)  # in place wherever it can
     G.insert(dev_u64(base))
     O.insert(base)
     steps = [("insert", fresh), ("insert", again), ("insert", np.concatenate([again, again])),
