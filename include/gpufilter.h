@@ -129,7 +129,7 @@ int filter_destroy(filter_t *f);
  *     tile. FILTER_TCF_PATH_AUTO takes TILED when the table has at least
  *     tcf_tiled_min_blocks blocks and the batch at least as many keys; with
  *     tcf_tiled_min_blocks = 0, for tables of 2^22 blocks or more unless the
- *     batch is small (at most 2^18 or 2^19 keys), and for removes of four keys
+ *     batch is small (at most 2^18 or 2^19 keys), and for removes of three keys
  *     a block or more on tables of 2^12 blocks or more.
  *   tcf_tile_target: tiled path, the expected candidates per tile, 128 ..
  *     1024 (0: 2048).

@@ -60,12 +60,13 @@ bool tcf_tiled(const filter_tuning &t, uint64_t nb, uint64_t n, bool del)
     // 32.7 by block, and 65533 of them a call 0.11 and 0.18 ms an insert and
     // remove; at 2^22 blocks 3.80 against 4.30 and 0.072 against 0.077. Below,
     // inserts are as fast by block or faster (2^20 blocks, 2^21 keys: 1.33 ms
-    // against 1.48). Removes of four keys a block or more are faster by unit on
+    // against 1.48). Removes of three keys a block or more are faster by unit on
     // any table, the unit step needing no scratch per block (2^20 blocks, 2^22
-    // keys: 0.67 ms against 0.87; 2^12 blocks, 2^14 keys 126 us against 139;
-    // 8-bit tags 0.77 ms against 1.72).
+    // keys: 0.67 ms against 0.87; 3.35e6 keys on 2^20 blocks of a group, all
+    // kernels, 0.47 and 0.58; 2^12 blocks, 2^14 keys 126 us against 139; 8-bit
+    // tags, 2^22 keys on 2^19 blocks, 0.77 ms against 1.72).
     if (tcf_few_keys(nb, n)) return false;
-    return nb >= (1ull << 22) || (del && nb >= (1ull << 12) && n >= 4 * nb);
+    return nb >= (1ull << 22) || (del && nb >= (1ull << 12) && n >= 3 * nb);
 }
 
 uint32_t tcf_tile_target(const filter_tuning &t) { return t.tcf_tile_target ? t.tcf_tile_target : 2048u; }

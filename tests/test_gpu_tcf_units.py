@@ -103,7 +103,7 @@ def test_later_phases_on_a_large_table(gf, oracle, copies):
     assert first_diff(G.export(), O.export()) is None
 
 
-@pytest.mark.parametrize("lg,n", [(16, 4 * (1 << 12)), (16, 4 * (1 << 12) - 1), (15, 8192)])
+@pytest.mark.parametrize("lg,n", [(16, 4 * (1 << 12)), (16, 3 * (1 << 12)), (16, 3 * (1 << 12) - 1), (15, 8192)])
 def test_auto_calls_leave_the_oracle_table(gf, oracle, lg, n):
     """Around the lines of the automatic choice, and of the one launch of the later phases."""
     keys = W.uniform_keys(lg, int(1.02 * (1 << lg)))
