@@ -2324,9 +2324,11 @@ static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_i
         }
         if (groups(nullptr)) return;
     }
-    fingerprint_for_sort(keys, n, Q.H, Q.fp_a, need_idx ? Q.idx_a : nullptr, Q.p, Q.radix_tmp, st);
-    radix_sort_u64(Q.fp_a, Q.fp_b, Q.fp_c, need_idx ? Q.idx_a : vals, Q.idx_b, Q.idx_c, n, Q.p, Q.radix_tmp,
-                   F->scan_tmp, F->ctr, st, true);
+    const uint32_t ibits = need_idx ? radix_pack_bits(n, Q.p) : 0;
+    uint32_t *idx = need_idx && !ibits ? Q.idx_a : nullptr;
+    fingerprint_for_sort(keys, n, Q.H, Q.fp_a, idx, ibits, Q.p, Q.radix_tmp, st);
+    radix_sort_u64(Q.fp_a, Q.fp_b, Q.fp_c, need_idx ? idx : vals, Q.idx_b, Q.idx_c, n, Q.p, Q.radix_tmp, F->scan_tmp,
+                   F->ctr, st, true, ibits);
     // groups: flags[n] = their number; flags[i] = the group of sorted element i (statuses only)
     rle_sorted_u64(Q.fp_b, n, Q.ufp, Q.ustart, need_idx ? Q.flags : nullptr, Q.flags + n, F->scan_tmp, F->ctr, st);
 }
@@ -2873,7 +2875,7 @@ struct GqfMemberDev {
 
 __global__ void gqf_group_fp_kernel(const uint64_t *__restrict__ keys, uint64_t n, const uint64_t *__restrict__ off,
                                     uint32_t nmem, const GqfMemberDev *__restrict__ gm, uint32_t pbits, uint64_t *fp,
-                                    uint32_t *idx)
+                                    uint32_t *idx, uint32_t ibits)
 {
     MemberCursor c(off, nmem, n);
     uint32_t cm = 0xffffffffu;
@@ -2883,7 +2885,8 @@ __global__ void gqf_group_fp_kernel(const uint64_t *__restrict__ keys, uint64_t 
             cm = c.m;
             H = gm[cm].H;
         }
-        fp[c.i] = ((uint64_t)cm << pbits) | fingerprint(__ldg(keys + c.i), H);
+        const uint64_t f = ((uint64_t)cm << pbits) | fingerprint(__ldg(keys + c.i), H);
+        fp[c.i] = ibits ? f << ibits | c.i : f;
         if (idx) idx[c.i] = (uint32_t)c.i;
     }
 }
@@ -3187,13 +3190,15 @@ static void group_prepare(filter_group *GR, const uint64_t *off, const uint64_t 
 {
     GqfState &Q = GR->gqf;
     const int g = grid_for(n, 256, 8);
+    const uint32_t ibits = need_idx ? radix_pack_bits(n, GR->pbits + GR->mbits) : 0;
+    uint32_t *idx = need_idx && !ibits ? Q.idx_a : nullptr;
     {
         gf::TraceScope ts_("gqf_group_fp_kernel", n, st);
         gqf_group_fp_kernel<<<g, 256, 0, st>>>(keys, n, off, GR->n, static_cast<const GqfMemberDev *>(GR->d_gmem),
-                                               GR->pbits, Q.fp_a, need_idx ? Q.idx_a : nullptr);
+                                               GR->pbits, Q.fp_a, idx, ibits);
     }
-    radix_sort_u64(Q.fp_a, Q.fp_b, Q.fp_c, need_idx ? Q.idx_a : nullptr, Q.idx_b, Q.idx_c, n, GR->pbits + GR->mbits,
-                   Q.radix_tmp, GR->scan_tmp, GR->ctr, st);
+    radix_sort_u64(Q.fp_a, Q.fp_b, Q.fp_c, idx, Q.idx_b, Q.idx_c, n, GR->pbits + GR->mbits, Q.radix_tmp, GR->scan_tmp,
+                   GR->ctr, st, false, ibits);
     rle_sorted_u64(Q.fp_b, n, Q.ufp, Q.ustart, need_idx ? Q.flags : nullptr, Q.flags + n, GR->scan_tmp, GR->ctr, st);
 }
 

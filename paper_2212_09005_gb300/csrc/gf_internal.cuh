@@ -243,11 +243,15 @@ size_t radix_tmp_words(uint64_t n);
 void radix_sort_u64(const uint64_t *keys_in, uint64_t *keys_out, uint64_t *keys_alt,
                     const uint32_t *vals_in, uint32_t *vals_out, uint32_t *vals_alt,
                     uint64_t n, uint32_t bits, uint32_t *tmp, uint64_t *scan_tmp,
-                    DevCounters *ctr, cudaStream_t st, bool first_hist_done = false);
+                    DevCounters *ctr, cudaStream_t st, bool first_hist_done = false, uint32_t ibits = 0);
+// Bits for the indices of n keys below `bits` sorted bits, 0 when both do not
+// fit into 64. With ibits, radix_sort_u64 takes packed keys and no values, sorts
+// from bit ibits on and writes the indices to vals_out.
+uint32_t radix_pack_bits(uint64_t n, uint32_t bits);
 // fp[i] = fingerprint(keys[i], H) (idx[i] = i when idx is set), with the
 // per-tile histogram of the lowest digit that radix_sort_u64(.., bits, tmp)
 // takes for its first pass
-void fingerprint_for_sort(const uint64_t *keys, uint64_t n, const PHash &H, uint64_t *fp, uint32_t *idx,
+void fingerprint_for_sort(const uint64_t *keys, uint64_t n, const PHash &H, uint64_t *fp, uint32_t *idx, uint32_t ibits,
                           uint32_t bits, uint32_t *tmp, cudaStream_t st);
 
 // ---------------------------------------------------------------------------

@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 from paper_2212_09005_gb300 import workloads as W
-from gpu_util import dev_u64, zeros_u64, host, first_diff
+from gpu_util import dev_u64, zeros_u8, zeros_u64, host, first_diff
 
 pytestmark = pytest.mark.gpu
 
@@ -82,3 +82,18 @@ def test_fingerprints_of_one_sliver(gf, oracle):
         getattr(O, op)(batch)
         d = first_diff(G.export(), O.export())
         assert d is None, (op, d)
+
+
+# (q, r, n): the batch index below the fingerprint, up to exactly 64 bits, and beside it above
+@pytest.mark.parametrize("q,r,n", [(13, 8, 4097), (18, 16, 70001), (26, 16, 1 << 22), (26, 16, (1 << 22) + 1)])
+def test_statuses_ride_with_the_sort(gf, oracle, q, r, n):
+    base = W.uniform_keys(50 + q, n - n // 8)
+    keys = np.concatenate([base, base[: n - len(base)]])  # some of them twice
+    np.random.default_rng(n).shuffle(keys)
+    O, G = oracle.GQF(q, r, seed=1), gf.GQF(q, r, seed=1, max_batch=n)
+    gone = np.concatenate([keys[: n // 2], keys[: n // 4], W.uniform_keys(51, n - n // 2 - n // 4)])
+    for op, ks in (("insert", keys), ("remove", gone)):
+        st = zeros_u8(n)
+        getattr(G, op)(dev_u64(ks), st)
+        assert np.array_equal(host(st), getattr(O, op)(ks)), op
+    assert first_diff(G.export(), O.export()) is None
