@@ -123,9 +123,10 @@ __device__ __forceinline__ uint32_t bin_of_tile(const uint32_t *__restrict__ fir
 
 // keys per unit: every CTA counts MH_TILE keys of one first-pass bin
 __global__ void __launch_bounds__(MP_T) msd_hist2(const uint64_t *__restrict__ v, MsdScratch s, uint32_t nb1,
-                                                  uint32_t shift, uint32_t bits2)
+                                                  uint32_t shift, uint32_t bits2, unsigned long long *units)
 {
     __shared__ uint32_t h[MP_BINS];
+    if (units && blockIdx.x == 0 && threadIdx.x == 0) *units = s.st1[nb1];  // (a phase may have fewer than its bound)
     const uint32_t j = bin_of_tile(s.htile1, nb1, blockIdx.x), nb = 1u << bits2;
     if (j == nb1) return;
     for (uint32_t b = threadIdx.x; b < nb; b += MP_T) h[b] = 0;
@@ -179,9 +180,10 @@ __global__ void __launch_bounds__(MP_BINS) msd_scan2(MsdScratch s, uint32_t nb1,
 template <bool FIRST, bool HASH>
 __global__ void __launch_bounds__(MP_T, 3) msd_part(const uint64_t *__restrict__ in, uint32_t n, PHash H, MsdScratch s,
                                                     uint32_t nb1, uint32_t shift, uint32_t bits,
-                                                    uint64_t *__restrict__ out)
+                                                    uint64_t *__restrict__ out, unsigned long long *units)
 {
     __shared__ PartSmem S;
+    if (!FIRST && units && blockIdx.x == 0 && threadIdx.x == 0) *units = s.st1[nb1];
     const uint32_t nb = 1u << bits;
     uint32_t base, end;
     uint32_t *cur;
@@ -221,16 +223,16 @@ void msd_second_pass(const MsdScratch &s, const uint64_t *in, uint64_t *out, uin
                      uint32_t bits2, const char *hist_name, const char *part_name, cudaStream_t st)
 {
     {
-        TraceScope ts_(hist_name, n, st);
-        msd_hist2<<<(unsigned)((n + MH_TILE - 1) / MH_TILE) + nb1, MP_T, 0, st>>>(in, s, nb1, shift, bits2);
+        TraceScope ts_(hist_name, 0, st, true);
+        msd_hist2<<<(unsigned)((n + MH_TILE - 1) / MH_TILE) + nb1, MP_T, 0, st>>>(in, s, nb1, shift, bits2, ts_.units());
     }
     {
         TraceScope ts_("msd_scan2", (uint64_t)nb1 << bits2, st);
         msd_scan2<<<nb1, MP_BINS, 0, st>>>(s, nb1, bits2);
     }
-    TraceScope ts_(part_name, n, st);
+    TraceScope ts_(part_name, 0, st, true);
     msd_part<false, false><<<(unsigned)((n + MP_TILE - 1) / MP_TILE) + nb1, MP_T, 0, st>>>(in, (uint32_t)n, PHash{}, s, nb1,
-                                                                                         shift, bits2, out);
+                                                                                         shift, bits2, out, ts_.units());
 }
 
 // ---------------------------------------------------------------------------
@@ -665,8 +667,8 @@ bool msd_groups(const uint64_t *keys, uint64_t n, const PHash *H, uint32_t bits,
     }
     {
         TraceScope ts_("msd_part", n, st);
-        if (H) msd_part<true, true><<<tiles, MP_T, 0, st>>>(keys, (uint32_t)n, h, s, 0, bits - b1, b1, buf_a);
-        else msd_part<true, false><<<tiles, MP_T, 0, st>>>(keys, (uint32_t)n, h, s, 0, bits - b1, b1, buf_a);
+        if (H) msd_part<true, true><<<tiles, MP_T, 0, st>>>(keys, (uint32_t)n, h, s, 0, bits - b1, b1, buf_a, nullptr);
+        else msd_part<true, false><<<tiles, MP_T, 0, st>>>(keys, (uint32_t)n, h, s, 0, bits - b1, b1, buf_a, nullptr);
     }
     if (two) msd_second_pass(s, buf_a, buf_b, n, 1u << b1, rbits, b2, "msd_hist2", "msd_part2", st);
     const uint32_t *ust = two ? s.st2 : s.st1;

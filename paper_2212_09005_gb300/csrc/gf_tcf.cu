@@ -3,20 +3,19 @@
 // Table: nb blocks of 32 bytes (one DRAM sector), B = 256 / f tags each, plus a
 // backing table of nbk buckets of 8 uint64 entries (Sec. 4.1, "Backing table").
 //
-// Query (Sec. 4): probe both candidate blocks with two 16-byte loads each and a
+// Query (Sec. 4): probe both candidate blocks with one 32-byte load each and a
 // SIMD compare (__vcmpeq2 / __vcmpeq4), then the backing bucket (L2-resident)
 // if the tag was in neither block.
 //
 // Bulk insert, deterministic mode (Sec. 4.1 shortcut + Sec. 4 two choices +
 // Sec. 4.1 backing table + Sec. 4.2 sorted blocks). Each block phase groups
-// its candidates by tile of consecutive blocks (one or two coalesced counting
-// passes), then one CTA per tile sorts them by block in shared memory and one
-// thread per block takes the k smallest (tag, batch index) candidates that
-// fit, merges them into its sorted block, and emits the rest to the next
-// phase:
+// its candidates by block (by units of blocks in shared memory, by a counting
+// sort over all blocks, or by one over the blocks that are touched, whichever
+// suits the table and the batch), then one thread per block takes the k
+// smallest (tag, batch index) candidates that fit, merges them into its sorted
+// block, and emits the rest to the next phase:
 //   A shortcut into b1 while fill + j < 3B/4, B the less-full block under the
-//   post-A fills, C the other block, D the backing bucket (few candidates:
-//   a counting sort over the touched buckets only).
+//   post-A fills, C the other block, D the backing bucket.
 // Blocks keep a fill byte array beside them so that the two-choice decision
 // reads 1 byte from L2 instead of a 32-byte sector from HBM.
 //

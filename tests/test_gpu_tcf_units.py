@@ -125,3 +125,30 @@ def test_few_keys_by_touched_blocks(gf, oracle, f, few):
     one = np.concatenate([base, np.repeat(hot[:1], cap + few)])
     check(G, O, [("insert", one), ("insert", np.concatenate([base[:3000], np.repeat(hot, 300)])),
                  ("remove", one[::-1]), ("remove", np.concatenate([base, np.repeat(hot, 200)])), ("insert", base)])
+
+
+@pytest.mark.parametrize("lg,n,path", [(18, 5000, 0), (18, 1 << 16, 1), (20, 1 << 17, 2)])
+def test_calls_captured_in_a_graph(gf, oracle, lg, n, path):
+    import torch
+
+    keys = W.uniform_keys(lg, 2 * n)
+    G, O = gf.TCF(lg, 16, seed=1, max_batch=n), oracle.TCF(lg, 16, seed=1)
+    G.set_tuning(tcf_path=path)
+    buf, st = dev_u64(keys[:n]), zeros_u8(n)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    graphs = {}
+    with torch.cuda.stream(s):
+        G.insert(buf, st)  # (outside a capture first: what a call sets up once)
+        G.remove(buf, st)
+        for op in ("insert", "remove"):
+            graphs[op] = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graphs[op], stream=s):
+                getattr(G, op)(buf, st)
+    torch.cuda.synchronize()
+    for op, ks in (("insert", keys[:n]), ("insert", keys[n:]), ("insert", keys[:n]), ("remove", keys[n:]), ("remove", keys[n:])):
+        buf.copy_(dev_u64(ks))
+        graphs[op].replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(host(st), getattr(O, op)(ks)), op
+        assert first_diff(G.export(), O.export()) is None, op
