@@ -1996,17 +1996,20 @@ __global__ void __launch_bounds__(256) gqf_group_counts(const uint32_t *__restri
 // ---------------------------------------------------------------------------
 // per-key status after a batch
 // ---------------------------------------------------------------------------
-// run_of[i] = group of sorted element i
+// run_of[i] = group of sorted element i. all = false: the statuses are zero (OK)
+// already and only the others are written, each a sector of its own (2^24 keys
+// removed from a group, all of them stored: 144 us with every status written).
 __global__ void gqf_status_kernel(uint64_t n, const uint32_t *__restrict__ run_of, const uint32_t *__restrict__ ustart,
                                   const uint32_t *__restrict__ sidx, const uint32_t *__restrict__ removed,
-                                  uint64_t m_keep, int del, uint8_t *status)
+                                  uint64_t m_keep, int del, bool all, uint8_t *status)
 {
+    static_assert(FILTER_KEY_OK == 0, "statuses are cleared to OK");
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         uint32_t g = run_of[i];
         uint8_t s;
         if (del) s = (i - ustart[g]) < removed[g] ? FILTER_KEY_OK : FILTER_KEY_NOT_FOUND;
         else s = (g < m_keep) ? FILTER_KEY_OK : FILTER_KEY_FULL;
-        status[sidx[i]] = s;
+        if (all || s != FILTER_KEY_OK) status[sidx[i]] = s;
     }
 }
 
@@ -2583,11 +2586,12 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
     if (n == 0) return FILTER_OK;
     GqfState &Q = F->gqf;
     uint32_t *sidx = nullptr;
-    // counts without statuses ride through the sort in place of the indices
-    const bool carry = counts != nullptr && status == nullptr;
+    // counts without statuses ride through the sort in place of the indices;
+    // other inserts need no indices unless some group does not fit
+    const bool carry = counts != nullptr && status == nullptr, need_idx = counts != nullptr && status != nullptr;
     MsdUnits units{};
     bool in_units = false;
-    gqf_prepare(F, keys, n, status != nullptr, st, &sidx, carry ? counts : nullptr, counts ? nullptr : &units, &in_units);
+    gqf_prepare(F, keys, n, need_idx, st, &sidx, carry ? counts : nullptr, counts ? nullptr : &units, &in_units);
     int rc;
     // the copies each group adds: its keys, or the sum of their counts
     const uint32_t *cstart = Q.ustart;
@@ -2614,6 +2618,7 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
         GF_CUDA(cudaGetLastError());
         cstart = cs;
     }
+    if (status) GF_CUDA(cudaMemsetAsync(status, FILTER_KEY_OK, n, st));
     // small batches: in place, region by region; larger ones: the merge. The
     // keys bound the groups, whose number is read back only when that decides.
     if (!in_units) {
@@ -2624,11 +2629,6 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
             bool done = false;
             if ((rc = gqf_insert_in_place(F, cstart, n, m, st, done))) return rc;
             if (done) {
-                if (status) {
-                    gf::TraceScope ts_("gqf_status_kernel", n, st);
-                    gqf_status_kernel<<<grid_for(n, 256, 8), 256, 0, st>>>(n, Q.flags, Q.ustart, sidx, Q.removed,
-                                                                          ~0ull, 0, status);
-                }
                 GF_CUDA(cudaGetLastError());
                 return FILTER_OK;
             }
@@ -2640,7 +2640,8 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
     if ((rc = read_dev(&F->ctr->overflow, &ovf, st))) return rc;
     uint64_t m_keep = ~0ull;
     if (ovf) {
-        if (in_units) gqf_prepare(F, keys, n, false, st, &sidx);  // one list, whose prefixes are tried
+        // one list, whose prefixes are tried, with the indices of its keys
+        if (in_units || (status && !need_idx)) gqf_prepare(F, keys, n, status != nullptr, st, &sidx);
         // keep the longest prefix of the sorted groups that fits (dry runs)
         uint32_t m = 0;
         if ((rc = read_dev(Q.flags + n, &m, st))) return rc;
@@ -2662,11 +2663,11 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
         GF_CUDA(cudaGetLastError());
     }
     Q.cur ^= 1;
-    if (status) {
+    if (status && ovf) {
         {
             gf::TraceScope ts_("gqf_status_kernel", n, st);
             gqf_status_kernel<<<grid_for(n, 256, 8), 256, 0, st>>>(n, Q.flags, Q.ustart, sidx, Q.removed, m_keep, 0,
-                                                                  status);
+                                                                  false, status);
         }
         GF_CUDA(cudaGetLastError());
     }
@@ -2736,7 +2737,9 @@ int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cud
     if (status) {
         {
             gf::TraceScope ts_("gqf_status_kernel", n, st);
-            gqf_status_kernel<<<grid_for(n, 256, 8), 256, 0, st>>>(n, Q.flags, Q.ustart, sidx, Q.removed, 0, 1, status);
+            const bool all = n <= GQF_SMALL;  // (a launch less)
+            if (!all) GF_CUDA(cudaMemsetAsync(status, FILTER_KEY_OK, n, st));
+            gqf_status_kernel<<<grid_for(n, 256, 8), 256, 0, st>>>(n, Q.flags, Q.ustart, sidx, Q.removed, 0, 1, all, status);
         }
         GF_CUDA(cudaGetLastError());
     }
@@ -3271,14 +3274,10 @@ int gqf_group_insert(filter_group *GR, const uint64_t *off, const uint64_t *keys
 {
     if (n == 0) return FILTER_OK;
     GqfState &Q = GR->gqf;
-    group_prepare(GR, off, keys, n, status != nullptr, st);
+    group_prepare(GR, off, keys, n, false, st);
     int rc = group_merge(GR, n, 0, st);
     if (rc) return rc;
-    if (status) {
-        gf::TraceScope ts_("gqf_status_kernel", n, st);
-        gqf_status_kernel<<<grid_for(n, 256, 8), 256, 0, st>>>(n, Q.flags, Q.ustart, Q.idx_b, Q.removed, ~0ull, 0,
-                                                              status);
-    }
+    if (status) GF_CUDA(cudaMemsetAsync(status, FILTER_KEY_OK, n, st));
     GF_CUDA(cudaMemsetAsync(&GR->ctr->pend[0], 0, 4, st));
     {
         gf::TraceScope ts_("gqf_group_overflow", GR->n, st);
@@ -3315,8 +3314,9 @@ int gqf_group_remove(filter_group *GR, const uint64_t *off, const uint64_t *keys
     int rc = group_merge(GR, n, 1, st);
     if (rc) return rc;
     if (status) {
+        GF_CUDA(cudaMemsetAsync(status, FILTER_KEY_OK, n, st));
         gf::TraceScope ts_("gqf_status_kernel", n, st);
-        gqf_status_kernel<<<grid_for(n, 256, 8), 256, 0, st>>>(n, Q.flags, Q.ustart, Q.idx_b, Q.removed, 0, 1, status);
+        gqf_status_kernel<<<grid_for(n, 256, 8), 256, 0, st>>>(n, Q.flags, Q.ustart, Q.idx_b, Q.removed, 0, 1, false, status);
     }
     GF_CUDA(cudaGetLastError());
     group_set_cur(GR, GR->cur ^ 1);
@@ -3343,13 +3343,13 @@ int gqf_group_update_async(filter_group *GR, const uint64_t *off, const uint64_t
 {
     if (n == 0) return FILTER_OK;
     GqfState &Q = GR->gqf;
-    group_prepare(GR, off, keys, n, status != nullptr, st);
+    group_prepare(GR, off, keys, n, status && del, st);
     int rc = group_merge(GR, n, del, st);
     if (rc) return rc;
-    if (status) {
+    if (status) GF_CUDA(cudaMemsetAsync(status, FILTER_KEY_OK, n, st));
+    if (status && del) {
         gf::TraceScope ts_("gqf_status_kernel", n, st);
-        gqf_status_kernel<<<grid_for(n, 256, 8), 256, 0, st>>>(n, Q.flags, Q.ustart, Q.idx_b, Q.removed,
-                                                              del ? 0 : ~0ull, del, status);
+        gqf_status_kernel<<<grid_for(n, 256, 8), 256, 0, st>>>(n, Q.flags, Q.ustart, Q.idx_b, Q.removed, 0, 1, false, status);
     }
     const int nb = GR->cur ^ 1;
     {
