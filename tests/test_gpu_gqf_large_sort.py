@@ -97,3 +97,18 @@ def test_statuses_ride_with_the_sort(gf, oracle, q, r, n):
         getattr(G, op)(dev_u64(ks), st)
         assert np.array_equal(host(st), getattr(O, op)(ks)), op
     assert first_diff(G.export(), O.export()) is None
+
+
+@pytest.mark.parametrize("q,n", [(11, 9000), (12, 14_001), (13, 3 * 8192)])
+def test_statuses_of_batches_that_do_not_fit(gf, oracle, q, n):
+    """Inserts carry no indices until some group does not fit: the keys past the kept prefix are FULL."""
+    keys = W.uniform_keys(70 + q, n)
+    keys = np.concatenate([keys, keys[:500]])
+    O, G = oracle.GQF(q, 16, seed=1), gf.GQF(q, 16, seed=1, max_batch=len(keys))
+    for part in (keys[: n // 8], keys):
+        st = zeros_u8(len(part))
+        G.insert(dev_u64(part), st)
+        want = O.insert(part)
+        assert np.array_equal(host(st), want)
+        assert first_diff(G.export(), O.export()) is None
+    assert (want != 0).any()
