@@ -4,7 +4,7 @@
 // {occupieds, runends, offset}, and an array of r-bit remainders.
 //
 // Bulk insert / delete (Sec. 5.3-5.4, Sec. 6.4): fingerprints are computed,
-// radix-sorted and reduced to <fingerprint, count> groups (the paper's
+// sorted and reduced to <fingerprint, count> groups (the paper's
 // map-reduce for skewed inputs). The groups are then merged into the table in
 // ONE pass over quotient tiles of TQ quotients instead of the paper's
 // even-odd region phases: a run of quotient x with encoded length L ends at
@@ -17,8 +17,9 @@
 // offsets into the other buffer. Every slot of the new buffer is written by
 // exactly one tile.
 //
-// Small batches (at most one group per 32 slots) are inserted in place over
-// even-odd regions instead (Sec. 5.3), and small deletes likewise (Sec. 6.4).
+// Small batches are inserted in place over even-odd regions instead (Sec. 5.3),
+// and small deletes likewise (Sec. 6.4); how small depends on the table's size
+// and load (gqf_goes_in_place).
 //
 // Counted insert (values through the counters, as in the CQF the paper
 // follows): each key brings a count; the counts ride through the sort (or are
