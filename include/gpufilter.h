@@ -130,7 +130,8 @@ int filter_destroy(filter_t *f);
  *     tcf_tiled_min_blocks blocks and the batch at least as many keys; with
  *     tcf_tiled_min_blocks = 0, for tables of 2^22 blocks or more unless the
  *     batch is small (at most 2^18 or 2^19 keys), and for removes of three keys
- *     a block or more on tables of 2^12 blocks or more.
+ *     a block or more on tables of 2^12 blocks or more. A group call whose keys
+ *     belong to a few members only leaves TILED for the touched blocks.
  *   tcf_tile_target: tiled path, the expected candidates per tile, 128 ..
  *     1024 (0: 2048).
  *   gqf_region_groups: GQF batches with at most this many distinct

@@ -43,13 +43,14 @@ struct DevCounters {
     unsigned int pend[8];         // TCF: pending-list lengths per phase
     unsigned int touched[4];      // TCF sparse phases: touched destinations
     unsigned int cursor[4];       // TCF sparse phases: records placed so far
-    unsigned int bar, pad;        // arrivals at the barriers of a cooperative launch
+    unsigned int bar;             // arrivals at the barriers of a cooperative launch
+    unsigned int uneven;          // TCF group calls: 1 when some unit has far more keys than its share
     long long gqf_end;            // GQF merge: end of the last run (dry runs)
     unsigned long long wflag;     // GQF counted insert: 1 if some count was 0
 };
-// a TCF bulk call clears its words, pend to bar, at once
+// a TCF bulk call clears its words, pend to uneven, at once
 static constexpr size_t CALL_WORDS_BYTES = 18 * sizeof(unsigned int);
-static_assert(offsetof(DevCounters, gqf_end) == offsetof(DevCounters, pend) + CALL_WORDS_BYTES, "pend to bar are adjacent");
+static_assert(offsetof(DevCounters, gqf_end) == offsetof(DevCounters, pend) + CALL_WORDS_BYTES, "pend to uneven are adjacent");
 
 // ---------------------------------------------------------------------------
 // Hashing (paper Sec. 5.1 fingerprint h; Sec. 4 block/tag hash). Bijective:
@@ -224,10 +225,11 @@ __device__ __forceinline__ uint32_t lookback_prefix(unsigned long long *st, uint
 // Generic device primitives (gf_prims.cu)
 // ---------------------------------------------------------------------------
 // In-place-safe exclusive scan of n uint32 (out may equal in). Needs
-// scan_tmp_words(n) words of temporary state. Values must sum below 2^32.
+// scan_tmp_words(n) words of temporary state. Values must sum below 2^32. gate:
+// a word on the device without which nothing is done (null: always).
 size_t scan_tmp_words(uint64_t n);
 void exclusive_scan_u32(const uint32_t *in, uint32_t *out, uint64_t n, uint64_t *tmp,
-                        DevCounters *ctr, cudaStream_t st);
+                        DevCounters *ctr, cudaStream_t st, const unsigned *gate = nullptr);
 
 // Run-length encoding of a sorted array: uniq[g] / start[g] for each run g,
 // start[m] = n and *m_out = m (the number of runs); run_of[i] (optional) =

@@ -100,8 +100,9 @@ size_t scan_tmp_words(uint64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE + 2; 
 
 __global__ void __launch_bounds__(SCAN_T) scan_kernel(const uint32_t *in, uint32_t *out, uint64_t n,
                                                       unsigned long long *tmp,
-                                                      unsigned long long *status)
+                                                      unsigned long long *status, const unsigned *gate)
 {
+    if (gate && !*gate) return;
     __shared__ uint32_t s_tile;
     __shared__ uint32_t s_warp[SCAN_T / 32];
     __shared__ uint32_t s_prefix;
@@ -185,14 +186,14 @@ void debug_wait_timeout(uint64_t *tmp, DevCounters *ctr, uint32_t limit, cudaStr
 }
 
 void exclusive_scan_u32(const uint32_t *in, uint32_t *out, uint64_t n, uint64_t *tmp,
-                        DevCounters *ctr, cudaStream_t st)
+                        DevCounters *ctr, cudaStream_t st, const unsigned *gate)
 {
     if (n == 0) return;
     uint64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
     cudaMemsetAsync(tmp, 0, (tiles + 1) * sizeof(uint64_t), st);
     TraceScope ts_("scan_kernel", n, st);
     scan_kernel<<<(unsigned)tiles, SCAN_T, 0, st>>>(in, out, n, (unsigned long long *)tmp,
-                                                   &ctr->status);
+                                                   &ctr->status, gate);
 }
 
 // ---------------------------------------------------------------------------

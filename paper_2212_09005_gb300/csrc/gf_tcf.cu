@@ -450,8 +450,10 @@ template <int SRC, int DST, bool SPARSE>
 __global__ void __launch_bounds__(TPB) tcf_group_hist(const uint64_t *__restrict__ keys, const TcfPrep prep,
                                                       uint64_t n_keys, const void *pend, const unsigned *npend,
                                                       TcfGeom G, const uint8_t *fill, uint32_t *cnt,
-                                                      uint32_t *tlist, uint32_t *tcount, unsigned long long *units)
+                                                      uint32_t *tlist, uint32_t *tcount, const unsigned *gate,
+                                                      unsigned long long *units)
 {
+    if (gate && !*gate) return;
     tcf_group_hist_body<SRC, DST, SPARSE>(keys, prep, n_keys, pend, npend, G, fill, cnt, tlist, tcount, units);
 }
 
@@ -549,8 +551,10 @@ __global__ void __launch_bounds__(TPB) tcf_group_scatter(const uint64_t *__restr
                                                          TcfGeom G,
                                                          const uint8_t *fill, uint32_t *cnt,
                                                          const uint32_t *__restrict__ off, uint64_t *rec,
-                                                         uint32_t *recI, unsigned long long *units)
+                                                         uint32_t *recI, const unsigned *gate,
+                                                         unsigned long long *units)
 {
+    if (gate && !*gate) return;
     tcf_group_scatter_body<SRC, DST>(keys, prep, n_keys, pend, npend, G, fill, cnt, off, rec, recI, units);
 }
 
@@ -769,9 +773,10 @@ template <int F>
 __global__ void __launch_bounds__(TPB) tcf_block_insert(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
                                                         const uint64_t *__restrict__ rec, int phase,
                                                         uint32_t cap, uint32_t *pend32, uint64_t *pend64,
-                                                        unsigned *npend, const TcfPrep prep,
+                                                        unsigned *npend, const TcfPrep prep, const unsigned *gate,
                                                         unsigned long long *units)
 {
+    if (gate && !*gate) return;
     tcf_block_insert_body<F>(G, blocks, fill, P, rec, phase, cap, pend32, pend64, npend, prep, units);
 }
 
@@ -1055,8 +1060,10 @@ __device__ __forceinline__ void tcf_block_remove_body(TcfGeom G, uint8_t *blocks
 template <int F>
 __global__ void __launch_bounds__(TPB) tcf_block_remove(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
                                                         const uint64_t *__restrict__ rec, uint32_t *pend32,
-                                                        unsigned *npend, unsigned long long *units)
+                                                        unsigned *npend, const unsigned *gate,
+                                                        unsigned long long *units)
 {
+    if (gate && !*gate) return;
     tcf_block_remove_body<F>(G, blocks, fill, P, rec, pend32, npend, units);
 }
 
@@ -1130,6 +1137,8 @@ struct SparseArgs {
     DevCounters *ctr;
     uint32_t unit_min;  // more candidates than this of the second phase went by unit
     bool first;         // the first phase is taken here too
+    const unsigned *uneven;  // set: all phases are taken here, or all but the first
+    bool first_done;
 };
 
 __device__ __forceinline__ unsigned ld_now(const unsigned *p) { return *(const volatile unsigned *)p; }
@@ -1222,12 +1231,13 @@ __global__ void __launch_bounds__(TPB, 4) tcf_sparse_insert_coop(const SparseArg
     unsigned *np = A.ctr->pend;
     SparseRun run{0, false};
     PhaseDst P;
-    if (A.first) {
+    const bool uneven = A.uneven && ld_now(A.uneven), all = A.first || uneven;  // (the same in every CTA)
+    if (A.first || (uneven && !A.first_done)) {
         if (!sparse_group<SRC_KEYS, DST_B1>(A, nullptr, nullptr, 0, nullptr, run, P)) return;
         tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 0, A.G.tsc, A.pend0, nullptr, &np[0], A.prep, nullptr);
         if (!sparse_next(A, run)) return;
     }
-    if (ld_now(&np[0]) <= A.unit_min) {
+    if (all || ld_now(&np[0]) <= A.unit_min) {
         if (!sparse_group<SRC_PEND_U32, DST_TARGET>(A, A.pend0, &np[0], 1, nullptr, run, P)) return;
         tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 1, A.G.B, nullptr, A.pend1, &np[1], A.prep, nullptr);
         if (!sparse_next(A, run)) return;
@@ -1245,12 +1255,13 @@ __global__ void __launch_bounds__(TPB, 4) tcf_sparse_remove_coop(const SparseArg
     unsigned *np = A.ctr->pend;
     SparseRun run{0, false};
     PhaseDst P;
-    if (A.first) {
+    const bool uneven = A.uneven && ld_now(A.uneven), all = A.first || uneven;  // (the same in every CTA)
+    if (A.first || (uneven && !A.first_done)) {
         if (!sparse_group<SRC_KEYS, DST_B1>(A, nullptr, nullptr, 0, nullptr, run, P)) return;
         tcf_block_remove_body<F>(A.G, A.blocks, A.fill, P, A.rec, A.pend0, &np[0], nullptr);
         if (!sparse_next(A, run)) return;
     }
-    if (ld_now(&np[0]) <= A.unit_min) {
+    if (all || ld_now(&np[0]) <= A.unit_min) {
         if (!sparse_group<SRC_PEND_U32, DST_B2>(A, A.pend0, &np[0], 1, nullptr, run, P)) return;
         tcf_block_remove_body<F>(A.G, A.blocks, A.fill, P, A.rec, A.pend2, &np[2], nullptr);
         if (!sparse_next(A, run)) return;
@@ -1472,12 +1483,16 @@ __device__ __forceinline__ uint64_t tu_item(const TuSrc &s, uint64_t j, const Tc
 
 template <int SRC>
 __global__ void __launch_bounds__(MP_T) tu_hist(const TuSrc s, TcfGeom G, TcfPrep P, const uint8_t *fill, TuGeom U,
-                                                MsdScratch M, unsigned long long *units)
+                                                MsdScratch M, const unsigned *uneven, unsigned long long *units)
 {
     __shared__ uint32_t h[MP_BINS];
+    const uint32_t nb = 1u << U.b1, shift = U.lbits + U.b2;
+    if (uneven && *uneven) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) M.tile1[nb] = M.htile1[nb] = 0;  // nothing for the second pass
+        return;
+    }
     const uint64_t n = tu_count(s);
     note_units(units, n);
-    const uint32_t nb = 1u << U.b1, shift = U.lbits + U.b2;
     for (uint32_t b = threadIdx.x; b < nb; b += MP_T) h[b] = 0;
     __syncthreads();
     for (uint64_t base = (uint64_t)blockIdx.x * MP_TILE; base < n; base += (uint64_t)gridDim.x * MP_TILE) {
@@ -1501,9 +1516,11 @@ __global__ void __launch_bounds__(MP_T) tu_hist(const TuSrc s, TcfGeom G, TcfPre
 // the first pass: a tile's records to the bins of their blocks' top bits
 template <int SRC>
 __global__ void __launch_bounds__(MP_T, 3) tu_part(const TuSrc s, TcfGeom G, TcfPrep P, const uint8_t *fill, TuGeom U,
-                                                   MsdScratch M, uint64_t *__restrict__ out, unsigned long long *units)
+                                                   MsdScratch M, uint64_t *__restrict__ out, const unsigned *uneven,
+                                                   unsigned long long *units)
 {
     __shared__ PartSmem S;
+    if (uneven && *uneven) return;
     const uint64_t n = tu_count(s), base = (uint64_t)blockIdx.x * MP_TILE;
     note_units(units, n);
     if (base >= n) return;
@@ -1919,6 +1936,7 @@ struct TuStep {
     const uint64_t *v;     // records by unit
     TuOut O;
     TuSrc src;
+    const unsigned *uneven;  // set: no phase goes by unit
     unsigned long long *units;
 };
 
@@ -2009,7 +2027,7 @@ __device__ __noinline__ void tu_big_unit(TuSmem &S, const TuStep &A, uint32_t un
 template <int F, bool DEL, int NEXT, bool ONE>
 __global__ void __launch_bounds__(TU_T, 3) tcf_unit_step(const __grid_constant__ TuStep A)
 {
-    if (tu_count(A.src) == 0) return;
+    if (tu_count(A.src) == 0 || (A.uneven && *A.uneven)) return;
     __shared__ __align__(16) TuSmem S;
     const uint32_t tsh = A.U.ibits, bsh = A.U.ibits + A.U.sbits, smask = (1u << A.U.sbits) - 1u;
     const uint64_t rmask = bsh + A.U.lbits >= 64 ? ~0ull : (1ull << (bsh + A.U.lbits)) - 1ull;
@@ -2307,6 +2325,7 @@ struct TcfBulk {
     uint64_t *scan_tmp;
     DevCounters *ctr;
     TcfPrep prep;
+    unsigned *uneven;  // unit path: where the call's keys turned out too uneven for it (null: not asked)
 };
 
 static TcfBulk bulk_of(const TcfState &T, uint64_t *scan_tmp, DevCounters *ctr, const TcfPrep &prep, uint64_t max_n,
@@ -2335,6 +2354,7 @@ static TcfBulk bulk_of(const TcfState &T, uint64_t *scan_tmp, DevCounters *ctr, 
     W.scan_tmp = scan_tmp;
     W.ctr = ctr;
     W.prep = prep;
+    W.uneven = nullptr;
     return W;
 }
 
@@ -2347,10 +2367,12 @@ static int group_grid(uint64_t n) { return grid_for(n, TPB, 8); }
 // scan over all destinations, then the scatter. Later phases see few
 // candidates and are sparse: only the touched destinations get a segment and
 // a list entry (slot: the phase's counters), so their per-destination kernel
-// visits those alone. `recI` (bucket phases) receives the batch indices.
+// visits those alone. `recI` (bucket phases) receives the batch indices. gate: a
+// word on the device without which the kernels do nothing (null: always).
 template <int SRC, int DST>
 static PhaseDst group_phase(const TcfBulk &T, const uint64_t *keys, uint64_t n, const void *pend,
-                            const unsigned *npend, int slot, uint32_t *recI, cudaStream_t st)
+                            const unsigned *npend, int slot, uint32_t *recI, cudaStream_t st,
+                            const unsigned *gate = nullptr)
 {
     const TcfGeom G = T.G;
     const int gk = group_grid(n);
@@ -2360,7 +2382,7 @@ static PhaseDst group_phase(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
     {
         gf::TraceScope ts_(SPARSE ? "tcf_group_hist_sparse" : "tcf_group_hist", n, st, SPARSE);
         tcf_group_hist<SRC, DST, SPARSE><<<gk, TPB, 0, st>>>(keys, T.prep, n, pend, npend, G, T.fill, T.cnt, T.tlist,
-                                                             T.tcount, ts_.units());
+                                                             T.tcount, gate, ts_.units());
     }
     if (SPARSE) {
         gf::TraceScope ts_("tcf_alloc", 0, st, true);
@@ -2370,13 +2392,13 @@ static PhaseDst group_phase(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
         P.seg = T.seg;
         P.nlist = &T.ctr->touched[slot];
     } else {
-        exclusive_scan_u32(T.cnt, T.off, ndst + 1, T.scan_tmp, T.ctr, st);
+        exclusive_scan_u32(T.cnt, T.off, ndst + 1, T.scan_tmp, T.ctr, st, gate);
         P.off = T.off;
     }
     {
         gf::TraceScope ts_(SPARSE ? "tcf_group_scatter_sparse" : "tcf_group_scatter", n, st, SPARSE);
         tcf_group_scatter<SRC, DST><<<gk, TPB, 0, st>>>(keys, T.prep, n, pend, npend, G, T.fill, T.cnt, T.off, T.rec,
-                                                        recI, ts_.units());
+                                                        recI, gate, ts_.units());
     }
     return P;
 }
@@ -2830,6 +2852,12 @@ static void tcf_sparse_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n
 template <int F, int GB = 0>
 static void tcf_sparse_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, cudaStream_t st);
 
+// Of an uneven call, the first phase over every block instead of the touched
+// ones? As in tcf_few_keys; only on large tables, where the five launches that an
+// even call then passes through (24 us) count for little: 2^24 keys in a quarter
+// of 1024 members of 2^18 slots, an insert 1015 us by touched blocks, 901 so.
+static bool uneven_dense(const TcfBulk &T, uint64_t n) { return T.uneven && T.G.nb > (1ull << 22) && n > T.G.nb / 2; }
+
 // the later phases in one launch; at most four CTAs per SM, which its launch
 // bounds keep resident together
 template <int F, bool DEL>
@@ -2837,11 +2865,30 @@ static void tcf_sparse_coop(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
                             bool first, cudaStream_t st)
 {
     SparseArgs A{keys, n, T.G, T.prep, T.blocks, T.fill, T.bk, T.cnt, T.off, T.tlist, T.tcount, T.dlist, T.pend0, T.pend2,
-                 T.rec, T.pend1, T.seg, status, T.ctr, unit_min, first};
+                 T.rec, T.pend1, T.seg, status, T.ctr, unit_min, first, T.uneven, uneven_dense(T, n)};
     void *args[] = {&A};
     gf::TraceScope ts_(DEL ? "tcf_sparse_remove" : "tcf_sparse_insert", n, st);
     const void *kernel = DEL ? (const void *)tcf_sparse_remove_coop<F> : (const void *)tcf_sparse_insert_coop<F>;
     cudaLaunchCooperativeKernel(kernel, dim3(grid_for(n, TPB * 2, 4)), dim3(TPB), args, 0, st);
+}
+
+// the first phase over every block: a shortcut into b1 (A), or removes from it (1)
+template <int F, bool DEL, int GB = 0>
+static void first_by_block(const TcfBulk &T, const uint64_t *keys, uint64_t n, cudaStream_t st,
+                           const unsigned *gate = nullptr)
+{
+    const TcfGeom G = T.G;
+    unsigned *np = T.ctr->pend;
+    const PhaseDst P = group_phase<SRC_KEYS, DST_B1>(T, keys, n, nullptr, nullptr, 0, nullptr, st, gate);
+    gf::TraceScope ts_(DEL ? "tcf_block_remove" : "tcf_block_insert", 0, st, true);
+    if constexpr (GB != 0)
+        gblock_phase<F, GB, DEL>(T, P, n, 0, DEL ? 0 : G.tsc, T.pend0, nullptr, &np[0], ts_.units(), st);
+    else if constexpr (DEL)
+        tcf_block_remove<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, T.pend0, &np[0], gate,
+                                                                   ts_.units());
+    else
+        tcf_block_insert<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, 0, G.tsc, T.pend0, nullptr,
+                                                                   &np[0], T.prep, gate, ts_.units());
 }
 
 // The per-block counting-sort path: each phase groups its candidates by
@@ -2857,16 +2904,7 @@ static void tcf_bulk_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
     cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
     if constexpr (GB == 0)
         if (tcf_few_keys(G.nb, n)) return tcf_sparse_coop<F, false>(T, keys, n, status, 0xffffffffu, true, st);
-    // A: shortcut into b1
-    PhaseDst P = group_phase<SRC_KEYS, DST_B1>(T, keys, n, nullptr, nullptr, 0, nullptr, st);
-    {
-        gf::TraceScope ts_("tcf_block_insert", 0, st, true);
-        if constexpr (GB == 0)
-            tcf_block_insert<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, 0, G.tsc, T.pend0,
-                                                                       nullptr, &np[0], T.prep, ts_.units());
-        else
-            gblock_phase<F, GB, false>(T, P, n, 0, G.tsc, T.pend0, nullptr, &np[0], ts_.units(), st);
-    }
+    first_by_block<F, false, GB>(T, keys, n, st);
     if constexpr (GB == 0)
         if (G.nb >= TCF_COOP_MIN_BLOCKS) return tcf_sparse_coop<F, false>(T, keys, n, status, 0xffffffffu, false, st);
     tcf_sparse_insert<F, GB>(T, keys, n, status, st);
@@ -2886,7 +2924,7 @@ static void tcf_sparse_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n
         gf::TraceScope ts_("tcf_block_insert_sparse", 0, st, true);
         if constexpr (GB == 0)
             tcf_block_insert<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, 1, G.B, nullptr,
-                                                                       T.pend1, &np[1], T.prep, ts_.units());
+                                                                       T.pend1, &np[1], T.prep, nullptr, ts_.units());
         else
             gblock_phase<F, GB, false>(T, P, n, 1, G.B, nullptr, T.pend1, &np[1], ts_.units(), st);
     }
@@ -2896,7 +2934,7 @@ static void tcf_sparse_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n
         gf::TraceScope ts_("tcf_block_insert_sparse", 0, st, true);
         if constexpr (GB == 0)
             tcf_block_insert<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, 2, G.B, T.pend2,
-                                                                       nullptr, &np[2], T.prep, ts_.units());
+                                                                       nullptr, &np[2], T.prep, nullptr, ts_.units());
         else
             gblock_phase<F, GB, false>(T, P, n, 2, G.B, T.pend2, nullptr, &np[2], ts_.units(), st);
     }
@@ -2917,16 +2955,7 @@ static void tcf_bulk_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
     cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
     if constexpr (GB == 0)
         if (tcf_few_keys(G.nb, n)) return tcf_sparse_coop<F, true>(T, keys, n, status, 0xffffffffu, true, st);
-    // 1: primary block
-    PhaseDst P = group_phase<SRC_KEYS, DST_B1>(T, keys, n, nullptr, nullptr, 0, nullptr, st);
-    {
-        gf::TraceScope ts_("tcf_block_remove", 0, st, true);
-        if constexpr (GB == 0)
-            tcf_block_remove<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, T.pend0, &np[0],
-                                                                       ts_.units());
-        else
-            gblock_phase<F, GB, true>(T, P, n, 0, 0, T.pend0, nullptr, &np[0], ts_.units(), st);
-    }
+    first_by_block<F, true, GB>(T, keys, n, st);
     if constexpr (GB == 0)
         if (G.nb >= TCF_COOP_MIN_BLOCKS) return tcf_sparse_coop<F, true>(T, keys, n, status, 0xffffffffu, false, st);
     tcf_sparse_remove<F, GB>(T, keys, n, status, st);
@@ -2945,7 +2974,7 @@ static void tcf_sparse_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n
         gf::TraceScope ts_("tcf_block_remove_sparse", 0, st, true);
         if constexpr (GB == 0)
             tcf_block_remove<F><<<dst_grid(P, n, G.nb), TPB, 0, st>>>(G, T.blocks, T.fill, P, T.rec, T.pend2, &np[2],
-                                                                       ts_.units());
+                                                                       nullptr, ts_.units());
         else
             gblock_phase<F, GB, true>(T, P, n, 0, 0, T.pend2, nullptr, &np[2], ts_.units(), st);
     }
@@ -3029,21 +3058,23 @@ static void tu_phase(const TcfBulk &T, const TuSrc &src, uint64_t n, uint32_t ca
     const TuGeom U = tu_geom(T.G, n, T.tile_target);
     const MsdScratch M = tu_scratch(T.tcur, T.max_n);
     const bool keys = SRC == TU_KEYS;
+    const unsigned *uneven = keys ? T.uneven : nullptr;  // (the later phases have no candidates then)
+    const bool known = keys && !uneven;  // the number of candidates
     const uint32_t nb1 = 1u << U.b1;
     const uint64_t tiles = (n + MP_TILE - 1) / MP_TILE;
     {
-        gf::TraceScope ts_(keys ? "tcf_tile_hist" : "tcf_tile_hist_pend", keys ? n : 0, st, !keys);
-        tu_hist<SRC><<<grid_for(tiles * MP_T, MP_T, 4), MP_T, 0, st>>>(src, T.G, T.prep, T.fill, U, M, ts_.units());
+        gf::TraceScope ts_(keys ? "tcf_tile_hist" : "tcf_tile_hist_pend", known ? n : 0, st, !known);
+        tu_hist<SRC><<<grid_for(tiles * MP_T, MP_T, 4), MP_T, 0, st>>>(src, T.G, T.prep, T.fill, U, M, uneven, ts_.units());
     }
     {
-        gf::TraceScope ts_(keys ? "tcf_tile_part" : "tcf_tile_part_pend", keys ? n : 0, st, !keys);
-        tu_part<SRC><<<(unsigned)tiles, MP_T, 0, st>>>(src, T.G, T.prep, T.fill, U, M, T.rec, ts_.units());
+        gf::TraceScope ts_(keys ? "tcf_tile_part" : "tcf_tile_part_pend", known ? n : 0, st, !known);
+        tu_part<SRC><<<(unsigned)tiles, MP_T, 0, st>>>(src, T.G, T.prep, T.fill, U, M, T.rec, uneven, ts_.units());
     }
     if (U.b2)
         msd_second_pass(M, T.rec, T.seg, n, nb1, U.lbits + U.sbits + U.ibits, U.b2, "tcf_tile_hist2", "tcf_tile_part2", st);
     gf::TraceScope ts_(DEL ? "tcf_tile_remove" : "tcf_tile_insert", 0, st, true);
     const TuStep A{T.G, T.prep, U, T.blocks, T.fill, U.b2 ? M.st2 : M.st1, 1u << U.k, cap, U.b2 ? T.seg : T.rec,
-                   TuOut{orec, oidx, nout, T.max_n, &T.ctr->status}, src, ts_.units()};
+                   TuOut{orec, oidx, nout, T.max_n, &T.ctr->status}, src, uneven, ts_.units()};
     const int g = grid_for((uint64_t)TU_T << U.k, TU_T, 3);
     if (U.lbits <= TU_BBITS) tcf_unit_step<F, DEL, NEXT, true><<<g, TU_T, 0, st>>>(A);
     else tcf_unit_step<F, DEL, NEXT, false><<<g, TU_T, 0, st>>>(A);
@@ -3066,7 +3097,7 @@ static void tcf_unit_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
     const TcfGeom G = T.G;
     unsigned *np = T.ctr->pend;
     const uint32_t unit_min = tu_unit_min(T, n);
-    cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
+    if (!T.uneven) cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
     // A: shortcut into b1 while fill < 3B/4; rejects keep b1
     tu_phase<F, false, TU_KEYS, TU_NX_SAME>(T, TuSrc{keys, nullptr, nullptr, nullptr, 0, n}, n, G.tsc, T.pend1, T.pend0,
                                             &np[0], st);
@@ -3078,6 +3109,7 @@ static void tcf_unit_insert(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
         tu_phase<F, false, TU_SAME, TU_NX_IDX>(T, TuSrc{nullptr, T.pb, T.pbi, &np[1], 0, n}, n, G.B, nullptr, T.pend2,
                                                &np[2], st);
     }
+    if (uneven_dense(T, n)) first_by_block<F, false>(T, keys, n, st, T.uneven);
     // B and C of fewer candidates, and D: backing buckets
     tcf_sparse_coop<F, false>(T, keys, n, status, unit_min, false, st);
 }
@@ -3087,7 +3119,7 @@ static void tcf_unit_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
 {
     unsigned *np = T.ctr->pend;
     const uint32_t unit_min = tu_unit_min(T, n);
-    cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
+    if (!T.uneven) cudaMemsetAsync(np, 0, CALL_WORDS_BYTES, st);
     // 1: primary block; misses go on to the secondary block
     tu_phase<F, true, TU_KEYS, TU_NX_OTHER>(T, TuSrc{keys, nullptr, nullptr, nullptr, 0, n}, n, 0, T.pend1, T.pend0, &np[0],
                                             st);
@@ -3095,6 +3127,7 @@ static void tcf_unit_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
     if (unit_min != 0xffffffffu)
         tu_phase<F, true, TU_SAME, TU_NX_IDX>(T, TuSrc{nullptr, T.pend1, T.pend0, &np[0], unit_min, n}, n, 0, nullptr,
                                               T.pend2, &np[2], st);
+    if (uneven_dense(T, n)) first_by_block<F, true>(T, keys, n, st, T.uneven);
     // 2 of fewer candidates, and 3: backing bucket; what is left is not found
     tcf_sparse_coop<F, true>(T, keys, n, status, unit_min, false, st);
 }
@@ -3242,10 +3275,40 @@ __device__ __forceinline__ TcfGeom member_geom(const TcfMember &M, uint32_t f)
     return G;
 }
 
+// Units are equal stretches of a group's blocks, and a call may bring its keys
+// to a few members only: one CTA would then read a unit of many thousand
+// candidates once for every range that it holds. A member's keys spread evenly
+// over its blocks, so the offsets tell. With a unit of more keys than a CTA holds
+// (less some five deviations) the partition is left out (its kernels return at
+// once), and the cooperative launch takes all phases by touched blocks. An
+// insert and a remove in us by unit / so, in 1024 members of 2^18 slots: 2^20 keys
+// in 8 of them 121400 + 167900 / 185 + 256, 2^22 in a quarter 872 + 1080 / 413 +
+// 420, 2^24 in a half 923 + 1179 / 873 + 1067; in all of them, by unit, 755 + 932.
+static constexpr uint64_t TU_UNEVEN = TU_CAP - 256;
+
+// the keys of the blocks below b, as the members' shares of blocks say
+__device__ __forceinline__ uint64_t keys_below(uint64_t b, const uint64_t *__restrict__ off, uint32_t nmem,
+                                               const TcfMember *__restrict__ mem)
+{
+    uint32_t lo = 0, hi = nmem;  // the last member that starts at or before b
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (mem[mid].block0 <= b) lo = mid;
+        else hi = mid;
+    }
+    const uint64_t in = b - mem[lo].block0, nb = mem[lo].nb, c = off[lo + 1] - off[lo];
+    return off[lo] + (in < nb ? in * c / nb : c);
+}
+
+// uneven: set when some unit of 2^lbits blocks has too many keys (null: not asked)
 __global__ void __launch_bounds__(TPB) tcf_group_prep(const uint64_t *__restrict__ keys, uint64_t n,
                                                       const uint64_t *__restrict__ off, uint32_t nmem,
-                                                      const TcfMember *__restrict__ mem, uint32_t f, TcfPrep out)
+                                                      const TcfMember *__restrict__ mem, uint32_t f, TcfPrep out,
+                                                      uint64_t nunits, uint32_t lbits, unsigned *uneven)
 {
+    if (uneven)
+        for (uint64_t u = blockIdx.x * (uint64_t)TPB + threadIdx.x; u < nunits; u += (uint64_t)gridDim.x * TPB)
+            if (keys_below((u + 1) << lbits, off, nmem, mem) - keys_below(u << lbits, off, nmem, mem) > TU_UNEVEN) *uneven = 1;
     MemberCursor c(off, nmem, n);
     uint32_t cm = 0xffffffffu;
     TcfMember M;
@@ -3437,17 +3500,23 @@ int tcf_group_op(filter_group *GR, int op, const uint64_t *off, const uint64_t *
         GF_CUDA(cudaGetLastError());
         return FILTER_OK;
     }
+    TcfBulk W = bulk_of(T, GR->scan_tmp, GR->ctr, GR->prep, GR->max_total, GR->tune);
+    const bool tiled = n > TS_CAP && tcf_tiled(GR->tune, T.G.nb, n, op != GROUP_INSERT) && tu_takes(T.G, n, W.tile_target);
+    const TuGeom U = tu_geom(T.G, n, W.tile_target);
+    if (tiled && GR->tune.tcf_path == FILTER_TCF_PATH_AUTO) {
+        W.uneven = &GR->ctr->uneven;
+        GF_CUDA(cudaMemsetAsync(GR->ctr->pend, 0, CALL_WORDS_BYTES, st));
+    }
     {
         gf::TraceScope ts_("tcf_group_prep", n, st);
-        tcf_group_prep<<<grid_for(n, TPB, 8), TPB, 0, st>>>(keys, n, off, GR->n, GR->d_tmem, T.G.f, GR->prep);
+        tcf_group_prep<<<grid_for(n, TPB, 8), TPB, 0, st>>>(keys, n, off, GR->n, GR->d_tmem, T.G.f, GR->prep, 1ull << U.k,
+                                                            U.lbits, W.uneven);
     }
-    const TcfBulk W = bulk_of(T, GR->scan_tmp, GR->ctr, GR->prep, GR->max_total, GR->tune);
     if (op == GROUP_INSERT ? tcf_small_call<false>(W, nullptr, n, out, st) : tcf_small_call<true>(W, nullptr, n, out, st)) {
         GF_CUDA(cudaGetLastError());
         return FILTER_OK;
     }
     if (out) GF_CUDA(cudaMemsetAsync(out, 0, n, st));
-    const bool tiled = tcf_tiled(GR->tune, T.G.nb, n, op != GROUP_INSERT) && tu_takes(T.G, n, tcf_tile_target(GR->tune));
     if (op == GROUP_INSERT) {
         if (T.G.f == 16) tiled ? tcf_unit_insert<16>(W, nullptr, n, out, st) : tcf_bulk_insert<16>(W, nullptr, n, out, st);
         else tiled ? tcf_unit_insert<8>(W, nullptr, n, out, st) : tcf_bulk_insert<8>(W, nullptr, n, out, st);
