@@ -1330,6 +1330,10 @@ __global__ void __launch_bounds__(MT, MERGE_CTAS) gqf_merge_group_kernel(const M
     merge_one<R>(A, S, s_tile - A.tile0);
 }
 
+// the word of ctr->pend that tells the number of groups with a merge's overflow
+// or a pre-check's verdict
+static constexpr int PRECHECK_GROUPS = 2;
+
 // What a merge starts from: no tile published, no overflow, no end, and (not in
 // dry runs) empty metadata: cleared by the launch before it in place of four
 // memsets (1000 keys in and out of 2^20 slots, two merges: 170 us before, 148
@@ -1338,6 +1342,7 @@ struct MergeClear {
     unsigned long long *ts;
     uint64_t words;
     DevCounters *ctr;
+    const uint32_t *pm;        // number of groups (device)
     unsigned long long *meta;  // null: dry run
     uint64_t meta_words;
 };
@@ -1347,6 +1352,7 @@ __device__ __forceinline__ void merge_clear(const MergeClear &c)
     const uint64_t i0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, step = (uint64_t)gridDim.x * blockDim.x;
     if (i0 == 0) {
         c.ctr->overflow = 0;
+        c.ctr->pend[PRECHECK_GROUPS] = *c.pm;
         c.ctr->gqf_end = -1;
     }
     for (uint64_t i = i0; i < c.words; i += step) c.ts[i] = 0;
@@ -1397,7 +1403,7 @@ __global__ void gqf_unit_tile_ranges(const uint64_t *__restrict__ ufp, MsdUnits 
         if (t * TQ < N) {
             const uint64_t u = t >> span;
             lo = units.st[u];
-            hi = lo + units.distinct[u];
+            hi = lo + (*clear.pm ? units.distinct[u] : 0u);  // (units given up have none)
             for (int side = 0; side < 2 && span; side++) {  // the tile's first group, then the next tile's
                 const uint64_t key = ((t + side) * TQ) << r;
                 uint32_t a = lo, b = hi;
@@ -1882,9 +1888,10 @@ __global__ void gqf_insert_phase(GView g, const uint64_t *__restrict__ ufp, cons
 
 // first group of every delete region (successor search)
 __global__ void gqf_region_ranges(const uint64_t *__restrict__ ufp, const uint32_t *pm, uint64_t N, uint32_t r,
-                                  uint64_t rq, uint64_t nreg, uint32_t *rlo)
+                                  uint64_t rq, uint64_t nreg, uint32_t *rlo, DevCounters *ctr)
 {
     const uint64_t m = *pm;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctr->pend[PRECHECK_GROUPS] = (uint32_t)m;
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t <= nreg;
          t += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t q0 = t * rq;
@@ -1904,12 +1911,14 @@ __global__ void gqf_region_ranges(const uint64_t *__restrict__ ufp, const uint32
 // the first gap at or after x + 1; a block's gaps are read off its own record
 // (gv_block_gap), so a thread makes one load per 64 slots of cluster instead
 // of two dependent ones per run (1000 groups at 85 % load: 90 -> 18 us). seen:
-// stored groups, and those of them whose cluster runs past their block.
+// stored groups, and those of them whose cluster runs past their block; then the
+// number of groups.
 template <int R>
 __global__ void gqf_delete_precheck(GView g, const uint64_t *__restrict__ ufp, const uint32_t *pm,
                                     unsigned long long *reach, unsigned *seen)
 {
     const uint64_t m = *pm;
+    if (blockIdx.x == 0 && threadIdx.x == 0) seen[PRECHECK_GROUPS] = (uint32_t)m;
     unsigned long long mine = 0;
     unsigned found = 0, crowded = 0;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
@@ -2334,8 +2343,9 @@ __global__ void __launch_bounds__(SM_T) gqf_small_prepare(const uint64_t *__rest
 // sort carries the batch indices (need_idx: statuses) or a caller's per-key
 // values (vals, without statuses); either ends in idx_b in sorted order. With
 // `units`, groups bound for the merge may be left in their units: *in_units
-// says whether they were.
-static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_idx, cudaStream_t st,
+// says whether they were. Unless by_digits, batches that the sort carries nothing
+// for go by units, which are given up (0 groups) when their values are not spread.
+static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_idx, bool by_digits, cudaStream_t st,
                         uint32_t **sorted_idx, const uint32_t *vals = nullptr, MsdUnits *units = nullptr,
                         bool *in_units = nullptr)
 {
@@ -2350,13 +2360,13 @@ static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_i
                                                            Q.merge_only ? nullptr : &F->ctr->pend[2]);
         return;
     }
-    if (!need_idx && !vals) {
+    if (!need_idx && !vals && !by_digits) {
         auto groups = [&](MsdUnits *in) {
             return msd_groups(keys, n, &Q.H, Q.p, Q.q > TQ_LOG ? Q.q - TQ_LOG : 0u, Q.fp_a, Q.fp_b, Q.ufp, Q.ustart,
                               Q.flags + n, Q.radix_tmp, radix_tmp_words(F->cfg.max_batch), F->ctr, st, in);
         };
-        // in place of the table, a batch needs its groups in one list; one
-        // twice past that bound may still turn out to have few distinct keys
+        // in place of the table, a batch needs its groups in one list; one up to
+        // four times past that bound may still turn out to have few distinct keys
         const bool dense = n > 4 * gqf_in_place_most(F->tune, Q.N) || Q.merge_only;
         if (units && dense && groups(units)) {
             *in_units = true;
@@ -2403,7 +2413,7 @@ static int gqf_merge(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m_l
     a.r = Q.r;
     a.del = del;
     a.dry = dry;
-    const MergeClear clear{Q.tile_state, Q.ntiles + 1, F->ctr,
+    const MergeClear clear{Q.tile_state, Q.ntiles + 1, F->ctr, Q.flags + n,
                            dry ? nullptr : reinterpret_cast<unsigned long long *>(Q.meta[nb]), Q.nblk * 4};
     const int g = grid_for(Q.nblk * 2 > Q.ntiles * 32 + 32 ? Q.nblk * 2 : Q.ntiles * 32 + 32, 256, 8);
     if (units) {
@@ -2452,16 +2462,18 @@ static uint64_t first_region(uint64_t m, uint64_t N)
     return rq;
 }
 
-// what a pre-check found: its verdict (a region that cannot, or the reach),
-// and its counts of places and of crowded ones
+// what a pre-check found: its verdict (a region that cannot, or the reach), its
+// counts of places and of crowded ones, and the number of groups (0: the units
+// were given up); after a merge, whether the table overflowed, and the groups
 struct Precheck {
     unsigned long long verdict;
-    unsigned seen[2];
+    unsigned seen[2], groups;
     bool crowded() const { return (uint64_t)seen[1] * 4 >= seen[0] && seen[0]; }
     bool warps(uint64_t m) const { return m <= GVW_FEW || (m <= GVW_MOST && crowded()); }
     bool merge(uint64_t m, uint64_t N) const { return crowded() && m * RQ_MIN > N; }
 };
-static_assert(offsetof(DevCounters, pend) == offsetof(DevCounters, overflow) + 8, "a pre-check's words are read together");
+static_assert(offsetof(DevCounters, pend) == offsetof(DevCounters, overflow) + 8 &&
+              offsetof(Precheck, groups) == 8 + 4 * PRECHECK_GROUPS, "a pre-check's words are read together");
 
 template <class T>
 static int read_dev(const T *d, T *h, cudaStream_t st);
@@ -2480,7 +2492,8 @@ static uint64_t gqf_crowded_most(uint64_t N, uint64_t late)
 }
 
 // Whether a batch of at most m groups goes in place as far as the table's load
-// says; m becomes its number of groups when that was read.
+// says; m becomes its number of groups when that was read (0: the units were
+// given up).
 static int gqf_goes_in_place(filter *F, uint64_t n, bool small, uint64_t &m, bool &in_place, cudaStream_t st)
 {
     GqfState &Q = F->gqf;
@@ -2519,8 +2532,8 @@ static int clear_precheck(DevCounters *ctr, cudaStream_t st)
 // Small batches go in place over even-odd regions; `done` is false when the
 // pre-check found, at every region size tried, a region whose inserts could
 // reach the region after next (or the table's end). m: at least the number
-// of groups.
-static int gqf_insert_in_place(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m, cudaStream_t st,
+// of groups; 0 afterwards when the units were given up (nothing was done).
+static int gqf_insert_in_place(filter *F, const uint32_t *cstart, uint64_t n, uint64_t &m, cudaStream_t st,
                                bool &done)
 {
     GqfState &Q = F->gqf;
@@ -2533,12 +2546,12 @@ static int gqf_insert_in_place(filter *F, const uint32_t *cstart, uint64_t n, ui
     for (uint64_t rq = first_region(m, Q.N);
          rq <= (uint64_t)RQ_MAX / 4 && m * rq <= gqf_region_groups(F->tune) * Q.N; rq <<= 2) {
         const uint64_t nreg = (Q.N + rq - 1) / rq;
+        if ((rc = clear_precheck(F->ctr, st))) return rc;
         {
             gf::TraceScope ts_("gqf_region_ranges", nreg + 1, st);
             gqf_region_ranges<<<grid_for(nreg + 1, 256, 4), 256, 0, st>>>(Q.ufp, Q.flags + n, Q.N, Q.r, rq, nreg,
-                                                                         Q.tile_lo);
+                                                                         Q.tile_lo, F->ctr);
         }
-        if ((rc = clear_precheck(F->ctr, st))) return rc;
         unsigned long long *d_bad = &F->ctr->overflow;
         if (pc.warps(m)) {  // as the last try saw the clusters
             gf::TraceScope ts_("gqf_insert_precheck_warp", nreg, st);
@@ -2561,6 +2574,10 @@ static int gqf_insert_in_place(filter *F, const uint32_t *cstart, uint64_t n, ui
             else gqf_insert_precheck<16><<<gr, 128, 0, st>>>(g, Q.ufp, Q.tile_lo, need, nreg, rq, d_bad, F->ctr->pend);
         }
         if ((rc = read_dev(reinterpret_cast<const Precheck *>(&F->ctr->overflow), &pc, st))) return rc;
+        if (pc.groups == 0) {
+            m = 0;
+            break;
+        }
         if (pc.merge(m, Q.N)) break;
         if (pc.verdict) continue;
         const bool warps = pc.warps(m);
@@ -2581,18 +2598,20 @@ static int gqf_insert_in_place(filter *F, const uint32_t *cstart, uint64_t n, ui
     return FILTER_OK;
 }
 
-int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t n, uint8_t *status,
-               cudaStream_t st)
+// by_digits: the sort, as in gqf_prepare. given_up: the units were, and nothing
+// was inserted.
+static int gqf_insert_by(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t n, uint8_t *status,
+                         bool by_digits, bool &given_up, cudaStream_t st)
 {
-    if (n == 0) return FILTER_OK;
     GqfState &Q = F->gqf;
+    given_up = false;
     uint32_t *sidx = nullptr;
     // counts without statuses ride through the sort in place of the indices;
     // other inserts need no indices unless some group does not fit
     const bool carry = counts != nullptr && status == nullptr, need_idx = counts != nullptr && status != nullptr;
     MsdUnits units{};
     bool in_units = false;
-    gqf_prepare(F, keys, n, need_idx, st, &sidx, carry ? counts : nullptr, counts ? nullptr : &units, &in_units);
+    gqf_prepare(F, keys, n, need_idx, by_digits, st, &sidx, carry ? counts : nullptr, counts ? nullptr : &units, &in_units);
     int rc;
     // the copies each group adds: its keys, or the sum of their counts
     const uint32_t *cstart = Q.ustart;
@@ -2626,23 +2645,25 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
         uint64_t m = n;
         bool in_place = false;
         if ((rc = gqf_goes_in_place(F, n, n <= GQF_SMALL, m, in_place, st))) return rc;
-        if (in_place) {
-            bool done = false;
-            if ((rc = gqf_insert_in_place(F, cstart, n, m, st, done))) return rc;
-            if (done) {
-                GF_CUDA(cudaGetLastError());
-                return FILTER_OK;
-            }
+        bool done = false;
+        if (in_place && m && (rc = gqf_insert_in_place(F, cstart, n, m, st, done))) return rc;
+        given_up = m == 0;
+        if (done || given_up) {
+            GF_CUDA(cudaGetLastError());
+            return FILTER_OK;
         }
     }
     rc = gqf_merge(F, cstart, n, ~0ull, 0, 0, st, in_units ? &units : nullptr);
     if (rc) return rc;
-    unsigned long long ovf = 0;
-    if ((rc = read_dev(&F->ctr->overflow, &ovf, st))) return rc;
+    Precheck pc{};
+    if ((rc = read_dev(reinterpret_cast<const Precheck *>(&F->ctr->overflow), &pc, st))) return rc;
+    given_up = pc.groups == 0;
+    if (given_up) return FILTER_OK;
+    const bool ovf = pc.verdict != 0;
     uint64_t m_keep = ~0ull;
     if (ovf) {
         // one list, whose prefixes are tried, with the indices of its keys
-        if (in_units || (status && !need_idx)) gqf_prepare(F, keys, n, status != nullptr, st, &sidx);
+        if (in_units || (status && !need_idx)) gqf_prepare(F, keys, n, status != nullptr, true, st, &sidx);
         // keep the longest prefix of the sorted groups that fits (dry runs)
         uint32_t m = 0;
         if ((rc = read_dev(Q.flags + n, &m, st))) return rc;
@@ -2675,19 +2696,30 @@ int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t
     return FILTER_OK;
 }
 
-int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cudaStream_t st)
+int gqf_insert(filter *F, const uint64_t *keys, const uint32_t *counts, uint64_t n, uint8_t *status, cudaStream_t st)
 {
     if (n == 0) return FILTER_OK;
+    bool given_up;
+    const int rc = gqf_insert_by(F, keys, counts, n, status, false, given_up, st);
+    return rc || !given_up ? rc : gqf_insert_by(F, keys, counts, n, status, true, given_up, st);
+}
+
+static int gqf_remove_by(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, bool by_digits, bool &given_up,
+                         cudaStream_t st)
+{
     GqfState &Q = F->gqf;
+    given_up = false;
     uint32_t *sidx = nullptr;
     MsdUnits units{};
     bool in_units = false;
-    gqf_prepare(F, keys, n, status != nullptr, st, &sidx, nullptr, &units, &in_units);
+    gqf_prepare(F, keys, n, status != nullptr, by_digits, st, &sidx, nullptr, &units, &in_units);
     int rc = FILTER_OK;
     // small batches: in place, cluster by cluster; large ones: full merge
     uint64_t m = n;  // at least the number of groups
     bool in_place = false;
     if (!in_units && (rc = gqf_goes_in_place(F, n, n <= GQF_SMALL, m, in_place, st))) return rc;
+    given_up = m == 0;
+    if (given_up) return FILTER_OK;
     bool done = false;
     if (in_place) {
         GView g{reinterpret_cast<Meta *>(Q.meta[Q.cur]), Q.rem[Q.cur], (long long)Q.N, (long long)Q.nslots,
@@ -2702,6 +2734,8 @@ int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cud
         }
         Precheck pc{};
         if ((rc = read_dev(reinterpret_cast<const Precheck *>(&F->ctr->overflow), &pc, st))) return rc;
+        given_up = pc.groups == 0;
+        if (given_up) return FILTER_OK;
         const bool warps = pc.warps(m);
         uint64_t rq = first_region(m, Q.N);
         while ((unsigned long long)rq < pc.verdict) rq <<= 1;
@@ -2710,7 +2744,7 @@ int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cud
             {
                 gf::TraceScope ts_("gqf_region_ranges", nreg + 1, st);
                 gqf_region_ranges<<<grid_for(nreg + 1, 256, 4), 256, 0, st>>>(Q.ufp, Q.flags + n, Q.N, Q.r, rq, nreg,
-                                                                             Q.tile_lo);
+                                                                             Q.tile_lo, F->ctr);
             }
             const uint64_t half = (nreg + 1) / 2;
             uint32_t *removed = status ? Q.removed : nullptr;
@@ -2733,6 +2767,12 @@ int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cud
     }
     if (!done) {
         if ((rc = gqf_merge(F, Q.ustart, n, ~0ull, 1, 0, st, in_units ? &units : nullptr))) return rc;
+        if (!status && !by_digits && n > GQF_SMALL && m == n) {  // sorted by units, and the groups not read yet
+            uint32_t groups = 0;
+            if ((rc = read_dev(Q.flags + n, &groups, st))) return rc;
+            given_up = groups == 0;
+            if (given_up) return FILTER_OK;
+        }
         Q.cur ^= 1;
     }
     if (status) {
@@ -2745,6 +2785,14 @@ int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cud
         GF_CUDA(cudaGetLastError());
     }
     return FILTER_OK;
+}
+
+int gqf_remove(filter *F, const uint64_t *keys, uint64_t n, uint8_t *status, cudaStream_t st)
+{
+    if (n == 0) return FILTER_OK;
+    bool given_up;
+    const int rc = gqf_remove_by(F, keys, n, status, false, given_up, st);
+    return rc || !given_up ? rc : gqf_remove_by(F, keys, n, status, true, given_up, st);
 }
 
 int gqf_count(filter *F, const uint64_t *keys, uint64_t n, uint64_t *counts, uint8_t *found, cudaStream_t st)

@@ -269,7 +269,8 @@ static constexpr int MP_BINS = 512;          // most bins of a pass
 // cleared before each
 struct MsdScratch {
     uint32_t *cnt1;     // first pass: values per bin
-    uint32_t *misc;     // [0] unit ticket, [1] squeezed chunks, [2] oversized units, [3] CTAs done
+    uint32_t *misc;     // [0] unit ticket, [1] squeezed chunks, [2] oversized units, [3] CTAs done,
+                        // [4] 1 when an oversized unit had too many distinct values
     uint64_t *look;     // look-back words of the units
     uint32_t *cnt2;     // second pass: values per unit
     uint32_t *st1, *cur1, *tile1, *htile1;  // first-pass bins: starts, cursors, first tiles of either kind
@@ -404,7 +405,9 @@ __device__ __forceinline__ void part_tile(PartSmem &S, const uint64_t (&v)[MP_I]
 // of their top k <= max_k bits: those of unit u are uniq / start [st[u], st[u] +
 // distinct[u]), with start[st[u] + distinct[u]] = st[u + 1] behind them, in tmp
 // until its next use. False (and nothing enqueued) for the sizes that it does
-// not take.
+// not take. *m_out = 0 when the values turned out crowded into a few units with
+// more distinct ones than a CTA takes: no group is written then, and the caller
+// sorts by digits.
 struct MsdUnits {
     const uint32_t *st, *distinct;
     uint32_t k;

@@ -17,7 +17,10 @@
 // Skew: the copies of a key all fall into one unit. A unit of more than MU_CAP
 // keys goes through a hash table in shared memory (its distinct values are
 // few) before the others are sorted, and one of more than MS_CHUNK keys is
-// squeezed to (value, copies) pairs before that, chunk by chunk.
+// squeezed to (value, copies) pairs before that, chunk by chunk. Where the
+// distinct values do not fit the table, the values are not spread as hashes are
+// (a stretch of a filter's enumeration put into another of its geometry): the
+// units are then given up, and the caller sorts by digits, whatever the values.
 #include "gf_internal.cuh"
 
 namespace gf {
@@ -30,7 +33,6 @@ static constexpr uint32_t MT_CAP = 4096;        // hash table: home slots
 static constexpr uint32_t MT_PAD = 256;         // and slots past the last one
 static constexpr uint32_t MT_PROBES = 192;      // hash table: longest probe
 static constexpr uint32_t MS_CHUNK = 16384;     // keys of a squeezed chunk
-static constexpr uint32_t MS_RAW = 0xffffffffu; // a chunk with too many distinct values stays as it is
 static constexpr uint32_t EMPTY = 0xffffffffu;  // (values below have at most 31 bits)
 
 static_assert(MP_BINS <= MP_T, "a thread per bin");
@@ -46,7 +48,7 @@ MsdScratch msd_scratch(uint32_t *base, uint64_t n, uint32_t k, bool two, bool lo
     };
     const uint64_t units = 1ull << k, chunks = 2 * (n / MS_CHUNK) + 2;
     s.cnt1 = take(MP_BINS);
-    s.misc = take(4);
+    s.misc = take(5);
     s.look = reinterpret_cast<uint64_t *>(take(lookback ? 2 * units : 0));
     s.cnt2 = take(two ? units : 0);
     s.zero_words = at;
@@ -243,11 +245,11 @@ void msd_second_pass(const MsdScratch &s, const uint64_t *in, uint64_t *out, uin
 struct Table {
     uint32_t *key, *cnt;  // MT_CAP + MT_PAD each
     uint32_t *over;       // set when a value found no slot
-    uint32_t lo, shift;   // home slot of v: (v - lo) >> shift
+    uint32_t shift;       // home slot of v: v >> shift
 
     __device__ __forceinline__ void add(uint32_t v, uint32_t w) const
     {
-        uint32_t p = (v - lo) >> shift;
+        uint32_t p = v >> shift;
         for (uint32_t t = 0; t < MT_PROBES && p < MT_CAP + MT_PAD; t++, p++) {
             uint32_t x = key[p];
             if (x == EMPTY) x = atomicCAS(&key[p], EMPTY, v);
@@ -255,9 +257,12 @@ struct Table {
                 atomicAdd(&cnt[p], w);
                 return;
             }
+            if (t % 16 == 15 && full()) return;
         }
         *over = 1;
     }
+    // some value found no slot (while others are added)
+    __device__ __forceinline__ bool full() const { return *(const volatile uint32_t *)over; }
     __device__ __forceinline__ void clear() const
     {
         for (uint32_t p = threadIdx.x; p < MT_CAP + MT_PAD; p += MU_T) {
@@ -287,22 +292,23 @@ struct RunCache {
 };
 
 // Squeezes the chunks of the units above MS_CHUNK keys to pairs (copies << 32
-// | low value bits), in place: copies of a hot key and a few distinct others. A chunk with too many of them stays as it is (MS_RAW).
+// | low value bits), in place: copies of a hot key and a few distinct others. A
+// chunk with more of them than the table takes gives the units up.
 __global__ void __launch_bounds__(MU_T) msd_squeeze(uint64_t *v, MsdScratch s, const uint32_t *__restrict__ st,
                                                     uint32_t rbits)
 {
     __shared__ uint32_t t_key[MT_CAP + MT_PAD], t_cnt[MT_CAP + MT_PAD], s_over, s_n;
     const uint32_t mask = (1u << rbits) - 1u;
-    const Table T{t_key, t_cnt, &s_over, 0u, rbits > 12 ? rbits - 12 : 0u};
+    const Table T{t_key, t_cnt, &s_over, rbits > 12 ? rbits - 12 : 0u};
     static_assert(MT_CAP == 1u << 12, "12 bits of home slot");
     for (uint32_t c = blockIdx.x; c < s.misc[1]; c += gridDim.x) {
         const uint32_t u = s.chunk_unit[c], i0 = st[u] + (c - s.chunk0[u]) * MS_CHUNK;
         const uint32_t end = min(i0 + MS_CHUNK, st[u + 1]);
         T.clear();
         if (threadIdx.x == 0) s_n = 0;
-        __syncthreads();
+        if (__syncthreads_or(s.misc[4])) return;
         RunCache run;
-        for (uint32_t base = i0; base < end; base += 8 * MU_T) {
+        for (uint32_t base = i0; base < end && !T.full(); base += 8 * MU_T) {
             uint64_t x[8];
 #pragma unroll
             for (int r = 0; r < 8; r++) {
@@ -316,27 +322,30 @@ __global__ void __launch_bounds__(MU_T) msd_squeeze(uint64_t *v, MsdScratch s, c
         run.flush(T);
         __syncthreads();
         if (s_over) {
-            if (threadIdx.x == 0) s.chunk_cnt[c] = MS_RAW;
-        } else {
-            for (uint32_t p = threadIdx.x; p < MT_CAP + MT_PAD; p += MU_T)
-                if (t_key[p] != EMPTY) v[i0 + atomicAdd(&s_n, 1u)] = ((uint64_t)t_cnt[p] << 32) | t_key[p];
-            __syncthreads();
-            if (threadIdx.x == 0) s.chunk_cnt[c] = s_n;
+            if (threadIdx.x == 0) s.misc[4] = 1;
+            return;
         }
+        for (uint32_t p = threadIdx.x; p < MT_CAP + MT_PAD; p += MU_T)
+            if (t_key[p] != EMPTY) v[i0 + atomicAdd(&s_n, 1u)] = ((uint64_t)t_cnt[p] << 32) | t_key[p];
+        __syncthreads();
+        if (threadIdx.x == 0) s.chunk_cnt[c] = s_n;
         __syncthreads();
     }
 }
 
-// Oversized units, a CTA each: every (value, copies) through the hash table,
-// in rounds over value ranges that fit it (one, unless the values are no
-// hashes). The distinct values are left in order in `spare` as pairs, their
-// number in distinct[u]. They have a launch of their own because a slow unit
-// would hold up the look-back of all that follow it.
+// Oversized units, a CTA each: every (value, copies) through the hash table.
+// The distinct values are left in order in `spare` as pairs, their number in
+// distinct[u]. They have a launch of their own because a slow unit would hold
+// up the look-back of all that follow it. A unit with more distinct values than
+// the table takes gives the units up: another round over its keys for each part
+// of them grows with the square of their number (2^16 keys spread over one unit
+// of 2^28 slots, an insert 95 ms by such rounds, 0.32 given up and sorted by digits).
 __global__ void __launch_bounds__(MU_T) msd_big(const uint64_t *__restrict__ v, MsdScratch s,
                                                 const uint32_t *__restrict__ st, uint32_t rbits, uint64_t *spare)
 {
     __shared__ uint32_t t_key[MT_CAP + MT_PAD], t_cnt[MT_CAP + MT_PAD], s_over, s_warp[MU_T / 32];
     const uint32_t mask = (1u << rbits) - 1u;
+    const Table T{t_key, t_cnt, &s_over, rbits > 12 ? rbits - 12 : 0u};
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (uint32_t k = blockIdx.x; k < s.misc[2]; k += gridDim.x) {
         const uint32_t u = s.big[k], s0 = st[u], c = st[u + 1] - s0;
@@ -345,67 +354,54 @@ __global__ void __launch_bounds__(MU_T) msd_big(const uint64_t *__restrict__ v, 
         // threads per chunk: few when the chunks are many, and hold little each
         uint32_t per = MU_T;
         while (per > 4 && (MU_T / per) < nch) per >>= 1;
-        uint32_t lo = 0, range = 1u << rbits, out = 0;  // (rbits <= 31)
-        while (lo < (1u << rbits)) {
-            uint32_t sh = 0;
-            while ((range >> sh) > MT_CAP) sh++;
-            const Table T{t_key, t_cnt, &s_over, lo, sh};
-            T.clear();
-            __syncthreads();
-            RunCache run;
-            for (uint32_t ch = threadIdx.x / per; ch < nch; ch += MU_T / per) {
-                const uint32_t left = squeezed ? s.chunk_cnt[ch0 + ch] : MS_RAW;
-                const uint64_t *p = v + s0 + ch * MS_CHUNK;
-                const uint32_t m = left == MS_RAW ? min(MS_CHUNK, c - ch * MS_CHUNK) : left;
-                for (uint32_t i = threadIdx.x % per; i < m; i += 8 * per) {
-                    uint64_t x[8];
+        T.clear();
+        if (__syncthreads_or(s.misc[4])) return;
+        RunCache run;
+        for (uint32_t ch = threadIdx.x / per; ch < nch; ch += MU_T / per) {
+            const uint64_t *p = v + s0 + ch * MS_CHUNK;
+            const uint32_t m = squeezed ? s.chunk_cnt[ch0 + ch] : c;
+            for (uint32_t i = threadIdx.x % per; i < m && !T.full(); i += 8 * per) {
+                uint64_t x[8];
 #pragma unroll
-                    for (int r = 0; r < 8; r++)
-                        if (i + r * per < m) x[r] = p[i + r * per];
+                for (int r = 0; r < 8; r++)
+                    if (i + r * per < m) x[r] = p[i + r * per];
 #pragma unroll
-                    for (int r = 0; r < 8; r++) {
-                        const uint32_t val = (uint32_t)x[r] & mask;
-                        if (i + r * per < m && val - lo < range)
-                            run.push(T, val, left == MS_RAW ? 1u : (uint32_t)(x[r] >> 32));
-                    }
-                }
+                for (int r = 0; r < 8; r++)
+                    if (i + r * per < m) run.push(T, (uint32_t)x[r] & mask, squeezed ? (uint32_t)(x[r] >> 32) : 1u);
             }
-            run.flush(T);
-            __syncthreads();
-            if (s_over && range > 1) {  // too many distinct values: half the range (a single value always fits)
-                range >>= 1;
-                __syncthreads();
-                continue;
-            }
-            // occupied slots below each warp's stretch of the table
-            constexpr uint32_t SPAN = (MT_CAP + MT_PAD) / (MU_T / 32);
-            static_assert(SPAN % 32 == 0, "whole warps of slots");
-            uint32_t mine = 0;
-            for (uint32_t q = 0; q < SPAN; q += 32)
-                mine += __popc(__ballot_sync(0xffffffffu, t_key[warp * SPAN + q + lane] != EMPTY));
-            if (lane == 0) s_warp[warp] = mine;
-            __syncthreads();
-            uint32_t pre = 0, total = 0;
-            for (int w = 0; w < MU_T / 32; w++) {
-                if (w < warp) pre += s_warp[w];
-                total += s_warp[w];
-            }
-            for (uint32_t q = 0; q < SPAN; q += 32) {
-                const uint32_t p = warp * SPAN + q + lane, x = t_key[p];
-                const unsigned occ = __ballot_sync(0xffffffffu, x != EMPTY);
-                if (x != EMPTY) {
-                    uint32_t r = pre + __popc(occ & ((1u << lane) - 1u));
-                    for (uint32_t j = p; j > 0 && t_key[j - 1] != EMPTY; j--) r -= t_key[j - 1] > x;
-                    for (uint32_t j = p + 1; j < MT_CAP + MT_PAD && t_key[j] != EMPTY; j++) r += t_key[j] < x;
-                    spare[s0 + out + r] = ((uint64_t)t_cnt[p] << 32) | x;
-                }
-                pre += __popc(occ);
-            }
-            out += total;
-            lo += range;
-            __syncthreads();
         }
-        if (threadIdx.x == 0) s.distinct[u] = out;
+        run.flush(T);
+        __syncthreads();
+        if (s_over) {
+            if (threadIdx.x == 0) s.misc[4] = 1;
+            return;
+        }
+        // occupied slots below each warp's stretch of the table
+        constexpr uint32_t SPAN = (MT_CAP + MT_PAD) / (MU_T / 32);
+        static_assert(SPAN % 32 == 0, "whole warps of slots");
+        uint32_t mine = 0;
+        for (uint32_t q = 0; q < SPAN; q += 32)
+            mine += __popc(__ballot_sync(0xffffffffu, t_key[warp * SPAN + q + lane] != EMPTY));
+        if (lane == 0) s_warp[warp] = mine;
+        __syncthreads();
+        uint32_t pre = 0, total = 0;
+        for (int w = 0; w < MU_T / 32; w++) {
+            if (w < warp) pre += s_warp[w];
+            total += s_warp[w];
+        }
+        for (uint32_t q = 0; q < SPAN; q += 32) {
+            const uint32_t p = warp * SPAN + q + lane, x = t_key[p];
+            const unsigned occ = __ballot_sync(0xffffffffu, x != EMPTY);
+            if (x != EMPTY) {
+                uint32_t r = pre + __popc(occ & ((1u << lane) - 1u));
+                for (uint32_t j = p; j > 0 && t_key[j - 1] != EMPTY; j--) r -= t_key[j - 1] > x;
+                for (uint32_t j = p + 1; j < MT_CAP + MT_PAD && t_key[j] != EMPTY; j++) r += t_key[j] < x;
+                spare[s0 + r] = ((uint64_t)t_cnt[p] << 32) | x;
+            }
+            pre += __popc(occ);
+        }
+        if (threadIdx.x == 0) s.distinct[u] = total;
+        __syncthreads();
     }
 }
 
@@ -524,7 +520,7 @@ __device__ __forceinline__ void unit_sort(UnitSmem &S, const uint32_t (&key)[MU_
 // units differ, 4.36 and 1.97 ms). CTAs stay and fetch the next unit's keys
 // while this one's groups are written. v: the keys by unit; pairs: the
 // oversized units' groups. Bound by instructions and the barriers between the
-// steps.
+// steps. Nothing is done, and *m_out stays 0, when the units were given up.
 template <bool ORDERED>
 __global__ void __launch_bounds__(MU_T, 6) msd_units(const uint64_t *__restrict__ v, MsdScratch s,
                                                      const uint32_t *__restrict__ st, uint32_t units, uint32_t rbits,
@@ -533,6 +529,7 @@ __global__ void __launch_bounds__(MU_T, 6) msd_units(const uint64_t *__restrict_
                                                      unsigned long long *status)
 {
     __shared__ __align__(16) UnitSmem S;
+    if (s.misc[4]) return;
     const uint32_t mask = (1u << rbits) - 1u, bs = rbits > MU_BBITS ? rbits - MU_BBITS : 0u;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long *look = reinterpret_cast<unsigned long long *>(s.look);
