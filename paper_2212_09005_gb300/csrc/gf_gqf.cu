@@ -2523,6 +2523,53 @@ static int gqf_goes_in_place(filter *F, uint64_t n, bool small, uint64_t &m, boo
     return FILTER_OK;
 }
 
+// the groups left in units as one list, a warp per unit; first: the groups
+// before each unit
+__global__ void gqf_units_list(const uint64_t *__restrict__ ufp, const uint32_t *__restrict__ ustart, MsdUnits units,
+                               const uint32_t *__restrict__ first, uint32_t n, uint64_t *__restrict__ list,
+                               uint32_t *__restrict__ lstart)
+{
+    const uint32_t u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (u >> units.k) return;
+    const uint32_t s = units.st[u], c = units.distinct[u], o = first[u];
+    for (uint32_t i = lane; i < c; i += 32) {
+        list[o + i] = ufp[s + i];
+        lstart[o + i] = ustart[s + i];
+    }
+    if (u == (1u << units.k) - 1 && lane == 0) lstart[o + c] = n;
+}
+
+// Groups left in units are bound for the merge, by the number of their keys. A
+// batch of few distinct keys goes in place all the same, its groups put into one
+// list. Not below 2^24 slots, where a merge takes no longer. Copies of 1000 keys,
+// an insert and a remove in us, merged / in place: 2^24 slots, 2^19 keys 290 + 262
+// / 283 + 135, 2^24 keys 571 + 543 / 562 + 414; 2^25, 2^21 556 + 527 / 304 + 196;
+// 2^26, 2^23 1012 + 990 / 358 + 271; 2^28, 2^26 4010 + 3952 / 1176 + 1130. A bound
+// that the caller set holds at all sizes. m becomes the number of groups when it
+// was read (0: the units were given up).
+static int gqf_units_in_place(filter *F, uint64_t n, const MsdUnits &units, uint64_t &m, bool &in_units, cudaStream_t st)
+{
+    GqfState &Q = F->gqf;
+    if (Q.merge_only || (!F->tune.gqf_region_groups && Q.N < (1ull << 24))) return FILTER_OK;
+    uint32_t groups = 0;
+    const int rc = read_dev(Q.flags + n, &groups, st);
+    if (rc) return rc;
+    m = groups;
+    if (m == 0 || m > gqf_in_place_most(F->tune, Q.N)) return FILTER_OK;
+    // the sort's buffers are free again; the ranges are not found yet
+    uint32_t *first = Q.tile_lo;
+    exclusive_scan_u32(units.distinct, first, 1ull << units.k, F->scan_tmp, F->ctr, st);
+    {
+        gf::TraceScope ts_("gqf_units_list", m, st);
+        gqf_units_list<<<(unsigned)((32ull << units.k) + 255) / 256, 256, 0, st>>>(Q.ufp, Q.ustart, units, first, (uint32_t)n,
+                                                                                  Q.fp_a, Q.idx_a);
+    }
+    GF_CUDA(cudaMemcpyAsync(Q.ufp, Q.fp_a, m * 8, cudaMemcpyDeviceToDevice, st));
+    GF_CUDA(cudaMemcpyAsync(Q.ustart, Q.idx_a, (m + 1) * 4, cudaMemcpyDeviceToDevice, st));
+    in_units = false;
+    return FILTER_OK;
+}
+
 static int clear_precheck(DevCounters *ctr, cudaStream_t st)
 {
     GF_CUDA(cudaMemsetAsync(&ctr->overflow, 0, sizeof(Precheck), st));
@@ -2641,18 +2688,20 @@ static int gqf_insert_by(filter *F, const uint64_t *keys, const uint32_t *counts
     if (status) GF_CUDA(cudaMemsetAsync(status, FILTER_KEY_OK, n, st));
     // small batches: in place, region by region; larger ones: the merge. The
     // keys bound the groups, whose number is read back only when that decides.
-    if (!in_units) {
-        uint64_t m = n;
+    uint64_t m = n;
+    if (in_units && (rc = gqf_units_in_place(F, n, units, m, in_units, st))) return rc;
+    if (!in_units && m) {
         bool in_place = false;
         if ((rc = gqf_goes_in_place(F, n, n <= GQF_SMALL, m, in_place, st))) return rc;
         bool done = false;
         if (in_place && m && (rc = gqf_insert_in_place(F, cstart, n, m, st, done))) return rc;
-        given_up = m == 0;
-        if (done || given_up) {
+        if (done) {
             GF_CUDA(cudaGetLastError());
             return FILTER_OK;
         }
     }
+    given_up = m == 0;
+    if (given_up) return FILTER_OK;
     rc = gqf_merge(F, cstart, n, ~0ull, 0, 0, st, in_units ? &units : nullptr);
     if (rc) return rc;
     Precheck pc{};
@@ -2717,7 +2766,8 @@ static int gqf_remove_by(filter *F, const uint64_t *keys, uint64_t n, uint8_t *s
     // small batches: in place, cluster by cluster; large ones: full merge
     uint64_t m = n;  // at least the number of groups
     bool in_place = false;
-    if (!in_units && (rc = gqf_goes_in_place(F, n, n <= GQF_SMALL, m, in_place, st))) return rc;
+    if (in_units && (rc = gqf_units_in_place(F, n, units, m, in_units, st))) return rc;
+    if (!in_units && m && (rc = gqf_goes_in_place(F, n, n <= GQF_SMALL, m, in_place, st))) return rc;
     given_up = m == 0;
     if (given_up) return FILTER_OK;
     bool done = false;
