@@ -18,7 +18,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgpufilter.so")
 SOURCES = ["gf_prims.cu", "gf_tcf.cu", "gf_gqf.cu", "gf_capi.cu", "gf_group.cu", "gf_serve.cu", "gf_noalloc.cu",
            "gf_batch.cu", "gf_msd.cu"]
-HEADERS = ["gf_internal.cuh", "gf_sched.h", "gf_packed.cuh", "gf_small.cuh"]
+HEADERS = ["gf_internal.cuh", "gf_sched.h", "gf_packed.cuh", "gf_small.cuh", "gf_coop.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVFLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 

@@ -31,6 +31,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "gf_coop.h"
 #include "gf_internal.cuh"
 #include "gf_packed.cuh"
 #include "gf_small.cuh"
@@ -2859,7 +2860,7 @@ static void tcf_sparse_remove(const TcfBulk &T, const uint64_t *keys, uint64_t n
 static bool uneven_dense(const TcfBulk &T, uint64_t n) { return T.uneven && T.G.nb > (1ull << 22) && n > T.G.nb / 2; }
 
 // the later phases in one launch; at most four CTAs per SM, which its launch
-// bounds keep resident together
+// bounds keep resident together (fewer where the stream has a part of the SMs)
 template <int F, bool DEL>
 static void tcf_sparse_coop(const TcfBulk &T, const uint64_t *keys, uint64_t n, uint8_t *status, uint32_t unit_min,
                             bool first, cudaStream_t st)
@@ -2869,7 +2870,10 @@ static void tcf_sparse_coop(const TcfBulk &T, const uint64_t *keys, uint64_t n, 
     void *args[] = {&A};
     gf::TraceScope ts_(DEL ? "tcf_sparse_remove" : "tcf_sparse_insert", n, st);
     const void *kernel = DEL ? (const void *)tcf_sparse_remove_coop<F> : (const void *)tcf_sparse_insert_coop<F>;
-    cudaLaunchCooperativeKernel(kernel, dim3(grid_for(n, TPB * 2, 4)), dim3(TPB), args, 0, st);
+    coop_launch(
+        grid_for(n, TPB * 2, 4), cudaErrorCooperativeLaunchTooLarge,
+        [&](int g) { return cudaLaunchCooperativeKernel(kernel, dim3(g), dim3(TPB), args, 0, st); },
+        [] { cudaGetLastError(); });
 }
 
 // the first phase over every block: a shortcut into b1 (A), or removes from it (1)
