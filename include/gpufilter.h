@@ -133,7 +133,7 @@ int filter_destroy(filter_t *f);
  *     a block or more on tables of 2^12 blocks or more. A group call whose keys
  *     belong to a few members only leaves TILED for the touched blocks.
  *   tcf_tile_target: tiled path, the expected candidates per tile, 128 ..
- *     1024 (0: 2048).
+ *     2048 (0: 2048).
  *   gqf_region_groups: GQF batches with at most this many distinct
  *     fingerprints per 256 quotients on average are inserted or removed in
  *     place (even-odd regions); denser ones take the merge (0: by the table's

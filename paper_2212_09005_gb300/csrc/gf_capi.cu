@@ -31,7 +31,7 @@ namespace gf {
 bool tuning_valid(const filter_tuning &t)
 {
     if (t.tcf_path > FILTER_TCF_PATH_TILED) return false;
-    if (t.tcf_tile_target && (t.tcf_tile_target < 128 || t.tcf_tile_target > 1024)) return false;
+    if (t.tcf_tile_target && (t.tcf_tile_target < 128 || t.tcf_tile_target > 2048)) return false;
     if (t.gqf_region_groups > 256) return false;
     return true;
 }

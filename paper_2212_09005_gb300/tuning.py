@@ -84,7 +84,7 @@ def struct(knobs: dict):
 # ---------------------------------------------------------------------------
 # Measurement
 # ---------------------------------------------------------------------------
-TCF_CANDIDATES = ((0, 0), (1, 0), (2, 512), (2, 1024))    # (tcf_path, tile target)
+TCF_CANDIDATES = ((0, 0), (1, 0), (2, 512), (2, 1024), (2, 2048))  # (tcf_path, tile target)
 AUTO_MARGIN = 0.97  # what another choice's time must be below, of the library's own
 GQF_CANDIDATES = (0, 1, 4, 8, 16)                          # region groups
 
