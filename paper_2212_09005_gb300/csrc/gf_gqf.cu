@@ -2454,11 +2454,18 @@ static int read_dev(const T *d, T *h, cudaStream_t st)
 // place by threads, 8.3 ms merged).
 static constexpr uint64_t GVW_FEW = 1u << 14, GVW_MOST = 1u << 18;
 
-// the smallest region tried: about one group each when warps take them anyway
+// The smallest region tried. A region's groups go one after another, and a group
+// opens its slots so: regions stay small, but on tables of so many that finding
+// them, a warp each, counts (2^20 of them 100 us): there, sixteen or more for a
+// group. An insert in us with about one region for a group / this way: 2^24 slots
+// at 70 % load, 1000 keys 144 / 80, three copies of each 269 / 132, 16000 keys 245
+// / 174; at 85 %, 300 keys 155 / 85, but 16000 keys, whose pre-check then fails
+// once, 406 / 479; 2^26 slots at 70 %, 4000 keys 175 / 134, at 40 %, 16000 143 /
+// 161; 2^28 slots at 70 %, 1000 keys 108 / 107, three copies of 4000 468 / 403.
 static uint64_t first_region(uint64_t m, uint64_t N)
 {
     uint64_t rq = RQ_MIN;
-    while (m <= GVW_FEW && rq < (uint64_t)RQ_MAX / 4 && m * rq * 4 <= N) rq <<= 2;
+    while (N > (1ull << 24) && m <= GVW_FEW && rq < (uint64_t)RQ_MAX / 4 && m * rq * 64 <= N) rq <<= 2;
     return rq;
 }
 
