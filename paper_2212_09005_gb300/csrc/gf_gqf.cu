@@ -397,7 +397,6 @@ __device__ __forceinline__ long long tile_lookback(unsigned long long *st, DevCo
         const long long v = ein + TB;
         const long long P = v > TA ? v : TA;
         atomicExch(&st[tile], (2ull << 62) | (unsigned long long)(P + 1));
-        atomicMax(&ctr->gqf_end, P);
     }
     return ein;
 }
@@ -867,8 +866,8 @@ struct FastSmem {
     uint32_t occ[TQ / 32], wpre[TQ / 32 + 1], nocc[TQ / 32], off[TBLK], rend[FOUT / 32];
     uint32_t sel[MT / 32];
     int wA[MT / 32], wB[MT / 32], wQ[MT / 32];
-    long long prev_end, os0;
-    uint32_t glo, ghi, yfirst, oldlen, err;
+    long long os0;
+    uint32_t glo, ghi, yfirst, oldlen;
 };
 
 // the group of an old run [.., e] at slot p: its value, count and slots
@@ -937,7 +936,6 @@ __device__ __forceinline__ bool merge_tile(const MergeArgs &a, FastSmem<R> &S, c
     } else if (tid == TBLK) {
         S.glo = a.tlo[tile];
         S.ghi = a.thi[tile];
-        S.err = 0;
         S.oldlen = 0;
     }
     for (int p = tid; p < (int)(FCAP / 32 + 1); p += MT) S.dead[p] = 0;
@@ -1334,7 +1332,7 @@ __global__ void __launch_bounds__(MT, MERGE_CTAS) gqf_merge_group_kernel(const M
 // or a pre-check's verdict
 static constexpr int PRECHECK_GROUPS = 2;
 
-// What a merge starts from: no tile published, no overflow, no end, and (not in
+// What a merge starts from: no tile published, no overflow, and (not in
 // dry runs) empty metadata: cleared by the launch before it in place of four
 // memsets (1000 keys in and out of 2^20 slots, two merges: 170 us before, 148
 // now).
@@ -1353,7 +1351,6 @@ __device__ __forceinline__ void merge_clear(const MergeClear &c)
     if (i0 == 0) {
         c.ctr->overflow = 0;
         c.ctr->pend[PRECHECK_GROUPS] = *c.pm;
-        c.ctr->gqf_end = -1;
     }
     for (uint64_t i = i0; i < c.words; i += step) c.ts[i] = 0;
     if (!c.meta) return;
@@ -1438,7 +1435,7 @@ static constexpr long long RQ_MAX = 1 << 16;
 // In-place batches are worth it only while each region thread has few groups
 // to apply one after another; past that the merge, whose cost does not grow
 // with the batch, is faster. The limit on the mean groups per region is a
-// tuning knob (gqf_region_groups, 8 by default).
+// tuning knob (gqf_region_groups; gqf_in_place_most and the table's load without).
 
 
 // ---------------------------------------------------------------------------
@@ -2362,7 +2359,7 @@ static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_i
     }
     if (!need_idx && !vals && !by_digits) {
         auto groups = [&](MsdUnits *in) {
-            return msd_groups(keys, n, &Q.H, Q.p, Q.q > TQ_LOG ? Q.q - TQ_LOG : 0u, Q.fp_a, Q.fp_b, Q.ufp, Q.ustart,
+            return msd_groups(keys, n, Q.H, Q.p, Q.q > TQ_LOG ? Q.q - TQ_LOG : 0u, Q.fp_a, Q.fp_b, Q.ufp, Q.ustart,
                               Q.flags + n, Q.radix_tmp, radix_tmp_words(F->cfg.max_batch), F->ctr, st, in);
         };
         // in place of the table, a batch needs its groups in one list; one up to
@@ -2481,9 +2478,6 @@ struct Precheck {
 };
 static_assert(offsetof(DevCounters, pend) == offsetof(DevCounters, overflow) + 8 &&
               offsetof(Precheck, groups) == 8 + 4 * PRECHECK_GROUPS, "a pre-check's words are read together");
-
-template <class T>
-static int read_dev(const T *d, T *h, cudaStream_t st);
 
 // Crowded tables merge from fewer groups, and without a pre-check. late: slots
 // that a block's offset is late, per mille: 820 at 70 % load, 1600 at 80 %, 2400
@@ -3064,7 +3058,6 @@ __global__ void gqf_group_reset(DevCounters *mctr, uint32_t n)
 {
     for (uint32_t m = blockIdx.x * blockDim.x + threadIdx.x; m < n; m += gridDim.x * blockDim.x) {
         mctr[m].overflow = 0;
-        mctr[m].gqf_end = -1;
     }
 }
 

@@ -45,12 +45,11 @@ struct DevCounters {
     unsigned int cursor[4];       // TCF sparse phases: records placed so far
     unsigned int bar;             // arrivals at the barriers of a cooperative launch
     unsigned int uneven;          // TCF group calls: 1 when some unit has far more keys than its share
-    long long gqf_end;            // GQF merge: end of the last run (dry runs)
     unsigned long long wflag;     // GQF counted insert: 1 if some count was 0
 };
 // a TCF bulk call clears its words, pend to uneven, at once
 static constexpr size_t CALL_WORDS_BYTES = 18 * sizeof(unsigned int);
-static_assert(offsetof(DevCounters, gqf_end) == offsetof(DevCounters, pend) + CALL_WORDS_BYTES, "pend to uneven are adjacent");
+static_assert(offsetof(DevCounters, wflag) == offsetof(DevCounters, pend) + CALL_WORDS_BYTES, "pend to uneven are adjacent");
 
 // ---------------------------------------------------------------------------
 // Hashing (paper Sec. 5.1 fingerprint h; Sec. 4 block/tag hash). Bijective:
@@ -365,7 +364,7 @@ struct PartSmem {
 };
 template <bool HOT, class Digit>
 __device__ __forceinline__ void part_tile(PartSmem &S, const uint64_t (&v)[MP_I], uint32_t cnt, uint32_t nb,
-                                          Digit digit, uint32_t *cur, uint64_t *__restrict__ out)
+                                          Digit digit, uint32_t *cur)
 {
     const int lane = threadIdx.x & 31;
     for (uint32_t b = threadIdx.x; b < nb; b += MP_T) S.cnt[b] = 0;
@@ -399,20 +398,19 @@ __device__ __forceinline__ void part_tile(PartSmem &S, const uint64_t (&v)[MP_I]
 
 // Distinct sorted values of n keys and the copies before each (gf_msd.cu): for
 // each group g, uniq[g] ascending and start[g] = the keys below it, start[m] =
-// n and *m_out = m. The values are the keys' fingerprints (H set), or the keys
-// themselves, of `bits` bits. buf_a and buf_b: n words each, spent; keys may be
-// buf_b. tmp: 32-bit words of scratch. With units_out, the groups stay in units
-// of their top k <= max_k bits: those of unit u are uniq / start [st[u], st[u] +
-// distinct[u]), with start[st[u] + distinct[u]] = st[u + 1] behind them, in tmp
-// until its next use. False (and nothing enqueued) for the sizes that it does
-// not take. *m_out = 0 when the values turned out crowded into a few units with
+// n and *m_out = m. The values are the keys' fingerprints, of `bits` bits. buf_a
+// and buf_b: n words each, spent. tmp: 32-bit words of scratch. With units_out,
+// the groups stay in units of their top k <= max_k bits: those of unit u are uniq
+// / start [st[u], st[u] + distinct[u]), with start[st[u] + distinct[u]] = st[u +
+// 1] behind them, in tmp until its next use. False (and nothing enqueued) for the
+// sizes that it does not take. *m_out = 0 when the values turned out crowded into a few units with
 // more distinct ones than a CTA takes: no group is written then, and the caller
 // sorts by digits.
 struct MsdUnits {
     const uint32_t *st, *distinct;
     uint32_t k;
 };
-bool msd_groups(const uint64_t *keys, uint64_t n, const PHash *H, uint32_t bits, uint32_t max_k, uint64_t *buf_a,
+bool msd_groups(const uint64_t *keys, uint64_t n, const PHash &H, uint32_t bits, uint32_t max_k, uint64_t *buf_a,
                 uint64_t *buf_b, uint64_t *uniq, uint32_t *start, uint32_t *m_out, uint32_t *tmp, uint64_t tmp_words,
                 DevCounters *ctr, cudaStream_t st, MsdUnits *units_out);
 

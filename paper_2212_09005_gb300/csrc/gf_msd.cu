@@ -75,14 +75,7 @@ MsdScratch msd_scratch(uint32_t *base, uint64_t n, uint32_t k, bool two, bool lo
 // ---------------------------------------------------------------------------
 // Histograms
 // ---------------------------------------------------------------------------
-template <bool HASH>
-__device__ __forceinline__ uint64_t msd_value(uint64_t key, const PHash &H)
-{
-    return HASH ? fingerprint(key, H) : key;
-}
-
-// keys per first-pass bin (value >> shift), one shared histogram per CTA
-template <bool HASH>
+// keys per first-pass bin (fingerprint >> shift), one shared histogram per CTA
 __global__ void __launch_bounds__(MP_T) msd_hist1(const uint64_t *__restrict__ keys, uint64_t n, PHash H,
                                                   uint32_t shift, uint32_t nb, MsdScratch s, bool two, uint32_t *m_out)
 {
@@ -101,7 +94,7 @@ __global__ void __launch_bounds__(MP_T) msd_hist1(const uint64_t *__restrict__ k
 #pragma unroll
         for (int r = 0; r < MP_I; r++) {
             const uint64_t i = base + r * MP_T + threadIdx.x;
-            if (i < n) atomicAdd(&h[(uint32_t)(msd_value<HASH>(v[r], H) >> shift)], 1u);
+            if (i < n) atomicAdd(&h[(uint32_t)(fingerprint(v[r], H) >> shift)], 1u);
         }
     }
     __syncthreads();
@@ -174,12 +167,12 @@ __global__ void __launch_bounds__(MP_BINS) msd_scan2(MsdScratch s, uint32_t nb1,
 }
 
 // ---------------------------------------------------------------------------
-// A partition pass. FIRST: tiles of the batch, keys hashed when HASH; else
-// tiles of a first-pass bin, whose keys go to its units. Bound by the
+// A partition pass. FIRST: tiles of the batch, whose keys are hashed; else
+// tiles of a first-pass bin, whose values go to its units. Bound by the
 // shared-memory pipe (80 % busy with the rank atomics and the staging; 16 bytes
 // a key at 4.4 TB/s); 48 warps per SM.
 // ---------------------------------------------------------------------------
-template <bool FIRST, bool HASH>
+template <bool FIRST>
 __global__ void __launch_bounds__(MP_T, 3) msd_part(const uint64_t *__restrict__ in, uint32_t n, PHash H, MsdScratch s,
                                                     uint32_t nb1, uint32_t shift, uint32_t bits,
                                                     uint64_t *__restrict__ out, unsigned long long *units)
@@ -209,8 +202,8 @@ __global__ void __launch_bounds__(MP_T, 3) msd_part(const uint64_t *__restrict__
     }
     if (FIRST)
 #pragma unroll
-        for (int r = 0; r < MP_I; r++) v[r] = msd_value<HASH>(v[r], H);
-    part_tile<!FIRST>(S, v, cnt, nb, [=](uint64_t x, int) { return (uint32_t)(x >> shift) & (nb - 1); }, cur, out);
+        for (int r = 0; r < MP_I; r++) v[r] = fingerprint(v[r], H);
+    part_tile<!FIRST>(S, v, cnt, nb, [=](uint64_t x, int) { return (uint32_t)(x >> shift) & (nb - 1); }, cur);
 #pragma unroll
     for (int r = 0; r < MP_I; r++) {
         const uint32_t i = r * MP_T + threadIdx.x;
@@ -233,7 +226,7 @@ void msd_second_pass(const MsdScratch &s, const uint64_t *in, uint64_t *out, uin
         msd_scan2<<<nb1, MP_BINS, 0, st>>>(s, nb1, bits2);
     }
     TraceScope ts_(part_name, 0, st, true);
-    msd_part<false, false><<<(unsigned)((n + MP_TILE - 1) / MP_TILE) + nb1, MP_T, 0, st>>>(in, (uint32_t)n, PHash{}, s, nb1,
+    msd_part<false><<<(unsigned)((n + MP_TILE - 1) / MP_TILE) + nb1, MP_T, 0, st>>>(in, (uint32_t)n, PHash{}, s, nb1,
                                                                                          shift, bits2, out, ts_.units());
 }
 
@@ -632,17 +625,17 @@ __global__ void __launch_bounds__(MU_T, 6) msd_units(const uint64_t *__restrict_
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-bool msd_groups(const uint64_t *keys, uint64_t n, const PHash *H, uint32_t bits, uint32_t max_k, uint64_t *buf_a,
+bool msd_groups(const uint64_t *keys, uint64_t n, const PHash &H, uint32_t bits, uint32_t max_k, uint64_t *buf_a,
                 uint64_t *buf_b, uint64_t *uniq, uint32_t *start, uint32_t *m_out, uint32_t *tmp, uint64_t tmp_words,
                 DevCounters *ctr, cudaStream_t st, MsdUnits *units_out)
 {
     if (n < 2048 || n >= (1ull << 30)) return false;
-    // units of 1024 to 2048 keys on average: a uniform batch's largest unit is
-    // eleven deviations below what a CTA sorts
+    // units of 1024 to 2048 keys on average: what a CTA sorts is eleven deviations
+    // above the mean of a uniform batch's units
     uint32_t k = 1;
     while (k < bits && (n >> k) > 2048) k++;
     const bool ordered = units_out == nullptr;
-    if (!ordered && k > max_k) {  // units at least as wide as asked for; a fifth more keys still fit
+    if (!ordered && k > max_k) {  // units at least as wide as asked for: means up to six deviations below the cap still fit
         if (k > max_k + 1 || (n >> max_k) > MU_CAP - 6 * 45) return false;
         k = max_k;
     }
@@ -651,7 +644,6 @@ bool msd_groups(const uint64_t *keys, uint64_t n, const PHash *H, uint32_t bits,
     if (k == 0 || k > 18 || rbits > 31) return false;
     const MsdScratch s = msd_scratch(tmp, n, k, two, ordered, true);
     if (s.words > tmp_words) return false;
-    const PHash h = H ? *H : PHash{};
     const uint32_t units = 1u << k;
     uint64_t *const v = two ? buf_b : buf_a, *const pairs = two ? buf_a : buf_b;
     cudaMemsetAsync(tmp, 0, s.zero_words * 4, st);
@@ -659,13 +651,11 @@ bool msd_groups(const uint64_t *keys, uint64_t n, const PHash *H, uint32_t bits,
     {
         TraceScope ts_("msd_hist1", n, st);
         const int g = grid_for(tiles * (uint64_t)MP_T, MP_T, 4);
-        if (H) msd_hist1<true><<<g, MP_T, 0, st>>>(keys, n, h, bits - b1, 1u << b1, s, two, m_out);
-        else msd_hist1<false><<<g, MP_T, 0, st>>>(keys, n, h, bits - b1, 1u << b1, s, two, m_out);
+        msd_hist1<<<g, MP_T, 0, st>>>(keys, n, H, bits - b1, 1u << b1, s, two, m_out);
     }
     {
         TraceScope ts_("msd_part", n, st);
-        if (H) msd_part<true, true><<<tiles, MP_T, 0, st>>>(keys, (uint32_t)n, h, s, 0, bits - b1, b1, buf_a, nullptr);
-        else msd_part<true, false><<<tiles, MP_T, 0, st>>>(keys, (uint32_t)n, h, s, 0, bits - b1, b1, buf_a, nullptr);
+        msd_part<true><<<tiles, MP_T, 0, st>>>(keys, (uint32_t)n, H, s, 0, bits - b1, b1, buf_a, nullptr);
     }
     if (two) msd_second_pass(s, buf_a, buf_b, n, 1u << b1, rbits, b2, "msd_hist2", "msd_part2", st);
     const uint32_t *ust = two ? s.st2 : s.st1;

@@ -1535,7 +1535,7 @@ __global__ void __launch_bounds__(MP_T, 3) tu_part(const TuSrc s, TcfGeom G, Tcf
         const uint32_t i = r * MP_T + threadIdx.x;
         if (i < cnt) bin[r] = (uint16_t)(tu_item<SRC>(s, base + i, G, P, fill, U, v[r]) >> shift);
     }
-    part_tile<false>(S, v, cnt, nb, [&](uint64_t, int r) { return (uint32_t)bin[r]; }, M.cur1, out);
+    part_tile<false>(S, v, cnt, nb, [&](uint64_t, int r) { return (uint32_t)bin[r]; }, M.cur1);
 #pragma unroll
     for (int r = 0; r < MP_I; r++) {
         const uint32_t i = r * MP_T + threadIdx.x;
