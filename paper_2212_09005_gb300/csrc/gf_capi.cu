@@ -10,6 +10,16 @@ const char *last_cuda_error();
 
 static cudaStream_t as_stream(void *s) { return static_cast<cudaStream_t>(s); }
 
+static void free_filter(filter *F)
+{
+    if (F->told_ev) cudaEventDestroy(F->told_ev);
+    if (F->told) cudaFreeHost(F->told);
+    gf::dev_free(F->ctr);
+    gf::dev_free(F->arena.base);
+    F->arena.base = nullptr;
+    delete F;
+}
+
 static bool valid(const filter_t *f) { return f != nullptr && f->arena.base != nullptr; }
 
 // every device buffer of the filter got an address
@@ -153,11 +163,15 @@ int filter_create(const filter_config *cfg, void *stream, filter_t **out)
     else rc = gf::gqf_setup(F, tb, sb, false);
     if (rc == FILTER_OK && F->arena.used > F->arena.size) rc = FILTER_ERR_INTERNAL;
     if (rc == FILTER_OK && !pointers_set(F)) rc = FILTER_ERR_INTERNAL;
+    if (rc == FILTER_OK && cfg->kind == FILTER_GQF &&
+        (cudaHostAlloc(reinterpret_cast<void **>(&F->told), sizeof(uint32_t), cudaHostAllocMapped) != cudaSuccess ||
+         cudaEventCreateWithFlags(&F->told_ev, cudaEventDisableTiming) != cudaSuccess)) {
+        cudaGetLastError();
+        rc = FILTER_ERR_OOM;
+    }
     if (rc == FILTER_OK) rc = (cfg->kind == FILTER_TCF) ? gf::tcf_clear(F, as_stream(stream)) : gf::gqf_clear(F, as_stream(stream));
     if (rc != FILTER_OK) {
-        gf::dev_free(F->ctr);
-        gf::dev_free(F->arena.base);
-        delete F;
+        free_filter(F);
         return rc;
     }
     *out = F;
@@ -169,10 +183,7 @@ int filter_destroy(filter_t *f)
     if (!f) return FILTER_OK;
     int rc = FILTER_OK;
     if (cudaDeviceSynchronize() != cudaSuccess) rc = FILTER_ERR_CUDA;
-    gf::dev_free(f->ctr);
-    gf::dev_free(f->arena.base);
-    f->arena.base = nullptr;
-    delete f;
+    free_filter(f);
     return rc;
 }
 

@@ -1341,6 +1341,7 @@ struct MergeClear {
     uint64_t words;
     DevCounters *ctr;
     const uint32_t *pm;        // number of groups (device)
+    uint32_t *told;            // the same for the host (null: not asked)
     unsigned long long *meta;  // null: dry run
     uint64_t meta_words;
 };
@@ -1351,6 +1352,7 @@ __device__ __forceinline__ void merge_clear(const MergeClear &c)
     if (i0 == 0) {
         c.ctr->overflow = 0;
         c.ctr->pend[PRECHECK_GROUPS] = *c.pm;
+        if (c.told) *(volatile uint32_t *)c.told = *c.pm;
     }
     for (uint64_t i = i0; i < c.words; i += step) c.ts[i] = 0;
     if (!c.meta) return;
@@ -2382,8 +2384,9 @@ static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_i
 
 // cstart: group g adds (or removes) cstart[g + 1] - cstart[g] copies
 // units: the groups' units where they were left in place (msd_groups)
+// tell: F->told has the number of groups after F->told_ev
 static int gqf_merge(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m_limit, int del, int dry,
-                     cudaStream_t st, const MsdUnits *units = nullptr)
+                     cudaStream_t st, const MsdUnits *units = nullptr, bool tell = false)
 {
     GqfState &Q = F->gqf;
     const int nb = Q.cur ^ 1;
@@ -2410,7 +2413,7 @@ static int gqf_merge(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m_l
     a.r = Q.r;
     a.del = del;
     a.dry = dry;
-    const MergeClear clear{Q.tile_state, Q.ntiles + 1, F->ctr, Q.flags + n,
+    const MergeClear clear{Q.tile_state, Q.ntiles + 1, F->ctr, Q.flags + n, tell ? F->told : nullptr,
                            dry ? nullptr : reinterpret_cast<unsigned long long *>(Q.meta[nb]), Q.nblk * 4};
     const int g = grid_for(Q.nblk * 2 > Q.ntiles * 32 + 32 ? Q.nblk * 2 : Q.ntiles * 32 + 32, 256, 8);
     if (units) {
@@ -2421,6 +2424,7 @@ static int gqf_merge(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m_l
         gf::TraceScope ts_("gqf_tile_ranges", Q.ntiles + 1, st);
         gqf_tile_ranges<<<g, 256, 0, st>>>(Q.ufp, Q.flags + n, m_limit, Q.N, Q.r, Q.ntiles, Q.tile_lo, clear);
     }
+    if (tell) GF_CUDA(cudaEventRecord(F->told_ev, st));
     {
         gf::TraceScope ts_("gqf_merge_kernel", 0, st, true);
         if (Q.r == 8) gqf_merge_kernel<8><<<(unsigned)Q.ntiles, MT, 0, st>>>(a, ts_.units());
@@ -2817,10 +2821,16 @@ static int gqf_remove_by(filter *F, const uint64_t *keys, uint64_t n, uint8_t *s
         }
     }
     if (!done) {
-        if ((rc = gqf_merge(F, Q.ustart, n, ~0ull, 1, 0, st, in_units ? &units : nullptr))) return rc;
-        if (!status && !by_digits && n > GQF_SMALL && m == n) {  // sorted by units, and the groups not read yet
+        // Sorted by units, and the groups not read yet: their number comes while the
+        // merge runs (2^17 keys removed from 2^20 slots 84 us without asking, 104
+        // with the number read back after the merge, 85 so).
+        const bool ask = !status && !by_digits && n > GQF_SMALL && m == n;
+        if ((rc = gqf_merge(F, Q.ustart, n, ~0ull, 1, 0, st, in_units ? &units : nullptr, ask && F->told))) return rc;
+        if (ask) {
             uint32_t groups = 0;
-            if ((rc = read_dev(Q.flags + n, &groups, st))) return rc;
+            if (F->told) GF_CUDA(cudaEventSynchronize(F->told_ev));
+            else if ((rc = read_dev(Q.flags + n, &groups, st))) return rc;
+            if (F->told) groups = *(volatile uint32_t *)F->told;
             given_up = groups == 0;
             if (given_up) return FILTER_OK;
         }

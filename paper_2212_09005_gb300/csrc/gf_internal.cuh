@@ -516,6 +516,10 @@ struct filter {
     TcfState tcf;
     GqfState gqf;
     int device = 0;
+    // GQF removes: a word of host memory that a merge's first launch writes the
+    // number of groups to, and the event after it (members of groups have none)
+    uint32_t *told = nullptr;
+    cudaEvent_t told_ev = nullptr;
 };
 
 // A group of filters of one kind sharing one allocation and one set of
