@@ -67,6 +67,7 @@ struct MergeArgs {
     const uint32_t *tlo;     // first group of each tile,
     const uint32_t *thi;     // and the end of its groups
     uint64_t m_limit;        // use groups [0, min(m, m_limit))
+    uint64_t least;          // nothing is merged with fewer groups (0: always)
     uint32_t *removed;       // delete: copies removed per group
     unsigned long long *ts;  // look-back state: [0] tile counter, then one status word per tile
     DevCounters *ctr;
@@ -1290,6 +1291,7 @@ __global__ void __launch_bounds__(MT, MERGE_CTAS) gqf_merge_kernel(const __grid_
 {
     __shared__ __align__(16) MergeShared<R> S;
     __shared__ unsigned s_tile;
+    if (a.least && *a.pm < a.least) return;
     if (threadIdx.x == 0) {
         s_tile = (unsigned)atomicAdd(&a.ts[0], 1ull);
         if (units && s_tile == 0) {
@@ -2384,9 +2386,9 @@ static void gqf_prepare(filter *F, const uint64_t *keys, uint64_t n, bool need_i
 
 // cstart: group g adds (or removes) cstart[g + 1] - cstart[g] copies
 // units: the groups' units where they were left in place (msd_groups)
-// tell: F->told has the number of groups after F->told_ev
+// tell: gqf_groups_told may be asked; least: nothing is merged with fewer groups
 static int gqf_merge(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m_limit, int del, int dry,
-                     cudaStream_t st, const MsdUnits *units = nullptr, bool tell = false)
+                     cudaStream_t st, const MsdUnits *units = nullptr, bool tell = false, uint64_t least = 0)
 {
     GqfState &Q = F->gqf;
     const int nb = Q.cur ^ 1;
@@ -2401,6 +2403,7 @@ static int gqf_merge(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m_l
     a.tlo = Q.tile_lo;
     a.thi = units ? Q.tile_lo + Q.ntiles : Q.tile_lo + 1;
     a.m_limit = m_limit;
+    a.least = least;
     a.removed = del ? Q.removed : nullptr;
     a.ts = Q.tile_state;
     a.ctr = F->ctr;
@@ -2424,7 +2427,7 @@ static int gqf_merge(filter *F, const uint32_t *cstart, uint64_t n, uint64_t m_l
         gf::TraceScope ts_("gqf_tile_ranges", Q.ntiles + 1, st);
         gqf_tile_ranges<<<g, 256, 0, st>>>(Q.ufp, Q.flags + n, m_limit, Q.N, Q.r, Q.ntiles, Q.tile_lo, clear);
     }
-    if (tell) GF_CUDA(cudaEventRecord(F->told_ev, st));
+    if (tell && F->told) GF_CUDA(cudaEventRecord(F->told_ev, st));
     {
         gf::TraceScope ts_("gqf_merge_kernel", 0, st, true);
         if (Q.r == 8) gqf_merge_kernel<8><<<(unsigned)Q.ntiles, MT, 0, st>>>(a, ts_.units());
@@ -2544,24 +2547,42 @@ __global__ void gqf_units_list(const uint64_t *__restrict__ ufp, const uint32_t 
     if (u == (1u << units.k) - 1 && lane == 0) lstart[o + c] = n;
 }
 
+// the number of groups, which the launches before the last merge have counted;
+// that merge goes on meanwhile (2^17 keys removed from 2^20 slots 84 us without
+// asking, 104 with the number read back after the merge, 85 so)
+static int gqf_groups_told(filter *F, uint64_t n, uint64_t &m, cudaStream_t st)
+{
+    uint32_t groups = 0;
+    if (F->told) {
+        GF_CUDA(cudaEventSynchronize(F->told_ev));
+        groups = *(volatile uint32_t *)F->told;
+    } else {
+        const int rc = read_dev(F->gqf.flags + n, &groups, st);
+        if (rc) return rc;
+    }
+    m = groups;
+    return FILTER_OK;
+}
+
 // Groups left in units are bound for the merge, by the number of their keys. A
-// batch of few distinct keys goes in place all the same, its groups put into one
-// list. Not below 2^24 slots, where a merge takes no longer. Copies of 1000 keys,
-// an insert and a remove in us, merged / in place: 2^24 slots, 2^19 keys 290 + 262
-// / 283 + 135, 2^24 keys 571 + 543 / 562 + 414; 2^25, 2^21 556 + 527 / 304 + 196;
-// 2^26, 2^23 1012 + 990 / 358 + 271; 2^28, 2^26 4010 + 3952 / 1176 + 1130. A bound
-// that the caller set holds at all sizes. m becomes the number of groups when it
-// was read (0: the units were given up).
-static int gqf_units_in_place(filter *F, uint64_t n, const MsdUnits &units, uint64_t &m, bool &in_units, cudaStream_t st)
+// batch of few distinct keys goes in place all the same: the merge is enqueued at
+// once, does nothing for so few groups, and they are put into one list. Not below
+// 2^24 slots, where a merge takes no longer. Copies of 1000 keys, an insert and a
+// remove in us, merged / in place: 2^24 slots, 2^19 keys 290 + 262 / 167 + 129, 2^24
+// keys 571 + 543 / 451 + 408; 2^25, 2^21 556 + 527 / 258 + 193; 2^26, 2^23 1012 +
+// 990 / 359 + 289; 2^28, 2^26 4010 + 3952 / 1260 + 1220. A bound that the caller
+// set holds at all sizes. m: the number of groups (0: the units were given up);
+// merged: they were.
+static int gqf_merge_units(filter *F, uint64_t n, const MsdUnits &units, int del, uint64_t &m, bool &merged, cudaStream_t st)
 {
     GqfState &Q = F->gqf;
-    if (Q.merge_only || (!F->tune.gqf_region_groups && Q.N < (1ull << 24))) return FILTER_OK;
-    uint32_t groups = 0;
-    const int rc = read_dev(Q.flags + n, &groups, st);
-    if (rc) return rc;
-    m = groups;
-    if (m == 0 || m > gqf_in_place_most(F->tune, Q.N)) return FILTER_OK;
-    // the sort's buffers are free again; the ranges are not found yet
+    const bool few = !Q.merge_only && (F->tune.gqf_region_groups || Q.N >= (1ull << 24));
+    const uint64_t most = few ? gqf_in_place_most(F->tune, Q.N) : 0;
+    int rc = gqf_merge(F, Q.ustart, n, ~0ull, del, 0, st, &units, true, most + 1);
+    if (rc || (rc = gqf_groups_told(F, n, m, st))) return rc;
+    merged = m > most;
+    if (merged || m == 0) return FILTER_OK;
+    // the sort's buffers are free again, and the ranges are found anew
     uint32_t *first = Q.tile_lo;
     exclusive_scan_u32(units.distinct, first, 1ull << units.k, F->scan_tmp, F->ctr, st);
     {
@@ -2571,7 +2592,6 @@ static int gqf_units_in_place(filter *F, uint64_t n, const MsdUnits &units, uint
     }
     GF_CUDA(cudaMemcpyAsync(Q.ufp, Q.fp_a, m * 8, cudaMemcpyDeviceToDevice, st));
     GF_CUDA(cudaMemcpyAsync(Q.ustart, Q.idx_a, (m + 1) * 4, cudaMemcpyDeviceToDevice, st));
-    in_units = false;
     return FILTER_OK;
 }
 
@@ -2694,8 +2714,9 @@ static int gqf_insert_by(filter *F, const uint64_t *keys, const uint32_t *counts
     // small batches: in place, region by region; larger ones: the merge. The
     // keys bound the groups, whose number is read back only when that decides.
     uint64_t m = n;
-    if (in_units && (rc = gqf_units_in_place(F, n, units, m, in_units, st))) return rc;
-    if (!in_units && m) {
+    bool merged = false;
+    if (in_units && (rc = gqf_merge_units(F, n, units, 0, m, merged, st))) return rc;
+    if (!merged && m) {
         bool in_place = false;
         if ((rc = gqf_goes_in_place(F, n, n <= GQF_SMALL, m, in_place, st))) return rc;
         bool done = false;
@@ -2707,8 +2728,7 @@ static int gqf_insert_by(filter *F, const uint64_t *keys, const uint32_t *counts
     }
     given_up = m == 0;
     if (given_up) return FILTER_OK;
-    rc = gqf_merge(F, cstart, n, ~0ull, 0, 0, st, in_units ? &units : nullptr);
-    if (rc) return rc;
+    if (!merged && (rc = gqf_merge(F, cstart, n, ~0ull, 0, 0, st))) return rc;
     Precheck pc{};
     if ((rc = read_dev(reinterpret_cast<const Precheck *>(&F->ctr->overflow), &pc, st))) return rc;
     given_up = pc.groups == 0;
@@ -2717,7 +2737,7 @@ static int gqf_insert_by(filter *F, const uint64_t *keys, const uint32_t *counts
     uint64_t m_keep = ~0ull;
     if (ovf) {
         // one list, whose prefixes are tried, with the indices of its keys
-        if (in_units || (status && !need_idx)) gqf_prepare(F, keys, n, status != nullptr, true, st, &sidx);
+        if (merged || (status && !need_idx)) gqf_prepare(F, keys, n, status != nullptr, true, st, &sidx);
         // keep the longest prefix of the sorted groups that fits (dry runs)
         uint32_t m = 0;
         if ((rc = read_dev(Q.flags + n, &m, st))) return rc;
@@ -2770,9 +2790,9 @@ static int gqf_remove_by(filter *F, const uint64_t *keys, uint64_t n, uint8_t *s
     int rc = FILTER_OK;
     // small batches: in place, cluster by cluster; large ones: full merge
     uint64_t m = n;  // at least the number of groups
-    bool in_place = false;
-    if (in_units && (rc = gqf_units_in_place(F, n, units, m, in_units, st))) return rc;
-    if (!in_units && m && (rc = gqf_goes_in_place(F, n, n <= GQF_SMALL, m, in_place, st))) return rc;
+    bool in_place = false, merged = false;
+    if (in_units && (rc = gqf_merge_units(F, n, units, 1, m, merged, st))) return rc;
+    if (!merged && m && (rc = gqf_goes_in_place(F, n, n <= GQF_SMALL, m, in_place, st))) return rc;
     given_up = m == 0;
     if (given_up) return FILTER_OK;
     bool done = false;
@@ -2821,19 +2841,12 @@ static int gqf_remove_by(filter *F, const uint64_t *keys, uint64_t n, uint8_t *s
         }
     }
     if (!done) {
-        // Sorted by units, and the groups not read yet: their number comes while the
-        // merge runs (2^17 keys removed from 2^20 slots 84 us without asking, 104
-        // with the number read back after the merge, 85 so).
-        const bool ask = !status && !by_digits && n > GQF_SMALL && m == n;
-        if ((rc = gqf_merge(F, Q.ustart, n, ~0ull, 1, 0, st, in_units ? &units : nullptr, ask && F->told))) return rc;
-        if (ask) {
-            uint32_t groups = 0;
-            if (F->told) GF_CUDA(cudaEventSynchronize(F->told_ev));
-            else if ((rc = read_dev(Q.flags + n, &groups, st))) return rc;
-            if (F->told) groups = *(volatile uint32_t *)F->told;
-            given_up = groups == 0;
-            if (given_up) return FILTER_OK;
-        }
+        // sorted by units, and the number of groups not known yet?
+        const bool ask = !merged && !status && !by_digits && n > GQF_SMALL && m == n;
+        if (!merged && (rc = gqf_merge(F, Q.ustart, n, ~0ull, 1, 0, st, nullptr, ask))) return rc;
+        if (ask && (rc = gqf_groups_told(F, n, m, st))) return rc;
+        given_up = m == 0;
+        if (given_up) return FILTER_OK;
         Q.cur ^= 1;
     }
     if (status) {
@@ -3285,6 +3298,7 @@ int gqf_group_setup(filter_group *GR, const filter_config *cfgs, uint64_t &bytes
                 a.tlo = Q.tile_lo + tile0[m];
                 a.thi = a.tlo + 1;
                 a.m_limit = ~0ull;
+                a.least = 0;
                 a.removed = del ? Q.removed : nullptr;
                 a.ts = Q.tile_state + tile0[m];
                 a.ctr = GR->mctr + m;
