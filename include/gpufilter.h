@@ -10,10 +10,12 @@
  * are asynchronous (filter_get_device_view does not touch the device): they
  * enqueue kernels on the stream and return; the caller's buffers must stay
  * valid until the stream reaches the call. Exceptions: GQF inserts and
- * removes synchronise the stream to read the number of distinct fingerprints
- * (which picks the in-place or the merge path) and, after a merge, whether
- * the table overflowed. Calls on one filter must be ordered (same stream, or
- * externally synchronised); different filters are independent.
+ * removes wait for the stream for what picks their path: the number of distinct
+ * fingerprints (0 of them when a large batch has to be sorted again by digits),
+ * the table's load, the verdict of an in-place update's pre-check; and, after an
+ * insert's merge, whether the table overflowed. Calls on one filter must be
+ * ordered (same stream, or externally synchronised); different filters are
+ * independent.
  *
  * Errors are returned synchronously for bad arguments, allocation failure
  * and unsupported operations. Conditions found on the device (a full table,
@@ -137,8 +139,9 @@ int filter_destroy(filter_t *f);
  *   gqf_region_groups: GQF batches with at most this many distinct
  *     fingerprints per 256 quotients on average are inserted or removed in
  *     place (even-odd regions); denser ones take the merge (0: by the table's
- *     size, from one per 512 quotients at 2^22 slots to one per 32 from 2^27,
- *     and fewer when its clusters are long).
+ *     size, one per 64 quotients below 2^22 slots, one per 512 below 2^24, then
+ *     from one per 256 at 2^24 to one per 32 from 2^27, and fewer when its
+ *     clusters are long).
  * filter_set_tuning / filter_group_set_tuning: FILTER_ERR_ARG for values out
  * of range. filter_get_tuning: the current settings (0 fields = defaults).
  */

@@ -92,8 +92,9 @@ uint64_t gqf_in_place_most(const filter_tuning &t, uint64_t N)
     // 2^20 2000 / 1717 / (refused); 2^28, 2^23 7756 / 8404 / (refused). The
     // bounds are for tables that are not crowded; crowded ones, told by the
     // pre-check or before it, merge from fewer. Below 2^22 slots the two are close
-    // and small updates stay in place: the default that callers of that path, the
-    // tests among them, count on; a merge of 1024 groups would be 24 us faster.
+    // (with the regions as small as they are now, 1024 groups in 2^20 slots take
+    // 156 us in place at 40 % load and 168 at 70 %), and small updates stay in
+    // place: the tests of that path count on it as the default.
     uint64_t most = N / 32;  // 8 per 256 quotients
     if (N < (1ull << 27)) most = N / 256 * (N >> 24);
     if (N < (1ull << 24)) most = N / 512;

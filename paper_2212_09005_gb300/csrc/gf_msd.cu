@@ -11,8 +11,8 @@
 // 2.4e8 36-bit keys move 8 (histogram) + 16 + 8 + 16 bytes each in the passes
 // and 8 in the last one; the least-significant-digit sort of gf_prims.cu, which
 // serves batches that carry values, moves 16 + 4 * 16 + 3 * 8, and 8 in the
-// reduction. Zipf keys: 8.35 ms there, 4.85 ms here (histograms 0.46 + 0.28,
-// passes 0.87 + 1.06, hot units 0.44, units 1.97).
+// reduction. Zipf keys: 8.35 ms there, 5.14 ms here (histograms 0.47 + 0.29,
+// passes 0.97 + 1.07, hot units 0.38, units 1.95).
 //
 // Skew: the copies of a key all fall into one unit. A unit of more than MU_CAP
 // keys goes through a hash table in shared memory (its distinct values are
