@@ -571,6 +571,7 @@ struct PhaseDst {
     const uint32_t *dlist;   // sparse: touched destinations
     const uint64_t *seg;     // sparse: start << 32 | count
     const unsigned *nlist;   // sparse: number of touched destinations
+    uint64_t nrec = 0;       // sparse: number of candidates (0: not told)
 };
 
 __device__ __forceinline__ uint64_t phase_count(const PhaseDst &P, uint64_t dense_n)
@@ -590,6 +591,60 @@ __device__ __forceinline__ uint64_t phase_dst(const PhaseDst &P, uint64_t j, uin
     s = P.off[j];
     e = P.off[j + 1];
     return j;
+}
+
+// Touched destinations of many candidates each (copies of a key) take long, and
+// lanes of a warp wait for one another: such a phase's destinations go round the
+// warps first, then to their lanes. 2^18 keys, a hundred copies of each, on 2^20
+// blocks, an insert and a remove: 1.32 and 3.55 ms with a warp's lanes side by
+// side, 0.51 and 0.58 so.
+__device__ __forceinline__ bool phase_spread(const PhaseDst &P, uint64_t nd) { return P.nrec >= 8 * nd && P.nrec; }
+
+// what this thread takes in the round from t0 on
+__device__ __forceinline__ uint64_t phase_pos(bool spread, uint64_t t0)
+{
+    const uint64_t warps = (uint64_t)gridDim.x * (TPB / 32);
+    const uint64_t w = blockIdx.x * (uint64_t)(TPB / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    return t0 + (spread ? lane * warps + w : w * 32 + lane);
+}
+
+// f(record) for each of [s, e), four loads in flight (one by one, each load's
+// latency counts: 32768 copies of one key, a remove 236 ms, 131 so)
+template <bool MANY, class Fn>
+__device__ __forceinline__ void each_record(const uint64_t *__restrict__ rec, uint32_t s, uint32_t e, Fn f)
+{
+    if constexpr (MANY) {
+        for (uint32_t q = s; q < e; q += 4) {
+            uint64_t r[4];
+#pragma unroll
+            for (uint32_t u = 0; u < 4; u++) r[u] = q + u < e ? rec[q + u] : 0ull;
+#pragma unroll
+            for (uint32_t u = 0; u < 4; u++)
+                if (q + u < e) f(r[u]);
+        }
+    } else {
+        for (uint32_t q = s; q < e; q++) f(rec[q]);
+    }
+}
+
+// the same for a bucket's candidates: f(entry, index). MANY: one at a time where
+// they are in shared memory, and few.
+template <bool MANY, class Entry, class Index, class Fn>
+__device__ __forceinline__ void each_candidate(uint32_t cnt, Entry entry, Index index, Fn f)
+{
+    constexpr uint32_t U = MANY ? 4 : 1;
+    for (uint32_t q = 0; q < cnt; q += U) {
+        uint64_t ee[U];
+        uint32_t ii[U];
+#pragma unroll
+        for (uint32_t u = 0; u < U; u++) {
+            ee[u] = q + u < cnt ? entry(q + u) : 0ull;
+            ii[u] = q + u < cnt ? index(q + u) : 0u;
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < U; u++)
+            if (q + u < cnt) f(ee[u], ii[u]);
+    }
 }
 
 // A warp reserves room for all its lanes' entries of a pending list with one
@@ -674,10 +729,81 @@ struct RejSink {
     }
 };
 
+// Candidates of one block or bucket above which a warp takes an insert's step
+// (copies of one key): 32768 of them in a batch of 2^18 took one thread 36 ms, a
+// warp 3.7.
+static constexpr uint32_t DST_HOT = 512;
+
+// the smallest (v, i) over the warp
+__device__ __forceinline__ void warp_min_pair(uint64_t &v, uint32_t &i)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const uint64_t y = __shfl_xor_sync(0xffffffffu, v, o);
+        const uint32_t k = __shfl_xor_sync(0xffffffffu, i, o);
+        if (y < v || (y == v && k < i)) {
+            v = y;
+            i = k;
+        }
+    }
+}
+
+// the insert step of block b with records [s, e) (the whole warp calls it): the
+// next smallest record once per free slot, then the rest into the pending list
+template <int F>
+__device__ __noinline__ void hot_block_insert(uint8_t *blocks, uint8_t *fill, uint64_t b, uint32_t f0, uint32_t cap,
+                                              const uint64_t *rec, uint32_t s, uint32_t e, int phase, uint32_t *pend32,
+                                              uint64_t *pend64, unsigned *npend, uint64_t nb, uint32_t vbits,
+                                              const TcfPrep prep)
+{
+    const uint32_t lane = threadIdx.x & 31, k = cap > f0 ? min(e - s, cap - f0) : 0u;
+    uint64_t thr = 0;
+    if (k) {
+        Blk<F> blk;
+        blk.load(blocks, b);
+        for (uint32_t j = 0; j < k; j++) {
+            uint64_t m = ~0ull;
+            uint32_t none = 0;
+#pragma unroll 4
+            for (uint32_t q = s + lane; q < e; q += 32) {
+                const uint64_t r = rec[q];
+                if ((j == 0 || r > thr) && r < m) m = r;
+            }
+            warp_min_pair(m, none);
+            thr = m;
+            uint64_t r8[8] = {thr, 0, 0, 0, 0, 0, 0, 0};
+            blk.merge_new(f0 + j, 1, r8);
+        }
+        if (lane == 0) {
+            blk.store(blocks, b);
+            fill[b] = (uint8_t)(f0 + k);
+        }
+    }
+    for (uint32_t q0 = s; q0 < e; q0 += 32) {
+        const uint64_t r = q0 + lane < e ? rec[q0 + lane] : 0ull;
+        const bool left = q0 + lane < e && !(k > 0 && r <= thr);
+        const unsigned lefts = __ballot_sync(0xffffffffu, left);
+        uint32_t base = 0;
+        if (lane == 0 && lefts) base = atomicAdd(npend, __popc(lefts));
+        base = __shfl_sync(0xffffffffu, base, 0) + __popc(lefts & ((1u << lane) - 1u));
+        if (!left) continue;
+        const uint32_t i = (uint32_t)r;
+        if (phase == 1) {  // the other block of the pair
+            const uint64_t alt = prep.bt ? (prep.bt[i] >> 32) + prep.b2[i] - b : b ^ tcf_g((uint32_t)(r >> 32) >> vbits, nb);
+            pend64[base] = (alt << 32) | i;
+        } else {
+            pend32[base] = i;
+        }
+    }
+    __syncwarp();
+}
+
 // The grid-stride loops of the per-block kernels step whole warps, so that
 // every lane reaches the sink's reserve in every iteration and its flush
 // after the last one.
-template <int F>
+// COOP: as the cooperative launch takes them, hot blocks by a warp and a phase's
+// destinations spread (the kernel over every block keeps its 48 registers without).
+template <int F, bool COOP>
 __device__ __forceinline__ void tcf_block_insert_body(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
                                                       const uint64_t *__restrict__ rec, int phase, uint32_t cap,
                                                       uint32_t *pend32, uint64_t *pend64, unsigned *npend,
@@ -689,8 +815,9 @@ __device__ __forceinline__ void tcf_block_insert_body(TcfGeom G, uint8_t *blocks
     const uint64_t nd = phase_count(P, G.nb);
     if (P.dlist) note_units(units, nd);  // units: blocks with candidates
     const uint64_t stride = (uint64_t)gridDim.x * TPB;
-    for (uint64_t j0 = blockIdx.x * (uint64_t)TPB + (threadIdx.x & ~31u); j0 < nd; j0 += stride) {
-        const uint64_t j = j0 + (threadIdx.x & 31);
+    const bool spread = COOP && phase_spread(P, nd);
+    for (uint64_t t0 = COOP ? 0 : blockIdx.x * (uint64_t)TPB + (threadIdx.x & ~31u); t0 < nd; t0 += stride) {
+        const uint64_t j = COOP ? phase_pos(spread, t0) : t0 + (threadIdx.x & 31);
         uint32_t s = 0, e = 0, k = 0, f0 = 0;
         uint64_t b = 0, thr = 0;  // records <= thr are accepted
         if (j < nd) {
@@ -700,6 +827,13 @@ __device__ __forceinline__ void tcf_block_insert_body(TcfGeom G, uint8_t *blocks
         if (units && !P.dlist) {
             const unsigned t = __ballot_sync(0xffffffffu, s != e);
             if ((threadIdx.x & 31) == 0 && t) atomicAdd(units, (unsigned long long)__popc(t));
+        }
+        for (unsigned hot = COOP ? __ballot_sync(0xffffffffu, e - s > DST_HOT) : 0u; hot; hot &= hot - 1) {
+            const int src = __ffs(hot) - 1;
+            hot_block_insert<F>(blocks, fill, __shfl_sync(0xffffffffu, b, src), __shfl_sync(0xffffffffu, f0, src), cap, rec,
+                                __shfl_sync(0xffffffffu, s, src), __shfl_sync(0xffffffffu, e, src), phase, pend32, pend64,
+                                npend, G.nb, G.vbits, prep);
+            if ((int)(threadIdx.x & 31) == src) s = e;
         }
         if (j < nd) {
             if (s != e) {
@@ -725,7 +859,7 @@ __device__ __forceinline__ void tcf_block_insert_body(TcfGeom G, uint8_t *blocks
                     blk.load(blocks, b);
                     uint64_t a[MAXSEL];
                     int have = 0;
-                    for (uint32_t q = s; q < e; q++) have = topk_push(a, have, (int)k, rec[q]);
+                    each_record<COOP>(rec, s, e, [&](uint64_t r) { have = topk_push(a, have, (int)k, r); });
                     thr = a[k - 1];
                     uint32_t t_out[B];
                     int ia = 0, ib = 0;
@@ -753,9 +887,8 @@ __device__ __forceinline__ void tcf_block_insert_body(TcfGeom G, uint8_t *blocks
         bool direct;
         uint32_t slot = sink.reserve(nrej, direct);
         if (nrej == 0) continue;
-        for (uint32_t q = s; q < e; q++) {
-            const uint64_t r = rec[q];
-            if (k > 0 && r <= thr) continue;
+        auto pass_on = [&](uint64_t r) {
+            if (k > 0 && r <= thr) return;
             const uint32_t i = (uint32_t)r;
             if (phase == 1) {
                 // the other block of the pair: b1 + b2 - b
@@ -765,7 +898,9 @@ __device__ __forceinline__ void tcf_block_insert_body(TcfGeom G, uint8_t *blocks
             } else {
                 sink.put(direct, slot, i);
             }
-        }
+        };
+        if (COOP && e - s > 8) each_record<COOP>(rec, s, e, pass_on);
+        else each_record<false>(rec, s, e, pass_on);
     }
     sink.flush();
 }
@@ -778,12 +913,12 @@ __global__ void __launch_bounds__(TPB) tcf_block_insert(TcfGeom G, uint8_t *bloc
                                                         unsigned long long *units)
 {
     if (gate && !*gate) return;
-    tcf_block_insert_body<F>(G, blocks, fill, P, rec, phase, cap, pend32, pend64, npend, prep, units);
+    tcf_block_insert_body<F, false>(G, blocks, fill, P, rec, phase, cap, pend32, pend64, npend, prep, units);
 }
 
 // One backing bucket q: cnt candidates (entry(j), index(j)) taken in (entry,
 // index) order while there is room; the rest are FULL
-template <class Entry, class Index>
+template <bool MANY, class Entry, class Index>
 __device__ __forceinline__ void bucket_insert_step(uint64_t *bk, uint64_t q, uint32_t cnt, Entry entry, Index index,
                                                    uint8_t *status, DevCounters *ctr)
 {
@@ -802,16 +937,14 @@ __device__ __forceinline__ void bucket_insert_step(uint64_t *bk, uint64_t q, uin
     for (uint32_t m = 0; m < k; m++) {
         uint64_t be = ~0ull;
         uint32_t bi = 0xffffffffu;
-        for (uint32_t j = 0; j < cnt; j++) {
-            uint64_t ee = entry(j);
-            uint32_t ii = index(j);
+        each_candidate<MANY>(cnt, entry, index, [&](uint64_t ee, uint32_t ii) {
             bool after = !have_prev || ee > pe || (ee == pe && ii > pi);
             bool better = ee < be || (ee == be && ii < bi);
             if (after && better) {
                 be = ee;
                 bi = ii;
             }
-        }
+        });
         acc_e[m] = be;
         pe = be;
         pi = bi;
@@ -831,22 +964,20 @@ __device__ __forceinline__ void bucket_insert_step(uint64_t *bk, uint64_t q, uin
     if (k > 0) atomicAdd(&ctr->backing, (unsigned long long)k);
     if (k < cnt) {
         // rejected: every pair after the k-th accepted one
-        for (uint32_t j = 0; j < cnt; j++) {
-            uint64_t ee = entry(j);
-            uint32_t ii = index(j);
+        each_candidate<MANY>(cnt, entry, index, [&](uint64_t ee, uint32_t ii) {
             bool acc = k > 0 && (ee < pe || (ee == pe && ii <= pi));
             if (!acc) {
                 if (status) status[ii] = FILTER_KEY_FULL;
                 atomicAdd(&ctr->failed, 1ull);
             }
-        }
+        });
         atomicOr(&ctr->status, ST_FULL);
     }
 }
 
 // One backing bucket q: per stored entry, the smallest batch indices among
 // the cnt candidates with that entry remove one copy each
-template <class Entry, class Index>
+template <bool MANY, class Entry, class Index>
 __device__ __forceinline__ void bucket_remove_step(const TcfGeom &G, uint64_t *bk, uint64_t q, uint32_t cnt, Entry entry,
                                                    Index index, uint8_t *status, DevCounters *ctr)
 {
@@ -873,8 +1004,9 @@ __device__ __forceinline__ void bucket_remove_step(const TcfGeom &G, uint64_t *b
     for (int d = 0; d < nd; d++) {
         uint64_t a[BK_W];
         int have = 0;
-        for (uint32_t j = 0; j < cnt; j++)
-            if (entry(j) == dv[d]) have = topk_push(a, have, (int)dc[d], (uint64_t)index(j));
+        each_candidate<MANY>(cnt, entry, index, [&](uint64_t v, uint32_t ii) {
+            if (v == dv[d]) have = topk_push(a, have, (int)dc[d], (uint64_t)ii);
+        });
         used[d] = (uint32_t)have;
         thr[d] = have ? (uint32_t)a[have - 1] : 0u;
     }
@@ -890,17 +1022,74 @@ __device__ __forceinline__ void bucket_remove_step(const TcfGeom &G, uint64_t *b
         for (int j = 0; j < (int)BK_W; j++) bk[q * BK_W + j] = outv[j];
         atomicAdd(&ctr->backing, (unsigned long long)(-(long long)removed));
     }
-    for (uint32_t j = 0; j < cnt; j++) {
-        uint64_t v = entry(j);
-        uint32_t ii = index(j);
+    if (!status) return;
+    each_candidate<MANY>(cnt, entry, index, [&](uint64_t v, uint32_t ii) {
         bool matched = false;
         for (int d = 0; d < nd; d++)
             if (dv[d] == v && used[d] > 0 && ii <= thr[d]) matched = true;
-        if (!matched && status) status[ii] = FILTER_KEY_NOT_FOUND;
+        if (!matched) status[ii] = FILTER_KEY_NOT_FOUND;
+    });
+}
+
+// the insert step of bucket q with cnt candidates, by the whole warp
+__device__ __noinline__ void hot_bucket_insert(uint64_t *bk, uint64_t q, uint32_t cnt, const uint64_t *rec,
+                                               const uint32_t *recI, uint8_t *status, DevCounters *ctr)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    uint64_t cur[BK_W], pe = 0;
+    uint32_t used = 0, pi = 0;
+#pragma unroll
+    for (int j = 0; j < (int)BK_W; j++) {
+        cur[j] = bk[q * BK_W + j];
+        used += cur[j] != 0;
     }
+    __syncwarp();
+    const uint32_t k = BK_W - used;  // (fewer than the candidates)
+    for (uint32_t m = 0; m < k; m++) {
+        uint64_t be = ~0ull;
+        uint32_t bi = 0xffffffffu;
+#pragma unroll 4
+        for (uint32_t j = lane; j < cnt; j += 32) {
+            const uint64_t ee = rec[j];
+            const uint32_t ii = recI[j];
+            if ((m == 0 || ee > pe || (ee == pe && ii > pi)) && (ee < be || (ee == be && ii < bi))) {
+                be = ee;
+                bi = ii;
+            }
+        }
+        warp_min_pair(be, bi);
+        pe = be;
+        pi = bi;
+        // into the sorted entries, free ones (0) last
+        uint64_t v = be;
+#pragma unroll
+        for (int j = 0; j < (int)BK_W; j++) {
+            const uint64_t x = cur[j];
+            if (v && (x == 0 || v < x)) {
+                cur[j] = v;
+                v = x;
+            }
+        }
+    }
+    if (lane == 0 && k) {
+#pragma unroll
+        for (int j = 0; j < (int)BK_W; j++) bk[q * BK_W + j] = cur[j];
+        atomicAdd(&ctr->backing, (unsigned long long)k);
+    }
+    for (uint32_t j = lane; j < cnt; j += 32) {
+        const uint64_t ee = rec[j];
+        const uint32_t ii = recI[j];
+        if (!(k > 0 && (ee < pe || (ee == pe && ii <= pi))) && status) status[ii] = FILTER_KEY_FULL;
+    }
+    if (lane == 0) {
+        atomicAdd(&ctr->failed, (unsigned long long)(cnt - k));
+        atomicOr(&ctr->status, ST_FULL);
+    }
+    __syncwarp();
 }
 
 // backing buckets of a phase: candidates (entry in rec, index in recI)
+template <bool HOT>
 __device__ __forceinline__ void tcf_bucket_insert_body(TcfGeom G, uint64_t *bk, PhaseDst P,
                                                        const uint64_t *__restrict__ rec,
                                                        const uint32_t *__restrict__ recI, uint8_t *status,
@@ -908,11 +1097,20 @@ __device__ __forceinline__ void tcf_bucket_insert_body(TcfGeom G, uint64_t *bk, 
 {
     const uint64_t nd = phase_count(P, G.nbk);
     note_units(units, nd);  // units: buckets with candidates
-    for (uint64_t j = blockIdx.x * (uint64_t)TPB + threadIdx.x; j < nd; j += (uint64_t)gridDim.x * TPB) {
-        uint32_t s, e;
-        const uint64_t q = phase_dst(P, j, s, e);
+    const bool spread = phase_spread(P, nd);
+    for (uint64_t t0 = 0; t0 < nd; t0 += (uint64_t)gridDim.x * TPB) {
+        const uint64_t j = phase_pos(spread, t0);
+        uint32_t s = 0, e = 0;
+        uint64_t q = 0;
+        if (j < nd) q = phase_dst(P, j, s, e);
+        for (unsigned hot = HOT ? __ballot_sync(0xffffffffu, e - s > DST_HOT) : 0u; hot; hot &= hot - 1) {
+            const int src = __ffs(hot) - 1;
+            const uint32_t hs = __shfl_sync(0xffffffffu, s, src), he = __shfl_sync(0xffffffffu, e, src);
+            hot_bucket_insert(bk, __shfl_sync(0xffffffffu, q, src), he - hs, rec + hs, recI + hs, status, ctr);
+            if ((int)(threadIdx.x & 31) == src) s = e;
+        }
         if (s == e) continue;
-        bucket_insert_step(bk, q, e - s, [&](uint32_t i) { return rec[s + i]; }, [&](uint32_t i) { return recI[s + i]; },
+        bucket_insert_step<true>(bk, q, e - s, [&](uint32_t i) { return rec[s + i]; }, [&](uint32_t i) { return recI[s + i]; },
                            status, ctr);
     }
 }
@@ -922,14 +1120,14 @@ __global__ void __launch_bounds__(TPB) tcf_bucket_insert(TcfGeom G, uint64_t *bk
                                                          const uint32_t *__restrict__ recI, uint8_t *status,
                                                          DevCounters *ctr, unsigned long long *units)
 {
-    tcf_bucket_insert_body(G, bk, P, rec, recI, status, ctr, units);
+    tcf_bucket_insert_body<false>(G, bk, P, rec, recI, status, ctr, units);
 }
 
 // ---------------------------------------------------------------------------
 // Bulk delete: per-block matching. For each tag present c times in the block,
 // the c smallest (tag, index) candidates with that tag remove one copy each.
 // ---------------------------------------------------------------------------
-template <int F>
+template <int F, bool COOP>
 __device__ __forceinline__ void tcf_block_remove_body(TcfGeom G, uint8_t *blocks, uint8_t *fill, PhaseDst P,
                                                       const uint64_t *__restrict__ rec, uint32_t *pend32,
                                                       unsigned *npend, unsigned long long *units)
@@ -941,8 +1139,9 @@ __device__ __forceinline__ void tcf_block_remove_body(TcfGeom G, uint8_t *blocks
     if (P.dlist) note_units(units, nd);  // units: blocks with candidates
     const uint32_t lm = Blk<F>::lane_mask(G.vmask);
     const uint64_t stride = (uint64_t)gridDim.x * TPB;
-    for (uint64_t j0 = blockIdx.x * (uint64_t)TPB + (threadIdx.x & ~31u); j0 < nd; j0 += stride) {
-        const uint64_t j = j0 + (threadIdx.x & 31);
+    const bool spread = COOP && phase_spread(P, nd);
+    for (uint64_t t0 = COOP ? 0 : blockIdx.x * (uint64_t)TPB + (threadIdx.x & ~31u); t0 < nd; t0 += stride) {
+        const uint64_t j = COOP ? phase_pos(spread, t0) : t0 + (threadIdx.x & 31);
         uint32_t s = 0, e = 0, nunm = 0, unm = 0;
         bool fast = false;
         uint64_t r8[8];  // fast path: the candidates, sorted
@@ -1011,10 +1210,9 @@ __device__ __forceinline__ void tcf_block_remove_body(TcfGeom G, uint8_t *blocks
                         uint64_t a[MAXSEL];
                         int have = 0;
                         uint64_t lo = (uint64_t)dt[d] << 32, hi = lo | 0xffffffffull;
-                        for (uint32_t q = s; q < e; q++) {
-                            uint64_t r = rec[q];
+                        each_record<COOP>(rec, s, e, [&](uint64_t r) {
                             if (r >= lo && r <= hi) have = topk_push(a, have, (int)dc[d], r);
-                        }
+                        });
                         used[d] = (uint32_t)have;
                         thr[d] = have ? a[have - 1] : 0;
                     }
@@ -1045,14 +1243,13 @@ __device__ __forceinline__ void tcf_block_remove_body(TcfGeom G, uint8_t *blocks
             for (int q = 0; q < 8; q++)
                 if ((unm >> q) & 1u) sink.put(direct, slot, (uint32_t)r8[q]);
         } else {
-            for (uint32_t q = s; q < e; q++) {
-                const uint64_t r = rec[q];
+            each_record<COOP>(rec, s, e, [&](uint64_t r) {
                 const uint32_t t = (uint32_t)(r >> 32);
                 bool matched = false;
                 for (int d = 0; d < ndt; d++)
                     if (dt[d] == t && used[d] > 0 && r <= thr[d]) matched = true;
                 if (!matched) sink.put(direct, slot, (uint32_t)r);
-            }
+            });
         }
     }
     sink.flush();
@@ -1065,7 +1262,7 @@ __global__ void __launch_bounds__(TPB) tcf_block_remove(TcfGeom G, uint8_t *bloc
                                                         unsigned long long *units)
 {
     if (gate && !*gate) return;
-    tcf_block_remove_body<F>(G, blocks, fill, P, rec, pend32, npend, units);
+    tcf_block_remove_body<F, false>(G, blocks, fill, P, rec, pend32, npend, units);
 }
 
 // backing buckets of a remove
@@ -1076,11 +1273,14 @@ __device__ __forceinline__ void tcf_bucket_remove_body(TcfGeom G, uint64_t *bk, 
 {
     const uint64_t nd = phase_count(P, G.nbk);
     note_units(units, nd);  // units: buckets with candidates
-    for (uint64_t j = blockIdx.x * (uint64_t)TPB + threadIdx.x; j < nd; j += (uint64_t)gridDim.x * TPB) {
+    const bool spread = phase_spread(P, nd);
+    for (uint64_t t0 = 0; t0 < nd; t0 += (uint64_t)gridDim.x * TPB) {
+        const uint64_t j = phase_pos(spread, t0);
+        if (j >= nd) continue;
         uint32_t s, e;
         const uint64_t q = phase_dst(P, j, s, e);
         if (s == e) continue;
-        bucket_remove_step(G, bk, q, e - s, [&](uint32_t i) { return rec[s + i]; },
+        bucket_remove_step<true>(G, bk, q, e - s, [&](uint32_t i) { return rec[s + i]; },
                            [&](uint32_t i) { return recI[s + i]; }, status, ctr);
     }
 }
@@ -1210,9 +1410,10 @@ __device__ __forceinline__ bool sparse_group(const SparseArgs &A, const void *pe
     DevCounters *c = A.ctr;
     const uint64_t m = SRC == SRC_KEYS ? A.n : (uint64_t)ld_now(npend);  // (the same in every CTA)
     if (m == 0) return false;
-    P = PhaseDst{nullptr, A.dlist, A.seg, &c->touched[slot]};
+    P = PhaseDst{nullptr, A.dlist, A.seg, &c->touched[slot], m};
     if (run.few || m <= SPARSE_FEW) {
         run.few = true;
+        P.nrec = 0;  // (the other CTAs' warps are gone)
         if (blockIdx.x != 0) return false;
         few_group<SRC, DST>(A, pend, (uint32_t)m, recI, &c->touched[slot]);
         __syncthreads();
@@ -1235,19 +1436,19 @@ __global__ void __launch_bounds__(TPB, 4) tcf_sparse_insert_coop(const SparseArg
     const bool uneven = A.uneven && ld_now(A.uneven), all = A.first || uneven;  // (the same in every CTA)
     if (A.first || (uneven && !A.first_done)) {
         if (!sparse_group<SRC_KEYS, DST_B1>(A, nullptr, nullptr, 0, nullptr, run, P)) return;
-        tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 0, A.G.tsc, A.pend0, nullptr, &np[0], A.prep, nullptr);
+        tcf_block_insert_body<F, true>(A.G, A.blocks, A.fill, P, A.rec, 0, A.G.tsc, A.pend0, nullptr, &np[0], A.prep, nullptr);
         if (!sparse_next(A, run)) return;
     }
     if (all || ld_now(&np[0]) <= A.unit_min) {
         if (!sparse_group<SRC_PEND_U32, DST_TARGET>(A, A.pend0, &np[0], 1, nullptr, run, P)) return;
-        tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 1, A.G.B, nullptr, A.pend1, &np[1], A.prep, nullptr);
+        tcf_block_insert_body<F, true>(A.G, A.blocks, A.fill, P, A.rec, 1, A.G.B, nullptr, A.pend1, &np[1], A.prep, nullptr);
         if (!sparse_next(A, run)) return;
         if (!sparse_group<SRC_PEND_U64, DST_ALT>(A, A.pend1, &np[1], 2, nullptr, run, P)) return;
-        tcf_block_insert_body<F>(A.G, A.blocks, A.fill, P, A.rec, 2, A.G.B, A.pend2, nullptr, &np[2], A.prep, nullptr);
+        tcf_block_insert_body<F, true>(A.G, A.blocks, A.fill, P, A.rec, 2, A.G.B, A.pend2, nullptr, &np[2], A.prep, nullptr);
         if (!sparse_next(A, run)) return;
     }
     if (!sparse_group<SRC_PEND_U32, DST_BUCKET>(A, A.pend2, &np[2], 3, A.pend0, run, P)) return;
-    tcf_bucket_insert_body(A.G, A.bk, P, A.rec, A.pend0, A.status, A.ctr, nullptr);
+    tcf_bucket_insert_body<true>(A.G, A.bk, P, A.rec, A.pend0, A.status, A.ctr, nullptr);
 }
 
 template <int F>
@@ -1259,12 +1460,12 @@ __global__ void __launch_bounds__(TPB, 4) tcf_sparse_remove_coop(const SparseArg
     const bool uneven = A.uneven && ld_now(A.uneven), all = A.first || uneven;  // (the same in every CTA)
     if (A.first || (uneven && !A.first_done)) {
         if (!sparse_group<SRC_KEYS, DST_B1>(A, nullptr, nullptr, 0, nullptr, run, P)) return;
-        tcf_block_remove_body<F>(A.G, A.blocks, A.fill, P, A.rec, A.pend0, &np[0], nullptr);
+        tcf_block_remove_body<F, true>(A.G, A.blocks, A.fill, P, A.rec, A.pend0, &np[0], nullptr);
         if (!sparse_next(A, run)) return;
     }
     if (all || ld_now(&np[0]) <= A.unit_min) {
         if (!sparse_group<SRC_PEND_U32, DST_B2>(A, A.pend0, &np[0], 1, nullptr, run, P)) return;
-        tcf_block_remove_body<F>(A.G, A.blocks, A.fill, P, A.rec, A.pend2, &np[2], nullptr);
+        tcf_block_remove_body<F, true>(A.G, A.blocks, A.fill, P, A.rec, A.pend2, &np[2], nullptr);
         if (!sparse_next(A, run)) return;
     }
     if (!sparse_group<SRC_PEND_U32, DST_BUCKET>(A, A.pend2, &np[2], 2, A.pend0, run, P)) return;
@@ -1390,8 +1591,8 @@ __global__ void __launch_bounds__(SM_T) tcf_small(const uint64_t *__restrict__ k
             const uint32_t x = index(q);
             return prep.bt ? prep.e[x] : tcf_entry(KeyInfo{b1[x], b2[x], slot[x]}, G.f);
         };
-        if (DEL) bucket_remove_step(G, bk, d, e - i, entry, index, status, ctr);
-        else bucket_insert_step(bk, d, e - i, entry, index, status, ctr);
+        if (DEL) bucket_remove_step<false>(G, bk, d, e - i, entry, index, status, ctr);
+        else bucket_insert_step<false>(bk, d, e - i, entry, index, status, ctr);
     }
 }
 
@@ -1410,7 +1611,12 @@ static constexpr int TU_T = 512;             // threads of a unit
 static constexpr uint32_t TU_CAP = 3072;     // candidates that a unit holds in shared memory
 static constexpr int TU_PER = TU_CAP / TU_T;
 static constexpr uint32_t TU_BBITS = 12, TU_BUCKETS = 1u << TU_BBITS;  // buckets they are grouped by: a block or a few
-static constexpr uint32_t TU_HOT = 64;       // candidates of one bucket above which the CTA takes them
+// Candidates of one bucket above which the CTA takes them, one bucket after
+// another: 20 us each, where a thread takes 0.2 us a candidate and other buckets go
+// beside it (42,000 keys with a hundred copies each on 2^22 blocks: 3.28 ms an
+// insert's step and 6.88 a remove's with 64, 0.33 and 0.69 so).
+static constexpr uint32_t TU_HOT = 512;
+static constexpr uint32_t TU_MANY = 16;  // and above which a remove skips the rest of a tag without copies left
 static uint64_t tcf_unit_words(uint64_t max_n);  // scratch words of calls of up to max_n keys
 static MsdScratch tu_scratch(uint32_t *base, uint64_t max_n);
 
@@ -1801,7 +2007,7 @@ __device__ __forceinline__ bool remove_tag16(uint32_t (&w)[8], uint32_t tt, uint
 // some do not fit. Remove: each candidate, smallest first, takes the first copy
 // of its tag. Those left are listed in S.left. Returns the algorithmic bytes
 // (64 per block changed, 32 per block only read, 2 per fill).
-template <int F, bool DEL, bool ONE>
+template <int F, bool DEL, bool ONE, bool MANY = false>
 __device__ __forceinline__ uint32_t tu_bucket(TuSmem &S, uint32_t s, uint32_t e, uint32_t lb, uint64_t b0,
                                               const TcfGeom &G, uint32_t tsh, uint32_t bsh, uint32_t smask,
                                               uint8_t *blocks, uint8_t *fill, uint32_t cap)
@@ -1894,6 +2100,16 @@ __device__ __forceinline__ uint32_t tu_bucket(TuSmem &S, uint32_t s, uint32_t e,
                 }
                 if (hit) {
                     removed++;
+                } else if constexpr (MANY) {  // no copy left: nor for the others of this tag
+                    uint64_t last = prev;
+                    for (uint32_t j = s; j < e; j++) {
+                        const uint64_t x = S.a[j];
+                        if (!mine(x) || x < prev || ((uint32_t)(x >> tsh) & smask) != tag) continue;
+                        S.left[atomicAdd(&S.nleft, 1u)] = (uint16_t)j;
+                        q += x != prev;
+                        last = x > last ? x : last;
+                    }
+                    prev = last;
                 } else {
                     uint32_t j = s;
                     while (S.a[j] != prev) j++;
@@ -1940,6 +2156,14 @@ struct TuStep {
     const unsigned *uneven;  // set: no phase goes by unit
     unsigned long long *units;
 };
+
+// a remove's steps of a bucket of many candidates
+template <int F, bool ONE>
+__device__ __noinline__ uint32_t tu_bucket_many(TuSmem &S, uint32_t s, uint32_t e, uint32_t lb, uint64_t b0, const TuStep &A)
+{
+    const uint32_t tsh = A.U.ibits, bsh = A.U.ibits + A.U.sbits, smask = (1u << A.U.sbits) - 1u;
+    return tu_bucket<F, true, ONE, true>(S, s, e, lb, b0, A.G, tsh, bsh, smask, A.blocks, A.fill, A.cap);
+}
 
 // the hot buckets in S.hot, by the whole CTA, block by block
 template <int F, bool DEL, int NEXT>
@@ -2008,6 +2232,7 @@ __device__ __noinline__ void tu_big_unit(TuSmem &S, const TuStep &A, uint32_t un
             for (uint32_t h = threadIdx.x; h < S.nhead; h += TU_T) {
                 const uint32_t bk = S.head[h], s = first[bk], e = first[bk + 1];
                 if (e - s > TU_HOT) S.hot[atomicAdd(&S.nhot, 1u)] = (uint16_t)bk;
+                else if (DEL && e - s > TU_MANY) tu_bucket_many<F, false>(S, s, e, bk, b0, A);
                 else tu_bucket<F, DEL, false>(S, s, e, bk, b0, A.G, tsh, bsh, smask, A.blocks, A.fill, A.cap);
             }
             __syncthreads();
@@ -2070,6 +2295,7 @@ __global__ void __launch_bounds__(TU_T, 3) tcf_unit_step(const __grid_constant__
         for (uint32_t h = threadIdx.x; h < heads; h += TU_T) {
             const uint32_t bk = S.head[h], s = first[bk], e = first[bk + 1];
             if (e - s > TU_HOT) S.hot[atomicAdd(&S.nhot, 1u)] = (uint16_t)bk;
+            else if (DEL && e - s > TU_MANY) bytes += tu_bucket_many<F, ONE>(S, s, e, bk, b0, A);
             else bytes += tu_bucket<F, DEL, ONE>(S, s, e, bk, b0, A.G, tsh, bsh, smask, A.blocks, A.fill, A.cap);
         }
         __syncthreads();
